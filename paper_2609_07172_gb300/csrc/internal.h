@@ -433,4 +433,11 @@ __host__ __device__ inline bool tw_rot(int t, int n) { return !(8 * t <= n || 8 
 int launch_conv3x3_tc(const void *in, int cin, const void *w, const float *bias, void *out, float *out32, int cout,
                       int n, int h, int wd, int relu, cudaStream_t st);
 
+// Weight and bias gradients of a 3x3 convolution on mma.sync (wgrad.cu):
+// whether it takes these tensors, and the two launches (at most max_parts
+// partials of 9 cin cout + cout floats in scratch).
+bool wgrad_mma_takes(const void *in, int cin, const void *dout, int cout);
+cudaError_t launch_wgrad_mma(const void *in, int cin, const void *dout, int cout, int n, int h, int wd, float *dw,
+                             float *dbias, float *scratch, int max_parts, cudaStream_t st);
+
 }  // namespace pp

@@ -122,8 +122,9 @@ __global__ void k_flip(const bf16 *__restrict__ w, bf16 *__restrict__ wt, int co
 
 constexpr int WG_CHUNK = 2048;   // pixels per weight-gradient partial
 
-// Weight and bias gradients of a 3x3 convolution, first stage: every thread
-// owns one (cout, cin) pair and sums dout[p][co] * in[p shifted][ci] over the
+// Weight and bias gradients of a 3x3 convolution whose channel counts are no
+// multiples of 8 or whose tensors are not 16-byte aligned (wgrad.cu takes the
+// others), first stage: every thread owns one (cout, cin) pair and sums dout[p][co] * in[p shifted][ci] over the
 // 9 taps for the pixels of one chunk, in FP32; partials[chunk][tap][co][ci].
 __global__ void __launch_bounds__(256)
 k_wgrad_partial(const bf16 *__restrict__ in, int cin, const bf16 *__restrict__ dout, int cout, int n, int h, int wd,
@@ -629,6 +630,10 @@ int pic_nn_conv3x3_wgrad(const void *in, int cin, const void *dout, int cout, in
         return PIC_POISSON_EINVAL;
     }
     const cudaStream_t st = (cudaStream_t)stream;
+    if (cin > 0 && cout > 0 && chunks > 0 && wgrad_mma_takes(in, cin, dout, cout)) {
+        PP_CUDA(launch_wgrad_mma(in, cin, dout, cout, n, h, wd, dw, dbias, scratch, chunks, st));
+        return PIC_POISSON_OK;
+    }
     float *part = scratch, *partb = scratch + (long)chunks * 9 * cout * cin;
     dim3 grid(chunks, (cout * cin + 255) / 256);
     k_wgrad_partial<<<grid, 256, 0, st>>>((const bf16 *)in, cin, (const bf16 *)dout, cout, n, h, wd, part, partb);
