@@ -41,6 +41,22 @@ int pic_nn_conv3x3(const void *in, int cin, const void *w, const float *bias, vo
  * cores, FP32 accumulation; any w), for comparison and as the fallback. */
 int pic_nn_conv3x3_mma_sync(const void *in, int cin, const void *w, const float *bias, void *out_bf16,
                             float *out_f32, int cout, int n, int h, int wd, int relu, void *stream);
+/*
+ * pic_nn_conv3x3 on the channel concatenation of an upsampled and a skip
+ * tensor: channels [0, cu) are `up` (BF16 [n,h/2,w/2,cu]) upsampled 2x
+ * (nearest), channels [cu, cu + cs) are `skip` (BF16 [n,h,w,cs]); h and w even.
+ * Where w is a multiple of 128 and the weights take at most 48 KB the
+ * convolution reads the two tensors as they are; elsewhere it writes the
+ * concatenation into the workspace `cat` (BF16 [n,h,w,cu+cs]) first.  Same
+ * result either way.
+ */
+int pic_nn_conv3x3_cat(const void *up, int cu, const void *skip, int cs, const void *w, const float *bias, void *cat,
+                       void *out_bf16, float *out_f32, int cout, int n, int h, int wd, int relu, void *stream);
+/* pic_nn_conv3x3 and pic_nn_pool2 of its BF16 output in one pass (two where the
+ * width or the weights rule out the tiles of two rows): pooled BF16
+ * [n,h/2,w/2,cout]; h and w even. */
+int pic_nn_conv3x3_pool(const void *in, int cin, const void *w, const float *bias, void *out_bf16, void *pooled,
+                        int cout, int n, int h, int wd, int relu, void *stream);
 /* Whether a bounded wait of the tcgen05 convolution ran out since the last
  * call: *status = 0 (none) or 1 + the role that gave up (0 TMA producer,
  * 1 MMA issuer, 2 epilogue, 3 / 4 the final drains); clears the flag.  Such a
@@ -61,6 +77,12 @@ size_t pic_nn_wgrad_scratch_floats(int cin, int cout, int n, int h, int wd);
  */
 int pic_nn_conv3x3_wgrad(const void *in, int cin, const void *dout, int cout, int n, int h, int wd, float *dw,
                          float *dbias, float *scratch, size_t scratch_floats, void *stream);
+
+/* The gradients of pic_nn_conv3x3_cat (scratch as for cin = cu + cs): cu, cs
+ * and cout multiples of 8, tensors 16-byte aligned. */
+int pic_nn_conv3x3_wgrad_cat(const void *up, int cu, const void *skip, int cs, const void *dout, int cout, int n,
+                             int h, int wd, float *dw, float *dbias, float *scratch, size_t scratch_floats,
+                             void *stream);
 
 /* dy = 0 where y <= 0 (ReLU backward, in place on dy; count elements). */
 int pic_nn_relu_bwd(const void *y, void *dy, long count, void *stream);

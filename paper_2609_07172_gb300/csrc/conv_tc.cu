@@ -61,8 +61,10 @@ struct ConvTCArgs {
     float *out32;
     int relu;
     int stages;                      // ring slots in use (<= TC_MAX_STAGES)
-    // halo variant (k_conv3x3_tc_halo): no-swizzle K-major operands
-    unsigned lbo_a;                  // bytes from one 8-channel group of the halo tile to the next
+    // halo variant (k_conv3x3_tc_halo): no-swizzle K-major weights
+    const bf16 *up;                  // CAT: channels [0, cu), of half the height and width
+    int cu;
+    bf16 *pool;                      // 2x2 averages of the output, or null
     unsigned lbo_b;                  // bytes from one 8-channel group of a tap's weights to the next
     unsigned w_bytes;                // all nine taps' weights (resident)
 };
@@ -131,18 +133,41 @@ __device__ __forceinline__ uint64_t smem_desc(unsigned addr, unsigned sbo, unsig
            ((uint64_t)1 << 46) | ((uint64_t)swz << 61);
 }
 
-__device__ __forceinline__ void umma_bf16(unsigned tmem_d, uint64_t a, uint64_t b, unsigned idesc, unsigned acc) {
+// One MMA, D (+)= A B, issued by the whole warp under a predicate (one lane's
+// `one` is 1), the descriptors' halves apart: the upper words are constants of
+// the kernel, the lower ones (start address >> 4) an addition per MMA.  Nothing
+// diverges, so the operands stay in uniform registers -- an MMA issued inside a
+// one-lane branch, its descriptors rebuilt from scratch, took about 360 cycles
+// of the issuing thread and bound the halo kernel (see below).
+__device__ __forceinline__ void umma_bf16_lo(unsigned tmem_d, unsigned alo, unsigned ahi, unsigned blo, unsigned bhi,
+                                             unsigned idesc, unsigned acc, unsigned one) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "setp.ne.b32 q, %7, 0;\n\t"
+        "mov.b64 da, {%1, %2};\n\t"
+        "mov.b64 db, {%3, %4};\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}" ::"r"(tmem_d),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc), "r"(one)
         : "memory");
 }
-// Arrive on `bar` once every MMA this thread issued before has completed.
-__device__ __forceinline__ void umma_commit(unsigned bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-                 : "memory");
+__device__ __forceinline__ unsigned elect_one() {
+    unsigned one;
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "elect.sync _|q, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(one));
+    return one;
+}
+// Arrive on `bar` once every MMA the elected lane issued before has completed.
+__device__ __forceinline__ void umma_commit_one(unsigned bar, unsigned one) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ne.b32 q, %1, 0;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar),
+        "r"(one)
+        : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -164,6 +189,11 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, float (&v)[16]) {
 __device__ __forceinline__ unsigned pack2(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<unsigned *>(&v);
+}
+
+// The two values of a packed BF16 pair.
+__device__ __forceinline__ float2 bf2(unsigned w) {
+    return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
 
 __device__ __forceinline__ void tile_origin(const ConvTCArgs &a, int tile, int &nn, int &x0, int &y0) {
@@ -252,38 +282,38 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
                 if (!mbar_wait(full0 + 8 * (j % S), (j / S) & 1u, never)) give_up(abort, 3);
         }
     } else if (warp == 5) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
-            unsigned it = 0, tc = 0;
-            bool ok = true;
-            for (int tile = blockIdx.x; ok && tile < a.tiles; tile += gridDim.x, ++tc) {
-                const unsigned buf = tc & 1u, u = tc >> 1;
-                if (!mbar_wait(tempty0 + 8 * buf, (u & 1u) ^ 1u, abort)) {
+        // ---------------- MMA issuer (the whole warp; one lane's MMAs and commits take effect)
+        const unsigned one = elect_one();
+        unsigned it = 0, tc = 0;
+        bool ok = true;
+        for (int tile = blockIdx.x; ok && tile < a.tiles; tile += gridDim.x, ++tc) {
+            const unsigned buf = tc & 1u, u = tc >> 1;
+            if (!mbar_wait(tempty0 + 8 * buf, (u & 1u) ^ 1u, abort)) {
+                give_up(abort, 1);
+                break;
+            }
+            tc_fence_after();
+            const unsigned d = tmem + buf * a.tmem_cols;
+            for (int k = 0; k < kiters; ++k, ++it) {
+                const unsigned s = it % S, us = it / S;
+                if (!mbar_wait(full0 + 8 * s, us & 1u, abort)) {
                     give_up(abort, 1);
+                    ok = false;
                     break;
                 }
                 tc_fence_after();
-                const unsigned d = tmem + buf * a.tmem_cols;
-                for (int k = 0; k < kiters; ++k, ++it) {
-                    const unsigned s = it % S, us = it / S;
-                    if (!mbar_wait(full0 + 8 * s, us & 1u, abort)) {
-                        give_up(abort, 1);
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const unsigned sa = stage0 + s * a.stage_bytes, sb = sa + a.a_bytes;
-                    for (int kk = 0; kk < a.kc / 16; ++kk)   // K = 16 BF16 = 32 bytes per MMA
-                        umma_bf16(d, smem_desc(sa + 32u * kk, a.sbo, a.swz), smem_desc(sb + 32u * kk, a.sbo, a.swz),
-                                  a.idesc, (k | kk) != 0 ? 1u : 0u);
-                    umma_commit(empty0 + 8 * s);   // the stage is free once these MMAs have read it
-                }
-                if (!ok) break;
-                umma_commit(tfull0 + 8 * buf);     // the tile's accumulator is complete
+                const unsigned sa = stage0 + s * a.stage_bytes;
+                const uint64_t da = smem_desc(sa, a.sbo, a.swz), db = smem_desc(sa + a.a_bytes, a.sbo, a.swz);
+                for (int kk = 0; kk < a.kc / 16; ++kk)   // K = 16 BF16 = 32 bytes per MMA
+                    umma_bf16_lo(d, (unsigned)da + 2u * kk, (unsigned)(da >> 32), (unsigned)db + 2u * kk,
+                                 (unsigned)(db >> 32), a.idesc, (k | kk) != 0 ? 1u : 0u, one);
+                umma_commit_one(empty0 + 8 * s, one);   // the stage is free once these MMAs have read it
             }
-            umma_commit(drain);
-            if (!mbar_wait(drain, 0, never)) give_up(abort, 4);
+            if (!ok) break;
+            umma_commit_one(tfull0 + 8 * buf, one);     // the tile's accumulator is complete
         }
+        umma_commit_one(drain, one);
+        if (!mbar_wait(drain, 0, never)) give_up(abort, 4);
     } else {
         // ---------------- epilogue: warp w drains TMEM lanes 32 w .. 32 w + 31
         const int row = threadIdx.x;   // pixel of the tile = TMEM lane
@@ -334,15 +364,43 @@ k_conv3x3_tc(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
     }
 }
 
-// Halo variant for image rows of 128 pixels or more (tiles of one row) and
-// small weight sets (the full- and half-resolution layers, which are bound by
-// data movement): per tile and chunk of KC channels, TMA brings the three input
-// rows y - 1 .. y + 1 over pixels x0 - 1 .. x0 + 128 once, as 8-channel groups
-// of 390 16-byte rows (no swizzle, K-major core matrices); the nine taps are
-// the same buffer seen from nine start rows, (1 + dy) * 130 + 1 + dx.  All
-// nine taps' weights stay resident from the CTA's start.  A tile then moves
-// 3 * 130 * cin instead of 9 * 128 * cin input values.
-__global__ void __launch_bounds__(TC_THREADS, 1)
+// Halo variant for image rows of 128 pixels or more and small weight sets (the
+// full- and half-resolution layers, which are bound by data movement).  A tile
+// is 128 pixels of two rows; per chunk of KC channels the four input rows
+// y - 1 .. y + 2 over pixels x0 - 1 .. x0 + 128 are staged once, one row of KC
+// channels per pixel (32- or 64-byte swizzle), and the nine taps of an output
+// row are the same buffer seen from nine start rows, (r + 1 + dy) * 130 + 1 +
+// dx: the swizzle is a function of the address bits, so a descriptor may start
+// at any pixel of a buffer aligned to the pattern.  All nine taps' weights stay
+// resident from the CTA's start.  A tile row then moves 2 * 130 * cin instead
+// of 9 * 128 * cin input values.
+//
+// What bounded it before (clock64 in the roles): the MMA thread, which built
+// two 64-bit descriptors per MMA inside a one-lane branch, about 360 cycles
+// each with 9 to 18 per row; and the TMA engine, one request per staged row of
+// 8 channels (780 to 1560 per output row at about 1.5 cycles).  65 samples of
+// 200 x 256: 16 -> 16 channels 114 us, 32 -> 16 169 us.  With uniform issue
+// (umma_bf16_lo), whole-pixel rows and two output rows per tile 60 and 77 us
+// (three and two CTAs per SM).  What is left: an MMA of N = 16 costs the 32
+// cycles of reading its 128 x 16 A operand (24 and 48 us), the staged rows about
+// 1.5 cycles each, the bytes 31 and 47 us.
+//
+// CAT: the input is two tensors, channels [0, cu) from `up`, an image of half
+// the height and width upsampled 2x (nearest), the others from `in` -- the
+// decoder's concatenation, which is never written.  Four expander warps load
+// up's pixels into registers a stage ahead and write each to the two pixels (and
+// rows) it covers (32 -> 16 channels on 65 x 200 x 256: 73 us, against 169 for
+// the convolution and 265 for writing the concatenation before).  MIX: a chunk holds 16 channels of each, in two buffers of
+// 32-byte rows (KC = 32); otherwise a chunk lies in one tensor.
+//
+// pool: the 2x2 averages of the (BF16) output, from the two rows of the tile.
+constexpr int TH_WX = TC_M + 2;                // pixels of a staged row
+constexpr int TH_ROWS = 4 * TH_WX;             // staged pixels
+constexpr int TH_EXPAND = 128;                 // expander threads (CAT)
+constexpr int TH_UPIX = 3 * (TC_M / 2 + 2);    // up's pixels under a tile
+
+template <int KC, bool CAT, bool MIX>
+__global__ void __launch_bounds__(TC_THREADS + (CAT ? TH_EXPAND : 0), 1)
 k_conv3x3_tc_halo(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, const ConvTCArgs a) {
     extern __shared__ __align__(1024) unsigned char dsm[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -361,12 +419,12 @@ k_conv3x3_tc_halo(const __grid_constant__ CUtensorMap ta, const __grid_constant_
     unsigned *tmem_slot = reinterpret_cast<unsigned *>(tail + 8 * (2 * TC_MAX_STAGES + 6));
     volatile int *abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
     volatile int *never = reinterpret_cast<volatile int *>(tmem_slot + 2);
-    const unsigned ncols = 2 * a.tmem_cols;
-    const int groups = a.kc / 8;                 // 8-channel groups per chunk
-    const int cgroups = a.cin / 8;               // per tap of the weights
+    float *bias = reinterpret_cast<float *>(tmem_slot + 4);           // [cout], zeros without a bias
+    const unsigned ncols = 4 * a.tmem_cols;      // two sets of two accumulators (the tile's rows)
+    const int cgroups = a.cin / 8;               // 8-channel groups per tap of the weights
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
-            mbar_init(full0 + 8 * s, 1);
+            mbar_init(full0 + 8 * s, CAT ? 1 + TH_EXPAND : 1);
             mbar_init(empty0 + 8 * s, 1);
         }
         for (int b = 0; b < 2; ++b) {
@@ -379,6 +437,7 @@ k_conv3x3_tc_halo(const __grid_constant__ CUtensorMap ta, const __grid_constant_
         *never = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    for (int c = threadIdx.x; c < a.cout; c += blockDim.x) bias[c] = a.bias ? a.bias[c] : 0.f;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(ncols)
@@ -410,10 +469,13 @@ k_conv3x3_tc_halo(const __grid_constant__ CUtensorMap ta, const __grid_constant_
                         break;
                     }
                     const unsigned sa = stage0 + s * a.stage_bytes;
+                    if (CAT && !MIX && c * KC < a.cu) {   // this chunk comes from the expanders alone
+                        mbar_arrive(full0 + 8 * s);
+                        continue;
+                    }
                     mbar_expect_tx(full0 + 8 * s, a.a_bytes);
-                    for (int g = 0; g < groups; ++g)
-                        tma_load_4d(sa + (unsigned)g * a.lbo_a, &ta, c * a.kc + 8 * g, x0 - 1, y0 - 1, nn,
-                                    full0 + 8 * s);
+                    tma_load_4d(MIX ? sa + a.stage_bytes / 2 : sa, &ta, MIX ? 0 : c * KC - a.cu, x0 - 1, y0 - 1, nn,
+                                full0 + 8 * s);
                 }
             }
             const unsigned first = it > (unsigned)S ? it - S : 0u;
@@ -422,83 +484,177 @@ k_conv3x3_tc_halo(const __grid_constant__ CUtensorMap ta, const __grid_constant_
             if (!mbar_wait(wbar, 0, never)) give_up(abort, 3);
         }
     } else if (warp == 5) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
-            unsigned it = 0, tc = 0;
-            bool ok = mbar_wait(wbar, 0, abort);
-            if (!ok) give_up(abort, 1);
+        // ---------------- MMA issuer (the whole warp; one lane's MMAs and commits take effect)
+        const unsigned one = elect_one();
+        unsigned it = 0, tc = 0;
+        bool ok = mbar_wait(wbar, 0, abort);
+        if (!ok) give_up(abort, 1);
+        tc_fence_after();
+        for (int tile = blockIdx.x; ok && tile < a.tiles; tile += gridDim.x, ++tc) {
+            const unsigned buf = tc & 1u, u = tc >> 1;
+            if (!mbar_wait(tempty0 + 8 * buf, (u & 1u) ^ 1u, abort)) {
+                give_up(abort, 1);
+                break;
+            }
             tc_fence_after();
-            for (int tile = blockIdx.x; ok && tile < a.tiles; tile += gridDim.x, ++tc) {
-                const unsigned buf = tc & 1u, u = tc >> 1;
-                if (!mbar_wait(tempty0 + 8 * buf, (u & 1u) ^ 1u, abort)) {
+            const unsigned d = tmem + 2u * buf * a.tmem_cols;
+            for (int c = 0; c < a.nchunks; ++c, ++it) {
+                const unsigned s = it % S, us = it / S;
+                if (!mbar_wait(full0 + 8 * s, us & 1u, abort)) {
                     give_up(abort, 1);
+                    ok = false;
                     break;
                 }
                 tc_fence_after();
-                const unsigned d = tmem + buf * a.tmem_cols;
-                for (int c = 0; c < a.nchunks; ++c, ++it) {
-                    const unsigned s = it % S, us = it / S;
-                    if (!mbar_wait(full0 + 8 * s, us & 1u, abort)) {
-                        give_up(abort, 1);
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const unsigned sa = stage0 + s * a.stage_bytes;
-                    for (int tap = 0; tap < 9; ++tap) {
-                        const unsigned row0 = (unsigned)((tap / 3) * (a.bx + 2) + tap % 3);   // (1 + dy) W' + 1 + dx
-                        for (int kk = 0; kk < a.kc / 16; ++kk) {   // K = 16: two 8-channel groups
-                            const unsigned adr = sa + 2u * kk * a.lbo_a + 16u * row0;
-                            const unsigned bdr = wbase + (unsigned)(tap * cgroups + c * groups + 2 * kk) * a.lbo_b;
-                            umma_bf16(d, smem_desc_plain(adr, a.lbo_a), smem_desc_plain(bdr, a.lbo_b), a.idesc,
-                                      (c | tap | kk) != 0 ? 1u : 0u);
-                        }
-                    }
-                    umma_commit(empty0 + 8 * s);
+                const unsigned sa = stage0 + s * a.stage_bytes;
+                constexpr int ROW = MIX ? 32 : KC * 2;                       // bytes of a staged pixel
+                const unsigned kstep = MIX ? a.stage_bytes / 2 >> 4 : 2u;    // the next 16 channels, 16-byte units
+                const uint64_t da = smem_desc(sa, a.sbo, a.swz), db = smem_desc_plain(wbase, a.lbo_b);
+                const unsigned alo = (unsigned)da, ahi = (unsigned)(da >> 32), bhi = (unsigned)(db >> 32);
+                const unsigned bstep = 2u * a.lbo_b >> 4, btap = (unsigned)cgroups * a.lbo_b >> 4;
+#pragma unroll 1
+                for (int r = 0; r < 2; ++r) {
+                    const unsigned ar = alo + (unsigned)r * (TH_WX * ROW / 16), dr = d + (unsigned)r * a.tmem_cols;
+                    unsigned blo = (unsigned)db + (unsigned)c * (KC / 16) * bstep;
+#pragma unroll
+                    for (int tap = 0; tap < 9; ++tap, blo += btap)
+#pragma unroll
+                        for (int kk = 0; kk < KC / 16; ++kk)   // K = 16 BF16 = 32 bytes per MMA
+                            umma_bf16_lo(dr, ar + ((tap / 3) * TH_WX + tap % 3) * (ROW / 16) + kk * kstep, ahi,
+                                         blo + kk * bstep, bhi, a.idesc, (c | tap | kk) != 0 ? 1u : 0u, one);
                 }
-                if (!ok) break;
-                umma_commit(tfull0 + 8 * buf);
+                umma_commit_one(empty0 + 8 * s, one);
             }
-            umma_commit(drain);
-            if (!mbar_wait(drain, 0, never)) give_up(abort, 4);
+            if (!ok) break;
+            umma_commit_one(tfull0 + 8 * buf, one);
         }
-    } else {
-        // ---------------- epilogue (as in k_conv3x3_tc; tiles are one row)
+        umma_commit_one(drain, one);
+        if (!mbar_wait(drain, 0, never)) give_up(abort, 4);
+    } else if (warp < 4) {
+        // ---------------- epilogue: warp w drains TMEM lanes 32 w .. 32 w + 31 (pixels) of the tile's two rows
         const int row = threadIdx.x;
         unsigned tc = 0;
         for (int tile = blockIdx.x; tile < a.tiles; tile += gridDim.x, ++tc) {
             const unsigned buf = tc & 1u, u = tc >> 1;
+            int nn, x0, y0;
+            tile_origin(a, tile, nn, x0, y0);
+            const size_t p = ((size_t)nn * a.h + y0) * a.wd + x0 + row;
+            const size_t pp = (((size_t)nn * (a.h >> 1) + (y0 >> 1)) * a.wd + x0 + row) >> 1;
             if (!mbar_wait(tfull0 + 8 * buf, u & 1u, abort)) {
                 give_up(abort, 2);
                 break;
             }
             tc_fence_after();
-            int nn, x0, y0;
-            tile_origin(a, tile, nn, x0, y0);
-            const size_t p = ((size_t)nn * a.h + y0) * a.wd + x0 + row;
-            const unsigned taddr = tmem + buf * a.tmem_cols + ((unsigned)(warp * 32) << 16);
+            const unsigned taddr = tmem + 2u * buf * a.tmem_cols + ((unsigned)(warp * 32) << 16);
             for (int c = 0; c < a.cout; c += 16) {
-                float v[16];
-                tmem_ld16(taddr + (unsigned)c, v);
+                unsigned q[2][8];
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    float t = v[e] + (a.bias ? a.bias[c + e] : 0.f);
-                    v[e] = a.relu ? fmaxf(t, 0.f) : t;
-                }
-                if (a.out) {
-                    uint4 *o = reinterpret_cast<uint4 *>(a.out + p * a.cout + c);
-                    o[0] = make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
-                    o[1] = make_uint4(pack2(v[8], v[9]), pack2(v[10], v[11]), pack2(v[12], v[13]),
-                                      pack2(v[14], v[15]));
-                }
-                if (a.out32) {
-                    float4 *o = reinterpret_cast<float4 *>(a.out32 + p * a.cout + c);
+                for (int r = 0; r < 2; ++r) {
+                    float v[16];
+                    tmem_ld16(taddr + (unsigned)r * a.tmem_cols + (unsigned)c, v);
+                    const bool valid = y0 + r < a.h;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                    for (int e = 0; e < 16; e += 4) {
+                        const float4 b = *reinterpret_cast<const float4 *>(bias + c + e);
+                        v[e] += b.x, v[e + 1] += b.y, v[e + 2] += b.z, v[e + 3] += b.w;
+                    }
+                    if (a.relu)
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) v[e] = fmaxf(v[e], 0.f);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) q[r][e] = pack2(v[2 * e], v[2 * e + 1]);
+                    const size_t o = (p + (size_t)r * a.wd) * a.cout + c;
+                    if (a.out && valid) {
+                        uint4 *w = reinterpret_cast<uint4 *>(a.out + o);
+                        w[0] = make_uint4(q[r][0], q[r][1], q[r][2], q[r][3]);
+                        w[1] = make_uint4(q[r][4], q[r][5], q[r][6], q[r][7]);
+                    }
+                    if (a.out32 && valid) {
+                        float4 *w = reinterpret_cast<float4 *>(a.out32 + o);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) w[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+                    }
+                }
+                if (a.pool) {   // (h even) this pixel and its right neighbour, both rows; even lanes store
+                    unsigned m[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const unsigned n0 = __shfl_down_sync(0xffffffffu, q[0][e], 1);
+                        const unsigned n1 = __shfl_down_sync(0xffffffffu, q[1][e], 1);
+                        const float2 f0 = bf2(q[0][e]), g0 = bf2(n0), f1 = bf2(q[1][e]), g1 = bf2(n1);
+                        m[e] = pack2(0.25f * (f0.x + g0.x + f1.x + g1.x), 0.25f * (f0.y + g0.y + f1.y + g1.y));
+                    }
+                    if ((lane & 1) == 0) {
+                        uint4 *w = reinterpret_cast<uint4 *>(a.pool + pp * a.cout + c);
+                        w[0] = make_uint4(m[0], m[1], m[2], m[3]);
+                        w[1] = make_uint4(m[4], m[5], m[6], m[7]);
+                    }
                 }
             }
             tc_fence_before();
             mbar_arrive(tempty0 + 8 * buf);
+        }
+    } else if (CAT) {
+        // ---------------- expanders: up's channels of a chunk, each pixel to the pixels and rows it covers
+        const int t = (int)threadIdx.x - TC_THREADS;
+        constexpr int G = (MIX ? 16 : KC) / 8;                        // 16-byte groups of a pixel
+        constexpr int NP = (TH_UPIX * G + TH_EXPAND - 1) / TH_EXPAND;  // pieces per thread
+        constexpr int UW = TC_M / 2 + 2;
+        constexpr int ROW = 16 * G;
+        const int uw = a.wd >> 1, uh = a.h >> 1;
+        uint4 v[NP];
+        auto load = [&](int tile, int c) {
+            int nn, x0, y0;
+            tile_origin(a, tile, nn, x0, y0);
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+                const int e = t + j * TH_EXPAND, g = e % G, px = e / G;
+                const int sy = px / UW, y = (y0 >> 1) - 1 + sy, x = (x0 >> 1) - 1 + (px - sy * UW);
+                v[j] = make_uint4(0u, 0u, 0u, 0u);
+                if (px < TH_UPIX && (unsigned)y < (unsigned)uh && (unsigned)x < (unsigned)uw)
+                    v[j] = __ldg(reinterpret_cast<const uint4 *>(
+                        a.up + (((size_t)nn * uh + y) * uw + x) * a.cu + (MIX ? 0 : c * KC) + 8 * g));
+            }
+        };
+        unsigned it = 0;
+        bool ok = true;
+        if ((int)blockIdx.x < a.tiles) load(blockIdx.x, 0);
+        for (int tile = blockIdx.x; ok && tile < a.tiles; tile += gridDim.x) {
+            for (int c = 0; c < a.nchunks; ++c, ++it) {
+                const unsigned s = it % S, u = it / S;
+                if (!mbar_wait(empty0 + 8 * s, (u & 1u) ^ 1u, abort)) {
+                    give_up(abort, 0);
+                    ok = false;
+                    break;
+                }
+                if (MIX || c * KC < a.cu) {
+                    const unsigned sa = stage0 + s * a.stage_bytes;
+#pragma unroll
+                    for (int j = 0; j < NP; ++j) {
+                        const int e = t + j * TH_EXPAND, g = e % G, px = e / G;
+                        const int sy = px / UW, sx = px - sy * UW;
+                        if (px >= TH_UPIX) continue;
+#pragma unroll
+                        for (int d = 0; d < 4; ++d) {
+                            // staged rows of up's row sy: 0; 1, 2; 3 -- staged pixels of column sx: 2 sx - 1, 2 sx
+                            const int r = sy == 0 ? 0 : (sy == 2 ? 3 : 1 + (d >> 1)), q = 2 * sx - 1 + (d & 1);
+                            if ((d >> 1 && sy != 1) || q < 0 || q >= TH_WX) continue;
+                            const unsigned pix = (unsigned)(r * TH_WX + q);
+                            const unsigned sw = ROW == 32 ? (pix >> 2) & 1u : (pix >> 1) & 3u;   // swizzled 16-byte group
+                            const unsigned at = sa + pix * ROW + (((unsigned)g ^ sw) << 4);
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(v[j].x), "r"(v[j].y),
+                                         "r"(v[j].z), "r"(v[j].w)
+                                         : "memory");
+                        }
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // to the MMA's proxy
+                }
+                mbar_arrive(full0 + 8 * s);
+                // the next chunk's pixels, in flight while the stage is used
+                int c1 = c + 1, t1 = tile;
+                if (c1 == a.nchunks) c1 = 0, t1 += gridDim.x;
+                if (t1 < a.tiles && (MIX || c1 * KC < a.cu)) load(t1, c1);
+            }
         }
     }
     tc_fence_before();
@@ -547,11 +703,17 @@ namespace {
 struct TCDeviceInfo {
     bool valid = false;
     int sms = 0, smem_sm = 0;
-    int regs[2] = {0, 0};   // k_conv3x3_tc, k_conv3x3_tc_halo
+    int regs[5] = {0, 0, 0, 0, 0};   // kTCKernels
 };
 TCDeviceInfo g_tc_info[64];
+// the generic variant, then the halo variants of 16 and 32 channels per chunk,
+// of two inputs, and of two inputs mixed in a chunk
+const void *const kTCKernels[5] = {
+    (const void *)k_conv3x3_tc, (const void *)k_conv3x3_tc_halo<16, false, false>,
+    (const void *)k_conv3x3_tc_halo<32, false, false>, (const void *)k_conv3x3_tc_halo<32, true, false>,
+    (const void *)k_conv3x3_tc_halo<32, true, true>};
 
-int conv_tc_occupancy(int which, size_t smem, unsigned tmem_cols_per_cta, int *grid_cap) {
+int conv_tc_occupancy(int which, int threads, size_t smem, unsigned tmem_cols_per_cta, int *grid_cap) {
     int dev = 0;
     PP_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) {
@@ -566,19 +728,19 @@ int conv_tc_occupancy(int which, size_t smem, unsigned tmem_cols_per_cta, int *g
     if (!info.valid) {
         PP_CUDA(cudaDeviceGetAttribute(&info.sms, cudaDevAttrMultiProcessorCount, dev));
         PP_CUDA(cudaDeviceGetAttribute(&info.smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
-        cudaFuncAttributes fa;
-        PP_CUDA(cudaFuncGetAttributes(&fa, (const void *)k_conv3x3_tc));
-        info.regs[0] = fa.numRegs;
-        PP_CUDA(cudaFuncGetAttributes(&fa, (const void *)k_conv3x3_tc_halo));
-        info.regs[1] = fa.numRegs;
+        for (int k = 0; k < 5; ++k) {
+            cudaFuncAttributes fa;
+            PP_CUDA(cudaFuncGetAttributes(&fa, kTCKernels[k]));
+            info.regs[k] = fa.numRegs;
+        }
         info.valid = true;
         std::lock_guard<std::mutex> lock(g_tc_mutex);
         g_tc_info[dev] = info;
     }
     // CTAs per SM: shared memory (1 KB reserved per CTA), registers, threads,
     // and tensor memory (512 columns per SM: no CTA waits for an allocation)
-    const int regs = std::max(1, (info.regs[which] + 7) & ~7) * TC_THREADS;
-    const int occ = std::min({(int)(info.smem_sm / (smem + 1024)), 65536 / regs, 2048 / TC_THREADS, 32,
+    const int regs = std::max(1, (info.regs[which] + 7) & ~7) * threads;
+    const int occ = std::min({(int)(info.smem_sm / (smem + 1024)), 65536 / regs, 2048 / threads, 32,
                               (int)(512u / tmem_cols_per_cta)});
     *grid_cap = info.sms * std::max(1, occ);
     return PIC_POISSON_OK;
@@ -596,28 +758,37 @@ int set_smem(const void *kernel, size_t smem) {
     return PIC_POISSON_OK;
 }
 
-// The halo variant's operands: no-swizzle 4-D boxes of 8 channels x 130
-// pixels x 3 rows of the input, 3-D boxes of 8 channels x cout of each tap's
-// weights.
+// The halo variant's operands: swizzled 4-D boxes of a chunk's channels x 130
+// pixels x 4 rows of the input, no-swizzle 3-D boxes of 8 channels x cout of
+// each tap's weights.  1 when two inputs do not split into its chunks.
 int launch_halo(ConvTCArgs a, const void *in, const void *w, EncodeTiledFn enc, cudaStream_t st) {
     a.kc = a.cin % 32 == 0 ? 32 : 16;
     a.nchunks = a.cin / a.kc;
-    const unsigned groups = (unsigned)a.kc / 8, rows = 3u * (unsigned)(a.bx + 2);
-    a.lbo_a = (rows * 16u + 127u) & ~127u;           // 128-byte aligned TMA destinations
-    a.a_bytes = groups * rows * 16u;                  // TMA bytes of one chunk
-    a.stage_bytes = (groups * a.lbo_a + 1023u) & ~1023u;
+    const bool cat = a.up != nullptr, mix = cat && a.cin == 32 && a.cu == 16;
+    if (cat && !mix && (a.kc != 32 || a.cu % 32)) return 1;
+    const int which = mix ? 4 : (cat ? 3 : (a.kc == 32 ? 2 : 1));
+    const int tma_kc = mix ? 16 : a.kc;               // channels of a TMA box
+    a.by = 2;
+    a.tiles_y = (a.h + 1) / 2;
+    const long tiles = (long)a.n * a.tiles_y * a.tiles_x;
+    a.tiles = (int)tiles;
+    a.a_bytes = (unsigned)(TH_ROWS * tma_kc * 2);      // TMA bytes of one chunk
+    const unsigned buf_bytes = (a.a_bytes + 1023u) & ~1023u;
+    a.stage_bytes = mix ? 2 * buf_bytes : buf_bytes;
+    a.swz = tma_kc == 32 ? 4u : 6u;                   // 64- or 32-byte pixel rows
+    a.sbo = 8u * (unsigned)(tma_kc * 2);
     a.lbo_b = (unsigned)a.cout * 16u;
     a.w_bytes = 9u * (unsigned)a.cout * (unsigned)a.cin * 2u;
     a.stages = a.kc == 16 ? 4 : 3;
     CUtensorMap ta, tb;
-    const cuuint64_t gdim_a[4] = {(cuuint64_t)a.cin, (cuuint64_t)a.wd, (cuuint64_t)a.h, (cuuint64_t)a.n};
-    const cuuint64_t gstr_a[3] = {(cuuint64_t)a.cin * 2, (cuuint64_t)a.cin * 2 * a.wd,
-                                  (cuuint64_t)a.cin * 2 * a.wd * a.h};
-    const cuuint32_t box_a[4] = {8, (cuuint32_t)(a.bx + 2), 3, 1};
+    const int cs = a.cin - a.cu;
+    const cuuint64_t gdim_a[4] = {(cuuint64_t)cs, (cuuint64_t)a.wd, (cuuint64_t)a.h, (cuuint64_t)a.n};
+    const cuuint64_t gstr_a[3] = {(cuuint64_t)cs * 2, (cuuint64_t)cs * 2 * a.wd, (cuuint64_t)cs * 2 * a.wd * a.h};
+    const cuuint32_t box_a[4] = {(cuuint32_t)tma_kc, (cuuint32_t)TH_WX, 4, 1};
     const cuuint32_t one[4] = {1, 1, 1, 1};
     if (enc(&ta, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(in), gdim_a, gstr_a, box_a, one,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            CU_TENSOR_MAP_INTERLEAVE_NONE, tma_kc == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return 1;
     const cuuint64_t gdim_b[3] = {(cuuint64_t)a.cin, (cuuint64_t)a.cout, 9};
     const cuuint64_t gstr_b[2] = {(cuuint64_t)a.cin * 2, (cuuint64_t)a.cin * 2 * a.cout};
@@ -627,13 +798,20 @@ int launch_halo(ConvTCArgs a, const void *in, const void *w, EncodeTiledFn enc, 
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return 1;
     const size_t smem = 1024 + ((a.w_bytes + 1023u) & ~1023u) + (size_t)a.stages * a.stage_bytes +
-                        8 * (2 * TC_MAX_STAGES + 6) + 16;
-    int rc = set_smem((const void *)k_conv3x3_tc_halo, smem);
+                        8 * (2 * TC_MAX_STAGES + 6) + 16 + 128 * sizeof(float);
+    int rc = set_smem(kTCKernels[which], smem);
     if (rc) return rc;
+    const int threads = TC_THREADS + (cat ? TH_EXPAND : 0);
     int cap = 0;
-    rc = conv_tc_occupancy(1, smem, 2u * a.tmem_cols, &cap);
+    rc = conv_tc_occupancy(which, threads, smem, 4u * a.tmem_cols, &cap);
     if (rc) return rc;
-    k_conv3x3_tc_halo<<<std::min(a.tiles, cap), TC_THREADS, smem, st>>>(ta, tb, a);
+    const int grid = std::min(a.tiles, cap);
+    switch (which) {
+    case 1: k_conv3x3_tc_halo<16, false, false><<<grid, threads, smem, st>>>(ta, tb, a); break;
+    case 2: k_conv3x3_tc_halo<32, false, false><<<grid, threads, smem, st>>>(ta, tb, a); break;
+    case 3: k_conv3x3_tc_halo<32, true, false><<<grid, threads, smem, st>>>(ta, tb, a); break;
+    default: k_conv3x3_tc_halo<32, true, true><<<grid, threads, smem, st>>>(ta, tb, a); break;
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_error("conv3x3 (tcgen05, halo) launch failed: %s", cudaGetErrorString(e));
@@ -657,12 +835,19 @@ int conv_tc_tile_x(int wd) {
 // runs the mma.sync kernel): cout a multiple of 16 up to 128, cin a multiple of
 // 16, a tileable width, 16-byte aligned tensors and the driver's tensor-map
 // encoder available.  0 on success, a PIC_POISSON_* error otherwise.
-int launch_conv3x3_tc(const void *in, int cin, const void *w, const float *bias, void *out, float *out32, int cout,
-                      int n, int h, int wd, int relu, cudaStream_t st) {
+// up: the first cu of the cin channels come from it (half the height and
+// width, upsampled 2x), the others from in; pool: also the 2x2 averages of the
+// output.  Only the halo variant takes these (1 otherwise).
+int launch_conv3x3_tc(const void *up, int cu, const void *in, int cin, const void *w, const float *bias, void *out,
+                      float *out32, void *pool, int cout, int n, int h, int wd, int relu, cudaStream_t st) {
     const int bx = conv_tc_tile_x(wd);
     if (!bx || cout % 16 || cout > 128 || cin % 16 || ((uintptr_t)in & 15) || ((uintptr_t)w & 15) ||
-        ((uintptr_t)out & 15) || ((uintptr_t)out32 & 15))
+        ((uintptr_t)out & 15) || ((uintptr_t)out32 & 15) || ((uintptr_t)up & 15) || ((uintptr_t)pool & 15))
         return 1;
+    // halo variant: rows of 128 pixels and weights small enough to stay resident
+    const unsigned w_all = 9u * (unsigned)cout * (unsigned)cin * 2u;
+    const bool halo = bx == TC_M && w_all <= 48u * 1024u;
+    if ((up || pool) && (!halo || h % 2)) return 1;
     EncodeTiledFn enc = encoder();
     if (!enc) return 1;
     ConvTCArgs a{};
@@ -695,9 +880,10 @@ int launch_conv3x3_tc(const void *in, int cin, const void *w, const float *bias,
     a.out = (bf16 *)out;
     a.out32 = out32;
     a.relu = relu;
-    // halo variant: one-row tiles and weights small enough to stay resident
-    const unsigned w_all = 9u * (unsigned)cout * (unsigned)cin * 2u;
-    if (a.by == 1 && w_all <= 48u * 1024u) return launch_halo(a, in, w, enc, st);
+    a.up = (const bf16 *)up;
+    a.cu = up ? cu : 0;
+    a.pool = (bf16 *)pool;
+    if (halo) return launch_halo(a, in, w, enc, st);
     const CUtensorMapSwizzle sw = a.kc == 64 ? CU_TENSOR_MAP_SWIZZLE_128B
                                              : (a.kc == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
     // activations: (c, x, y, n), zero fill outside
@@ -723,7 +909,7 @@ int launch_conv3x3_tc(const void *in, int cin, const void *w, const float *bias,
     int rc = set_smem((const void *)k_conv3x3_tc, smem);
     if (rc) return rc;
     int cap = 0;
-    rc = conv_tc_occupancy(0, smem, 2u * a.tmem_cols, &cap);
+    rc = conv_tc_occupancy(0, TC_THREADS, smem, 2u * a.tmem_cols, &cap);
     if (rc) return rc;
     const int grid = std::min(a.tiles, cap);
     k_conv3x3_tc<<<grid, TC_THREADS, smem, st>>>(ta, tb, a);

@@ -429,15 +429,17 @@ __host__ __device__ inline bool tw_rot(int t, int n) { return !(8 * t <= n || 8 
 
 // 3x3 convolution on the tcgen05 tensor cores (conv_tc.cu): 0 on success, 1
 // when the shape or alignment is not taken (run the mma.sync kernel), else a
-// PIC_POISSON_* error.
-int launch_conv3x3_tc(const void *in, int cin, const void *w, const float *bias, void *out, float *out32, int cout,
-                      int n, int h, int wd, int relu, cudaStream_t st);
+// PIC_POISSON_* error.  up: see pic_nn_conv3x3_cat (null: one input); pool:
+// see pic_nn_conv3x3_pool (null: none).
+int launch_conv3x3_tc(const void *up, int cu, const void *in, int cin, const void *w, const float *bias, void *out,
+                      float *out32, void *pool, int cout, int n, int h, int wd, int relu, cudaStream_t st);
 
 // Weight and bias gradients of a 3x3 convolution on mma.sync (wgrad.cu):
 // whether it takes these tensors, and the two launches (at most max_parts
 // partials of 9 cin cout + cout floats in scratch).
-bool wgrad_mma_takes(const void *in, int cin, const void *dout, int cout);
-cudaError_t launch_wgrad_mma(const void *in, int cin, const void *dout, int cout, int n, int h, int wd, float *dw,
+// up: see pic_nn_conv3x3_cat (null: one input).
+bool wgrad_mma_takes(const void *up, int cu, const void *in, int cin, const void *dout, int cout);
+cudaError_t launch_wgrad_mma(const void *up, int cu, const void *in, int cin, const void *dout, int cout, int n, int h, int wd, float *dw,
                              float *dbias, float *scratch, int max_parts, cudaStream_t st);
 
 }  // namespace pp

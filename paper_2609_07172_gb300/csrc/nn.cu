@@ -9,6 +9,9 @@
 // N-tile).
 #include <cuda_bf16.h>
 
+#include <cstdint>
+#include <initializer_list>
+
 #include "internal.h"
 #include "pic_poisson_nn.h"
 
@@ -176,14 +179,51 @@ __global__ void k_wgrad_reduce(const float *__restrict__ part, const float *__re
     }
 }
 
-__global__ void k_relu_bwd(const bf16 *__restrict__ y, bf16 *__restrict__ dy, long count) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < count && !(__bfloat162float(y[e]) > 0.f)) dy[e] = __float2bfloat16(0.f);
+// The element-wise kernels between the convolutions move BF16 tensors once
+// and are bound by memory: a thread takes V = 8 channels of a pixel (16-byte
+// accesses), or one where a channel count, stride or offset is no multiple of
+// 8 or a tensor not 16-byte aligned (V = 1).  With one channel (two bytes) per
+// thread a training batch (16 x 200 x 256) spent 700 us in these passes and the
+// loss, with eight 130 us; of the forward pass's on 65 x 200 x 256, 915 us then,
+// 25 are left (on its smaller images), because the convolutions pool and
+// concatenate themselves (pic_nn_conv3x3_pool, _cat).
+template <int V> struct Pack;
+template <> struct Pack<8> {
+    uint4 q;
+    __device__ __forceinline__ void load(const bf16 *p) { q = *reinterpret_cast<const uint4 *>(p); }
+    __device__ __forceinline__ void store(bf16 *p) const { *reinterpret_cast<uint4 *>(p) = q; }
+    __device__ __forceinline__ float get(int e) const {
+        const unsigned w = (e >> 1) == 0 ? q.x : (e >> 1) == 1 ? q.y : (e >> 1) == 2 ? q.z : q.w;
+        return __uint_as_float((e & 1) ? (w & 0xffff0000u) : (w << 16));
+    }
+    __device__ __forceinline__ void set(const float (&v)[8]) {
+        q = make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
+    }
+};
+template <> struct Pack<1> {
+    bf16 b;
+    __device__ __forceinline__ void load(const bf16 *p) { b = *p; }
+    __device__ __forceinline__ void store(bf16 *p) const { *p = b; }
+    __device__ __forceinline__ float get(int) const { return __bfloat162float(b); }
+    __device__ __forceinline__ void set(const float (&v)[1]) { b = __float2bfloat16(v[0]); }
+};
+
+template <int V> __global__ void k_relu_bwd(const bf16 *__restrict__ y, bf16 *__restrict__ dy, long count) {
+    const long e = ((long)blockIdx.x * blockDim.x + threadIdx.x) * V;
+    if (e >= count) return;
+    Pack<V> py, pd;
+    py.load(y + e);
+    pd.load(dy + e);
+    float v[V];
+#pragma unroll
+    for (int c = 0; c < V; ++c) v[c] = py.get(c) > 0.f ? pd.get(c) : 0.f;
+    pd.set(v);
+    pd.store(dy + e);
 }
 
 // 2x2 average pooling (NHWC) and its adjoint.
-__global__ void k_pool(const bf16 *__restrict__ in, bf16 *__restrict__ out, int n, int h, int wd, int c) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+template <int V> __global__ void k_pool(const bf16 *__restrict__ in, bf16 *__restrict__ out, int n, int h, int wd, int c) {
+    const long e = ((long)blockIdx.x * blockDim.x + threadIdx.x) * V;
     const int h2 = h / 2, w2 = wd / 2;
     const long total = (long)n * h2 * w2 * c;
     if (e >= total) return;
@@ -194,13 +234,21 @@ __global__ void k_pool(const bf16 *__restrict__ in, bf16 *__restrict__ out, int 
     const int y = (int)(t % h2);
     const long b = t / h2;
     const bf16 *s = in + ((b * h + 2 * y) * wd + 2 * x) * c + ch;
-    const float v = __bfloat162float(s[0]) + __bfloat162float(s[c]) + __bfloat162float(s[(long)wd * c]) +
-                    __bfloat162float(s[(long)wd * c + c]);
-    out[e] = __float2bfloat16(0.25f * v);
+    Pack<V> p0, p1, p2, p3;
+    p0.load(s);
+    p1.load(s + c);
+    p2.load(s + (long)wd * c);
+    p3.load(s + (long)wd * c + c);
+    float v[V];
+#pragma unroll
+    for (int q = 0; q < V; ++q) v[q] = 0.25f * (p0.get(q) + p1.get(q) + p2.get(q) + p3.get(q));
+    p0.set(v);
+    p0.store(out + e);
 }
 
+template <int V>
 __global__ void k_pool_bwd(const bf16 *__restrict__ dout, bf16 *__restrict__ din, int n, int h, int wd, int c) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long e = ((long)blockIdx.x * blockDim.x + threadIdx.x) * V;
     const long total = (long)n * h * wd * c;
     if (e >= total) return;
     const int ch = (int)(e % c);
@@ -209,14 +257,21 @@ __global__ void k_pool_bwd(const bf16 *__restrict__ dout, bf16 *__restrict__ din
     t /= wd;
     const int y = (int)(t % h);
     const long b = t / h;
-    din[e] = __float2bfloat16(0.25f * __bfloat162float(dout[((b * (h / 2) + y / 2) * (wd / 2) + x / 2) * c + ch]));
+    Pack<V> p;
+    p.load(dout + ((b * (h / 2) + y / 2) * (wd / 2) + x / 2) * c + ch);
+    float v[V];
+#pragma unroll
+    for (int q = 0; q < V; ++q) v[q] = 0.25f * p.get(q);
+    p.set(v);
+    p.store(din + e);
 }
 
 // Nearest-neighbour 2x upsampling of `in` (h x w, c channels) into channels
 // [0, c) of `out` (2h x 2w, cstride channels), and the adjoint (sum of the
 // 2x2 block) back from those channels.
+template <int V>
 __global__ void k_up(const bf16 *__restrict__ in, bf16 *__restrict__ out, int n, int h, int wd, int c, int cstride) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long e = ((long)blockIdx.x * blockDim.x + threadIdx.x) * V;
     const long total = (long)n * 4 * h * wd * c;
     if (e >= total) return;
     const int ch = (int)(e % c);
@@ -225,12 +280,15 @@ __global__ void k_up(const bf16 *__restrict__ in, bf16 *__restrict__ out, int n,
     t /= 2 * wd;
     const int y = (int)(t % (2 * h));
     const long b = t / (2 * h);
-    out[((b * 2 * h + y) * 2 * wd + x) * cstride + ch] = in[((b * h + y / 2) * wd + x / 2) * c + ch];
+    Pack<V> p;
+    p.load(in + ((b * h + y / 2) * wd + x / 2) * c + ch);
+    p.store(out + ((b * 2 * h + y) * 2 * wd + x) * cstride + ch);
 }
 
+template <int V>
 __global__ void k_up_bwd(const bf16 *__restrict__ dout, int cstride, bf16 *__restrict__ din, int n, int h, int wd,
                          int c) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long e = ((long)blockIdx.x * blockDim.x + threadIdx.x) * V;
     const long total = (long)n * h * wd * c;
     if (e >= total) return;
     const int ch = (int)(e % c);
@@ -241,39 +299,57 @@ __global__ void k_up_bwd(const bf16 *__restrict__ dout, int cstride, bf16 *__res
     const long b = t / h;
     const bf16 *s = dout + ((b * 2 * h + 2 * y) * 2 * wd + 2 * x) * cstride + ch;
     const long rs = 2L * wd * cstride;
-    din[e] = __float2bfloat16(__bfloat162float(s[0]) + __bfloat162float(s[cstride]) + __bfloat162float(s[rs]) +
-                              __bfloat162float(s[rs + cstride]));
+    Pack<V> p0, p1, p2, p3;
+    p0.load(s);
+    p1.load(s + cstride);
+    p2.load(s + rs);
+    p3.load(s + rs + cstride);
+    float v[V];
+#pragma unroll
+    for (int q = 0; q < V; ++q) v[q] = p0.get(q) + p1.get(q) + p2.get(q) + p3.get(q);
+    p0.set(v);
+    p0.store(din + e);
 }
 
 // Copy c channels between NHWC tensors with different channel strides and offsets.
+template <int V>
 __global__ void k_copy_ch(const bf16 *__restrict__ src, int sstride, int soff, bf16 *__restrict__ dst, int dstride,
                           int doff, long pixels, int c) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long e = ((long)blockIdx.x * blockDim.x + threadIdx.x) * V;
     if (e >= pixels * c) return;
     const long p = e / c;
     const int ch = (int)(e - p * c);
-    dst[p * dstride + doff + ch] = src[p * sstride + soff + ch];
+    Pack<V> q;
+    q.load(src + p * sstride + soff + ch);
+    q.store(dst + p * dstride + doff + ch);
 }
 
 // Mean-squared error over the first `used` of `c` channels; gradient (BF16,
 // channel layout of the prediction, zero on unused channels) and per-block
 // loss partials.
+template <int V>
 __global__ void __launch_bounds__(256) k_mse(const float *__restrict__ pred, const float *__restrict__ target,
                                              long pixels, int c, int used, bf16 *__restrict__ dpred,
                                              float *__restrict__ part) {
     __shared__ float red[8];
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long e = ((long)blockIdx.x * blockDim.x + threadIdx.x) * V;
     float l = 0.f;
     if (e < pixels * c) {
         const long p = e / c;
         const int ch = (int)(e - p * c);
-        float g = 0.f;
-        if (ch < used) {
-            const float d = pred[e] - target[p * used + ch];
-            l = d * d;
-            g = 2.f * d / (float)(pixels * used);
+        float g[V];
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            g[q] = 0.f;
+            if (ch + q < used) {
+                const float d = pred[e + q] - target[p * used + ch + q];
+                l = fmaf(d, d, l);
+                g[q] = 2.f * d / (float)(pixels * used);
+            }
         }
-        dpred[e] = __float2bfloat16(g);
+        Pack<V> o;
+        o.set(g);
+        o.store(dpred + e);
     }
     for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = l;
@@ -314,9 +390,17 @@ __global__ void k_adam(float *__restrict__ w, const float *__restrict__ g, float
     if (wb) wb[e] = __float2bfloat16(wi);
 }
 
-__global__ void k_add(bf16 *__restrict__ a, const bf16 *__restrict__ b, long count) {
-    const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < count) a[e] = __float2bfloat16(__bfloat162float(a[e]) + __bfloat162float(b[e]));
+template <int V> __global__ void k_add(bf16 *__restrict__ a, const bf16 *__restrict__ b, long count) {
+    const long e = ((long)blockIdx.x * blockDim.x + threadIdx.x) * V;
+    if (e >= count) return;
+    Pack<V> pa, pb;
+    pa.load(a + e);
+    pb.load(b + e);
+    float v[V];
+#pragma unroll
+    for (int c = 0; c < V; ++c) v[c] = pa.get(c) + pb.get(c);
+    pa.set(v);
+    pa.store(a + e);
 }
 
 __global__ void k_f32_to_bf16(const float *__restrict__ a, bf16 *__restrict__ b, long count) {
@@ -552,6 +636,16 @@ __global__ void k_axpy_alpha(const double2 *__restrict__ x, const double2 *__res
 
 inline unsigned grid1(long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
+// Whether 16-byte accesses reach every 8-channel group: counts, strides and
+// offsets c, the tensors' addresses p.
+inline bool by8(std::initializer_list<long> c, std::initializer_list<const void *> p) {
+    for (long v : c)
+        if (v % 8) return false;
+    for (const void *q : p)
+        if ((uintptr_t)q & 15) return false;
+    return true;
+}
+
 }  // namespace
 }  // namespace pp
 
@@ -572,7 +666,7 @@ int pic_nn_conv3x3(const void *in, int cin, const void *w, const float *bias, vo
                    int n, int h, int wd, int relu, void *stream) {
     clear_error();
     if (in && w && (out_bf16 || out_f32) && cin > 0 && cout > 0 && n > 0 && h > 0 && wd > 0) {
-        const int rc = launch_conv3x3_tc(in, cin, w, bias, out_bf16, out_f32, cout, n, h, wd, relu,
+        const int rc = launch_conv3x3_tc(nullptr, 0, in, cin, w, bias, out_bf16, out_f32, nullptr, cout, n, h, wd, relu,
                                          (cudaStream_t)stream);
         if (rc != 1) return rc;   // done on the tcgen05 tensor cores, or an error
     }
@@ -603,6 +697,38 @@ int pic_nn_conv3x3_mma_sync(const void *in, int cin, const void *w, const float 
     return PIC_POISSON_OK;
 }
 
+int pic_nn_conv3x3_cat(const void *up, int cu, const void *skip, int cs, const void *w, const float *bias, void *cat,
+                       void *out_bf16, float *out_f32, int cout, int n, int h, int wd, int relu, void *stream) {
+    clear_error();
+    if (!up || !skip || !w || !cat || (!out_bf16 && !out_f32) || cu <= 0 || cs <= 0 || cout <= 0 || n <= 0 || h <= 0 ||
+        wd <= 0 || h % 2 || wd % 2) {
+        set_error("conv3x3_cat: need up, skip, w, cat, an output, positive channel counts and even h and w");
+        return PIC_POISSON_EINVAL;
+    }
+    int rc = launch_conv3x3_tc(up, cu, skip, cu + cs, w, bias, out_bf16, out_f32, nullptr, cout, n, h, wd, relu,
+                               (cudaStream_t)stream);
+    if (rc != 1) return rc;
+    rc = pic_nn_up2(up, cat, n, h / 2, wd / 2, cu, cu + cs, 0, stream);
+    if (rc) return rc;
+    rc = pic_nn_copy_channels(skip, cs, 0, cat, cu + cs, cu, (long)n * h * wd, cs, stream);
+    if (rc) return rc;
+    return pic_nn_conv3x3(cat, cu + cs, w, bias, out_bf16, out_f32, cout, n, h, wd, relu, stream);
+}
+
+int pic_nn_conv3x3_pool(const void *in, int cin, const void *w, const float *bias, void *out_bf16, void *pooled,
+                        int cout, int n, int h, int wd, int relu, void *stream) {
+    clear_error();
+    if (!in || !w || !out_bf16 || !pooled || cin <= 0 || cout <= 0 || n <= 0 || h <= 0 || wd <= 0 || h % 2 || wd % 2) {
+        set_error("conv3x3_pool: need in, w, both outputs, positive channel counts and even h and w");
+        return PIC_POISSON_EINVAL;
+    }
+    int rc = launch_conv3x3_tc(nullptr, 0, in, cin, w, bias, out_bf16, nullptr, pooled, cout, n, h, wd, relu,
+                               (cudaStream_t)stream);
+    if (rc != 1) return rc;
+    rc = pic_nn_conv3x3(in, cin, w, bias, out_bf16, nullptr, cout, n, h, wd, relu, stream);
+    return rc ? rc : pic_nn_pool2(out_bf16, pooled, n, h, wd, cout, 0, stream);
+}
+
 int pic_nn_flip_weights(const void *w, int cout, int cin, void *wt, void *stream) {
     clear_error();
     if (!w || !wt || cout <= 0 || cin <= 0) {
@@ -630,8 +756,8 @@ int pic_nn_conv3x3_wgrad(const void *in, int cin, const void *dout, int cout, in
         return PIC_POISSON_EINVAL;
     }
     const cudaStream_t st = (cudaStream_t)stream;
-    if (cin > 0 && cout > 0 && chunks > 0 && wgrad_mma_takes(in, cin, dout, cout)) {
-        PP_CUDA(launch_wgrad_mma(in, cin, dout, cout, n, h, wd, dw, dbias, scratch, chunks, st));
+    if (cin > 0 && cout > 0 && chunks > 0 && wgrad_mma_takes(nullptr, 0, in, cin, dout, cout)) {
+        PP_CUDA(launch_wgrad_mma(nullptr, 0, in, cin, dout, cout, n, h, wd, dw, dbias, scratch, chunks, st));
         return PIC_POISSON_OK;
     }
     float *part = scratch, *partb = scratch + (long)chunks * 9 * cout * cin;
@@ -642,8 +768,27 @@ int pic_nn_conv3x3_wgrad(const void *in, int cin, const void *dout, int cout, in
     return PIC_POISSON_OK;
 }
 
+int pic_nn_conv3x3_wgrad_cat(const void *up, int cu, const void *skip, int cs, const void *dout, int cout, int n,
+                             int h, int wd, float *dw, float *dbias, float *scratch, size_t scratch_floats,
+                             void *stream) {
+    clear_error();
+    if (!up || !skip || !dout || !dw || !scratch || cu <= 0 || cs <= 0 || cout <= 0 || n <= 0 || h <= 0 || wd <= 0 ||
+        h % 2 || wd % 2 || !wgrad_mma_takes(up, cu, skip, cu + cs, dout, cout) ||
+        scratch_floats < pic_nn_wgrad_scratch_floats(cu + cs, cout, n, h, wd)) {
+        set_error("conv3x3_wgrad_cat: need channel counts in multiples of 8, even h and w, 16-byte aligned tensors and "
+                  "the scratch of pic_nn_wgrad_scratch_floats");
+        return PIC_POISSON_EINVAL;
+    }
+    const int chunks = (int)(((long)n * h * wd + WG_CHUNK - 1) / WG_CHUNK);
+    PP_CUDA(launch_wgrad_mma(up, cu, skip, cu + cs, dout, cout, n, h, wd, dw, dbias, scratch, chunks,
+                             (cudaStream_t)stream));
+    return PIC_POISSON_OK;
+}
+
 int pic_nn_relu_bwd(const void *y, void *dy, long count, void *stream) {
-    k_relu_bwd<<<grid1(count), 256, 0, (cudaStream_t)stream>>>((const bf16 *)y, (bf16 *)dy, count);
+    const cudaStream_t st = (cudaStream_t)stream;
+    if (by8({count}, {y, dy})) k_relu_bwd<8><<<grid1(count / 8), 256, 0, st>>>((const bf16 *)y, (bf16 *)dy, count);
+    else k_relu_bwd<1><<<grid1(count), 256, 0, st>>>((const bf16 *)y, (bf16 *)dy, count);
     NN_CHECK();
     return PIC_POISSON_OK;
 }
@@ -654,24 +799,41 @@ int pic_nn_pool2(const void *in, void *out, int n, int h, int wd, int c, int bac
         set_error("pool2: h and w must be even");
         return PIC_POISSON_EINVAL;
     }
-    if (!backward) k_pool<<<grid1((long)n * (h / 2) * (wd / 2) * c), 256, 0, st>>>((const bf16 *)in, (bf16 *)out, n, h, wd, c);
-    else k_pool_bwd<<<grid1((long)n * h * wd * c), 256, 0, st>>>((const bf16 *)in, (bf16 *)out, n, h, wd, c);
+    const bf16 *I = (const bf16 *)in;
+    bf16 *O = (bf16 *)out;
+    const bool v8 = by8({c}, {in, out});
+    const long work = (long)n * (backward ? (long)h * wd : (long)(h / 2) * (wd / 2)) * c;
+    if (!backward && v8) k_pool<8><<<grid1(work / 8), 256, 0, st>>>(I, O, n, h, wd, c);
+    else if (!backward) k_pool<1><<<grid1(work), 256, 0, st>>>(I, O, n, h, wd, c);
+    else if (v8) k_pool_bwd<8><<<grid1(work / 8), 256, 0, st>>>(I, O, n, h, wd, c);
+    else k_pool_bwd<1><<<grid1(work), 256, 0, st>>>(I, O, n, h, wd, c);
     NN_CHECK();
     return PIC_POISSON_OK;
 }
 
 int pic_nn_up2(const void *in, void *out, int n, int h, int wd, int c, int cstride, int backward, void *stream) {
     const cudaStream_t st = (cudaStream_t)stream;
-    if (!backward) k_up<<<grid1((long)n * 4 * h * wd * c), 256, 0, st>>>((const bf16 *)in, (bf16 *)out, n, h, wd, c, cstride);
-    else k_up_bwd<<<grid1((long)n * h * wd * c), 256, 0, st>>>((const bf16 *)in, cstride, (bf16 *)out, n, h, wd, c);
+    const bf16 *I = (const bf16 *)in;
+    bf16 *O = (bf16 *)out;
+    const bool v8 = by8({c, cstride}, {in, out});
+    const long work = (long)n * (backward ? 1 : 4) * h * wd * c;
+    if (!backward && v8) k_up<8><<<grid1(work / 8), 256, 0, st>>>(I, O, n, h, wd, c, cstride);
+    else if (!backward) k_up<1><<<grid1(work), 256, 0, st>>>(I, O, n, h, wd, c, cstride);
+    else if (v8) k_up_bwd<8><<<grid1(work / 8), 256, 0, st>>>(I, cstride, O, n, h, wd, c);
+    else k_up_bwd<1><<<grid1(work), 256, 0, st>>>(I, cstride, O, n, h, wd, c);
     NN_CHECK();
     return PIC_POISSON_OK;
 }
 
 int pic_nn_copy_channels(const void *src, int sstride, int soff, void *dst, int dstride, int doff, long pixels, int c,
                          void *stream) {
-    k_copy_ch<<<grid1(pixels * c), 256, 0, (cudaStream_t)stream>>>((const bf16 *)src, sstride, soff, (bf16 *)dst,
-                                                                     dstride, doff, pixels, c);
+    const cudaStream_t st = (cudaStream_t)stream;
+    const bf16 *S = (const bf16 *)src;
+    bf16 *D = (bf16 *)dst;
+    if (by8({c, sstride, soff, dstride, doff}, {src, dst}))
+        k_copy_ch<8><<<grid1(pixels * c / 8), 256, 0, st>>>(S, sstride, soff, D, dstride, doff, pixels, c);
+    else
+        k_copy_ch<1><<<grid1(pixels * c), 256, 0, st>>>(S, sstride, soff, D, dstride, doff, pixels, c);
     NN_CHECK();
     return PIC_POISSON_OK;
 }
@@ -679,8 +841,10 @@ int pic_nn_copy_channels(const void *src, int sstride, int soff, void *dst, int 
 int pic_nn_mse(const float *pred, const float *target, long pixels, int c, int used, void *dpred, float *scratch,
                float *loss, void *stream) {
     const cudaStream_t st = (cudaStream_t)stream;
-    const unsigned nb = grid1(pixels * c);
-    k_mse<<<nb, 256, 0, st>>>(pred, target, pixels, c, used, (bf16 *)dpred, scratch);
+    const bool v8 = by8({c}, {dpred});
+    const unsigned nb = grid1(v8 ? pixels * c / 8 : pixels * c);
+    if (v8) k_mse<8><<<nb, 256, 0, st>>>(pred, target, pixels, c, used, (bf16 *)dpred, scratch);
+    else k_mse<1><<<nb, 256, 0, st>>>(pred, target, pixels, c, used, (bf16 *)dpred, scratch);
     k_sum_f<<<1, 1024, 0, st>>>(scratch, (int)nb, pixels * used, loss);
     NN_CHECK();
     return PIC_POISSON_OK;
@@ -696,7 +860,9 @@ int pic_nn_adam(float *w, const float *g, float *m, float *v, long count, float 
 }
 
 int pic_nn_add(void *a, const void *b, long count, void *stream) {
-    k_add<<<grid1(count), 256, 0, (cudaStream_t)stream>>>((bf16 *)a, (const bf16 *)b, count);
+    const cudaStream_t st = (cudaStream_t)stream;
+    if (by8({count}, {a, b})) k_add<8><<<grid1(count / 8), 256, 0, st>>>((bf16 *)a, (const bf16 *)b, count);
+    else k_add<1><<<grid1(count), 256, 0, st>>>((bf16 *)a, (const bf16 *)b, count);
     NN_CHECK();
     return PIC_POISSON_OK;
 }

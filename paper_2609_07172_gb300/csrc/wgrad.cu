@@ -43,7 +43,8 @@ constexpr int WG_MAX_IN = (64 + 2) * (8 + 2);    // halo pixels of the largest t
 constexpr int WG_STAGE = (WG_MAX_IN + WG_PIX) * 32;
 
 struct WgradArgs {
-    const bf16 *in;
+    const bf16 *in, *up;          // input; channels [0, cu) from up, of half the height and width, upsampled 2x
+    int cu;
     const bf16 *dout;
     int cin, cout, n, h, wd;
     int tx, ty;                   // tile: tx pixels by ty rows, tx ty = WG_PIX
@@ -91,7 +92,11 @@ __device__ __forceinline__ void load_tile(const WgradArgs &a, int t, unsigned sm
         const int p = e >> 1, half = e & 1;
         const int r = p / wx, y = y0 + r - 1, x = x0 + (p - r * wx) - 1, c = ci0 + 8 * half;
         const bool ok = (unsigned)y < (unsigned)a.h && (unsigned)x < (unsigned)a.wd && c < a.cin;
-        cp16(pix_addr(sm, p, half), a.in + (ok ? ((img + y) * a.wd + x) * a.cin + c : 0), ok);
+        const bf16 *src = a.in;
+        if (ok)
+            src = c < a.cu ? a.up + (((size_t)s * (a.h >> 1) + (y >> 1)) * (a.wd >> 1) + (x >> 1)) * a.cu + c
+                           : a.in + ((img + y) * a.wd + x) * (a.cin - a.cu) + (c - a.cu);
+        cp16(pix_addr(sm, p, half), src, ok);
     }
     const unsigned sd = sm + WG_MAX_IN * 32;
     const int sh = __ffs(a.tx) - 1;
@@ -208,14 +213,17 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce_split(const float *__restr
 
 // 16-byte loads of eight channels: channel counts are multiples of 8 and the
 // tensors 16-byte aligned; the caller's scalar kernel takes the rest.
-bool wgrad_mma_takes(const void *in, int cin, const void *dout, int cout) {
-    return cin % 8 == 0 && cout % 8 == 0 && (((uintptr_t)in | (uintptr_t)dout) & 15) == 0;
+bool wgrad_mma_takes(const void *up, int cu, const void *in, int cin, const void *dout, int cout) {
+    return cin % 8 == 0 && cu % 8 == 0 && cout % 8 == 0 &&
+           (((uintptr_t)in | (uintptr_t)up | (uintptr_t)dout) & 15) == 0;
 }
 
-cudaError_t launch_wgrad_mma(const void *in, int cin, const void *dout, int cout, int n, int h, int wd, float *dw,
+cudaError_t launch_wgrad_mma(const void *up, int cu, const void *in, int cin, const void *dout, int cout, int n, int h, int wd, float *dw,
                              float *dbias, float *scratch, int max_parts, cudaStream_t st) {
     WgradArgs a{};
     a.in = (const bf16 *)in;
+    a.up = (const bf16 *)up;
+    a.cu = up ? cu : 0;
     a.dout = (const bf16 *)dout;
     a.cin = cin;
     a.cout = cout;

@@ -34,9 +34,12 @@ OUT_USED = 2
 _SIGS = {
     "pic_nn_conv3x3": "vivvvvi iiiiv",
     "pic_nn_conv3x3_mma_sync": "vivvvvi iiiiv",
+    "pic_nn_conv3x3_pool": "vivvvv iiiiiv",
+    "pic_nn_conv3x3_cat": "vivivvvvv iiiiiv",
     "pic_nn_conv_tc_status": "v",
     "pic_nn_flip_weights": "viivv",
     "pic_nn_conv3x3_wgrad": "viviiiivvvsv",
+    "pic_nn_conv3x3_wgrad_cat": "vivivi iiivvvsv",
     "pic_nn_relu_bwd": "vvlv",
     "pic_nn_pool2": "vviiiiiv",
     "pic_nn_up2": "vviiiiiiv",
@@ -192,22 +195,31 @@ class UNet:
         s = b["levels"]
         self._x = x
         st = _st()
-        self._conv("e0", x, 16, b["e0"], 16, n, s[0], True)
-        _ok(lib.pic_nn_pool2(P(b["e0"]), P(b["p0"]), n, *s[0], 16, 0, st))
-        self._conv("e1", b["p0"], 16, b["e1"], 32, n, s[1], True)
-        _ok(lib.pic_nn_pool2(P(b["e1"]), P(b["p1"]), n, *s[1], 32, 0, st))
-        self._conv("e2", b["p1"], 32, b["e2"], 64, n, s[2], True)
-        _ok(lib.pic_nn_pool2(P(b["e2"]), P(b["p2"]), n, *s[2], 64, 0, st))
+        src, cin = x, 16
+        for lv, (name, cout) in enumerate((("e0", 16), ("e1", 32), ("e2", 64))):
+            pooled = b["p%d" % lv]
+            if self.conv_entry == "pic_nn_conv3x3":
+                _ok(lib.pic_nn_conv3x3_pool(P(src), cin, P(self.wb[name]), P(self.b[name]), P(b[name]), P(pooled), cout,
+                                            n, *s[lv], 1, st))
+            else:
+                self._conv(name, src, cin, b[name], cout, n, s[lv], True)
+                _ok(lib.pic_nn_pool2(P(b[name]), P(pooled), n, *s[lv], cout, 0, st))
+            src, cin = pooled, cout
         self._conv("b1", b["p2"], 64, b["b1"], 128, n, s[3], True)
         self._conv("b2", b["b1"], 128, b["b2"], 64, n, s[3], True)
         for lo, hi, cu, cs, src in ((3, 2, 64, 128, ("b2", "e2", "c2")), (2, 1, 32, 64, ("d2", "e1", "c1")),
                                     (1, 0, 16, 32, ("d1", "e0", "c0"))):
             up, skip, cat = src
+            dname = {"c2": "d2", "c1": "d1", "c0": "d0"}[cat]
+            cout = {"d2": 32, "d1": 16, "d0": 16}[dname]
+            if self.conv_entry == "pic_nn_conv3x3":
+                # reads up and skip as they are on wide images, without writing the concatenation
+                _ok(lib.pic_nn_conv3x3_cat(P(b[up]), cu, P(b[skip]), cs - cu, P(self.wb[dname]), P(self.b[dname]),
+                                           P(b[cat]), P(b[dname]), None, cout, n, *s[hi], 1, st))
+                continue
             _ok(lib.pic_nn_up2(P(b[up]), P(b[cat]), n, *s[lo], cu, cs, 0, st))
             _ok(lib.pic_nn_copy_channels(P(b[skip]), cs - cu, 0, P(b[cat]), cs, cu, n * s[hi][0] * s[hi][1],
                                          cs - cu, st))
-            dname = {"c2": "d2", "c1": "d1", "c0": "d0"}[cat]
-            cout = {"d2": 32, "d1": 16, "d0": 16}[dname]
             self._conv(dname, b[cat], cs, b[dname], cout, n, s[hi], True)
         self._conv("out", b["d0"], 16, None, 16, n, s[0], False, y32=b["y"])
         return b["y"]
@@ -237,7 +249,8 @@ class UNet:
                                                         ("d1", "c1", 64, 16, 1, "d2", "e1", 32),
                                                         ("d2", "c2", 128, 32, 2, "b2", "e2", 64)):
             relu_bwd(b[dname], b["g" + dname])
-            wgrad(dname, b[cat], cin, b["g" + dname], cout, lv)
+            _ok(lib.pic_nn_conv3x3_wgrad_cat(P(b[up]), cu, P(b[skip]), cin - cu, P(b["g" + dname]), cout, n, *s[lv],
+                                             P(self.gw[dname]), P(self.gb[dname]), P(wg), nwg, st))
             self._conv(dname, b["g" + dname], cout, b["g" + cat], cin, n, s[lv], False, transposed=True)
             pix = n * s[lv][0] * s[lv][1]
             _ok(lib.pic_nn_copy_channels(P(b["g" + cat]), cin, cu, P(b["g" + skip]), cin - cu, 0, pix, cin - cu, st))
