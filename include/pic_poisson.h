@@ -346,12 +346,12 @@ int pic_poisson_solve_host(pic_poisson_plan_t plan, const double *rho_host, doub
  * density (nz + 1, ntheta, nr + 1) FP64 (node (c, j, a) at z-face c, alpha
  * j dalpha, r-face a), which the caller zeroes before a step's first species.
  * Each thread sums its 4 consecutive particles of one cell in registers, lanes
- * of a warp holding the same cell add their sums with register shuffles, and
- * one lane per run of equal cells issues the eight FP64 atomics, so
- * cell-sorted particles are cheapest; any order is correct (the order of the
- * additions, hence rounding, varies from run to run).  The weights' products
- * and those sums are double-float (about 48 significant bits, ~1e-14
- * relative); cell, offset and the atomics are binary64.
+ * of a warp holding the same cell add their sums with register shuffles, runs
+ * of radially neighbouring cells share their common corners, and one lane per
+ * run of equal cells issues the FP64 atomics, so cell-sorted particles are
+ * cheapest; any order is correct (the order of the atomics, hence rounding,
+ * varies from run to run).  Offsets, weights' products and those sums are
+ * 64-bit fixed point (2^-54 of a particle); the atomics are binary64.
  * Particles outside the domain deposit nothing.  On non-uniform faces
  * (r_faces, z_faces) the cell is the one the face arrays define (max{a :
  * face[a] <= x}, found by a lookup guess and exact binary64 comparisons) and

@@ -8,19 +8,32 @@
 // zeta) adds W w_r w_alpha w_z / V_nu to each of the cell's eight corner
 // nodes (w^(0) = 1 - t, w^(1) = t; V_nu the node's cylindrical control
 // volume, from cell centre to cell centre in r and z and cut at the walls, a
-// full dalpha in alpha).  Aggregation (Eq. warp_aggregated_cic): a thread
-// first sums, in registers, its consecutive particles that share a cell;
-// then lanes whose last cells agree -- runs of equal cell labels in lane
-// order, which cell-sorted input makes long -- add their sums with a
-// segmented scan of register shuffles, and the last lane of each run issues
-// the run's eight FP64 atomic additions, each divided by the node's volume
-// once.  The weights' products and the sums are double-float (df.h, about
-// 48 bits, on the FP32 pipe); the particle's cell and offset and the final
-// per-node values are binary64.  All weights and corners stay; only the
-// order of the additions changes.  Particles outside the domain deposit
-// nothing.
+// full dalpha in alpha).  Aggregation (Eq. warp_aggregated_cic): a thread first
+// sums its consecutive particles that share a cell; then lanes whose last
+// cells agree -- runs of equal cell labels in lane order, which cell-sorted
+// input makes long -- add their sums with a segmented scan of register
+// shuffles; a run whose cell is the radial neighbour of the run before it takes
+// over that run's four outer corners (the same nodes), across the warps of the
+// block too; and the last lane of each run issues the run's FP64 atomic
+// additions, each divided by the node's volume once: four per cell of sorted
+// input instead of eight.  Particles outside the domain deposit nothing.
 //
-// Non-uniform faces and composite domains (k_deposit_faces): the cell comes
+// Fixed point.  The FP64 unit (1/64 of the FP32 rate) bound this kernel: about
+// 23 of its instructions per particle for the position and 16 per cell for the
+// corners, 5.8 of the 5.8 ms per 105 M particles.  Offsets in the cell, their
+// products and every sum are 64-bit integers instead (scale 2^-54): a cell's
+// particles are summed as the eight moments 1, x, y, z, xy, xz, yz, xyz -- sums
+// that round nothing -- and the corner weights follow from them by exact
+// subtractions.  A particle's products are within 2^-54 of exact, where the
+// double-float products before were within 2^-48 relative.  The position goes
+// to a cell and an offset by one 64-bit multiplication; a particle near a cell
+// boundary (2^-24 of a cell) or outside takes the binary64 arithmetic, which
+// alone decides those cases.  210 M cell-sorted particles of two species, 4 per
+// cell and species, at 512 x 128 x 400: 11.6 ms, now 2.25 (integer instructions and
+// their issue, both two thirds busy; against a quadruple-precision deposit the nodes
+// are within 5.6e-14 as before, the largest error 2.0e-13 instead of 4.8e-13).
+//
+// Non-uniform faces and composite domains (FACES): the cell comes
 // from the face arrays (a bin lookup guesses, binary64 comparisons decide),
 // the offsets from the cell's own faces; in a composite domain (Sec. 2.2) a
 // particle in an inactive cell deposits nothing and a node's volume counts
@@ -35,27 +48,41 @@
 // integral of the half cell (f_lo, f_hi below, f_lo + f_hi = 1), the
 // azimuthal and axial ones are 1/2; so charge is conserved exactly:
 // sum_q rho_q V_q = charge * sum_nu n_nu V_nu.
+#include <algorithm>
 #include <cmath>
+#include <cstdint>
 
-#include "df.h"
 #include "plan.h"
 
 namespace pp {
 namespace {
 
+typedef unsigned long long u64;
+
+// One uniform axis in fixed point: x -> X = x 2^(62 - E) (|x| < 2^E over the
+// domain), D = X - base in [0, span), and D 2^sh K / 2^64 = the position in
+// cells with F fraction bits.
+struct FixAxis {
+    long long base;
+    u64 span, K;
+    int e1;                 // E + 1023
+    int sh, F;
+};
+
 struct DepositArgs {
     int nr, nt, nz;
     long long np;
     double r_in, z0, inv_dr, inv_da, inv_dz;
-    float w_hi, w_lo;       // the weight W 2^-w_exp in double-float, in [1, 2)
-    int w_exp;
+    FixAxis fr, fa, fz;
+    double wscale;          // the weight times 2^-54
+    int vec;                // the arrays allow 16-byte loads
     const double *r, *al, *z;
     const double *inv_vr;   // [nr + 1] 1 / (radial integral of r dr of node a's interval)
     const double *inv_vz;   // [nz + 1] 1 / (dalpha * axial length of node c's interval)
     double *nodes;          // (nz + 1, nt, nr + 1)
 };
 
-// Non-uniform faces or a composite domain (k_deposit_faces): the cell is found
+// Non-uniform faces or a composite domain: the cell is found
 // on the face arrays -- a lookup bin guesses it, exact comparisons settle it.
 struct DepositGeo {
     const double *rf, *zf;          // faces [nr + 1], [nz + 1]
@@ -84,190 +111,270 @@ __device__ __forceinline__ int find_cell(double x, const double *f, int n, const
 }
 
 constexpr int DEP_PPT = 4;   // consecutive particles per thread
+constexpr int DEP_THREADS = 256;
 
-// The eight corner contributions W w_r w_alpha w_z 2^-w_exp (corner index
-// 4 dz + 2 dalpha + dr) of offsets (xr, xa, xz) in the cell, in double-float
-// on the FP32 pipe -- the deposit's FP64 instructions were its bound.
-__device__ __forceinline__ bool weights8(const DepositArgs &a, double xr, double xa, double xz, df c[8]) {
-    const df r1 = split_scaled(xr, 1023), r0 = split_scaled(1.0 - xr, 1023);
-    const df a1 = split_scaled(xa, 1023), a0 = split_scaled(1.0 - xa, 1023);
-    const df z1 = split_scaled(xz, 1023), z0 = split_scaled(1.0 - xz, 1023);
-    const df w = {a.w_hi, a.w_lo};
-    const df wz0 = df_mul(w, z0), wz1 = df_mul(w, z1);
-    const df q00 = df_mul(wz0, a0), q01 = df_mul(wz0, a1), q10 = df_mul(wz1, a0), q11 = df_mul(wz1, a1);
-    c[0] = df_mul(q00, r0);
-    c[1] = df_mul(q00, r1);
-    c[2] = df_mul(q01, r0);
-    c[3] = df_mul(q01, r1);
-    c[4] = df_mul(q10, r0);
-    c[5] = df_mul(q10, r1);
-    c[6] = df_mul(q11, r0);
-    c[7] = df_mul(q11, r1);
-    return true;
+// A particle in its cell: indices and offsets, 64 fraction bits.
+struct Place {
+    int ir, ia, iz;
+    u64 x, y, z;
+};
+
+// A binary64 offset in [0, 1] as a 64-bit fraction (cut; 1 becomes 1 - 2^-64).
+__device__ __forceinline__ u64 frac64(double f) {
+    const unsigned hi = (unsigned)__double2hiint(f), lo = (unsigned)__double2loint(f);
+    const int s = 1022 - (int)((hi >> 20) & 0x7ffu);   // 0 for [1/2, 1)
+    if (s < 0) return ~0ull;
+    if (s > 63) return 0ull;
+    return ((((u64)((hi & 0xfffffu) | 0x100000u)) << 32 | lo) << 11) >> s;
 }
 
-// Cell and corner contributions of particle p; false when p is absent or
-// outside.  The position arithmetic (cell, offset in the cell) is binary64.
-__device__ __forceinline__ bool cic_weights(const DepositArgs &a, long long p, int &ir, int &ia, int &iz, df c[8]) {
-    if (p >= a.np) return false;
-    const double tr = (a.r[p] - a.r_in) * a.inv_dr, ta = a.al[p] * a.inv_da, tz = (a.z[p] - a.z0) * a.inv_dz;
+// Cell and offset of x on a uniform axis; false where the binary64 arithmetic
+// has to decide: outside, not finite, or within 2^-24 of a cell boundary.
+__device__ __forceinline__ bool fix_place(const FixAxis &a, double x, int &cell, u64 &f) {
+    const int hi = __double2hiint(x);
+    const unsigned lo = (unsigned)__double2loint(x);
+    const int s = a.e1 - ((hi >> 20) & 0x7ff);
+    u64 X = ((((u64)((hi & 0xfffff) | 0x100000)) << 32 | lo) << 10) >> min(max(s, 0), 63);
+    if (hi < 0) X = 0ull - X;
+    const u64 D = X - (u64)a.base;
+    const u64 t = __umul64hi(D << a.sh, a.K);
+    cell = (int)(t >> a.F);
+    f = t << (64 - a.F);
+    return s >= 1 && D < a.span && (unsigned)(f >> 32) + 0x100u >= 0x200u;
+}
+
+// Cell and offsets of particle (r, al, z) by binary64 arithmetic; false when
+// it is outside.
+__device__ __noinline__ bool place_exact(const DepositArgs &a, double r, double al, double z, Place &q) {
+    const double tr = (r - a.r_in) * a.inv_dr, ta = al * a.inv_da, tz = (z - a.z0) * a.inv_dz;
     const double fr = floor(tr), fa = floor(ta), fz = floor(tz);
     // in range before any conversion (NaN compares false)
     if (!(fr >= 0.0 && fr < (double)a.nr && fa >= 0.0 && fa < (double)a.nt && fz >= 0.0 && fz < (double)a.nz))
         return false;
-    ir = (int)fr;
-    ia = (int)fa;
-    iz = (int)fz;
-    const double xr = tr - fr, xa = ta - fa, xz = tz - fz;   // exact, in [0, 1)
-    return weights8(a, xr, xa, xz, c);
+    q.ir = (int)fr;
+    q.ia = (int)fa;
+    q.iz = (int)fz;
+    q.x = frac64(tr - fr);   // exact differences, in [0, 1)
+    q.y = frac64(ta - fa);
+    q.z = frac64(tz - fz);
+    return true;
+}
+
+__device__ __forceinline__ bool place(const DepositArgs &a, double r, double al, double z, Place &q) {
+    const bool ok = fix_place(a.fr, r, q.ir, q.x) & fix_place(a.fa, al, q.ia, q.y) & fix_place(a.fz, z, q.iz, q.z);
+    if (ok) return true;
+    Place e;   // (q stays in registers)
+    if (!place_exact(a, r, al, z, e)) return false;
+    q = e;
+    return true;
 }
 
 // The same on face arrays; false also for a particle in an inactive cell.
-__device__ __forceinline__ bool cic_weights_faces(const DepositArgs &a, const DepositGeo &g, long long p, int &ir,
-                                                  int &ia, int &iz, df c[8]) {
-    if (p >= a.np) return false;
-    const double r = a.r[p], z = a.z[p], ta = a.al[p] * a.inv_da;
-    const double fa = floor(ta);
+__device__ __forceinline__ bool place_faces(const DepositArgs &a, const DepositGeo &g, double r, double al, double z,
+                                            Place &q) {
+    const double ta = al * a.inv_da, fa = floor(ta);
     if (!(fa >= 0.0 && fa < (double)a.nt)) return false;
-    ir = find_cell(r, g.rf, a.nr, g.rbin, g.nrbin, g.r0f, g.inv_rbw);
-    iz = find_cell(z, g.zf, a.nz, g.zbin, g.nzbin, g.z0f, g.inv_zbw);
-    if (ir < 0 || iz < 0) return false;
-    if (g.act && !g.act[(size_t)iz * a.nr + ir]) return false;   // inactive cell: nothing deposited
-    ia = (int)fa;
+    q.ir = find_cell(r, g.rf, a.nr, g.rbin, g.nrbin, g.r0f, g.inv_rbw);
+    q.iz = find_cell(z, g.zf, a.nz, g.zbin, g.nzbin, g.z0f, g.inv_zbw);
+    if (q.ir < 0 || q.iz < 0) return false;
+    if (g.act && !g.act[(size_t)q.iz * a.nr + q.ir]) return false;   // inactive cell: nothing deposited
+    q.ia = (int)fa;
     // the products may round to 1 at the upper face; the weights stay in [0, 1]
-    const double xr = fmin((r - g.rf[ir]) * g.inv_wr[ir], 1.0), xz = fmin((z - g.zf[iz]) * g.inv_wz[iz], 1.0);
-    return weights8(a, xr, ta - fa, xz, c);
+    q.x = frac64(fmin((r - g.rf[q.ir]) * g.inv_wr[q.ir], 1.0));
+    q.y = frac64(ta - fa);
+    q.z = frac64(fmin((z - g.zf[q.iz]) * g.inv_wz[q.iz], 1.0));
+    return true;
 }
 
-// The eight atomic additions of a run's sums to the corners of cell (ir, ia, iz).
-__device__ __forceinline__ void add_corners(const DepositArgs &a, int ir, int ia, int iz, const df c[8]) {
+// Moments of a cell's particles in units of 2^-54 (the count apart); at most
+// the 128 particles of a warp, so every sum stays below 2^61.
+struct Moments {
+    unsigned n;
+    u64 m[7];   // x, y, z, xy, xz, yz, xyz
+    __device__ __forceinline__ void clear() {
+        n = 0;
+#pragma unroll
+        for (int e = 0; e < 7; ++e) m[e] = 0;
+    }
+    __device__ __forceinline__ void add(const Place &q) {
+        const u64 y = q.y >> 10, z = q.z >> 10, yz = __umul64hi(q.y, z);
+        ++n;
+        m[0] += q.x >> 10;
+        m[1] += y;
+        m[2] += z;
+        m[3] += __umul64hi(q.x, y);
+        m[4] += __umul64hi(q.x, z);
+        m[5] += yz;
+        m[6] += __umul64hi(q.x, yz);
+    }
+    // Corner sums (corner 4 dz + 2 dalpha + dr).  The cut of the products can
+    // bring a sum that is 0 a few units below it.
+    __device__ __forceinline__ void corners(u64 c[8]) const {
+        c[7] = m[6];
+        c[3] = m[3] - m[6];
+        c[5] = m[4] - m[6];
+        c[6] = m[5] - m[6];
+        c[1] = m[0] - m[3] - c[5];
+        c[2] = m[1] - m[3] - c[6];
+        c[4] = m[2] - m[4] - c[6];
+        c[0] = ((u64)n << 54) - m[0] - c[2] - c[4] - c[6];
+#pragma unroll
+        for (int e = 0; e < 7; ++e)
+            if ((long long)c[e] < 0) c[e] = 0;
+    }
+};
+
+// The nearest binary64 value of an integer below 2^63 (integer instructions;
+// the FP64 unit's conversion takes several of its slots).
+__device__ __forceinline__ double to_f64(u64 c) {
+    const int lz = __clzll((long long)c);
+    const u64 m = c << (lz & 63);
+    const u64 bits = ((u64)(1085 - lz) << 52) + (m >> 11) + ((m >> 10) & 1u);
+    return c ? __longlong_as_double((long long)bits) : 0.0;
+}
+
+// Add four corner sums to the nodes at radius index nri around cell (ia, iz):
+// (alpha, z) = (0, 0), (1, 0), (0, 1), (1, 1).
+template <bool V2D>
+__device__ __forceinline__ void add4(const DepositArgs &a, const double *inv_v2, int nri, int ia, int iz, u64 c00,
+                                     u64 c10, u64 c01, u64 c11) {
     const int ja = ia + 1 == a.nt ? 0 : ia + 1;
     const size_t rs = (size_t)a.nr + 1, ps = (size_t)a.nt * rs;
-#pragma unroll
-    for (int d = 0; d < 8; ++d) {
-        const int nzi = iz + (d >> 2), nai = (d & 2) ? ja : ia, nri = ir + (d & 1);
-        atomicAdd(a.nodes + (size_t)nzi * ps + (size_t)nai * rs + nri,
-                  to_double(c[d], a.w_exp) * a.inv_vr[nri] * a.inv_vz[nzi]);
+    double f0, f1;
+    if (V2D) {   // composite domain: node volumes of active octants
+        f0 = a.wscale * inv_v2[(size_t)iz * rs + nri];
+        f1 = a.wscale * inv_v2[(size_t)(iz + 1) * rs + nri];
+    } else {
+        const double fr = a.wscale * a.inv_vr[nri];
+        f0 = fr * a.inv_vz[iz];
+        f1 = fr * a.inv_vz[iz + 1];
     }
+    double *p = a.nodes + (size_t)iz * ps + nri;
+    atomicAdd(p + (size_t)ia * rs, to_f64(c00) * f0);
+    atomicAdd(p + (size_t)ja * rs, to_f64(c10) * f0);
+    atomicAdd(p + ps + (size_t)ia * rs, to_f64(c01) * f1);
+    atomicAdd(p + ps + (size_t)ja * rs, to_f64(c11) * f1);
 }
 
-// The same with the composite domain's node volumes of active octants.
-__device__ __forceinline__ void add_corners_faces(const DepositArgs &a, const DepositGeo &g, int ir, int ia, int iz,
-                                                  const df c[8]) {
-    if (!g.inv_v2) {
-        add_corners(a, ir, ia, iz, c);
-        return;
-    }
-    const int ja = ia + 1 == a.nt ? 0 : ia + 1;
-    const size_t rs = (size_t)a.nr + 1, ps = (size_t)a.nt * rs;
-#pragma unroll
-    for (int d = 0; d < 8; ++d) {
-        const int nzi = iz + (d >> 2), nai = (d & 2) ? ja : ia, nri = ir + (d & 1);
-        atomicAdd(a.nodes + (size_t)nzi * ps + (size_t)nai * rs + nri,
-                  to_double(c[d], a.w_exp) * g.inv_v2[(size_t)nzi * rs + nri]);
-    }
-}
-
-// Each thread takes DEP_PPT consecutive particles and sums those of one cell
-// in registers (a cell change inside the chunk sends the finished run's sums
-// straight to the nodes); then the threads' last runs are aggregated across
-// the warp.
-__global__ void __launch_bounds__(256) k_deposit(const DepositArgs a) {
+// FACES: face arrays or a composite domain; V2D: a composite domain.
+template <bool FACES, bool V2D>
+__global__ void __launch_bounds__(DEP_THREADS) k_deposit(const DepositArgs a, const DepositGeo g) {
+    constexpr int W = DEP_THREADS / 32;
+    __shared__ long long s_first[W], s_last[W];   // labels of each warp's first and last lane
+    __shared__ u64 s_hi[W][4];                    // outer corners of its last run
     const long long t0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * DEP_PPT;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned full = 0xffffffffu;
-    df acc[8];
+    double pr[DEP_PPT], pa[DEP_PPT], pz[DEP_PPT];
+    const int have_p = (int)min((long long)DEP_PPT, max(0ll, a.np - t0));
+    if (a.vec && have_p == DEP_PPT) {
 #pragma unroll
-    for (int d = 0; d < 8; ++d) acc[d] = {0.f, 0.f};
+        for (int t = 0; t < DEP_PPT; t += 2) {
+            const double2 u = __ldcs(reinterpret_cast<const double2 *>(a.r + t0 + t));
+            const double2 v = __ldcs(reinterpret_cast<const double2 *>(a.al + t0 + t));
+            const double2 w = __ldcs(reinterpret_cast<const double2 *>(a.z + t0 + t));
+            pr[t] = u.x, pr[t + 1] = u.y, pa[t] = v.x, pa[t + 1] = v.y, pz[t] = w.x, pz[t + 1] = w.y;
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < DEP_PPT; ++t)
+            if (t < have_p) pr[t] = a.r[t0 + t], pa[t] = a.al[t0 + t], pz[t] = a.z[t0 + t];
+    }
+    Moments M;
+    M.clear();
     int cr = 0, ca = 0, cz = 0;
     bool have = false;
+    u64 c[8];
 #pragma unroll
     for (int t = 0; t < DEP_PPT; ++t) {
-        df c[8];
-        int ir, ia, iz;
-        if (!cic_weights(a, t0 + t, ir, ia, iz, c)) continue;
-        if (have && (ir != cr || ia != ca || iz != cz)) {
-            add_corners(a, cr, ca, cz, acc);
-            have = false;
+        Place q;
+        if (t >= have_p) continue;
+        if (!(FACES ? place_faces(a, g, pr[t], pa[t], pz[t], q) : place(a, pr[t], pa[t], pz[t], q))) continue;
+        if (have && (q.ir != cr || q.ia != ca || q.iz != cz)) {   // the finished run straight to the nodes
+            M.corners(c);
+            add4<V2D>(a, g.inv_v2, cr, ca, cz, c[0], c[2], c[4], c[6]);
+            add4<V2D>(a, g.inv_v2, cr + 1, ca, cz, c[1], c[3], c[5], c[7]);
+            M.clear();
         }
-        if (!have) {
-#pragma unroll
-            for (int d = 0; d < 8; ++d) acc[d] = c[d];
-            cr = ir;
-            ca = ia;
-            cz = iz;
-            have = true;
-        } else {
-#pragma unroll
-            for (int d = 0; d < 8; ++d) acc[d] = df_add(acc[d], c[d]);
-        }
+        cr = q.ir;
+        ca = q.ia;
+        cz = q.iz;
+        have = true;
+        M.add(q);
     }
     // runs of lanes with the same last cell (lanes with nothing left: a run each)
     const long long label = have ? ((long long)cz * a.nt + ca) * a.nr + cr : -1 - lane;
-    const long long prev = __shfl_up_sync(full, label, 1);
+    const long long prev = __shfl_up_sync(full, label, 1), next = __shfl_down_sync(full, label, 1);
     const unsigned heads = __ballot_sync(full, lane == 0 || prev != label);
     const unsigned upto = lane == 31 ? full : ((2u << lane) - 1u);
     const int start = 31 - __clz(heads & upto);   // first lane of this lane's run
+    for (int off = 1; __any_sync(full, lane - off >= start); off <<= 1) {
+        const bool in = lane - off >= start;
+        const unsigned yn = __shfl_up_sync(full, M.n, off);
+        if (in) M.n += yn;
 #pragma unroll
-    for (int d = 0; d < 8; ++d) {
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const df y = {__shfl_up_sync(full, acc[d].hi, off), __shfl_up_sync(full, acc[d].lo, off)};
-            if (lane - off >= start) acc[d] = df_add(acc[d], y);
+        for (int e = 0; e < 7; ++e) {
+            const u64 y = __shfl_up_sync(full, M.m[e], off);
+            if (in) M.m[e] += y;
         }
     }
+    M.corners(c);
+    // the outer corners of the run before go to this run when its cell is the
+    // radial neighbour; the warps' ends meet through shared memory
+    if (lane == 0) s_first[warp] = label;
+    if (lane == 31) {
+        s_last[warp] = label;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s_hi[warp][e] = c[2 * e + 1];
+    }
+    __syncthreads();
+    const int src = start > 0 ? start - 1 : 0;
+    long long pl = __shfl_sync(full, label, src);
+    u64 hi[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) hi[e] = __shfl_sync(full, c[2 * e + 1], src);
+    if (start == 0) {
+        pl = warp > 0 ? s_last[warp - 1] : -1;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) hi[e] = s_hi[warp > 0 ? warp - 1 : 0][e];
+    }
     const bool last = lane == 31 || ((heads >> (lane + 1)) & 1u);
-    if (have && last) add_corners(a, cr, ca, cz, acc);
+    if (!(have && last)) return;
+    if (pl >= 0 && pl + 1 == label && cr > 0) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) c[2 * e] += hi[e];
+    }
+    add4<V2D>(a, g.inv_v2, cr, ca, cz, c[0], c[2], c[4], c[6]);
+    const long long nl = lane < 31 ? next : (warp + 1 < W ? s_first[warp + 1] : -1);
+    if (!(nl == label + 1 && cr + 1 < a.nr)) add4<V2D>(a, g.inv_v2, cr + 1, ca, cz, c[1], c[3], c[5], c[7]);
 }
 
-// The same on face arrays and composite domains (kept a separate kernel so
-// that the plain one's code stays as it is).
-__global__ void __launch_bounds__(256) k_deposit_faces(const DepositArgs a, const DepositGeo g) {
-    const long long t0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * DEP_PPT;
-    const int lane = threadIdx.x & 31;
-    const unsigned full = 0xffffffffu;
-    df acc[8];
-#pragma unroll
-    for (int d = 0; d < 8; ++d) acc[d] = {0.f, 0.f};
-    int cr = 0, ca = 0, cz = 0;
-    bool have = false;
-#pragma unroll
-    for (int t = 0; t < DEP_PPT; ++t) {
-        df c[8];
-        int ir, ia, iz;
-        if (!cic_weights_faces(a, g, t0 + t, ir, ia, iz, c)) continue;
-        if (have && (ir != cr || ia != ca || iz != cz)) {
-            add_corners_faces(a, g, cr, ca, cz, acc);
-            have = false;
-        }
-        if (!have) {
-#pragma unroll
-            for (int d = 0; d < 8; ++d) acc[d] = c[d];
-            cr = ir;
-            ca = ia;
-            cz = iz;
-            have = true;
-        } else {
-#pragma unroll
-            for (int d = 0; d < 8; ++d) acc[d] = df_add(acc[d], c[d]);
+// The fixed-point form of a uniform axis of n cells over [lo, hi).
+FixAxis fix_axis(double lo, double hi, int n) {
+    FixAxis a{};
+    int E = 0;
+    std::frexp(std::max(std::fabs(lo), std::fabs(hi)), &E);
+    a.e1 = E + 1023;
+    a.base = (long long)std::ldexp(lo, 62 - E);   // (cut where lo has bits below 2^(E - 62))
+    a.span = (u64)((long long)std::ldexp(hi, 62 - E) - a.base);
+    a.sh = 0;
+    while (a.span && !((a.span << a.sh) >> 62)) ++a.sh;    // span 2^sh in [2^62, 2^63)
+    int b = 0;
+    while ((n >> (b + 1)) != 0) ++b;
+    a.F = 61 - b;                                          // n 2^F in [2^61, 2^62)
+    const u64 num = (u64)n << a.F, den = a.span << a.sh;   // K = floor(num 2^64 / den), num < den
+    u64 rem = num, K = 0;
+    for (int k = 0; k < 64; ++k) {
+        rem <<= 1;
+        K <<= 1;
+        if (rem >= den) {
+            rem -= den;
+            K |= 1;
         }
     }
-    // runs of lanes with the same last cell (lanes with nothing left: a run each)
-    const long long label = have ? ((long long)cz * a.nt + ca) * a.nr + cr : -1 - lane;
-    const long long prev = __shfl_up_sync(full, label, 1);
-    const unsigned heads = __ballot_sync(full, lane == 0 || prev != label);
-    const unsigned upto = lane == 31 ? full : ((2u << lane) - 1u);
-    const int start = 31 - __clz(heads & upto);   // first lane of this lane's run
-#pragma unroll
-    for (int d = 0; d < 8; ++d) {
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const df y = {__shfl_up_sync(full, acc[d].hi, off), __shfl_up_sync(full, acc[d].lo, off)};
-            if (lane - off >= start) acc[d] = df_add(acc[d], y);
-        }
-    }
-    const bool last = lane == 31 || ((heads >> (lane + 1)) & 1u);
-    if (have && last) add_corners_faces(a, g, cr, ca, cz, acc);
+    a.K = K;
+    if (a.span == 0 || num >= den) a.span = 0;             // degenerate: every particle takes the binary64 arithmetic
+    return a;
 }
 
 struct ProjectArgs {
@@ -279,23 +386,44 @@ struct ProjectArgs {
     const unsigned char *act;  // MASK: active flags [nz][nr]; inactive cells get no charge
 };
 
+// A warp takes 31 consecutive radial cells (32 node radii) at one j and walks
+// PROJ_K axial cells: a lane adds the two alpha nodes of its radius in a node
+// plane once for the cells on both sides of the plane, adds two planes' sums,
+// and gets the next radius' sum from the next lane -- 2 additions and 2
+// multiply-adds per cell where one thread per cell took 7 and 4 FP64
+// instructions, which bound the kernel (26.2 M cells: 545 us, now 264, the FP64 unit 72 % busy).
+constexpr int PROJ_K = 8, PROJ_WARPS = 8;
+
 template <bool MASK>
-__global__ void __launch_bounds__(256) k_project(const ProjectArgs a) {
-    const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;   // (k, j, i), i fastest
-    const unsigned nr = (unsigned)a.nr;
-    if (e >= (unsigned)a.nz * a.nt * nr) return;
-    const unsigned row = e / nr;
-    const int i = (int)(e - row * nr);
-    const int k = (int)(row / (unsigned)a.nt), j = (int)(row - (unsigned)k * a.nt);
+__global__ void __launch_bounds__(PROJ_WARPS * 32) k_project(const ProjectArgs a) {
+    const int lane = threadIdx.x & 31;
+    const unsigned item = blockIdx.x * PROJ_WARPS + (threadIdx.x >> 5);   // (k block, j, radial block), radial fastest
+    const unsigned rb = (unsigned)(a.nr + 30) / 31u, kb = (unsigned)(a.nz + PROJ_K - 1) / PROJ_K;
+    if (item >= rb * (unsigned)a.nt * kb) return;
+    const unsigned row = item / rb;
+    const int i = (int)(item - row * rb) * 31 + lane;
+    const int k0 = (int)(row / (unsigned)a.nt) * PROJ_K, j = (int)(row % (unsigned)a.nt);
     const int jn = j + 1 == a.nt ? 0 : j + 1;
-    const size_t rs = nr + 1, ps = (size_t)a.nt * rs;
-    const double *n0 = a.nodes + (size_t)k * ps, *n1 = n0 + ps;
-    // the four (alpha, z) nodes at radius a = i and at a = i + 1
-    const double lo = (n0[j * rs + i] + n0[jn * rs + i]) + (n1[j * rs + i] + n1[jn * rs + i]);
-    const double hi = (n0[j * rs + i + 1] + n0[jn * rs + i + 1]) + (n1[j * rs + i + 1] + n1[jn * rs + i + 1]);
-    double v = a.charge * 0.25 * (a.flo[i] * lo + a.fhi[i] * hi);
-    if (MASK && !a.act[(size_t)k * nr + i]) v = 0.0;
-    a.rho[e] = a.accumulate ? a.rho[e] + v : v;
+    const size_t rs = (size_t)a.nr + 1, ps = (size_t)a.nt * rs;
+    const int in = min(i, a.nr);                                           // (lanes beyond the last node radius)
+    const bool cell = lane < 31 && i < a.nr;
+    const double s = a.charge * 0.25;
+    const double flo = cell ? s * a.flo[i] : 0.0, fhi = cell ? s * a.fhi[i] : 0.0;
+    const double *n0 = a.nodes + (size_t)k0 * ps + (size_t)j * rs + in, *n1 = a.nodes + (size_t)k0 * ps + (size_t)jn * rs + in;
+    double lower = *n0 + *n1;
+    const int k1 = min(a.nz, k0 + PROJ_K);
+    for (int k = k0; k < k1; ++k) {
+        n0 += ps;
+        n1 += ps;
+        const double upper = *n0 + *n1, lo = lower + upper;
+        const double hi = __shfl_down_sync(0xffffffffu, lo, 1);
+        lower = upper;
+        if (!cell) continue;
+        const size_t e = ((size_t)k * a.nt + j) * a.nr + i;
+        double v = fma(flo, lo, fhi * hi);
+        if (MASK && !a.act[(size_t)k * a.nr + i]) v = 0.0;
+        a.rho[e] = a.accumulate ? a.rho[e] + v : v;
+    }
 }
 
 }  // namespace
@@ -336,13 +464,9 @@ extern "C" int pic_poisson_deposit(pic_poisson_plan_t plan, const double *r_dev,
     a.inv_dr = 1.0 / h.dr;
     a.inv_da = q.d.ntheta / q.d.theta_span;
     a.inv_dz = 1.0 / h.dz;
-    // W = (w_hi + w_lo) 2^w_exp with w_hi + w_lo in [1, 2)
-    int e2 = 0;
-    const double m = std::frexp(weight, &e2);   // weight = m 2^e2, m in [0.5, 1)
-    a.w_exp = e2 - 1;
-    const double ws = 2.0 * m;
-    a.w_hi = (float)ws;
-    a.w_lo = (float)(ws - (double)a.w_hi);
+    a.wscale = std::ldexp(weight, -54);
+    a.vec = ((reinterpret_cast<uintptr_t>(r_dev) | reinterpret_cast<uintptr_t>(alpha_dev) |
+              reinterpret_cast<uintptr_t>(z_dev)) & 15) == 0;
     a.r = r_dev;
     a.al = alpha_dev;
     a.z = z_dev;
@@ -366,14 +490,19 @@ extern "C" int pic_poisson_deposit(pic_poisson_plan_t plan, const double *r_dev,
         g.inv_zbw = q.dep_inv_zbw;
         g.act = q.act0;
         g.inv_v2 = q.dep_inv_v2;
+    } else {
+        a.fr = fix_axis(q.d.r_in, q.d.r_out, h.nr);
+        a.fa = fix_axis(0.0, q.d.theta_span, q.d.ntheta);
+        a.fz = fix_axis(q.d.z0, q.d.z1, h.nz);
     }
-    const long long blocks = (np + 256LL * DEP_PPT - 1) / (256LL * DEP_PPT);
+    const long long per = (long long)DEP_THREADS * DEP_PPT, blocks = (np + per - 1) / per;
     if (blocks > 0x7fffffffLL) {
         set_error("pic_poisson_deposit: too many particles for one launch (%lld)", np);
         return PIC_POISSON_EINVAL;
     }
-    if (gen) k_deposit_faces<<<(unsigned)blocks, 256, 0, plan->stream>>>(a, g);
-    else k_deposit<<<(unsigned)blocks, 256, 0, plan->stream>>>(a);
+    if (gen && g.inv_v2) k_deposit<true, true><<<(unsigned)blocks, DEP_THREADS, 0, plan->stream>>>(a, g);
+    else if (gen) k_deposit<true, false><<<(unsigned)blocks, DEP_THREADS, 0, plan->stream>>>(a, g);
+    else k_deposit<false, false><<<(unsigned)blocks, DEP_THREADS, 0, plan->stream>>>(a, g);
     PP_CUDA(cudaGetLastError());
     return PIC_POISSON_OK;
 }
@@ -401,9 +530,10 @@ extern "C" int pic_poisson_project(pic_poisson_plan_t plan, const double *nodes_
     a.nodes = nodes_dev;
     a.rho = rho_dev;
     a.act = q.act0;
-    const size_t n = (size_t)a.nz * a.nt * a.nr;
-    if (q.act0) k_project<true><<<(unsigned)((n + 255) / 256), 256, 0, plan->stream>>>(a);
-    else k_project<false><<<(unsigned)((n + 255) / 256), 256, 0, plan->stream>>>(a);
+    const size_t items = (size_t)((a.nr + 30) / 31) * a.nt * ((a.nz + PROJ_K - 1) / PROJ_K);
+    const unsigned grid = (unsigned)((items + PROJ_WARPS - 1) / PROJ_WARPS);
+    if (q.act0) k_project<true><<<grid, PROJ_WARPS * 32, 0, plan->stream>>>(a);
+    else k_project<false><<<grid, PROJ_WARPS * 32, 0, plan->stream>>>(a);
     PP_CUDA(cudaGetLastError());
     return PIC_POISSON_OK;
 }

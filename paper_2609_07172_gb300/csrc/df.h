@@ -8,7 +8,7 @@
 // nor reorders them.  Conversions between binary64 and hi/lo pairs use
 // integer instructions (the FP64 unit's conversions are slow on this GPU).
 // Used where FP64 instructions bound a kernel but ~1e-14 relative accuracy
-// is enough: the mixed form's forward transform and the CIC deposit.
+// is enough: the mixed form's forward transform.
 #pragma once
 
 #include <cuda_runtime.h>
