@@ -252,8 +252,7 @@ int pic_poisson_set_stream(pic_poisson_plan_t plan, void *stream);
  * rho_dev and phi_dev may not alias.  `info` may be NULL.  The norms are
  * binary64 sums of squares: right-hand sides whose entries lie outside about
  * 1e-150 .. 1e150 (underflowing or overflowing squares) are not supported.
- * The mixed form computes the forward transform in double-float arithmetic
- * (b to about 1e-14 relative; its result stays within 1e-10 of the FP64 one).
+ * The mixed form's result stays within 1e-10 of the FP64 one.
  */
 int pic_poisson_solve(pic_poisson_plan_t plan, const double *rho_dev, double *phi_dev, double tol,
                       pic_poisson_info *info);

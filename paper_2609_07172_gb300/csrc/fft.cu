@@ -17,18 +17,26 @@
 // Problems of a batch may differ in size and N_theta; the dynamic shared
 // memory is sized for the largest.
 //
-// FP64 runs at 1/64 of the FP32 rate on this GPU, so the transforms are bound
-// by FP64 instructions and are written to issue few of them:
-//  * a butterfly top +- w bot with w = rho a (1 + i b) (see tw_rot) costs six
-//    multiply-adds: u = bot + i b bot (two), top +- a rho u (four) -- instead
-//    of a four-operation complex product and four additions; rho is applied
-//    with integer instructions, so no FP64 instruction depends on a branch;
-//  * the first stages, whose twiddles are 1 and -i (+i inverse), are
-//    additions only;
-//  * each thread applies two consecutive radix-2 stages to four values held
-//    in registers, halving the shared-memory round trips and barriers;
-//  * the unpack (pack) of the real transform treats modes m and M - m
-//    together, sharing one twiddle product.
+// Fixed point.  In binary64 the transforms were bound by the FP64 unit (89 %
+// busy, 12 % of the bandwidth); every value between the conversions is a 64-bit
+// integer instead (fixed.h).  A column's scale is set by the sum of its inputs'
+// magnitudes, which bounds every intermediate value: the largest integer stays
+// below 2^61 and one unit lies 2^-61 of that sum away -- for 128 inputs of equal
+// size 2^-54 of one of them -- and additions round nothing.  Against a
+// quadruple-precision transform of 8 to 256 points (plasma charge, smooth, spiked
+// and near-constant columns) the results are within 4.6e-17 to 6.1e-17 forward
+// and 1.3e-17 to 1.2e-16 inverse (relative L2), where binary64 butterflies had
+// 8.1e-17 to 2.7e-16 both ways.  A butterfly is 16 integer multiply-adds and
+// some 30 other integer instructions instead of six binary64 multiply-adds, 384
+// issue slots of a scheduler.  Each thread applies two consecutive radix-2 stages to four
+// values held in registers, halving the shared-memory round trips and barriers;
+// the unpack (pack) of the real transform treats modes m and M - m together,
+// sharing one twiddle product.  A column that holds an infinity or a NaN comes
+// out as NaN.
+// 512 x 128 x 400: forward 586 -> 312 us (with b_hat and the norm, in a solve,
+// 653 -> 330), inverse 496 -> 272 us; both now bound by integer instructions
+// and their latency (ALU pipe 44 to 48 %, three CTAs per SM).
+#include "fixed.h"
 #include "internal.h"
 
 namespace pp {
@@ -36,9 +44,10 @@ namespace {
 
 constexpr int TI = FFT_TI;
 constexpr int LD = TI + 1;   // padded row of the transform buffer (conflict-free 16-byte lanes)
+constexpr int NW = FFT_THREADS / 32;
 
-__device__ __forceinline__ int bitrev(int n, int log2M) {
-    return log2M == 0 ? 0 : (int)(__brev((unsigned)n) >> (32 - log2M));
+template <int LG> __device__ __forceinline__ int bitrev(int n) {
+    return LG == 0 ? 0 : (int)(__brev((unsigned)n) >> (32 - LG));
 }
 
 __device__ __forceinline__ int find_problem(const unsigned *__restrict__ start, int n, unsigned blk) {
@@ -51,90 +60,133 @@ __device__ __forceinline__ int find_problem(const unsigned *__restrict__ start, 
     return lo;
 }
 
-// -x when c (sign bit flipped with an integer instruction).
-__device__ __forceinline__ double flip_if(double x, bool c) {
-    return __hiloint2double(__double2hiint(x) ^ (c ? (int)0x80000000 : 0), __double2loint(x));
+struct ci {
+    fx x, y;
+};
+
+// w = e^{-i theta} (INVERSE: e^{+i theta}) as limbs of cos, -sin and +sin.
+struct Tw {
+    Limbs c, s, n;
+};
+template <bool INVERSE> __device__ __forceinline__ Tw twiddle(const int4 *__restrict__ tw, int t) {
+    const int4 u = tw[2 * t], v = tw[2 * t + 1];
+    const Limbs minus = {u.z, u.w}, plus = {v.x, v.y};   // -sin, +sin
+    return {{u.x, u.y}, INVERSE ? plus : minus, INVERSE ? minus : plus};
+}
+// w z; |z| < 2^61 in either part
+__device__ __forceinline__ ci tw_mul(const Tw &w, ci z) {
+    return {fx_mul2(z.x, w.c, z.y, w.n), fx_mul2(z.y, w.c, z.x, w.s)};
 }
 
-// v with w z = a v for the twiddle entry ab = (a, b) of w (INVERSE: of
-// conj w); rot: the entry's rotation flag (tw_rot).
-template <bool INVERSE>
-__device__ __forceinline__ double2 tw_v(double2 ab, bool rot, double2 z) {
-    const double b = INVERSE ? -ab.y : ab.y;
-    const double ux = fma(-b, z.y, z.x), uy = fma(b, z.x, z.y);   // u = z + i b z
-    // rho u with rho = -i (forward) or +i (inverse) when rot, 1 otherwise
-    const double vx = rot ? uy : ux, vy = rot ? ux : uy;
-    return make_double2(flip_if(vx, rot && INVERSE), flip_if(vy, rot && !INVERSE));
+__device__ __forceinline__ void add_sub(ci &a, ci &b) {
+    const ci x = a;
+    a = {x.x + b.x, x.y + b.y};
+    b = {x.x - b.x, x.y - b.y};
+}
+// (top, bot) <- (top + w bot, top - w bot)
+__device__ __forceinline__ void bfly(ci &top, ci &bot, const Tw &w) {
+    bot = tw_mul(w, bot);
+    add_sub(top, bot);
+}
+template <bool INVERSE> __device__ __forceinline__ ci quarter(ci z) {   // times -i (inverse: +i)
+    return INVERSE ? ci{-z.y, z.x} : ci{z.y, -z.x};
 }
 
-// Radix-2 butterfly (top, bot) <- (top + w bot, top - w bot), w = e^{-+2 pi i t / M}.
-template <bool INVERSE>
-__device__ __forceinline__ void bfly(double2 &top, double2 &bot, int t, int M, const double2 *__restrict__ tw) {
-    const double2 ab = tw[t];
-    const double2 v = tw_v<INVERSE>(ab, tw_rot(t, M), bot);
-    const double2 x = top;
-    top = make_double2(fma(ab.x, v.x, x.x), fma(ab.x, v.y, x.y));
-    bot = make_double2(fma(-ab.x, v.x, x.x), fma(-ab.x, v.y, x.y));
+__device__ __forceinline__ ci ld(const double2 *p) {
+    const longlong2 v = *reinterpret_cast<const longlong2 *>(p);
+    return {v.x, v.y};
 }
-
-__device__ __forceinline__ void add_sub(double2 &a, double2 &b) {
-    const double2 x = a;
-    a = make_double2(x.x + b.x, x.y + b.y);
-    b = make_double2(x.x - b.x, x.y - b.y);
-}
+__device__ __forceinline__ void st(double2 *p, ci z) { *reinterpret_cast<longlong2 *>(p) = make_longlong2(z.x, z.y); }
 
 // In-place radix-2 DIT FFT of length M on buf[M][LD] (bit-reversed input),
 // two stages (h, 2h) per pass on four values per thread.  The first pass
 // (or the first single stage when log2 M is odd) has twiddles 1 and -i only
-// and is done with additions.  INVERSE: conjugated twiddles.
-template <bool INVERSE>
-__device__ __forceinline__ void fft_stages(double2 *buf, const double2 *__restrict__ tw, int M, int log2M, int lane,
-                                           int warp, int nw) {
-    int h;
-    if (log2M & 1) {   // single stage h = 1
-        for (int q = warp; q < (M >> 1); q += nw) {
-            double2 a = buf[(2 * q) * LD + lane], b = buf[(2 * q + 1) * LD + lane];
+// and is done with additions.  INVERSE: conjugated twiddles.  tw: e^{-2 pi i
+// t / 2M}.  A warp's lanes hold columns, so its twiddles are uniform.
+template <bool INVERSE, int LG>
+__device__ __forceinline__ void fft_stages(double2 *buf, const int4 *__restrict__ tw, int lane, int warp) {
+    constexpr int M = 1 << LG;
+    if constexpr (LG & 1) {   // single stage h = 1
+#pragma unroll
+        for (int q0 = 0; q0 < (M >> 1); q0 += NW) {
+            const int q = q0 + warp;
+            if ((M >> 1) % NW && q >= (M >> 1)) break;
+            double2 *x = buf + 2 * q * LD + lane;
+            ci a = ld(x), b = ld(x + LD);
             add_sub(a, b);
-            buf[(2 * q) * LD + lane] = a;
-            buf[(2 * q + 1) * LD + lane] = b;
+            st(x, a);
+            st(x + LD, b);
         }
-        h = 2;
-    } else {           // stages 1 and 2: four-point DFTs
-        for (int q = warp; q < (M >> 2); q += nw) {
+    } else if constexpr (M >= 4) {   // stages 1 and 2: four-point DFTs
+#pragma unroll
+        for (int q0 = 0; q0 < (M >> 2); q0 += NW) {
+            const int q = q0 + warp;
+            if ((M >> 2) % NW && q >= (M >> 2)) break;
             double2 *x = buf + 4 * q * LD + lane;
-            double2 a0 = x[0], a1 = x[LD], a2 = x[2 * LD], a3 = x[3 * LD];
+            ci a0 = ld(x), a1 = ld(x + LD), a2 = ld(x + 2 * LD), a3 = ld(x + 3 * LD);
             add_sub(a0, a1);
             add_sub(a2, a3);
             add_sub(a0, a2);
-            a3 = INVERSE ? make_double2(-a3.y, a3.x) : make_double2(a3.y, -a3.x);   // w = -i (+i)
+            a3 = quarter<INVERSE>(a3);
             add_sub(a1, a3);
-            x[0] = a0;
-            x[LD] = a1;
-            x[2 * LD] = a2;
-            x[3 * LD] = a3;
+            st(x, a0);
+            st(x + LD, a1);
+            st(x + 2 * LD, a2);
+            st(x + 3 * LD, a3);
         }
-        h = 4;
     }
     __syncthreads();
-    for (; 4 * h <= M; h <<= 2) {
-        for (int q = warp; q < (M >> 2); q += nw) {
+#pragma unroll
+    for (int h = LG & 1 ? 2 : 4; 4 * h <= M; h <<= 2) {
+#pragma unroll 2
+        for (int q0 = 0; q0 < (M >> 2); q0 += NW) {
+            const int q = q0 + warp;
+            if ((M >> 2) % NW && q >= (M >> 2)) break;
             const int p = q & (h - 1);
             const int g = (q - p) << 2;   // (q / h) * 4h
             double2 *x = buf + (g + p) * LD + lane;
-            double2 a0 = x[0], a1 = x[h * LD], a2 = x[2 * h * LD], a3 = x[3 * h * LD];
-            const int t1 = p * (M / (2 * h));          // W_{2h}^p
-            bfly<INVERSE>(a0, a1, t1, M, tw);
-            bfly<INVERSE>(a2, a3, t1, M, tw);
-            const int t2 = p * (M / (4 * h));          // W_{4h}^p and W_{4h}^{p+h}
-            bfly<INVERSE>(a0, a2, t2, M, tw);
-            bfly<INVERSE>(a1, a3, t2 + (M >> 2), M, tw);
-            x[0] = a0;
-            x[h * LD] = a1;
-            x[2 * h * LD] = a2;
-            x[3 * h * LD] = a3;
+            ci a0 = ld(x), a1 = ld(x + h * LD), a2 = ld(x + 2 * h * LD), a3 = ld(x + 3 * h * LD);
+            const Tw w1 = twiddle<INVERSE>(tw, p * (M / h));          // W_{2h}^p
+            bfly(a0, a1, w1);
+            bfly(a2, a3, w1);
+            const Tw w2 = twiddle<INVERSE>(tw, p * (M / (2 * h)));    // W_{4h}^p; W_{4h}^{p+h} = -i (+i) times it
+            bfly(a0, a2, w2);
+            a3 = quarter<INVERSE>(tw_mul(w2, a3));
+            add_sub(a1, a3);
+            st(x, a0);
+            st(x + h * LD, a1);
+            st(x + 2 * h * LD, a2);
+            st(x + 3 * h * LD, a3);
         }
         __syncthreads();
     }
+}
+
+// Bounds of a column (lane) over the block's warps: the largest exponent
+// field, then the bits bl of the sum of magnitudes in units of 2^(em - 1043),
+// sum < 2^bl of them.  HALVES: of the larger of the two sums over the even and
+// the odd warps.  w: [FFT_THREADS / 32][32] words of shared memory each.
+__device__ __forceinline__ int column_max(int v, int *w, int lane, int warp) {
+    w[warp * 32 + lane] = v;
+    __syncthreads();
+    int m = 0;
+#pragma unroll
+    for (int q = 0; q < NW; ++q) m = max(m, w[q * 32 + lane]);
+    return m;
+}
+__device__ __forceinline__ unsigned magnitude(double x, int em) {
+    return ((((unsigned)__double2hiint(x) & 0xfffffu) | 0x100000u) >> min(em - f64_exp(x), 31)) + 1u;
+}
+template <bool HALVES> __device__ __forceinline__ int column_bits(unsigned v, int *w, int lane, int warp) {
+    w[warp * 32 + lane] = (int)v;
+    __syncthreads();
+    unsigned s0 = 0, s1 = 0;
+#pragma unroll
+    for (int q = 0; q < NW; q += 2) {
+        s0 += (unsigned)w[q * 32 + lane];
+        s1 += (unsigned)w[q * 32 + 32 + lane];
+    }
+    return 32 - __clz((int)(HALVES ? max(s0, s1) : s0 + s1));
 }
 
 // Sum of v over the block, valid in thread 0; sh holds blockDim doubles.  The
@@ -153,85 +205,104 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
     return s;
 }
 
-__global__ void __launch_bounds__(FFT_THREADS) k_forward(const FFTTab *__restrict__ tab, double *__restrict__ partials) {
-    extern __shared__ double2 sm[];
-    __shared__ double red[FFT_THREADS];
-    const int pr = find_problem(tab->start, tab->n, blockIdx.x);
-    const FFTProb P = tab->p[pr];
-    const int nr = P.nr, nt = P.nt, nz = P.nz;
-    const int M = nt >> 1, nm = M + 1;
+// LG = log2 M: the loops' bounds and the shared-memory offsets are constants.
+template <int LG>
+__device__ __forceinline__ void forward_body(const FFTProb &P, int lb, double2 *sm, double *red, int *wmax, int *wsum,
+                                             double *__restrict__ partials) {
+    constexpr int M = 1 << LG, nt = 2 * M, nm = M + 1;
+    const int nr = P.nr, nz = P.nz;
     double2 *buf = sm;              // [M][LD]
     double2 *outb = sm + M * LD;    // [TI][nm]
 
     const int tiles = (nr + TI - 1) / TI;
-    const int lb = (int)(blockIdx.x - tab->start[pr]);
     const int k = lb / tiles;
     const int i0 = (lb - k * tiles) * TI;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = i0 + lane;
     const bool valid = i < nr;
 
     const double *src = P.rho + (size_t)k * nt * nr + i;
-    for (int n = warp; n < M; n += nw) {
+    int em = 0;
+#pragma unroll 4
+    for (int n = warp; n < M; n += NW) {
         double a = 0.0, b = 0.0;
         if (valid) {
             a = src[(size_t)(2 * n) * nr];
             b = src[(size_t)(2 * n + 1) * nr];
         }
-        buf[bitrev(n, P.log2M) * LD + lane] = make_double2(a, b);
+        em = max(em, max(f64_exp(a), f64_exp(b)));
+        buf[bitrev<LG>(n) * LD + lane] = make_double2(a, b);
+    }
+    em = column_max(em, wmax, lane, warp);
+    unsigned mag = 0;
+#pragma unroll 4
+    for (int n = warp; n < M; n += NW) {   // (a thread's own entries: no barrier between these passes)
+        const double2 v = buf[bitrev<LG>(n) * LD + lane];
+        mag += magnitude(v.x, em) + magnitude(v.y, em);
+    }
+    const int bl = column_bits<false>(mag, wsum, lane, warp);
+#pragma unroll 4
+    for (int n = warp; n < M; n += NW) {
+        double2 *e = buf + bitrev<LG>(n) * LD + lane;
+        const double2 v = *e;
+        // sum of magnitudes < 2^61
+        st(e, {f64_to_fx(v.x, em - f64_exp(v.x) + bl - 19), f64_to_fx(v.y, em - f64_exp(v.y) + bl - 19)});
     }
     __syncthreads();
-    fft_stages<false>(buf, (const double2 *)P.tw, M, P.log2M, lane, warp, nw);
+    fft_stages<false, LG>(buf, P.tw, lane, warp);
 
     // Unpack, modes m and M - m together (W = e^{-2 pi i / N}, hs = s_i / (2N)):
     //   S = Z_m + conj Z_{M-m},  D = Z_m - conj Z_{M-m},  T = W^m D,
     //   X_m = hs (S - i T),  X_{M-m} = hs conj(S + i T);
     // X_0 = 2 hs (Re Z_0 + Im Z_0), X_M = 2 hs (Re Z_0 - Im Z_0), both exactly real.
-    const double2 *tw2 = (const double2 *)P.tw2;
+    // |S - i T| = 2 |sum of the inputs times roots of unity| < 2^62; D is halved
+    // for the product.  hs multiplies as a 63-bit mantissa.
     // s_i, or per cell in a composite domain (zero outside its patches)
     const size_t si = valid ? (P.s_rows ? (size_t)k * nr + i : (size_t)i) : 0;
     const double hs = (P.s ? P.s[si] : 1.0) * P.half_inv_n;
+    const fx hm = f64_exp(hs) ? (hs < 0.0 ? -(fx)f64_mant(hs) : (fx)f64_mant(hs)) : 0;
+    const int be = em + bl - 18 + f64_exp(hs) - 1021;     // biased exponent of r hm = 2^63 2^64
+    const bool bad = em == 0x7ff;
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    auto out = [&](fx r, int e) { return bad ? nan : fx_to_f64(__mul64hi(r, hm), e); };
     double acc_in = 0.0, acc_edge = 0.0;   // Parseval weight 2 (0 < m < M) and 1 (m = 0, M)
     double2 *ob = outb + lane * nm;
-    for (int m = 1 + warp; 2 * m < M; m += nw) {
-        const double2 A = buf[m * LD + lane], B = buf[(M - m) * LD + lane];
-        const double2 S = make_double2(hs * (A.x + B.x), hs * (A.y - B.y));
-        const double2 D = make_double2(A.x - B.x, A.y + B.y);
-        const double2 ab = tw2[m];
-        const double2 v = tw_v<false>(ab, tw_rot(m, nt), D);   // T = ab.x v
-        const double g = hs * ab.x;
-        const double2 xm = make_double2(fma(g, v.y, S.x), fma(-g, v.x, S.y));
-        const double2 xp = make_double2(fma(-g, v.y, S.x), -fma(g, v.x, S.y));
+    for (int m = 1 + warp; 2 * m < M; m += NW) {
+        const ci A = ld(buf + m * LD + lane), B = ld(buf + (M - m) * LD + lane);
+        const ci S = {A.x + B.x, A.y - B.y};
+        const ci T = tw_mul(twiddle<false>(P.tw, m), {(A.x - B.x) >> 1, (A.y + B.y) >> 1});   // W^m D / 2
+        const double2 xm = make_double2(out(S.x + 2 * T.y, be), out(S.y - 2 * T.x, be));
+        const double2 xp = make_double2(out(S.x - 2 * T.y, be), out(-S.y - 2 * T.x, be));
         ob[m] = xm;
         ob[M - m] = xp;
         acc_in = fma(xm.x, xm.x, fma(xm.y, xm.y, acc_in));
         acc_in = fma(xp.x, xp.x, fma(xp.y, xp.y, acc_in));
     }
     if (warp == 0) {
-        const double2 z = buf[lane];
-        double x0 = (z.x + z.y) * (2.0 * hs);
-        const double xM = (z.x - z.y) * (2.0 * hs);
+        const ci z = ld(buf + lane);
+        double x0 = out(z.x + z.y, be + 1);
+        const double xM = out(z.x - z.y, be + 1);
         if (P.bD && valid) x0 += P.bD[(size_t)k * nr + i];
         acc_edge = fma(x0, x0, fma(xM, xM, acc_edge));
         ob[0] = make_double2(x0, 0.0);
         ob[M] = make_double2(xM, 0.0);
     }
-    if (M >= 2 && warp == nw - 1) {   // m = M/2 pairs with itself: X = 2 hs conj Z
-        const double2 z = buf[(M >> 1) * LD + lane];
-        const double2 x = make_double2((2.0 * hs) * z.x, -(2.0 * hs) * z.y);
+    if (M >= 2 && warp == NW - 1) {   // m = M/2 pairs with itself: X = 2 hs conj Z
+        const ci z = ld(buf + (M >> 1) * LD + lane);
+        const double2 x = make_double2(out(z.x, be + 1), out(-z.y, be + 1));
         ob[M >> 1] = x;
         acc_in = fma(x.x, x.x, fma(x.y, x.y, acc_in));
     }
     __syncthreads();
     const int ncols = min(TI, nr - i0);
     double2 *dst = P.b + ((size_t)k * nr + i0) * nm;
-    for (int f = threadIdx.x; f < ncols * nm; f += blockDim.x) dst[f] = outb[f];
+    for (int f = threadIdx.x; f < ncols * nm; f += FFT_THREADS) dst[f] = outb[f];
     if (P.bh && P.invd) {
         // b_hat = b / diag for the smoother (row class of plane k, cells i0.., all modes)
         const int cls = P.rcls ? P.rcls[k] : (k == 0 ? 0 : (k == nz - 1 ? P.ncls - 1 : 1));
         const double *inv = P.invd + ((size_t)cls * nr + i0) * nm;
         double2 *dh = P.bh + ((size_t)k * nr + i0) * nm;
-        for (int f = threadIdx.x; f < ncols * nm; f += blockDim.x) {
+        for (int f = threadIdx.x; f < ncols * nm; f += FFT_THREADS) {
             const double2 x = outb[f];
             const double v = inv[f];
             dh[f] = make_double2(x.x * v, x.y * v);
@@ -243,63 +314,117 @@ __global__ void __launch_bounds__(FFT_THREADS) k_forward(const FFTTab *__restric
     }
 }
 
-__global__ void __launch_bounds__(FFT_THREADS) k_inverse(const FFTTab *__restrict__ tab) {
-    extern __shared__ double2 sm[];
-    const int pr = find_problem(tab->start, tab->n, blockIdx.x);
-    const FFTProb P = tab->p[pr];
-    const int nr = P.nr, nt = P.nt;
-    const int M = nt >> 1, nm = M + 1;
+template <int LG>
+__device__ __forceinline__ void inverse_body(const FFTProb &P, int lb, double2 *sm, int *wmax, int *wsum) {
+    constexpr int M = 1 << LG, nt = 2 * M, nm = M + 1;
+    const int nr = P.nr;
     double2 *buf = sm;              // [M][LD]
     double2 *inb = sm + M * LD;     // [TI][nm]
 
     const int tiles = (nr + TI - 1) / TI;
-    const int lb = (int)(blockIdx.x - tab->start[pr]);
     const int k = lb / tiles;
     const int i0 = (lb - k * tiles) * TI;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = i0 + lane;
     const bool valid = i < nr;
     const int ncols = min(TI, nr - i0);
 
     const double2 *src = P.uhat + ((size_t)k * nr + i0) * nm;
-    for (int f = threadIdx.x; f < TI * nm; f += blockDim.x)
+    for (int f = threadIdx.x; f < TI * nm; f += FFT_THREADS)
         inb[f] = f < ncols * nm ? src[f] : make_double2(0.0, 0.0);
     __syncthreads();
+
+    // The column's bounds; X_0 and X_M enter through their real parts only.
+    const double2 *ib = inb + lane * nm;
+    int em = 0;
+    for (int m = warp; m <= M; m += NW) {
+        const double2 x = ib[m];
+        em = max(em, max(f64_exp(x.x), m == 0 || m == M ? 0 : f64_exp(x.y)));
+    }
+    em = column_max(em, wmax, lane, warp);
+    unsigned mag = 0;
+    for (int m = warp; m <= M; m += NW) {
+        const double2 x = ib[m];
+        mag += magnitude(x.x, em) + (m == 0 || m == M ? 0u : magnitude(x.y, em));
+    }
+    const int bl = column_bits<true>(mag, wsum, lane, warp);
+    // Sums of magnitudes of the even and of the odd modes < 2^59 (a warp's modes
+    // have its parity, and so do m and M - m): the packed values of one parity and
+    // their partial sums, all that a twiddle multiplies, stay below 2^61, the
+    // last stage's sums of both below 2^62.
+    auto in = [&](double v) { return f64_to_fx(v, em - f64_exp(v) + bl - 17); };
 
     // Pack, modes m and M - m together (w = e^{+2 pi i / N}):
     //   S = X_m + conj X_{M-m},  D = X_m - conj X_{M-m},  T = w^m D,
     //   Z_m = S + i T,  Z_{M-m} = conj(S - i T);
-    // X_0 and X_M enter through their real parts only: Z_0 = (X_0 + X_M) + i (X_0 - X_M).
-    const double2 *tw2 = (const double2 *)P.tw2;
-    const double2 *ib = inb + lane * nm;
-    for (int m = 1 + warp; 2 * m < M; m += nw) {
-        const double2 A = ib[m], B = ib[M - m];
-        const double2 S = make_double2(A.x + B.x, A.y - B.y);
-        const double2 D = make_double2(A.x - B.x, A.y + B.y);
-        const double2 ab = tw2[m];
-        const double2 v = tw_v<true>(ab, tw_rot(m, nt), D);   // T = ab.x v
-        buf[bitrev(m, P.log2M) * LD + lane] = make_double2(fma(-ab.x, v.y, S.x), fma(ab.x, v.x, S.y));
-        buf[bitrev(M - m, P.log2M) * LD + lane] = make_double2(fma(ab.x, v.y, S.x), fma(ab.x, v.x, -S.y));
+    // Z_0 = (X_0 + X_M) + i (X_0 - X_M).
+    for (int m = 1 + warp; 2 * m < M; m += NW) {
+        const double2 a = ib[m], b = ib[M - m];
+        const ci A = {in(a.x), in(a.y)}, B = {in(b.x), in(b.y)};
+        const ci S = {A.x + B.x, A.y - B.y};
+        const ci T = tw_mul(twiddle<true>(P.tw, m), {A.x - B.x, A.y + B.y});
+        st(buf + bitrev<LG>(m) * LD + lane, {S.x - T.y, S.y + T.x});
+        st(buf + bitrev<LG>(M - m) * LD + lane, {S.x + T.y, T.x - S.y});
     }
     if (warp == 0) {
-        const double a = ib[0].x, b = ib[M].x;
-        buf[lane] = make_double2(a + b, a - b);
+        const fx a = in(ib[0].x), b = in(ib[M].x);
+        st(buf + lane, {a + b, a - b});
     }
-    if (M >= 2 && warp == nw - 1) {   // m = M/2 pairs with itself: Z = 2 conj X
+    if (M >= 2 && warp == NW - 1) {   // m = M/2 pairs with itself: Z = 2 conj X
         const double2 x = ib[M >> 1];
-        buf[bitrev(M >> 1, P.log2M) * LD + lane] = make_double2(x.x + x.x, -(x.y + x.y));
+        st(buf + bitrev<LG>(M >> 1) * LD + lane, {2 * in(x.x), -2 * in(x.y)});
     }
     __syncthreads();
-    fft_stages<true>(buf, (const double2 *)P.tw, M, P.log2M, lane, warp, nw);
+    fft_stages<true, LG>(buf, P.tw, lane, warp);
 
     if (valid) {
+        const int be = em + bl - 16;
+        const bool bad = em == 0x7ff;
+        const double nan = __longlong_as_double(0x7ff8000000000000ll);
         double *dst = P.phi + (size_t)k * nt * nr + i;
-        for (int n = warp; n < M; n += nw) {
-            const double2 z = buf[n * LD + lane];
-            dst[(size_t)(2 * n) * nr] = z.x;
-            dst[(size_t)(2 * n + 1) * nr] = z.y;
+    #pragma unroll 4
+    for (int n = warp; n < M; n += NW) {
+            const ci z = ld(buf + n * LD + lane);
+            dst[(size_t)(2 * n) * nr] = bad ? nan : fx_to_f64(z.x, be);
+            dst[(size_t)(2 * n + 1) * nr] = bad ? nan : fx_to_f64(z.y, be);
         }
     }
+}
+
+// One instantiation per azimuthal size of a batch's problems.
+#define PP_FFT_SWITCH(CALL)            \
+    switch (P.log2M) {                 \
+    case 0: CALL(0); break;            \
+    case 1: CALL(1); break;            \
+    case 2: CALL(2); break;            \
+    case 3: CALL(3); break;            \
+    case 4: CALL(4); break;            \
+    case 5: CALL(5); break;            \
+    case 6: CALL(6); break;            \
+    default: CALL(7); break;           \
+    }
+
+__global__ void __launch_bounds__(FFT_THREADS, 3) k_forward(const FFTTab *__restrict__ tab, double *__restrict__ partials) {
+    extern __shared__ double2 sm[];
+    __shared__ double red[FFT_THREADS];
+    __shared__ int wmax[FFT_THREADS], wsum[FFT_THREADS];
+    const int pr = find_problem(tab->start, tab->n, blockIdx.x);
+    const FFTProb P = tab->p[pr];
+    const int lb = (int)(blockIdx.x - tab->start[pr]);
+#define PP_CALL(LG) forward_body<LG>(P, lb, sm, red, wmax, wsum, partials)
+    PP_FFT_SWITCH(PP_CALL)
+#undef PP_CALL
+}
+
+__global__ void __launch_bounds__(FFT_THREADS, 3) k_inverse(const FFTTab *__restrict__ tab) {
+    extern __shared__ double2 sm[];
+    __shared__ int wmax[FFT_THREADS], wsum[FFT_THREADS];
+    const int pr = find_problem(tab->start, tab->n, blockIdx.x);
+    const FFTProb P = tab->p[pr];
+    const int lb = (int)(blockIdx.x - tab->start[pr]);
+#define PP_CALL(LG) inverse_body<LG>(P, lb, sm, wmax, wsum)
+    PP_FFT_SWITCH(PP_CALL)
+#undef PP_CALL
 }
 
 // Mode-layout initial iterate: b = guess, each CTA copying the cells of its

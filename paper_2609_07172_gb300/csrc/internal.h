@@ -165,9 +165,7 @@ struct DefectTab {                // mixed precision: FP64 level 0 and FP32 leve
 // Azimuthal transforms of one problem's finest level.
 struct FFTProb {
     int nr, nt, nz, nm, ncls, log2M;
-    const double *tw;             // [max(M/2,1)] e^{-2 pi i t / M}, M = nt / 2, as (scale, ratio) pairs
-    const double *tw2;            // [M+1] e^{-2 pi i m / nt}, same form (see tw_rot)
-    const float4 *twf, *tw2f;     // the same tables in double-float, (a_hi, a_lo, b_hi, b_lo)
+    const int4 *tw;               // [M+1][2] e^{-2 pi i m / nt}, M = nt / 2: limbs (fixed.h) of cos, -sin; +sin, 0
     double half_inv_n;            // 1 / (2 nt)
     const double *s;              // [nr] s_i (Eq. mode_rhs), [nz][nr] when s_rows; null: plain 1/N transform
     int s_rows;                   // composite domain: s per cell, 0 outside the patches
@@ -239,8 +237,6 @@ struct PsumTab {
 // table's total block count (start[n]); tables live in device memory.
 cudaError_t launch_forward(const FFTTab *tab, unsigned grid, size_t smem, double *partials, cudaStream_t st);
 cudaError_t launch_inverse(const FFTTab *tab, unsigned grid, size_t smem, cudaStream_t st);
-// The forward transform in double-float arithmetic (fft_df.cu), for the mixed form.
-cudaError_t launch_forward_df(const FFTTab *tab, unsigned grid, size_t smem, double *partials, cudaStream_t st);
 // b = guess for every problem of the table (mode-layout initial iterates).
 cudaError_t launch_copy_guess(const FFTTab *tab, unsigned grid, cudaStream_t st);
 
@@ -417,15 +413,6 @@ __device__ __forceinline__ void thomas_rows(T *ws, const T *ps, const T *cs, con
 constexpr int FFT_TI = 32;        // radial columns per transform CTA
 constexpr int FFT_THREADS = 256;
 size_t fft_smem_bytes(int nt);
-
-// Twiddle tables of the transforms hold w = e^{-i theta}, theta = 2 pi t / n,
-// as a scale and a ratio: w = rho a (1 + i b) with a = cos theta', b =
-// -tan theta', theta' = theta - rot pi/2 and rho = (-i)^rot, where rot = 1
-// for theta in (pi/4, 3 pi/4) keeps |b| <= 1.  A complex product w z then
-// costs two multiply-adds, u = z + i b z, plus the scale a, which folds into
-// the butterfly's own multiply-adds; the factor rho is a swap of the parts
-// of u and a sign, done with integer instructions.
-__host__ __device__ inline bool tw_rot(int t, int n) { return !(8 * t <= n || 8 * t >= 3 * n); }
 
 // 3x3 convolution on the tcgen05 tensor cores (conv_tc.cu): 0 on success, 1
 // when the shape or alignment is not taken (run the mma.sync kernel), else a

@@ -749,10 +749,7 @@ void carve(pic_poisson_plan_s &P, Carver &c) {
         if (mixed) carve_coarse(q, c, q.cf);
         else carve_coarse(q, c, q.cd);
         const int M = nt / 2;
-        q.tw = (const double *)c.take<double2>(std::max(M / 2, 1));
-        q.tw2 = (const double *)c.take<double2>(M + 1);
-        q.twf = c.take<float4>(std::max(M / 2, 1));
-        q.tw2f = c.take<float4>(M + 1);
+        q.tw = c.take<int4>(2 * (size_t)(M + 1));
         q.s0 = c.take<double>(q.lv[0].act.empty() ? q.lv[0].nr : (size_t)q.lv[0].nr * q.lv[0].nz);
         q.bD0 = c.take<double>((size_t)q.lv[0].nr * q.lv[0].nz);
         q.mask0 = q.lv[0].act.empty() ? nullptr : c.take<double>((size_t)q.lv[0].nr * q.lv[0].nz);
@@ -1071,28 +1068,19 @@ int upload(pic_poisson_plan_s &P) {
             else put(q.cf);
         }
         const int nt = q.d.ntheta, M = nt / 2;
-        std::vector<double> tw(2 * std::max(M / 2, 1), 0.0), tw2(2 * (M + 1), 0.0);
-        auto scale_ratio = [](double *out, int t, int n) {   // e^{-2 pi i t / n} as (a, b), see tw_rot
-            const double th = 2.0 * kPi * t / n - (tw_rot(t, n) ? 0.5 * kPi : 0.0);
-            out[0] = std::cos(th);
-            out[1] = -std::tan(th);
-        };
-        for (int t = 0; t < M / 2; ++t) scale_ratio(&tw[2 * t], t, M);
-        if (M / 2 == 0) tw[0] = 1.0;
-        for (int m = 0; m <= M; ++m) scale_ratio(&tw2[2 * m], m, nt);
-        to_dev(tw, q.tw, st, err);
-        to_dev(tw2, q.tw2, st, err);
-        // double-float copies: each binary64 entry as hi = its binary32 rounding, lo = the rest rounded
-        auto split = [](const std::vector<double> &v) {   // binary32 values, held exactly in binary64
-            std::vector<double> f(2 * v.size());
-            for (size_t e = 0; e < v.size(); ++e) {
-                f[2 * e] = (double)(float)v[e];
-                f[2 * e + 1] = (double)(float)(v[e] - f[2 * e]);
-            }
-            return f;
-        };
-        to_dev(split(tw), (float *)q.twf, st, err);
-        to_dev(split(tw2), (float *)q.tw2f, st, err);
+        std::vector<int> tw(8 * (size_t)(M + 1), 0);   // e^{-2 pi i m / nt} in limbs
+        for (int m = 0; m <= M; ++m) {
+            auto limbs = [&](long double v, int *o) {
+                const long long f = std::llrintl(std::ldexp(v, 61));
+                o[0] = (int)(f >> 31);
+                o[1] = (int)(f & 0x7fffffff);
+            };
+            const long double th = 2.0L * acosl(-1.0L) * m / nt;
+            limbs(cosl(th), &tw[8 * m]);
+            limbs(-sinl(th), &tw[8 * m + 2]);
+            limbs(sinl(th), &tw[8 * m + 4]);
+        }
+        ints_to_dev(tw, (const int *)q.tw, st, err);
         // level-0 right-hand-side factors: s_i (Eq. mode_rhs) and b^D (Eq. boundary_rhs_appendix)
         const LevelHost &h = q.lv[0];
         std::vector<double> s(h.nr), bD((size_t)h.nr * h.nz, 0.0);
@@ -1244,9 +1232,6 @@ int upload(pic_poisson_plan_s &P) {
         while ((1 << lg) < q.d.ntheta / 2) ++lg;
         fp.log2M = lg;
         fp.tw = q.tw;
-        fp.tw2 = q.tw2;
-        fp.twf = q.twf;
-        fp.tw2f = q.tw2f;
         fp.half_inv_n = 0.5 / q.d.ntheta;
         FFTProb f = fp, g = fp, iv = fp;
         f.s = q.s0;
