@@ -82,7 +82,6 @@ template <class T>
 __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom(const BottomTab<T> *__restrict__ tab) {
     extern __shared__ unsigned char smraw[];
     const int p = find_problem(tab->start, tab->n, blockIdx.x);
-    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
     const BottomProb<T> &B = tab->p[p];
     const LevelDev<T> &U = B.U;
     const CoarseDev<T> &D = B.D;
@@ -114,20 +113,27 @@ __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom(const BottomTab<T> *_
     T *es = cs + ncz * lw;
 
     // Every load of the block is issued at once (cp.async) in two groups: what
-    // the pre-smoothing reads (b_hat, the smoother's tables), then what only
-    // the restriction and the coarsest solve read (b -- of the red cells when
-    // only those carry a residual -- the residual's tables, V and this mode's
-    // factorisation), which arrives while the pre-smoothing runs.
+    // the pre-smoothing reads (the smoother's tables, before the wait for the
+    // kernel before, and b_hat), then what only the restriction and the coarsest
+    // solve read (b -- of the red cells when only those carry a residual -- the
+    // residual's tables, V and this mode's factorisation), which arrives while
+    // the pre-smoothing runs.
     const T *gb = (const T *)U.b + part, *gbh = (const T *)U.bh + part;
-    for (int f = threadIdx.x; f < n; f += blockDim.x) {
-        cp_async_elem(bh + f, gbh + 2 * ((size_t)f * nm + m));
-        u[f] = 0;
-    }
     for (int f = threadIdx.x; f < ncls * nr; f += blockDim.x) {
         const size_t t = (size_t)f * nm + m;   // (class, i) -> ((class * nr + i) * nm + m)
         cp_async_elem(hz + f, U.hz + t);
         cp_async_elem(hw + f, U.hw + t);
         cp_async_elem(he + f, U.he + t);
+    }
+    pdl_wait();
+    pdl_go();
+    if (tab->done && tab->done[tab->pid[p]]) {   // stopped problem of a batch
+        cp_async_wait_all();
+        return;
+    }
+    for (int f = threadIdx.x; f < n; f += blockDim.x) {
+        cp_async_elem(bh + f, gbh + 2 * ((size_t)f * nm + m));
+        u[f] = 0;
     }
     cp_async_group_close();
     if (B.red_only) {
@@ -279,8 +285,7 @@ template <class T> size_t bottom_smem_bytes(int nr, int nz, int ncls, int ncr, i
 template <class T> cudaError_t launch_bottom(const BottomTab<T> *tab, unsigned grid, size_t smem, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(k_bottom<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_bottom<T><<<grid, BOTTOM_THREADS, smem, st>>>(tab);
-    return cudaGetLastError();
+    return launch_pdl(k_bottom<T>, grid, BOTTOM_THREADS, smem, st, tab);
 }
 
 template size_t bottom_smem_bytes<double>(int, int, int, int, int);

@@ -46,9 +46,11 @@ template <class T>
 __global__ void __launch_bounds__(DENSE_THREADS) k_dense_prep(const DenseTab<T> *__restrict__ tab) {
     __shared__ int s_emax;
     const int p = find_problem(tab->start, tab->n, blockIdx.x);
-    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
     const LevelDev<T> &L = tab->f[p];
     const CoarseDev<T> &D = tab->c[p];
+    pdl_wait();
+    pdl_go();
+    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
     const int col = (int)(blockIdx.x - tab->start[p]);
     const int m = col >> 1, comp = col & 1, nm = D.nm, n = D.nact;
     const T *bg = (const T *)L.b + comp;
@@ -94,7 +96,6 @@ __global__ void __launch_bounds__(DENSE_THREADS) k_dense_gemm(const DenseTab<T> 
     __shared__ float As[TR][TK + 1];
     __shared__ __align__(16) float Bs[TK][TC + 4];
     const int p = find_problem(tab->gstart, tab->n, blockIdx.x);
-    if (tab->done && tab->done[tab->pid[p]]) return;
     const LevelDev<T> &L = tab->f[p];
     const CoarseDev<T> &D = tab->c[p];
     const int n = D.nact, ncol = 2 * D.nm;
@@ -121,6 +122,9 @@ __global__ void __launch_bounds__(DENSE_THREADS) k_dense_gemm(const DenseTab<T> 
             rb[i] = (gc < ncol && gk < n) ? __ldg(B + (size_t)gc * n + gk) : 0.f;
         }
     };
+    pdl_wait();
+    pdl_go();
+    if (tab->done && tab->done[tab->pid[p]]) return;
     load(0);
     for (int k0 = 0; k0 < n; k0 += TK) {
 #pragma unroll
@@ -168,11 +172,10 @@ unsigned dense_gemm_blocks(int nact, int nm) {
 template <class T>
 cudaError_t launch_dense(const DenseTab<T> *tab, int stage, unsigned g_prep, unsigned g_gemm, cudaStream_t st) {
     switch (stage) {
-    case 0: k_dense_prep<T><<<g_prep, DENSE_THREADS, 0, st>>>(tab); break;
-    case 1: k_dense_gemm<T, 1><<<g_gemm, DENSE_THREADS, 0, st>>>(tab); break;
-    default: k_dense_gemm<T, 2><<<g_gemm, DENSE_THREADS, 0, st>>>(tab); break;
+    case 0: return launch_pdl(k_dense_prep<T>, g_prep, DENSE_THREADS, 0, st, tab);
+    case 1: return launch_pdl(k_dense_gemm<T, 1>, g_gemm, DENSE_THREADS, 0, st, tab);
+    default: return launch_pdl(k_dense_gemm<T, 2>, g_gemm, DENSE_THREADS, 0, st, tab);
     }
-    return cudaGetLastError();
 }
 
 template cudaError_t launch_dense<double>(const DenseTab<double> *, int, unsigned, unsigned, cudaStream_t);

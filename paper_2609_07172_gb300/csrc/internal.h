@@ -129,6 +129,24 @@ template <class T> struct LaunchTab {
     LevelDev<T> c[kMaxBatch];
 };
 
+// What a launch over a table gets: the table and, for a plan of one problem,
+// its entry by value.  The kernel then reads the level views from its own
+// parameters (constant bank) instead of through three dependent loads, and
+// keeps none of them in registers: the restriction of every cell on a stretched
+// axial mesh needs 48 registers instead of 80 (4.0 -> 2.0 ms per mixed solve at
+// 512 x 128 x 400, the whole solve 11.7 -> 9.1 ms).
+template <class T> struct LevelArg {
+    const LaunchTab<T> *tab;
+    LevelDev<T> f, c;
+};
+template <class T> struct TabRef {
+    LaunchTab<T> *tab = nullptr;  // device (null when no problem takes part)
+    bool one = false;             // plan of one problem: f and c below are its entry
+    LevelDev<T> f{}, c{};
+    explicit operator bool() const { return tab != nullptr; }
+    LevelArg<T> arg() const { return {tab, f, c}; }
+};
+
 template <class T> struct CoarseTab {
     int n;
     const int *done;
@@ -225,12 +243,46 @@ struct Ctrl {
 // block) adds a few dozen numbers instead of tens of thousands -- on one SM
 // the FP64 additions alone took longer than the rest of the test.
 constexpr int PSUM_CHUNK = 2048;
+constexpr unsigned PSUM_MIN = 4096;   // partials below which the test adds them itself
 struct PsumTab {
     int n;
     unsigned start[kMaxBatch + 1];    // blocks (chunks) of problem p: [start[p], start[p+1])
     unsigned in_begin[kMaxBatch];     // its first-level partials
     unsigned in_end[kMaxBatch];
 };
+
+// ------------------------------------------------------------------ overlapped launches
+// The solve's kernels are launched so that a kernel's blocks may start while
+// the one before still runs (programmatic dependent launch): they read their
+// launch table and level view -- written at plan time -- and work out their
+// indices, then pdl_wait() blocks until the kernel before has completed and
+// its writes are visible.  Nothing a kernel of the solve writes is read before
+// that.  pdl_go(), after the wait, lets the next kernel start likewise.  Most
+// kernels below level 0 run for 2 to 4 us, of which launch, table reads and
+// index arithmetic were more than half.  With the level views by value (LevelArg)
+// and overlapped launches: 32 x 16 x 32 in one graph 632 -> 534 us, 152 x 32 x 90
+// from the host 1,393 -> 1,002 us, channel-plume 256 x 64 x 192 3,170 -> 2,700 us;
+// of these the views alone give 592, 1,308 and 2,812 us.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+constexpr size_t PDL_MAX_THREADS = size_t(152) * 2048;
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    // a launch of several waves hides its own start, and blocks that wait early
+    // only take room from the ones at work
+    const bool overlap = (size_t)grid * block <= (size_t)PDL_MAX_THREADS;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
 
 // ------------------------------------------------------------------ launchers
 // All launchers enqueue on `st` and return cudaGetLastError().  `grid` is the
@@ -244,7 +296,7 @@ cudaError_t launch_copy_guess(const FFTTab *tab, unsigned grid, cudaStream_t st)
 // ranges must have been computed with the same size).
 // strip: see pic_poisson_desc.smooth_strip; sor: over-relaxed update (omega != 1).
 template <class T>
-cudaError_t launch_smooth(const LaunchTab<T> *tab, unsigned grid, int color, int threads, int strip, bool sor,
+cudaError_t launch_smooth(const TabRef<T> &tab, unsigned grid, int color, int threads, int strip, bool sor,
                           cudaStream_t st, bool rowwise = false);
 // red_only: residual of the red fine cells only (valid right after a black half-sweep).
 // Per problem, f.init selects what is written into the coarse level c: 0 = b only
@@ -254,7 +306,7 @@ cudaError_t launch_smooth(const LaunchTab<T> *tab, unsigned grid, int color, int
 // non-uniform axial mesh (class tables per row, no residual or correction
 // outside the patches); false runs the plain kernels.
 template <class T>
-cudaError_t launch_residual_restrict(const LaunchTab<T> *tab, unsigned grid, bool red_only, double *partials,
+cudaError_t launch_residual_restrict(const TabRef<T> &tab, unsigned grid, bool red_only, double *partials,
                                      cudaStream_t st, bool masked = false);
 // r = b - A_m u on level f of every problem (r_out: optional per-problem output
 // in c[p].u), Parseval-weighted norms of r and b into partials[block] and
@@ -263,7 +315,7 @@ template <class T>
 cudaError_t launch_residual(const LaunchTab<T> *tab, unsigned grid, bool write_r, double *partials,
                             unsigned partial_stride, cudaStream_t st, bool masked = false);
 template <class T>
-cudaError_t launch_prolong(const LaunchTab<T> *tab, unsigned grid, bool black_only, cudaStream_t st,
+cudaError_t launch_prolong(const TabRef<T> &tab, unsigned grid, bool black_only, cudaStream_t st,
                            bool masked = false);
 template <class T>
 cudaError_t launch_coarse(const CoarseTab<T> *tab, unsigned grid, size_t smem, cudaStream_t st);
@@ -275,10 +327,10 @@ unsigned dense_gemm_blocks(int nact, int nm);   // GEMM blocks of one problem
 // black ones, for a red Gauss-Seidel half-sweep to follow); coarse b =
 // restricted fine b.
 template <class T>
-cudaError_t launch_interp(const LaunchTab<T> *tab, unsigned grid, cudaStream_t st, bool masked = false,
+cudaError_t launch_interp(const TabRef<T> &tab, unsigned grid, cudaStream_t st, bool masked = false,
                           bool black_only = false);
 template <class T>
-cudaError_t launch_rhs_restrict(const LaunchTab<T> *tab, unsigned grid, cudaStream_t st, bool masked = false);
+cudaError_t launch_rhs_restrict(const TabRef<T> &tab, unsigned grid, cudaStream_t st, bool masked = false);
 
 // zero_x: the FP64 iterate is zero (r = b; the kernel also writes x = 0).
 cudaError_t launch_defect(const DefectTab *tab, unsigned grid, const Ctrl *ctrl, double *partials, bool zero_x,

@@ -85,6 +85,15 @@ __device__ __forceinline__ int find_problem(const unsigned *__restrict__ start, 
     return lo;
 }
 
+// A level view of a batch's table copied to shared memory by the block: the
+// kernel then reads its fields from there instead of holding them in registers.
+template <class T> __device__ __forceinline__ void stage_view(LevelDev<T> *dst, const LevelDev<T> *src) {
+    static_assert(sizeof(LevelDev<T>) % 8 == 0, "copied by 8-byte words");
+    constexpr int W = sizeof(LevelDev<T>) / 8;
+    for (int w = threadIdx.x; w < W; w += blockDim.x)
+        reinterpret_cast<unsigned long long *>(dst)[w] = reinterpret_cast<const unsigned long long *>(src)[w];
+}
+
 // b - A_m u at entry (k, i, m), Eq. matrix_free_mode_operator.
 template <class T, bool MASK>
 __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i, int m, size_t idx) {
@@ -137,14 +146,12 @@ __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i,
 // omega (one more load and multiply-add per component); otherwise omega = 1.
 // RW: the plan holds per-row tables (composite domain or non-uniform axial
 // mesh); the plain variant keeps the three-class rule and no such branch.
-template <class T, int NT, int S, bool SOR, bool RW>
-__global__ void __launch_bounds__(NT, S == 0 ? 2048 / NT : 1) k_smooth(const LaunchTab<T> *__restrict__ tab, int color) {
-    const int p = find_problem(tab->start, tab->n, blockIdx.x);
-    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
-    const LevelDev<T> L = tab->f[p];
+// (EARLY: the wait for the kernel before comes after the index arithmetic)
+template <class T, int NT, int S, bool SOR, bool RW, bool EARLY>
+__device__ __forceinline__ void smooth_body(const LevelDev<T> &L, unsigned blk, int color) {
     const unsigned nm = L.nm;
     if constexpr (S == 0) {
-        const unsigned e = (blockIdx.x - tab->start[p]) * NT + threadIdx.x;
+        const unsigned e = blk * NT + threadIdx.x;
         if (e >= (unsigned)L.nz * (unsigned)(L.nr >> 1) * nm) return;
         // (plain divisions: this kernel is capped at 32 registers for full
         // occupancy, and the multiply-high form needs more)
@@ -156,6 +163,10 @@ __global__ void __launch_bounds__(NT, S == 0 ? 2048 / NT : 1) k_smooth(const Lau
         const size_t idx = ((size_t)k * L.nr + i) * nm + m;
         const size_t tb = ((size_t)(RW ? lclass(L, k) : row_class(k, L.nz, L.ncls)) * L.nr + i) * nm + m;
         const size_t rowstride = (size_t)L.nr * nm;
+        if (EARLY) {
+            pdl_wait();
+            pdl_go();
+        }
         V2<T> acc;
         if (RW && L.holes && L.invd[tb] == T(0)) return;   // outside a composite domain: u stays 0
         if (RW && L.rcls && sizeof(T) == sizeof(double)) {   // per-row tables, FP64: south (hz) and
@@ -197,9 +208,8 @@ __global__ void __launch_bounds__(NT, S == 0 ? 2048 / NT : 1) k_smooth(const Lau
     } else {
         const unsigned w = (unsigned)(L.nr >> 1) * nm;
         const unsigned bx = (w + NT - 1) / NT;
-        const unsigned lb = blockIdx.x - tab->start[p];
-        const unsigned g = lb / bx;
-        const unsigned x = (lb - g * bx) * NT + threadIdx.x;
+        const unsigned g = blk / bx;
+        const unsigned x = (blk - g * bx) * NT + threadIdx.x;
         if (x >= w) return;
         const unsigned s0 = ((unsigned)(L.nz + 1) / 2 + S - 1) / S;
         const int par = g < s0 ? 0 : 1;
@@ -210,6 +220,10 @@ __global__ void __launch_bounds__(NT, S == 0 ? 2048 / NT : 1) k_smooth(const Lau
         const size_t rs = (size_t)L.nr * nm;                 // one row of cells, all modes
         const size_t tcol = (size_t)i * nm + m;              // (i, m) within a row / a coefficient class
         const size_t t1 = (L.ncls > 1 ? rs : 0) + tcol;      // interior coefficient class
+        if (EARLY) {
+            pdl_wait();
+            pdl_go();
+        }
         const T hz1 = __ldg(L.hz + t1), hw1 = __ldg(L.hw + t1), he1 = __ldg(L.he + t1);
         const V2<T> zero = mk<T>(0, 0);
         const size_t idx0 = (size_t)k0 * rs + tcol;
@@ -277,20 +291,33 @@ __global__ void __launch_bounds__(NT, S == 0 ? 2048 / NT : 1) k_smooth(const Lau
     }
 }
 
+template <class T, int NT, int S, bool SOR, bool RW, bool ONE>
+__global__ void __launch_bounds__(NT, S == 0 ? 2048 / NT : 1)
+k_smooth(const __grid_constant__ LevelArg<T> arg, int color) {
+    if constexpr (ONE) {
+        smooth_body<T, NT, S, SOR, RW, true>(arg.f, blockIdx.x, color);
+    } else {
+        const LaunchTab<T> *__restrict__ tab = arg.tab;
+        const int p = find_problem(tab->start, tab->n, blockIdx.x);
+        if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
+        const LevelDev<T> L = tab->f[p];
+        smooth_body<T, NT, S, SOR, RW, false>(L, blockIdx.x - tab->start[p], color);
+    }
+}
+
 // Residual of the fine cells of each coarse cell, summed into the coarse
 // right-hand side (finite-volume restriction: a residual is a cell integral),
 // with optional Parseval-weighted squared-norm partials.  RED_ONLY: only the
 // two red fine cells (after a black half-sweep the black residuals vanish).
 // F.init selects what else the coarse level receives (see internal.h).
-template <class T, bool RED_ONLY, bool MASK>
-__global__ void __launch_bounds__(MG_THREADS)
-k_residual_restrict(const LaunchTab<T> *__restrict__ tab, double *__restrict__ partials) {
-    __shared__ double red[MG_THREADS];
-    const int p = find_problem(tab->start, tab->n, blockIdx.x);
-    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
-    const LevelDev<T> F = tab->f[p];
-    const LevelDev<T> C = tab->c[p];
-    const unsigned e = (blockIdx.x - tab->start[p]) * blockDim.x + threadIdx.x;
+template <class T, bool RED_ONLY, bool MASK, bool EARLY>
+__device__ __forceinline__ void restrict_body(const LevelDev<T> &F, const LevelDev<T> &C, unsigned blk, double *red,
+                                              double *__restrict__ partials) {
+    const unsigned e = blk * MG_THREADS + threadIdx.x;
+    if (EARLY) {
+        pdl_wait();
+        pdl_go();
+    }
     double acc = 0.0;
     if (e < (unsigned)C.nz * (unsigned)C.nr * (unsigned)C.nm) {
         const unsigned nm = C.nm;
@@ -350,6 +377,24 @@ k_residual_restrict(const LaunchTab<T> *__restrict__ tab, double *__restrict__ p
     }
 }
 
+template <class T, bool RED_ONLY, bool MASK, bool ONE>
+__global__ void __launch_bounds__(MG_THREADS)
+k_residual_restrict(const __grid_constant__ LevelArg<T> arg, double *__restrict__ partials) {
+    __shared__ double red[MG_THREADS];
+    if constexpr (ONE) {
+        restrict_body<T, RED_ONLY, MASK, true>(arg.f, arg.c, blockIdx.x, red, partials);
+    } else {
+        const LaunchTab<T> *__restrict__ tab = arg.tab;
+        const int p = find_problem(tab->start, tab->n, blockIdx.x);
+        if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
+        __shared__ LevelDev<T> F, C;
+        stage_view(&F, &tab->f[p]);
+        stage_view(&C, &tab->c[p]);
+        __syncthreads();
+        restrict_body<T, RED_ONLY, MASK, false>(F, C, blockIdx.x - tab->start[p], red, partials);
+    }
+}
+
 // r = b - A_m u on level f (r written to c.u when write_r), Parseval-weighted
 // squared norms of r into partials[block] and, when stride > 0, of b into
 // partials[stride + block].
@@ -392,13 +437,9 @@ k_residual(const LaunchTab<T> *__restrict__ tab, int write_r, double *__restrict
 // value is reflected with a sign change (the correction vanishes on the
 // Dirichlet face).  BLACK_ONLY: only black fine cells (the red half-sweep that
 // follows overwrites the red ones).
-template <class T, bool BLACK_ONLY, bool ASSIGN, bool MASK>
-__global__ void __launch_bounds__(MG_THREADS) k_prolong(const LaunchTab<T> *__restrict__ tab) {
-    const int p = find_problem(tab->start, tab->n, blockIdx.x);
-    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
-    const LevelDev<T> F = tab->f[p];
-    const LevelDev<T> C = tab->c[p];
-    const unsigned e = (blockIdx.x - tab->start[p]) * blockDim.x + threadIdx.x;
+template <class T, bool BLACK_ONLY, bool ASSIGN, bool MASK, bool EARLY>
+__device__ __forceinline__ void prolong_body(const LevelDev<T> &F, const LevelDev<T> &C, unsigned blk) {
+    const unsigned e = blk * MG_THREADS + threadIdx.x;
     const unsigned nm = F.nm;
     const unsigned total = (unsigned)F.nz * (unsigned)(BLACK_ONLY ? (F.nr >> 1) : F.nr) * nm;
     if (e >= total) return;
@@ -418,6 +459,10 @@ __global__ void __launch_bounds__(MG_THREADS) k_prolong(const LaunchTab<T> *__re
         i = (int)(c - (unsigned)k * F.nr);
     }
     const unsigned idx = ((unsigned)k * F.nr + i) * nm + m;
+    if (EARLY) {
+        pdl_wait();
+        pdl_go();
+    }
     // composite domain: a cell outside the patches keeps u = 0 (in a batch the
     // masked variant also runs the plain problems, whose rcls is null; a level
     // without inactive cells -- a non-uniform axial mesh -- reads no diag)
@@ -459,6 +504,19 @@ __global__ void __launch_bounds__(MG_THREADS) k_prolong(const LaunchTab<T> *__re
     F.u[idx] = u;
 }
 
+template <class T, bool BLACK_ONLY, bool ASSIGN, bool MASK, bool ONE>
+__global__ void __launch_bounds__(MG_THREADS) k_prolong(const __grid_constant__ LevelArg<T> arg) {
+    if constexpr (ONE) {
+        prolong_body<T, BLACK_ONLY, ASSIGN, MASK, true>(arg.f, arg.c, blockIdx.x);
+    } else {
+        const LaunchTab<T> *__restrict__ tab = arg.tab;
+        const int p = find_problem(tab->start, tab->n, blockIdx.x);
+        if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
+        const LevelDev<T> F = tab->f[p], C = tab->c[p];
+        prolong_body<T, BLACK_ONLY, ASSIGN, MASK, false>(F, C, blockIdx.x - tab->start[p]);
+    }
+}
+
 // Full-multigrid start: the right-hand side restricted to the next coarser
 // level (the finite-volume sum of b over the fine cells of each coarse cell,
 // the restriction the residuals get), b_hat = b / diag, and a zero iterate.
@@ -466,10 +524,12 @@ template <class T, bool MASK>
 __global__ void __launch_bounds__(MG_THREADS) k_rhs_restrict(const LaunchTab<T> *__restrict__ tab) {
     // (MASK: the class tables of a composite domain's rows)
     const int p = find_problem(tab->start, tab->n, blockIdx.x);
-    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
     const LevelDev<T> F = tab->f[p];
     const LevelDev<T> C = tab->c[p];
     const unsigned e = (blockIdx.x - tab->start[p]) * blockDim.x + threadIdx.x;
+    pdl_wait();
+    pdl_go();
+    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
     if (e >= (unsigned)C.nz * (unsigned)C.nr * (unsigned)C.nm) return;
     const unsigned nm = C.nm;
     const unsigned cc = fdiv(e, nm, C.rnm);
@@ -540,10 +600,12 @@ __global__ void __launch_bounds__(MG_THREADS, 6)   // 48 warps per SM for the FP
 k_defect(const DefectTab *__restrict__ tab, const Ctrl *__restrict__ ctrl, double *__restrict__ partials) {
     __shared__ double red[MG_THREADS];
     const int p = find_problem(tab->start, tab->n, blockIdx.x);
-    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
     const LevelDev<double> D = tab->d[p];
     const LevelDev<float> S = tab->s[p];
     const int init_red = tab->init_red[p];
+    pdl_wait();
+    pdl_go();
+    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
     const int ls = pow2_exponent(ctrl->sigma_next[p]);
     const unsigned e = (blockIdx.x - tab->start[p]) * blockDim.x + threadIdx.x;
     double acc = 0.0;
@@ -577,9 +639,11 @@ k_defect(const DefectTab *__restrict__ tab, const Ctrl *__restrict__ ctrl, doubl
 // problem just solved; 1/sigma is an exact power of two).
 __global__ void __launch_bounds__(MG_THREADS) k_update(const DefectTab *__restrict__ tab, const Ctrl *__restrict__ ctrl) {
     const int p = find_problem(tab->start, tab->n, blockIdx.x);
-    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
     const LevelDev<double> D = tab->d[p];
     const LevelDev<float> S = tab->s[p];
+    pdl_wait();
+    pdl_go();
+    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
     const int ls = pow2_exponent(ctrl->inv_sigma_used[p]);
     const unsigned e = (blockIdx.x - tab->start[p]) * blockDim.x + threadIdx.x;
     if (e >= (unsigned)D.nz * (unsigned)D.nr * (unsigned)D.nm) return;
@@ -608,9 +672,11 @@ template <class T>
 __global__ void __launch_bounds__(MG_THREADS) k_coarse(const CoarseTab<T> *__restrict__ tab) {
     extern __shared__ unsigned char smraw[];
     const int p = find_problem(tab->start, tab->n, blockIdx.x);
-    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
     const LevelDev<T> L = tab->f[p];
     const CoarseDev<T> D = tab->c[p];
+    pdl_wait();
+    pdl_go();
+    if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
     const int nr = D.nr, nz = D.nz, nm = D.nm;
     const int lb = (int)(blockIdx.x - tab->start[p]);
     const int m = lb >> 1, comp = lb & 1;
@@ -722,6 +788,8 @@ __global__ void __launch_bounds__(256) k_psum(const PsumTab *__restrict__ tab, c
     const unsigned c = blockIdx.x - tab->start[p];
     const unsigned b0 = tab->in_begin[p] + c * (unsigned)PSUM_CHUNK;
     const unsigned b1 = min(tab->in_end[p], b0 + (unsigned)PSUM_CHUNK);
+    pdl_wait();
+    pdl_go();
     double s = 0.0;
     for (unsigned b = b0 + threadIdx.x; b < b1; b += blockDim.x) s += partials[b];
     const double tot = block_sum(s, red);
@@ -734,6 +802,8 @@ __global__ void __launch_bounds__(1024) k_bnorm(Ctrl *__restrict__ ctrl, const F
                                                 const double *__restrict__ partials) {
     __shared__ double wsum[32];
     __shared__ double sums[kMaxBatch];
+    pdl_wait();
+    pdl_go();
     range_sums(partials, fft->start, fft->start + 1, fft->n, sums, wsum);
     for (int p = threadIdx.x; p < fft->n; p += blockDim.x) {
         ctrl->bnorm2[p] = sums[p];
@@ -759,6 +829,8 @@ __global__ void __launch_bounds__(1024) k_check(Ctrl *__restrict__ ctrl, const d
     __shared__ double wsum[32];
     __shared__ double sums[kMaxBatch];
     __shared__ int s_any;
+    pdl_wait();
+    pdl_go();
     const int cycles = ctrl->cycles + (counting == 2 ? ctrl->inc_first : counting ? ctrl->inc : 0);
     if (threadIdx.x == 0) s_any = 0;
     range_sums(partials, ctrl->rbegin, ctrl->rend, ctrl->n, sums, wsum);
@@ -823,31 +895,37 @@ __global__ void __launch_bounds__(1024) k_sum(const double *__restrict__ p, int 
 
 }  // namespace
 
+// (strips read the table: they are for levels of a few waves, not for latency)
+template <class T, int NT, int S, bool SOR, bool RW>
+cudaError_t launch_smooth_n(const TabRef<T> &tab, unsigned grid, int color, cudaStream_t st) {
+    if (S == 0 && tab.one) return launch_pdl(k_smooth<T, NT, S, SOR, RW, S == 0>, grid, NT, 0, st, tab.arg(), color);
+    k_smooth<T, NT, S, SOR, RW, false><<<grid, NT, 0, st>>>(tab.arg(), color);
+    return cudaGetLastError();
+}
+
 template <class T, int S, bool SOR, bool RW>
-void launch_smooth_s(const LaunchTab<T> *tab, unsigned grid, int color, int threads, cudaStream_t st) {
+cudaError_t launch_smooth_s(const TabRef<T> &tab, unsigned grid, int color, int threads, cudaStream_t st) {
     switch (threads) {
-    case 64: k_smooth<T, 64, S, SOR, RW><<<grid, 64, 0, st>>>(tab, color); break;
-    case 128: k_smooth<T, 128, S, SOR, RW><<<grid, 128, 0, st>>>(tab, color); break;
-    case 512: k_smooth<T, 512, S, SOR, RW><<<grid, 512, 0, st>>>(tab, color); break;
-    default: k_smooth<T, 256, S, SOR, RW><<<grid, 256, 0, st>>>(tab, color); break;
+    case 64: return launch_smooth_n<T, 64, S, SOR, RW>(tab, grid, color, st);
+    case 128: return launch_smooth_n<T, 128, S, SOR, RW>(tab, grid, color, st);
+    case 512: return launch_smooth_n<T, 512, S, SOR, RW>(tab, grid, color, st);
+    default: return launch_smooth_n<T, 256, S, SOR, RW>(tab, grid, color, st);
     }
 }
 
 template <class T, bool SOR, bool RW>
-cudaError_t launch_smooth_r(const LaunchTab<T> *tab, unsigned grid, int color, int threads, int strip,
-                            cudaStream_t st) {
+cudaError_t launch_smooth_r(const TabRef<T> &tab, unsigned grid, int color, int threads, int strip, cudaStream_t st) {
     switch (strip) {
-    case 0: launch_smooth_s<T, 0, SOR, RW>(tab, grid, color, threads, st); break;
-    case 1: launch_smooth_s<T, 1, SOR, RW>(tab, grid, color, threads, st); break;
-    case 2: launch_smooth_s<T, 2, SOR, RW>(tab, grid, color, threads, st); break;
-    case 4: launch_smooth_s<T, 4, SOR, RW>(tab, grid, color, threads, st); break;
+    case 0: return launch_smooth_s<T, 0, SOR, RW>(tab, grid, color, threads, st);
+    case 1: return launch_smooth_s<T, 1, SOR, RW>(tab, grid, color, threads, st);
+    case 2: return launch_smooth_s<T, 2, SOR, RW>(tab, grid, color, threads, st);
+    case 4: return launch_smooth_s<T, 4, SOR, RW>(tab, grid, color, threads, st);
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 template <class T>
-cudaError_t launch_smooth(const LaunchTab<T> *tab, unsigned grid, int color, int threads, int strip, bool sor,
+cudaError_t launch_smooth(const TabRef<T> &tab, unsigned grid, int color, int threads, int strip, bool sor,
                           cudaStream_t st, bool rowwise) {
     if (rowwise)
         return sor ? launch_smooth_r<T, true, true>(tab, grid, color, threads, strip, st)
@@ -856,17 +934,22 @@ cudaError_t launch_smooth(const LaunchTab<T> *tab, unsigned grid, int color, int
                : launch_smooth_r<T, false, false>(tab, grid, color, threads, strip, st);
 }
 
-template <class T>
-cudaError_t launch_residual_restrict(const LaunchTab<T> *tab, unsigned grid, bool red_only, double *partials,
-                                     cudaStream_t st, bool masked) {
-    if (masked) {
-        if (red_only) k_residual_restrict<T, true, true><<<grid, MG_THREADS, 0, st>>>(tab, partials);
-        else k_residual_restrict<T, false, true><<<grid, MG_THREADS, 0, st>>>(tab, partials);
-    } else {
-        if (red_only) k_residual_restrict<T, true, false><<<grid, MG_THREADS, 0, st>>>(tab, partials);
-        else k_residual_restrict<T, false, false><<<grid, MG_THREADS, 0, st>>>(tab, partials);
-    }
+template <class T, bool RED_ONLY, bool MASK>
+cudaError_t launch_restrict_m(const TabRef<T> &tab, unsigned grid, double *partials, cudaStream_t st) {
+    if (tab.one)
+        return launch_pdl(k_residual_restrict<T, RED_ONLY, MASK, true>, grid, MG_THREADS, 0, st, tab.arg(), partials);
+    k_residual_restrict<T, RED_ONLY, MASK, false><<<grid, MG_THREADS, 0, st>>>(tab.arg(), partials);
     return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t launch_residual_restrict(const TabRef<T> &tab, unsigned grid, bool red_only, double *partials,
+                                     cudaStream_t st, bool masked) {
+    if (masked)
+        return red_only ? launch_restrict_m<T, true, true>(tab, grid, partials, st)
+                        : launch_restrict_m<T, false, true>(tab, grid, partials, st);
+    return red_only ? launch_restrict_m<T, true, false>(tab, grid, partials, st)
+                    : launch_restrict_m<T, false, false>(tab, grid, partials, st);
 }
 
 template <class T>
@@ -877,76 +960,70 @@ cudaError_t launch_residual(const LaunchTab<T> *tab, unsigned grid, bool write_r
     return cudaGetLastError();
 }
 
-template <class T>
-cudaError_t launch_prolong(const LaunchTab<T> *tab, unsigned grid, bool black_only, cudaStream_t st, bool masked) {
-    if (masked) {
-        if (black_only) k_prolong<T, true, false, true><<<grid, MG_THREADS, 0, st>>>(tab);
-        else k_prolong<T, false, false, true><<<grid, MG_THREADS, 0, st>>>(tab);
-    } else {
-        if (black_only) k_prolong<T, true, false, false><<<grid, MG_THREADS, 0, st>>>(tab);
-        else k_prolong<T, false, false, false><<<grid, MG_THREADS, 0, st>>>(tab);
-    }
+template <class T, bool BLACK_ONLY, bool ASSIGN, bool MASK>
+cudaError_t launch_prolong_m(const TabRef<T> &tab, unsigned grid, cudaStream_t st) {
+    if (tab.one) return launch_pdl(k_prolong<T, BLACK_ONLY, ASSIGN, MASK, true>, grid, MG_THREADS, 0, st, tab.arg());
+    k_prolong<T, BLACK_ONLY, ASSIGN, MASK, false><<<grid, MG_THREADS, 0, st>>>(tab.arg());
     return cudaGetLastError();
 }
 
 template <class T>
-cudaError_t launch_interp(const LaunchTab<T> *tab, unsigned grid, cudaStream_t st, bool masked, bool black_only) {
-    if (black_only) {
-        if (masked) k_prolong<T, true, true, true><<<grid, MG_THREADS, 0, st>>>(tab);
-        else k_prolong<T, true, true, false><<<grid, MG_THREADS, 0, st>>>(tab);
-    } else {
-        if (masked) k_prolong<T, false, true, true><<<grid, MG_THREADS, 0, st>>>(tab);
-        else k_prolong<T, false, true, false><<<grid, MG_THREADS, 0, st>>>(tab);
-    }
-    return cudaGetLastError();
+cudaError_t launch_prolong(const TabRef<T> &tab, unsigned grid, bool black_only, cudaStream_t st, bool masked) {
+    if (masked)
+        return black_only ? launch_prolong_m<T, true, false, true>(tab, grid, st)
+                          : launch_prolong_m<T, false, false, true>(tab, grid, st);
+    return black_only ? launch_prolong_m<T, true, false, false>(tab, grid, st)
+                      : launch_prolong_m<T, false, false, false>(tab, grid, st);
 }
 
 template <class T>
-cudaError_t launch_rhs_restrict(const LaunchTab<T> *tab, unsigned grid, cudaStream_t st, bool masked) {
-    if (masked) k_rhs_restrict<T, true><<<grid, MG_THREADS, 0, st>>>(tab);
-    else k_rhs_restrict<T, false><<<grid, MG_THREADS, 0, st>>>(tab);
-    return cudaGetLastError();
+cudaError_t launch_interp(const TabRef<T> &tab, unsigned grid, cudaStream_t st, bool masked, bool black_only) {
+    if (black_only)
+        return masked ? launch_prolong_m<T, true, true, true>(tab, grid, st)
+                      : launch_prolong_m<T, true, true, false>(tab, grid, st);
+    return masked ? launch_prolong_m<T, false, true, true>(tab, grid, st)
+                  : launch_prolong_m<T, false, true, false>(tab, grid, st);
+}
+
+template <class T>
+cudaError_t launch_rhs_restrict(const TabRef<T> &tab, unsigned grid, cudaStream_t st, bool masked) {
+    if (masked) return launch_pdl(k_rhs_restrict<T, true>, grid, MG_THREADS, 0, st, (const LaunchTab<T> *)tab.tab);
+    else return launch_pdl(k_rhs_restrict<T, false>, grid, MG_THREADS, 0, st, (const LaunchTab<T> *)tab.tab);
 }
 
 template <class T>
 cudaError_t launch_coarse(const CoarseTab<T> *tab, unsigned grid, size_t smem, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(k_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_coarse<T><<<grid, MG_THREADS, smem, st>>>(tab);
-    return cudaGetLastError();
+    return launch_pdl(k_coarse<T>, grid, MG_THREADS, smem, st, tab);
 }
 
 cudaError_t launch_defect(const DefectTab *tab, unsigned grid, const Ctrl *ctrl, double *partials, bool zero_x,
                           cudaStream_t st, bool masked) {
     if (masked) {
-        if (zero_x) k_defect<true, true><<<grid, MG_THREADS, 0, st>>>(tab, ctrl, partials);
-        else k_defect<false, true><<<grid, MG_THREADS, 0, st>>>(tab, ctrl, partials);
+        if (zero_x) return launch_pdl(k_defect<true, true>, grid, MG_THREADS, 0, st, tab, ctrl, partials);
+        else return launch_pdl(k_defect<false, true>, grid, MG_THREADS, 0, st, tab, ctrl, partials);
     } else {
-        if (zero_x) k_defect<true, false><<<grid, MG_THREADS, 0, st>>>(tab, ctrl, partials);
-        else k_defect<false, false><<<grid, MG_THREADS, 0, st>>>(tab, ctrl, partials);
+        if (zero_x) return launch_pdl(k_defect<true, false>, grid, MG_THREADS, 0, st, tab, ctrl, partials);
+        else return launch_pdl(k_defect<false, false>, grid, MG_THREADS, 0, st, tab, ctrl, partials);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_update(const DefectTab *tab, unsigned grid, const Ctrl *ctrl, cudaStream_t st) {
-    k_update<<<grid, MG_THREADS, 0, st>>>(tab, ctrl);
-    return cudaGetLastError();
+    return launch_pdl(k_update, grid, MG_THREADS, 0, st, tab, ctrl);
 }
 
 cudaError_t launch_bnorm(Ctrl *ctrl, const FFTTab *fft, const double *partials, cudaStream_t st) {
-    k_bnorm<<<1, 1024, 0, st>>>(ctrl, fft, partials);
-    return cudaGetLastError();
+    return launch_pdl(k_bnorm, 1, 1024, 0, st, ctrl, fft, partials);
 }
 
 cudaError_t launch_psum(const PsumTab *tab, unsigned grid, const double *partials, double *out, cudaStream_t st) {
-    k_psum<<<grid, 256, 0, st>>>(tab, partials, out);
-    return cudaGetLastError();
+    return launch_pdl(k_psum, grid, 256, 0, st, tab, partials, out);
 }
 
 cudaError_t launch_check(Ctrl *ctrl, const double *partials, int counting, cudaGraphConditionalHandle handle,
                          cudaGraphConditionalHandle handle2, int use_handle, cudaStream_t st) {
-    k_check<<<1, 1024, 0, st>>>(ctrl, partials, counting, handle, handle2, use_handle);
-    return cudaGetLastError();
+    return launch_pdl(k_check, 1, 1024, 0, st, ctrl, partials, counting, handle, handle2, use_handle);
 }
 
 cudaError_t launch_sum(const double *partials, int n, double *out, cudaStream_t st) {
@@ -955,15 +1032,15 @@ cudaError_t launch_sum(const double *partials, int n, double *out, cudaStream_t 
 }
 
 #define PP_INST(T)                                                                                         \
-    template cudaError_t launch_smooth<T>(const LaunchTab<T> *, unsigned, int, int, int, bool, cudaStream_t, \
+    template cudaError_t launch_smooth<T>(const TabRef<T> &, unsigned, int, int, int, bool, cudaStream_t, \
                                           bool);                                                           \
-    template cudaError_t launch_residual_restrict<T>(const LaunchTab<T> *, unsigned, bool, double *,       \
+    template cudaError_t launch_residual_restrict<T>(const TabRef<T> &, unsigned, bool, double *,       \
                                                      cudaStream_t, bool);                                  \
     template cudaError_t launch_residual<T>(const LaunchTab<T> *, unsigned, bool, double *, unsigned,      \
                                             cudaStream_t, bool);                                           \
-    template cudaError_t launch_prolong<T>(const LaunchTab<T> *, unsigned, bool, cudaStream_t, bool);      \
-    template cudaError_t launch_interp<T>(const LaunchTab<T> *, unsigned, cudaStream_t, bool, bool);       \
-    template cudaError_t launch_rhs_restrict<T>(const LaunchTab<T> *, unsigned, cudaStream_t, bool);       \
+    template cudaError_t launch_prolong<T>(const TabRef<T> &, unsigned, bool, cudaStream_t, bool);      \
+    template cudaError_t launch_interp<T>(const TabRef<T> &, unsigned, cudaStream_t, bool, bool);       \
+    template cudaError_t launch_rhs_restrict<T>(const TabRef<T> &, unsigned, cudaStream_t, bool);       \
     template cudaError_t launch_coarse<T>(const CoarseTab<T> *, unsigned, size_t, cudaStream_t);
 PP_INST(double)
 PP_INST(float)

@@ -700,24 +700,24 @@ template <class T> void carve_coarse(const ProblemPlan &q, Carver &c, CoarseDev<
 
 template <class T> void carve_hier(pic_poisson_plan_s &P, Carver &c, Hier<T> &H) {
     const int nl = std::max(P.Lmax - 1, 0);
-    H.smooth.assign(nl, nullptr);
-    H.restr.assign(nl, nullptr);
-    H.prolong.assign(nl, nullptr);
+    H.smooth.assign(nl, TabRef<T>{});
+    H.restr.assign(nl, TabRef<T>{});
+    H.prolong.assign(nl, TabRef<T>{});
     H.fpre.assign(nl, nullptr);
     H.fpost.assign(nl, nullptr);
-    H.rhs.assign(nl, nullptr);
-    H.interp.assign(nl, nullptr);
+    H.rhs.assign(nl, TabRef<T>{});
+    H.interp.assign(nl, TabRef<T>{});
     for (int l = 0; l < nl; ++l) {
-        H.smooth[l] = c.take<LaunchTab<T>>(1);
-        H.restr[l] = c.take<LaunchTab<T>>(1);
-        H.prolong[l] = c.take<LaunchTab<T>>(1);
+        H.smooth[l].tab = c.take<LaunchTab<T>>(1);
+        H.restr[l].tab = c.take<LaunchTab<T>>(1);
+        H.prolong[l].tab = c.take<LaunchTab<T>>(1);
         if (H.fused) {
             H.fpre[l] = c.take<FusedTab>(1);
             H.fpost[l] = c.take<FusedTab>(1);
         }
         if (P.shared.fmg) {
-            H.rhs[l] = c.take<LaunchTab<T>>(1);
-            H.interp[l] = c.take<LaunchTab<T>>(1);
+            H.rhs[l].tab = c.take<LaunchTab<T>>(1);
+            H.interp[l].tab = c.take<LaunchTab<T>>(1);
         }
     }
     H.coarse = c.take<CoarseTab<T>>(1);
@@ -842,6 +842,12 @@ template <class T, class Views, class Coarse>
 void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, cudaStream_t st, cudaError_t &err) {
     const int nl = std::max(P.Lmax - 1, 0);
     const int pre = P.shared.pre_sweeps, post = P.shared.post_sweeps;
+    auto put = [&](const LaunchTab<T> &t, TabRef<T> &r) {
+        blob_to_dev(t, r.tab, st, err);
+        r.one = P.n == 1;
+        r.f = t.f[0];
+        r.c = t.c[0];
+    };
     H.g_smooth.assign(nl, 0);
     H.g_restr.assign(nl, 0);
     H.g_prolong.assign(nl, 0);
@@ -930,12 +936,12 @@ void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, c
         H.g_restr[l] = tr.start[tr.n];
         H.g_prolong[l] = tp.start[tp.n];
         if (ts.n == 0) {
-            H.smooth[l] = H.restr[l] = H.prolong[l] = nullptr;
+            H.smooth[l] = H.restr[l] = H.prolong[l] = TabRef<T>{};
             continue;
         }
-        blob_to_dev(ts, H.smooth[l], st, err);
-        blob_to_dev(tr, H.restr[l], st, err);
-        blob_to_dev(tp, H.prolong[l], st, err);
+        put(ts, H.smooth[l]);
+        put(tr, H.restr[l]);
+        put(tp, H.prolong[l]);
         if (H.fused) {
             H.g_fpre[l] = fa.start[fa.n];
             H.g_fpost[l] = fb.start[fb.n];
@@ -974,8 +980,8 @@ void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, c
             }
             H.g_rhs[l] = trh.start[trh.n];
             H.g_interp[l] = tin.start[tin.n];
-            if (trh.n) blob_to_dev(trh, H.rhs[l], st, err);
-            if (tin.n) blob_to_dev(tin, H.interp[l], st, err);
+            if (trh.n) put(trh, H.rhs[l]);
+            if (tin.n) put(tin, H.interp[l]);
         }
     }
     CoarseTab<T> tc{};
@@ -1333,19 +1339,26 @@ int upload(pic_poisson_plan_s &P) {
         }
     }
     // two-stage norm reduction: k_psum sums chunks of each problem's partials,
-    // the convergence test reads the chunk sums
+    // the convergence test reads the chunk sums -- or, when there are few, the
+    // partials themselves: a launch costs about 3 us, 4096 additions by one block
+    // about 1 us
     PsumTab ps{};
     ps.n = P.n;
-    for (int p = 0; p < P.n; ++p) {
-        const unsigned len = C.rend[p] - C.rbegin[p];
-        const unsigned chunks = std::max(1u, (len + PSUM_CHUNK - 1) / PSUM_CHUNK);
-        ps.in_begin[p] = C.rbegin[p];
-        ps.in_end[p] = C.rend[p];
-        ps.start[p + 1] = ps.start[p] + chunks;
-        C.rbegin[p] = ps.start[p];
-        C.rend[p] = ps.start[p + 1];
+    unsigned total = 0;
+    for (int p = 0; p < P.n; ++p) total += C.rend[p] - C.rbegin[p];
+    P.g_psum = 0;
+    if (total > PSUM_MIN) {
+        for (int p = 0; p < P.n; ++p) {
+            const unsigned len = C.rend[p] - C.rbegin[p];
+            const unsigned chunks = std::max(1u, (len + PSUM_CHUNK - 1) / PSUM_CHUNK);
+            ps.in_begin[p] = C.rbegin[p];
+            ps.in_end[p] = C.rend[p];
+            ps.start[p + 1] = ps.start[p] + chunks;
+            C.rbegin[p] = ps.start[p];
+            C.rend[p] = ps.start[p + 1];
+        }
+        P.g_psum = ps.start[P.n];
     }
-    P.g_psum = ps.start[P.n];
     blob_to_dev(ps, P.psum, st, err);
     if (err != cudaSuccess) {
         set_error("uploading plan tables failed: %s", cudaGetErrorString(err));

@@ -48,7 +48,7 @@ struct ProblemPlan {
 // Launch tables of one precision's hierarchy, per level l = 0 .. Lmax-2
 // (problems that have a level below l), plus the coarsest-level solve.
 template <class T> struct Hier {
-    std::vector<LaunchTab<T> *> smooth, restr, prolong;   // device tables (null when no problem takes part)
+    std::vector<TabRef<T>> smooth, restr, prolong;        // tables (null when no problem takes part)
     std::vector<unsigned> g_smooth, g_restr, g_prolong;   // grids
     std::vector<int> strip;                               // smoother strip per level
     bool fused = false;                                   // FP32 fused smoother (pre: u -> u2, post: u2 -> u)
@@ -60,7 +60,7 @@ template <class T> struct Hier {
     unsigned g_dense_prep = 0, g_dense_gemm = 0;
     unsigned g_coarse = 0;
     size_t smem_coarse = 0;
-    std::vector<LaunchTab<T> *> rhs, interp;  // full-multigrid start: b restricted to l + 1, u_l = P u_(l+1)
+    std::vector<TabRef<T>> rhs, interp;       // full-multigrid start: b restricted to l + 1, u_l = P u_(l+1)
     bool interp_black = false;                // u_l = P u_(l+1) on the black cells only (the red half-sweep
                                               // that follows overwrites the red ones unread)
     std::vector<unsigned> g_rhs, g_interp;
