@@ -18,6 +18,7 @@
 // changes.
 #include <algorithm>
 
+#include "fixed.h"
 #include "internal.h"
 
 namespace pp {
@@ -37,8 +38,12 @@ __device__ __forceinline__ int row_class(int k, int nz, int ncls) {
     return k == 0 ? 0 : (k == nz - 1 ? ncls - 1 : 1);
 }
 
+// FX (binary64, the imaginary part): in fixed point, as the level kernels
+// compute imaginary parts (fixed.h); the tables then hold its coefficients.
+__device__ __forceinline__ int2 coef(double v) { return make_int2(__double2loint(v), __double2hiint(v)); }
+
 // One red-black half-sweep of colour `color` on U (one real part, shared memory).
-template <class T>
+template <class T, bool FX>
 __device__ void half_sweep(T *u, const T *bh, const T *hz, const T *hw, const T *he, int nr, int nz, int ncls,
                            int color) {
     const int hr = nr >> 1, ncell = nz * hr;
@@ -47,6 +52,11 @@ __device__ void half_sweep(T *u, const T *bh, const T *hz, const T *hw, const T 
         const int i = 2 * (c - k * hr) + ((k + color) & 1);
         const int f = k * nr + i;
         const int tb = row_class(k, nz, ncls) * nr + i;
+        if constexpr (FX) {
+            u[f] = fx_update(bh[f], k > 0 ? u[f - nr] : 0.0, k < nz - 1 ? u[f + nr] : 0.0, i > 0 ? u[f - 1] : 0.0,
+                             i < nr - 1 ? u[f + 1] : 0.0, coef(hz[tb]), coef(hw[tb]), coef(he[tb]));
+            continue;
+        }
         T s = 0;
         if (k > 0) s = u[f - nr];
         if (k < nz - 1) {
@@ -62,10 +72,14 @@ __device__ void half_sweep(T *u, const T *bh, const T *hz, const T *hw, const T 
 }
 
 // b - A_m u at cell (k, i) of U (as residual_at in mg.cu).
-template <class T>
+template <class T, bool FX>
 __device__ __forceinline__ T residual(const T *u, const T *b, const T *cw, const T *ce, const T *cz, const T *dg,
-                                      int k, int i, int nr, int nz, int ncls) {
+                                      int k, int i, int nr, int nz, int ncls, int q) {
     const int f = k * nr + i;
+    if constexpr (FX)
+        return fx_residual(b[f], k > 0 ? u[f - nr] : 0.0, k < nz - 1 ? u[f + nr] : 0.0, i > 0 ? u[f - 1] : 0.0,
+                           i < nr - 1 ? u[f + 1] : 0.0, u[f], coef(cz[i]), coef(cw[i]), coef(ce[i]),
+                           coef(dg[row_class(k, nz, ncls) * nr + i]), q);
     T s = 0;
     if (k > 0) s = u[f - nr];
     if (k < nz - 1) {
@@ -78,10 +92,8 @@ __device__ __forceinline__ T residual(const T *u, const T *b, const T *cw, const
     return fma(-dg[row_class(k, nz, ncls) * nr + i], u[f], acc);
 }
 
-template <class T>
-__global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom(const BottomTab<T> *__restrict__ tab) {
-    extern __shared__ unsigned char smraw[];
-    const int p = find_problem(tab->start, tab->n, blockIdx.x);
+template <class T, bool FX>
+__device__ __forceinline__ void bottom_body(const BottomTab<T> *__restrict__ tab, int p, unsigned char *smraw) {
     const BottomProb<T> &B = tab->p[p];
     const LevelDev<T> &U = B.U;
     const CoarseDev<T> &D = B.D;
@@ -121,9 +133,15 @@ __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom(const BottomTab<T> *_
     const T *gb = (const T *)U.b + part, *gbh = (const T *)U.bh + part;
     for (int f = threadIdx.x; f < ncls * nr; f += blockDim.x) {
         const size_t t = (size_t)f * nm + m;   // (class, i) -> ((class * nr + i) * nm + m)
-        cp_async_elem(hz + f, U.hz + t);
-        cp_async_elem(hw + f, U.hw + t);
-        cp_async_elem(he + f, U.he + t);
+        if constexpr (FX) {   // (coefficients of fixed.h, 8 bytes like binary64 values)
+            cp_async_elem(hz + f, reinterpret_cast<const T *>(U.hzw + t));
+            cp_async_elem(hw + f, reinterpret_cast<const T *>(U.hzw + t) + 1);
+            cp_async_elem(he + f, reinterpret_cast<const T *>(U.hev + t));
+        } else {
+            cp_async_elem(hz + f, U.hz + t);
+            cp_async_elem(hw + f, U.hw + t);
+            cp_async_elem(he + f, U.he + t);
+        }
     }
     pdl_wait();
     pdl_go();
@@ -145,11 +163,21 @@ __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom(const BottomTab<T> *_
     } else {
         for (int f = threadIdx.x; f < n; f += blockDim.x) cp_async_elem(b + f, gb + 2 * ((size_t)f * nm + m));
     }
-    for (int f = threadIdx.x; f < ncls * nr; f += blockDim.x) cp_async_elem(dg + f, U.diag + (size_t)f * nm + m);
-    for (int i = threadIdx.x; i < nr; i += blockDim.x) {
-        cp_async_elem(cw + i, U.cw + i);
-        cp_async_elem(ce + i, U.ce + i);
-        cp_async_elem(cz + i, U.cz + i);
+    if constexpr (FX) {
+        for (int f = threadIdx.x; f < ncls * nr; f += blockDim.x)
+            cp_async_elem(dg + f, reinterpret_cast<const T *>(U.rdg + (size_t)f * nm + m));
+        for (int i = threadIdx.x; i < nr; i += blockDim.x) {
+            cp_async_elem(cz + i, reinterpret_cast<const T *>(U.rzw + i));
+            cp_async_elem(cw + i, reinterpret_cast<const T *>(U.rzw + i) + 1);
+            cp_async_elem(ce + i, reinterpret_cast<const T *>(U.rev + i));
+        }
+    } else {
+        for (int f = threadIdx.x; f < ncls * nr; f += blockDim.x) cp_async_elem(dg + f, U.diag + (size_t)f * nm + m);
+        for (int i = threadIdx.x; i < nr; i += blockDim.x) {
+            cp_async_elem(cw + i, U.cw + i);
+            cp_async_elem(ce + i, U.ce + i);
+            cp_async_elem(cz + i, U.cz + i);
+        }
     }
     for (int f = threadIdx.x; f < hzc * ncz; f += blockDim.x) cp_async_elem(Vs + f, D.V + f);
     {
@@ -168,8 +196,8 @@ __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom(const BottomTab<T> *_
     // pre-smoothing from zero (the restriction's fused first red half-sweep
     // gives the same values as the red half-sweep done here)
     for (int s = 0; s < B.pre; ++s) {
-        half_sweep(u, bh, hz, hw, he, nr, nz, ncls, 0);
-        half_sweep(u, bh, hz, hw, he, nr, nz, ncls, 1);
+        half_sweep<T, FX>(u, bh, hz, hw, he, nr, nz, ncls, 0);
+        half_sweep<T, FX>(u, bh, hz, hw, he, nr, nz, ncls, 1);
     }
     cp_async_group_wait<0>();
     __syncthreads();
@@ -188,7 +216,7 @@ __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom(const BottomTab<T> *_
                 k = fz * K + (fr == 2 ? (c >> 1) : c);
                 i = fr * I + (fr == 2 ? (c & 1) : 0);
             }
-            const T r = residual(u, b, cw, ce, cz, dg, k, i, nr, nz, ncls);
+            const T r = residual<T, FX>(u, b, cw, ce, cz, dg, k, i, nr, nz, ncls, U.rq);
             sum = c == 0 ? r : sum + r;
         }
         bc[e] = sum;
@@ -256,22 +284,37 @@ __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom(const BottomTab<T> *_
                 const T c1 = bc[K * ncr + Ix], c2 = bc[Kx * ncr + I], c3 = bc[Kx * ncr + Ix];
                 const T w1 = iin ? T(0.1875) : T(-0.1875), w2 = kin ? T(0.1875) : T(-0.1875);
                 const T w3 = iin == kin ? T(0.0625) : T(-0.0625);
-                v = fma(w3, c3, fma(w2, c2, fma(w1, c1, fma(T(0.5625), c0, v))));
+                if constexpr (FX) v = fx_bilinear(v, c0, c1, c2, c3, !iin, !kin);
+                else v = fma(w3, c3, fma(w2, c2, fma(w1, c1, fma(T(0.5625), c0, v))));
             } else {
                 const T c1 = cz2 ? bc[Kx * ncr + I] : bc[K * ncr + Ix];
                 const T w1 = (cz2 ? kin : iin) ? T(0.25) : T(-0.25);
-                v = fma(w1, c1, fma(T(0.75), c0, v));
+                if constexpr (FX) v = fx_linear(v, c0, c1, cz2 ? !kin : !iin);
+                else v = fma(w1, c1, fma(T(0.75), c0, v));
             }
             u[k * nr + i] = v;
         }
     }
     __syncthreads();
     for (int s = 0; s < B.post; ++s) {
-        half_sweep(u, bh, hz, hw, he, nr, nz, ncls, 0);
-        half_sweep(u, bh, hz, hw, he, nr, nz, ncls, 1);
+        half_sweep<T, FX>(u, bh, hz, hw, he, nr, nz, ncls, 0);
+        half_sweep<T, FX>(u, bh, hz, hw, he, nr, nz, ncls, 1);
     }
     T *gu = (T *)U.u + part;
     for (int f = threadIdx.x; f < n; f += blockDim.x) gu[2 * ((size_t)f * nm + m)] = u[f];
+}
+
+template <class T>
+__global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom(const BottomTab<T> *__restrict__ tab) {
+    extern __shared__ unsigned char smraw[];
+    const int p = find_problem(tab->start, tab->n, blockIdx.x);
+    if constexpr (sizeof(T) == sizeof(double)) {
+        if ((blockIdx.x - tab->start[p]) & 1u && tab->p[p].U.rzw) {
+            bottom_body<T, true>(tab, p, smraw);
+            return;
+        }
+    }
+    bottom_body<T, false>(tab, p, smraw);
 }
 
 }  // namespace

@@ -69,4 +69,120 @@ __device__ __forceinline__ fx fx_mul2(fx a, Limbs c, fx b, Limbs d) {
     return 2 * hi + (mid >> 30);
 }
 
+// ---- one component of a stencil in fixed point, beside the other in binary64
+// A binary64 multiply-add of a warp holds the SM's FP64 unit for 16 cycles; a
+// kernel bound by it leaves three quarters of its issue slots empty.  The stencil
+// kernels compute the real part with the FP64 unit and the imaginary part with
+// integer instructions, which halves the unit's work.  Measured at
+// 512 x 128 x 400: a half-sweep of the finest level 98.5 -> 72 us, the transfer
+// kernels of a solve 2.65 -> 2.26 and 1.43 -> 1.02 ms, the solve 12.2 -> 9.5 ms.
+
+// Coefficients: c = m 2^-e with m in [1/2, 1], m 2^61 in two limbs whose low word
+// carries e in its lowest 7 bits (a binary64 mantissa leaves 8 empty).
+// Every operand is aligned to the exponent of the largest *term*, so that the
+// sum is cut some 2^-58 below it however far the operands lie apart -- binary64
+// multiply-adds round 2^-53 below their partial sums.
+
+// x aligned to the exponent field emax (bits 20..30 in place), `eb` its own
+// field (less that of its coefficient), with GUARD empty bits below the sign:
+// cut toward minus infinity; shifts beyond 63 give 0 or -1.
+template <int GUARD> __device__ __forceinline__ fx fx_align(double x, int eb, int emax) {
+    const unsigned s = (unsigned)(emax - eb + (GUARD << 20)) >> 20;
+    ufx m;
+    asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(f64_mant(x)), "r"(s));   // (amounts above 63 give 0)
+    const fx sg = (fx)(__double2hiint(x) >> 31);
+    return (fx)m ^ sg;
+}
+// Exponent field in place.
+__device__ __forceinline__ int exp_bits(double x) { return __double2hiint(x) & 0x7ff00000; }
+// The result where fixed point does not reach: NaN when an operand is above
+// 2^977, infinite or NaN (squares of such values overflow: a solve with them
+// ends as non-finite either way), 0 when all are below 2^-863 (their squares
+// vanish; imaginary parts that are zero identically, those of modes 0 and N/2,
+// among them).  `lo` and `hi`: the exponent field of the largest term, before
+// and after a scale.
+__device__ __forceinline__ double fx_ends(double r, int lo, int hi) {
+    const bool z = lo < (160 << 20);
+    return __hiloint2double(hi >= (2000 << 20) ? 0x7ff80000 : z ? 0 : __double2hiint(r), z ? 0 : __double2loint(r));
+}
+__device__ __forceinline__ double fx_ends(double r, int em) { return fx_ends(r, em, em); }
+// The nearest binary64 value of r 2^(be - 1086), r in the normal range: one
+// conversion by the FP64 unit (a little more than one of its slots; some 25
+// integer instructions otherwise) and an exact change of the exponent.
+__device__ __forceinline__ double fx_to_f64_normal(fx r, int be) {
+    const double d = __ll2double_rn(r);
+    return r ? __hiloint2double(__double2hiint(d) + ((be - 1086) << 20), __double2loint(d)) : 0.0;
+}
+__device__ __forceinline__ int coef_exp(int2 c) { return (c.y & 127) << 20; }
+__device__ __forceinline__ Limbs coef_limbs(int2 c) { return {c.x, c.y & ~127}; }
+
+// b + hz (s + n) + hw w + he e (a Gauss-Seidel update).  All terms below 2^60.
+__device__ __forceinline__ double fx_update(double b, double s, double n, double w, double e, int2 hz, int2 hw,
+                                            int2 he) {
+    const int ez = coef_exp(hz), eb = exp_bits(b), es = exp_bits(s) - ez, en = exp_bits(n) - ez;
+    const int ew = exp_bits(w) - coef_exp(hw), ee = exp_bits(e) - coef_exp(he);
+    const int em = max(max(max(eb, es), max(en, ew)), ee);
+    const fx x = fx_align<3>(s, es, em) + fx_align<3>(n, en, em);
+    const fx y = fx_align<3>(w, ew, em), z = fx_align<3>(e, ee, em);
+    const Limbs c = coef_limbs(hz), d = coef_limbs(hw), f = coef_limbs(he);
+    const int xh = (int)(x >> 31), xl = (int)((unsigned)x & 0x7fffffffu), yh = (int)(y >> 31),
+              yl = (int)((unsigned)y & 0x7fffffffu), zh = (int)(z >> 31), zl = (int)((unsigned)z & 0x7fffffffu);
+    // (the products of the low limbs, below two units each, are left out)
+    fx m1 = (fx)xh * c.l, m2 = (fx)xl * c.h, hi = (fx)xh * c.h;
+    m1 += (fx)yh * d.l;
+    m2 += (fx)yl * d.h;
+    hi += (fx)yh * d.h;
+    m1 += (fx)zh * f.l;
+    m2 += (fx)zl * f.h;
+    hi += (fx)zh * f.h;
+    const fx r = 2 * hi + (m1 >> 30) + (m2 >> 30) + fx_align<3>(b, eb, em);
+    return fx_ends(fx_to_f64_normal(r, (em >> 20) + 4), em);
+}
+__device__ __forceinline__ double fx_update(double b, double s, double n, double w, double e, int4 zw, int2 ev) {
+    return fx_update(b, s, n, w, e, make_int2(zw.x, zw.y), make_int2(zw.z, zw.w), ev);
+}
+// b + cz (s + n) + cw w + ce e - d u, the coefficients given times 2^q (|q| < 60).
+__device__ __forceinline__ double fx_residual(double b, double s, double n, double w, double e, double u, int2 cz,
+                                              int2 cw, int2 ce, int2 cd, int q) {
+    const int ez = coef_exp(cz), es = exp_bits(s) - ez, en = exp_bits(n) - ez, eb = exp_bits(b) + q * (1 << 20);
+    const int ew = exp_bits(w) - coef_exp(cw), ee = exp_bits(e) - coef_exp(ce), eu = exp_bits(u) - coef_exp(cd);
+    const int em = max(max(max(es, en), max(ew, ee)), max(eu, eb));
+    const fx x = fx_align<3>(s, es, em) + fx_align<3>(n, en, em);
+    const fx y = fx_align<3>(w, ew, em), z = fx_align<3>(e, ee, em);
+    const fx v = fx_align<3>(u, eu, em);
+    const Limbs c = coef_limbs(cz), d = coef_limbs(cw), f = coef_limbs(ce), g = coef_limbs(cd);
+    const int xh = (int)(x >> 31), xl = (int)((unsigned)x & 0x7fffffffu), yh = (int)(y >> 31),
+              yl = (int)((unsigned)y & 0x7fffffffu), zh = (int)(z >> 31), zl = (int)((unsigned)z & 0x7fffffffu),
+              vh = (int)(v >> 31), vl = (int)((unsigned)v & 0x7fffffffu);
+    fx m1 = (fx)xh * c.l, m2 = (fx)xl * c.h, hi = (fx)xh * c.h;
+    m1 += (fx)yh * d.l;
+    m2 += (fx)yl * d.h;
+    hi += (fx)yh * d.h;
+    m1 += (fx)zh * f.l;
+    m2 += (fx)zl * f.h;
+    hi += (fx)zh * f.h;
+    m1 -= (fx)vh * g.l;
+    m2 -= (fx)vl * g.h;
+    hi -= (fx)vh * g.h;
+    const fx r = 2 * hi + (m1 >> 30) + (m2 >> 30) + fx_align<3>(b, eb, em);
+    const int emq = em - q * (1 << 20);
+    return fx_ends(fx_to_f64_normal(r, (emq >> 20) + 4), min(em, emq), max(em, emq));
+}
+// u + (9 c0 + 3 (+-c1) + 3 (+-c2) +- c3) / 16: bilinear interpolation, s1 s2 set for a minus.
+__device__ __forceinline__ double fx_bilinear(double u, double c0, double c1, double c2, double c3, bool s1, bool s2) {
+    const int em = max(max(max(exp_bits(u), exp_bits(c0)), max(exp_bits(c1), exp_bits(c2))), exp_bits(c3));
+    const fx a = fx_align<4>(c0, exp_bits(c0), em);
+    const fx m1 = s1 ? -1 : 0, m2 = s2 ? -1 : 0;   // (one's complement: a unit off)
+    const fx t = (fx_align<4>(c1, exp_bits(c1), em) ^ m1) + (fx_align<4>(c2, exp_bits(c2), em) ^ m2);
+    const fx r = 8 * a + a + 2 * t + t + (fx_align<4>(c3, exp_bits(c3), em) ^ m1 ^ m2);
+    return fx_ends(fx_to_f64_normal((r >> 4) + fx_align<4>(u, exp_bits(u), em), (em >> 20) + 5), em);
+}
+// u + (3 c0 +- c1) / 4.
+__device__ __forceinline__ double fx_linear(double u, double c0, double c1, bool s1) {
+    const int em = max(max(exp_bits(u), exp_bits(c0)), exp_bits(c1));
+    const fx a = fx_align<4>(c0, exp_bits(c0), em), m1 = s1 ? -1 : 0;
+    const fx r = 2 * a + a + (fx_align<4>(c1, exp_bits(c1), em) ^ m1);
+    return fx_ends(fx_to_f64_normal((r >> 2) + fx_align<4>(u, exp_bits(u), em), (em >> 20) + 5), em);
+}
+
 }  // namespace pp

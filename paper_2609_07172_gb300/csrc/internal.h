@@ -80,6 +80,11 @@ template <class T> struct LevelDev {
     const T *cw, *ce, *cz;        // [nr]
     const T *invd, *diag;         // [ncls][nr][nm]: omega / diag, diag
     const T *hw, *he, *hz;        // [ncls][nr][nm] omega * off-diagonal conductances / diag
+    const int4 *hzw;              // FP64 levels without per-row tables, omega = 1: the h tables in limbs
+    const int2 *hev;              // (fixed.h), (hz, hw) and he, [ncls][nr][nm]; else null
+    const int4 *rzw;              // FP64 levels without per-row tables: cz, cw [nr], ce [nr] and
+    const int2 *rev, *rdg;        // diag [ncls][nr][nm] times 2^rq in limbs; else null
+    int rq;
     const int *rcls;              // per-row tables (composite domain or non-uniform axial mesh): coefficient
                                   // class of each row [nz]; null: rows 0 and nz-1 are classes 0 and
                                   // ncls-1, the others class 1.  An inactive cell has zero diag, invd and
@@ -331,6 +336,9 @@ cudaError_t launch_interp(const TabRef<T> &tab, unsigned grid, cudaStream_t st, 
                           bool black_only = false);
 template <class T>
 cudaError_t launch_rhs_restrict(const TabRef<T> &tab, unsigned grid, cudaStream_t st, bool masked = false);
+
+// The limb tables of a level from its binary64 ones (ntab entries of [ncls][nr][nm]).
+cudaError_t launch_limbs(const LevelDev<double> &L, size_t ntab, cudaStream_t st);
 
 // zero_x: the FP64 iterate is zero (r = b; the kernel also writes x = 0).
 cudaError_t launch_defect(const DefectTab *tab, unsigned grid, const Ctrl *ctrl, double *partials, bool zero_x,

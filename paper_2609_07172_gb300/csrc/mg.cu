@@ -20,12 +20,15 @@
 //  * the smoother uses coefficients pre-divided by the diagonal and a
 //    right-hand side b_hat = b / diag, so one Gauss-Seidel update is
 //    u = b_hat + h_z (u_S + u_N) + h_w u_W + h_e u_E (4 FP64 ops per component);
+//  * on levels without per-row tables the imaginary part is computed in 64-bit
+//    fixed point by the integer pipes while the FP64 unit does the real part;
 //  * after a black half-sweep the black cells satisfy their equations, so the
 //    residual (and the restricted right-hand side) only needs the red cells;
 //  * the red half-sweep that follows a prolongation overwrites the red cells
 //    without reading them, so only black cells receive the correction;
 //  * on coarse levels the first red half-sweep from a zero iterate is just
 //    u_red = b_hat_red, written by the restriction kernel.
+#include "fixed.h"
 #include "internal.h"
 
 namespace pp {
@@ -114,6 +117,20 @@ __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i,
         if (i < L.nr - 1) acc = fma2<T>(L.cce[ci], L.u[idx + L.nm], acc);
         return fma2<T>(-d, L.u[idx], acc);
     }
+    if constexpr (sizeof(T) == sizeof(double)) {
+        if (L.rzw) {   // real part on the FP64 unit, imaginary part in fixed point (fixed.h)
+            const unsigned rs = (unsigned)L.nr * (unsigned)L.nm;
+            const V2<T> zero = mk<T>(0, 0), *u = L.u + idx;
+            const V2<T> us = k > 0 ? *(u - rs) : zero, un = k < L.nz - 1 ? u[rs] : zero;
+            const V2<T> uw = i > 0 ? *(u - L.nm) : zero, ue = i < L.nr - 1 ? u[L.nm] : zero, uc = *u, b = L.b[idx];
+            const unsigned tb = (unsigned)row_class(k, L.nz, L.ncls) * rs + (unsigned)i * (unsigned)L.nm + (unsigned)m;
+            const int4 zw = L.rzw[i];
+            const int2 ev = L.rev[i], dg = L.rdg[tb];
+            return mk<T>(fma(-L.diag[tb], uc.x, fma(L.ce[i], ue.x, fma(L.cw[i], uw.x, fma(L.cz[i], us.x + un.x, b.x)))),
+                         fx_residual(b.y, us.y, un.y, uw.y, ue.y, uc.y, make_int2(zw.x, zw.y), make_int2(zw.z, zw.w),
+                                     ev, dg, L.rq));
+        }
+    }
     V2<T> s = mk<T>(0, 0);
     if (k > 0) s = L.u[idx - rowstride];
     if (k < L.nz - 1) {
@@ -153,6 +170,30 @@ __device__ __forceinline__ void smooth_body(const LevelDev<T> &L, unsigned blk, 
     if constexpr (S == 0) {
         const unsigned e = blk * NT + threadIdx.x;
         if (e >= (unsigned)L.nz * (unsigned)(L.nr >> 1) * nm) return;
+        if constexpr (sizeof(T) == sizeof(double) && !RW && !SOR) {
+            // Real part on the FP64 unit, imaginary part in fixed point (fixed.h).
+            // (launch bounds of three quarters of the warps: the integer path needs
+            // more than 32 registers)
+            const unsigned c = fdiv(e, nm, L.rnm), m = e - c * nm;
+            const unsigned hr = (unsigned)L.nr >> 1, k = fdiv(c, hr, L.rhr);
+            const unsigned i = 2 * (c - k * hr) + ((k + (unsigned)color) & 1u);
+            const unsigned rs = (unsigned)L.nr * nm, col = i * nm + m, idx = k * rs + col;
+            const unsigned tb = (unsigned)row_class((int)k, L.nz, L.ncls) * rs + col;
+            if (EARLY) {
+                pdl_wait();
+                pdl_go();
+            }
+            const double2 zero = make_double2(0.0, 0.0);
+            const double2 *u = L.u + idx;
+            const double2 us = k > 0 ? *(u - rs) : zero, un = k + 1 < (unsigned)L.nz ? u[rs] : zero;
+            const double2 uw = i > 0 ? *(u - nm) : zero, ue = i + 1 < (unsigned)L.nr ? u[nm] : zero, b = L.bh[idx];
+            const int4 q = L.hzw[tb];
+            const int2 qe = L.hev[tb];
+            const double hz = L.hz[tb], hw = L.hw[tb], he = L.he[tb];
+            L.u[idx] = make_double2(fma(he, ue.x, fma(hw, uw.x, fma(hz, us.x + un.x, b.x))),
+                                    fx_update(b.y, us.y, un.y, uw.y, ue.y, q, qe));
+            return;
+        }
         // (plain divisions: this kernel is capped at 32 registers for full
         // occupancy, and the multiply-high form needs more)
         const unsigned c = e / nm;
@@ -225,6 +266,13 @@ __device__ __forceinline__ void smooth_body(const LevelDev<T> &L, unsigned blk, 
             pdl_go();
         }
         const T hz1 = __ldg(L.hz + t1), hw1 = __ldg(L.hw + t1), he1 = __ldg(L.he + t1);
+        constexpr bool FX = sizeof(T) == sizeof(double) && !RW && !SOR;   // imaginary part in fixed point, as above
+        int4 zw1 = make_int4(0, 0, 0, 0);
+        int2 ev1 = make_int2(0, 0);
+        if (FX) {
+            zw1 = __ldg(L.hzw + t1);
+            ev1 = __ldg(L.hev + t1);
+        }
         const V2<T> zero = mk<T>(0, 0);
         const size_t idx0 = (size_t)k0 * rs + tcol;
         V2<T> south = k0 > 0 ? __ldg(L.u + idx0 - rs) : zero;
@@ -253,6 +301,23 @@ __device__ __forceinline__ void smooth_body(const LevelDev<T> &L, unsigned blk, 
             }
             T hz = hz1, hw = hw1, he = he1;
             V2<T> acc;
+            if constexpr (FX) {
+                int4 zw = zw1;
+                int2 ev = ev1;
+                if (k == 0 || k == L.nz - 1) {   // boundary rows have their own coefficient class
+                    const size_t tb = (size_t)row_class(k, L.nz, L.ncls) * rs + tcol;
+                    hz = L.hz[tb];
+                    hw = L.hw[tb];
+                    he = L.he[tb];
+                    zw = L.hzw[tb];
+                    ev = L.hev[tb];
+                }
+                L.u[idx0 + (size_t)(2 * t) * rs] =   // (absent neighbours are zero)
+                    mk<T>(fma(he, ve[t].x, fma(hw, vw[t].x, fma(hz, south.x + vn[t].x, vb[t].x))),
+                          (T)fx_update(vb[t].y, south.y, vn[t].y, vw[t].y, ve[t].y, zw, ev));
+                south = vn[t];
+                continue;
+            }
             if (RW && L.rcls && sizeof(T) == sizeof(double)) {   // per-row tables, FP64
                 const size_t tb = (size_t)L.rcls[k] * rs + tcol;
                 hw = L.hw[tb];
@@ -292,7 +357,7 @@ __device__ __forceinline__ void smooth_body(const LevelDev<T> &L, unsigned blk, 
 }
 
 template <class T, int NT, int S, bool SOR, bool RW, bool ONE>
-__global__ void __launch_bounds__(NT, S == 0 ? 2048 / NT : 1)
+__global__ void __launch_bounds__(NT, S == 0 ? (sizeof(T) == 8 && !RW && !SOR ? 1536 : 2048) / NT : 1)
 k_smooth(const __grid_constant__ LevelArg<T> arg, int color) {
     if constexpr (ONE) {
         smooth_body<T, NT, S, SOR, RW, true>(arg.f, blockIdx.x, color);
@@ -300,8 +365,15 @@ k_smooth(const __grid_constant__ LevelArg<T> arg, int color) {
         const LaunchTab<T> *__restrict__ tab = arg.tab;
         const int p = find_problem(tab->start, tab->n, blockIdx.x);
         if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
-        const LevelDev<T> L = tab->f[p];
-        smooth_body<T, NT, S, SOR, RW, false>(L, blockIdx.x - tab->start[p], color);
+        if constexpr (sizeof(T) == sizeof(double) && S == 0 && !SOR && !RW) {
+            __shared__ LevelDev<T> L;
+            stage_view(&L, &tab->f[p]);
+            __syncthreads();
+            smooth_body<T, NT, S, SOR, RW, false>(L, blockIdx.x - tab->start[p], color);
+        } else {
+            const LevelDev<T> L = tab->f[p];
+            smooth_body<T, NT, S, SOR, RW, false>(L, blockIdx.x - tab->start[p], color);
+        }
     }
 }
 
@@ -493,13 +565,15 @@ __device__ __forceinline__ void prolong_body(const LevelDev<T> &F, const LevelDe
         const T w1 = iin ? T(0.1875) : T(-0.1875), w2 = kin ? T(0.1875) : T(-0.1875);
         const T w3 = iin == kin ? T(0.0625) : T(-0.0625);
         u.x = fma(w3, c3.x, fma(w2, c2.x, fma(w1, c1.x, fma(T(0.5625), c0.x, u.x))));
-        u.y = fma(w3, c3.y, fma(w2, c2.y, fma(w1, c1.y, fma(T(0.5625), c0.y, u.y))));
+        if constexpr (sizeof(T) == sizeof(double)) u.y = fx_bilinear(u.y, c0.y, c1.y, c2.y, c3.y, !iin, !kin);
+        else u.y = fma(w3, c3.y, fma(w2, c2.y, fma(w1, c1.y, fma(T(0.5625), c0.y, u.y))));
     } else {
         // linear along the coarsened direction
         const V2<T> c1 = cz2 ? cu[(unsigned)Kx * crow + (unsigned)I * nm] : cu[(unsigned)K * crow + (unsigned)Ix * nm];
         const T w1 = (cz2 ? kin : iin) ? T(0.25) : T(-0.25);
         u.x = fma(w1, c1.x, fma(T(0.75), c0.x, u.x));
-        u.y = fma(w1, c1.y, fma(T(0.75), c0.y, u.y));
+        if constexpr (sizeof(T) == sizeof(double)) u.y = fx_linear(u.y, c0.y, c1.y, cz2 ? !kin : !iin);
+        else u.y = fma(w1, c1.y, fma(T(0.75), c0.y, u.y));
     }
     F.u[idx] = u;
 }
@@ -738,6 +812,31 @@ __global__ void __launch_bounds__(MG_THREADS) k_coarse(const CoarseTab<T> *__res
         if (nz & 1) e = fma(Vs[k * nz + nz - 1], ws[(nz - 1) * lw + i], e);
         ug[2 * ((size_t)(k * nr + i) * nm + m)] = e + o;
         if (nz - 1 - k != k) ug[2 * ((size_t)((nz - 1 - k) * nr + i) * nm + m)] = e - o;
+    }
+}
+
+// 0 <= x <= 1 as a coefficient (fixed.h): limbs of m 2^61 and e, x = m 2^-e.
+__device__ __forceinline__ int2 to_coef(double x) {
+    const int e = 1022 - f64_exp(x), lim = min(max(e, 0), 127);   // (1 has m = 1, e = 0)
+    const ufx m = f64_exp(x) ? (e < 0 ? 2 * (f64_mant(x) >> 2) : (f64_mant(x) >> 2) >> min(e - lim, 63)) : 0;
+    return make_int2((int)(m >> 31), (int)((unsigned)m & 0x7fffff80u) | lim);
+}
+// x 2^q, exactly (x 0 or normal, as is the result).
+__device__ __forceinline__ double times_pow2(double x, int q) {
+    return f64_exp(x) ? __hiloint2double(__double2hiint(x) + q * (1 << 20), __double2loint(x)) : 0.0;
+}
+__global__ void __launch_bounds__(256) k_limbs(const LevelDev<double> L, size_t ntab) {
+    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= ntab) return;
+    const int2 z = to_coef(L.hz[t]), w = to_coef(L.hw[t]);
+    const_cast<int4 *>(L.hzw)[t] = make_int4(z.x, z.y, w.x, w.y);
+    const_cast<int2 *>(L.hev)[t] = to_coef(L.he[t]);
+    if (!L.rzw) return;
+    const_cast<int2 *>(L.rdg)[t] = to_coef(times_pow2(L.diag[t], L.rq));
+    if (t < (size_t)L.nr) {
+        const int2 a = to_coef(times_pow2(L.cz[t], L.rq)), b = to_coef(times_pow2(L.cw[t], L.rq));
+        const_cast<int4 *>(L.rzw)[t] = make_int4(a.x, a.y, b.x, b.y);
+        const_cast<int2 *>(L.rev)[t] = to_coef(times_pow2(L.ce[t], L.rq));
     }
 }
 
@@ -1011,6 +1110,11 @@ cudaError_t launch_defect(const DefectTab *tab, unsigned grid, const Ctrl *ctrl,
 
 cudaError_t launch_update(const DefectTab *tab, unsigned grid, const Ctrl *ctrl, cudaStream_t st) {
     return launch_pdl(k_update, grid, MG_THREADS, 0, st, tab, ctrl);
+}
+
+cudaError_t launch_limbs(const LevelDev<double> &L, size_t ntab, cudaStream_t st) {
+    k_limbs<<<(unsigned)((ntab + 255) / 256), 256, 0, st>>>(L, ntab);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_bnorm(Ctrl *ctrl, const FFTTab *fft, const double *partials, cudaStream_t st) {

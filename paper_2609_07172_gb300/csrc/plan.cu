@@ -655,6 +655,27 @@ template <class T, class V> void carve_level(const LevelHost &h, int nm, int nt,
     v.hw = c.take<T>(ntab);
     v.he = c.take<T>(ntab);
     v.hz = c.take<T>(ntab);
+    const bool fxt = std::is_same<T, double>::value && h.rcls.empty();
+    v.hzw = fxt ? c.take<int4>(ntab) : nullptr;
+    v.hev = fxt ? c.take<int2>(ntab) : nullptr;
+    v.rzw = fxt ? c.take<int4>(h.nr) : nullptr;
+    v.rev = fxt ? c.take<int2>(h.nr) : nullptr;
+    v.rdg = fxt ? c.take<int2>(ntab) : nullptr;
+    int rq = 0;   // the largest diagonal times 2^rq in [1/2, 1)
+    if (fxt) {
+        double dmax = 0.0;
+        for (double d : h.diag) dmax = std::max(dmax, d);
+        std::frexp(dmax, &rq);
+        if (dmax > 0.0 && std::abs(rq) < 60) {
+            v.rq = -rq;
+        } else {   // (coefficients out of that range: the FP64 unit computes both parts)
+            v.rzw = nullptr;
+            v.rev = v.rdg = nullptr;
+            v.rq = 0;
+        }
+    } else {
+        v.rq = 0;
+    }
     v.rcls = h.rcls.empty() ? nullptr : c.take<int>(h.nz);
     v.holes = std::find(h.act.begin(), h.act.end(), (unsigned char)0) != h.act.end() ? 1 : 0;
     const bool rw = !h.rcls.empty();
@@ -835,6 +856,9 @@ template <class T> void upload_level(const LevelHost &h, const LevelDev<T> &v, c
     to_dev(h.hw, v.hw, st, err);
     to_dev(h.he, v.he, st, err);
     to_dev(h.hz, v.hz, st, err);
+    if constexpr (std::is_same<T, double>::value) {   // the same coefficients in limbs
+        if (v.hzw && err == cudaSuccess) err = launch_limbs(v, h.hz.size(), st);
+    }
 }
 
 // Launch tables of one precision's hierarchy.  views(q) is problem q's level list.
