@@ -119,9 +119,9 @@ typedef struct {
     int smooth_fused;          /* mixed precision: 1 runs each pre- or post-smoothing of an FP32 level
                                   (1 or 2 sweeps, omega = 1, even nr) as one fused pass; 0 separate
                                   half-sweeps */
-    int local_bottom;          /* 0: the level above the coarsest and the coarsest solve run per mode in
-                                  one block's shared memory where they fit (omega = 1, 3 or more levels);
-                                  -1: never (separate launches) */
+    int local_bottom;          /* 0: the lower levels -- at least the level above the coarsest and the
+                                  coarsest solve, of small problems all of them -- run per mode in shared
+                                  memory where they fit (omega = 1); -1: never (separate launches) */
     int fmg;                   /* FP64: 1 starts a solve with a full-multigrid pass: from a zero iterate,
                                   the right-hand side restricted to every level, coarsest solve, then
                                   prolongation and one V-cycle per level up to the finest; from a given

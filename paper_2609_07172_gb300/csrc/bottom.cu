@@ -18,6 +18,7 @@
 // changes.
 #include <algorithm>
 
+#include "coarse.h"
 #include "fixed.h"
 #include "internal.h"
 
@@ -105,7 +106,7 @@ __device__ __forceinline__ void bottom_body(const BottomTab<T> *__restrict__ tab
 
     // shared memory (element type T): U: u, b_hat, b [n]; tables [ncls][nr] x 4, [nr] x 3;
     // C: right-hand side / correction [nc]; separable solve: w [ncz][ncr + 1], V [ceil(ncz/2)][ncz],
-    // this mode's Thomas factorisation piv, cpr [ncz][ncr + 1] and the off-diagonal e [ncr]
+    // this mode's factorisation piv, cpr, f [ncz][ncr + 1], Q [ncz][TRI_Q], exponents [ncr]
     T *u = (T *)smraw;
     T *bh = u + n;
     T *b = bh + n;
@@ -117,12 +118,14 @@ __device__ __forceinline__ void bottom_body(const BottomTab<T> *__restrict__ tab
     T *ce = cw + nr;
     T *cz = ce + nr;
     T *bc = cz + nr;
-    const int lw = ncr + 1, hzc = ncz - ncz / 2, hc = ncz / 2;
+    const int lw = ncr + 1, hzc = ncz - ncz / 2;
     T *ws = bc + nc;
     T *Vs = ws + ncz * lw;
     T *ps = Vs + hzc * ncz;
     T *cs = ps + ncz * lw;
-    T *es = cs + ncz * lw;
+    T *fs = cs + ncz * lw;
+    T *Qs = fs + ncz * lw;
+    int *ecol = (int *)(Qs + ncz * TRI_Q);
 
     // Every load of the block is issued at once (cp.async) in two groups: what
     // the pre-smoothing reads (the smoother's tables, before the wait for the
@@ -179,15 +182,18 @@ __device__ __forceinline__ void bottom_body(const BottomTab<T> *__restrict__ tab
             cp_async_elem(cz + i, U.cz + i);
         }
     }
-    for (int f = threadIdx.x; f < hzc * ncz; f += blockDim.x) cp_async_elem(Vs + f, D.V + f);
+    const T *V = D.Vl ? (const T *)D.Vl : D.V;
+    for (int f = threadIdx.x; f < hzc * ncz; f += blockDim.x) cp_async_elem(Vs + f, V + f);
     {
-        const T *gp = D.piv + (size_t)m * ncz * ncr, *gc = D.cpr + (size_t)m * ncz * ncr;
+        const size_t base = (size_t)m * ncz * ncr;
         for (int f = threadIdx.x; f < ncz * ncr; f += blockDim.x) {
             const int j = f / ncr, i = f - j * ncr;
-            cp_async_elem(ps + j * lw + i, gp + f);
-            cp_async_elem(cs + j * lw + i, gc + f);
+            cp_async_elem(ps + j * lw + i, D.piv + base + f);
+            cp_async_elem(cs + j * lw + i, D.cpr + base + f);
+            cp_async_elem(fs + j * lw + i, D.f + base + f);
         }
-        for (int i = threadIdx.x; i + 1 < ncr; i += blockDim.x) cp_async_elem(es + i, D.e + i);
+        if (ncr > TRI_SERIAL)
+            for (int f = threadIdx.x; f < ncz * TRI_Q; f += blockDim.x) cp_async_elem(Qs + f, D.fq + (size_t)m * ncz * TRI_Q + f);
     }
     cp_async_group_close();
     cp_async_group_wait<1>();
@@ -223,38 +229,11 @@ __device__ __forceinline__ void bottom_body(const BottomTab<T> *__restrict__ tab
     }
     __syncthreads();
 
-    // exact solve on C (the separable, mirror-folded solve of k_coarse)
-    for (int f = threadIdx.x; f < hc * ncr; f += blockDim.x) {
-        const int k = f / ncr, i = f - k * ncr;
-        const T lo = bc[k * ncr + i], hi = bc[(ncz - 1 - k) * ncr + i];
-        bc[k * ncr + i] = lo + hi;
-        bc[(ncz - 1 - k) * ncr + i] = lo - hi;
-    }
+    // exact solve on C (the separable, mirror-folded solve of k_coarse), correction into bc
+    coarse_forward(bc, ws, Vs, ecol, ncr, ncz, lw);
+    tri_rows<T, 1>(ws, ps, fs, cs, Qs, ncz, ncr, lw);
     __syncthreads();
-    for (int f = threadIdx.x; f < nc; f += blockDim.x) {
-        const int j = f / ncr, i = f - j * ncr;
-        T a = 0;
-        if ((j & 1) == 0) {
-            for (int k = 0; k < hzc; ++k) a = fma(Vs[k * ncz + j], bc[k * ncr + i], a);
-        } else {
-            for (int k = 0; k < hc; ++k) a = fma(Vs[k * ncz + j], bc[(ncz - 1 - k) * ncr + i], a);
-        }
-        ws[j * lw + i] = a;
-    }
-    __syncthreads();
-    thomas_rows(ws, ps, cs, es, ncz, ncr, lw);
-    __syncthreads();
-    for (int f = threadIdx.x; f < hzc * ncr; f += blockDim.x) {   // correction into bc
-        const int k = f / ncr, i = f - k * ncr;
-        T e = 0, o = 0;
-        for (int j = 0; j + 1 < ncz; j += 2) {
-            e = fma(Vs[k * ncz + j], ws[j * lw + i], e);
-            o = fma(Vs[k * ncz + j + 1], ws[(j + 1) * lw + i], o);
-        }
-        if (ncz & 1) e = fma(Vs[k * ncz + ncz - 1], ws[(ncz - 1) * lw + i], e);
-        bc[k * ncr + i] = e + o;
-        if (ncz - 1 - k != k) bc[(ncz - 1 - k) * ncr + i] = e - o;
-    }
+    coarse_back(ws, Vs, ecol, ncr, ncz, lw, [&](int k, int i, T v) { bc[k * ncr + i] = v; });
     __syncthreads();
 
     // prolongation of the correction (as k_prolong; black cells only when the
@@ -321,8 +300,8 @@ __global__ void __launch_bounds__(BOTTOM_THREADS) k_bottom(const BottomTab<T> *_
 
 template <class T> size_t bottom_smem_bytes(int nr, int nz, int ncls, int ncr, int ncz) {
     const size_t n = (size_t)nr * nz, nc = (size_t)ncr * ncz;
-    return (3 * n + 4 * (size_t)ncls * nr + 3 * (size_t)nr + nc + 3 * (size_t)ncz * (ncr + 1) +
-            (size_t)(ncz - ncz / 2) * ncz + (size_t)ncr) * sizeof(T);
+    return (3 * n + 4 * (size_t)ncls * nr + 3 * (size_t)nr + nc + 4 * (size_t)ncz * (ncr + 1) +
+            (size_t)(ncz - ncz / 2) * ncz + (size_t)ncz * TRI_Q + (size_t)ncr) * sizeof(T);
 }
 
 template <class T> cudaError_t launch_bottom(const BottomTab<T> *tab, unsigned grid, size_t smem, cudaStream_t st) {

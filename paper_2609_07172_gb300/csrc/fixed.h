@@ -185,4 +185,30 @@ __device__ __forceinline__ double fx_linear(double u, double c0, double c1, bool
     return fx_ends(fx_to_f64_normal((r >> 2) + fx_align<4>(u, exp_bits(u), em), (em >> 20) + 5), em);
 }
 
+
+// Sums of products of a column's values, aligned to the column's largest exponent
+// (fx_align<5>: below 2^58), with constants |c| <= 1 as c 2^61 = h 2^31 + l,
+// |l| <= 2^30.  Up to 64 products with sum |c| <= 8: three multiply-adds of the
+// integer pipe each in place of one that holds the FP64 unit for 16 cycles, and
+// sums that do not depend on their order.
+struct FxSum {
+    fx hi = 0, m1 = 0, m2 = 0;
+};
+__device__ __forceinline__ int2 fx_split(fx x) {
+    const int h = (int)((x + (1ll << 30)) >> 31);
+    return make_int2(h, (int)(x - ((fx)h << 31)));
+}
+__device__ __forceinline__ int4 fx_split2(fx x, fx y) {
+    const int2 a = fx_split(x), b = fx_split(y);
+    return make_int4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void fx_mac(FxSum &s, int xh, int xl, int2 c) {
+    s.hi += (fx)xh * c.x;
+    s.m1 += (fx)xh * c.y;
+    s.m2 += (fx)xl * c.x;
+}
+__device__ __forceinline__ fx fx_total(const FxSum &s) { return 2 * s.hi + (s.m1 >> 30) + (s.m2 >> 30); }
+// A total as binary64, em the column's exponent field.
+__device__ __forceinline__ double fx_column(fx r, int em) { return fx_ends(fx_to_f64_normal(r, (em >> 20) + 6), em); }
+
 }  // namespace pp

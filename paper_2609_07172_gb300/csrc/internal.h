@@ -98,12 +98,15 @@ template <class T> struct LevelDev {
 };
 
 // Coarsest level: separable direct solve (z eigenbasis, tridiagonal in r).
+constexpr int TRI_Q = 48;         // products of factors per row of the tridiagonal solves (coarse.h)
 template <class T> struct CoarseDev {
     int nr, nz, nm;
     const T *V;                   // [nz][nz] orthonormal eigenvectors of the axial operator, V[k*nz+j]
+    const int2 *Vl;               // FP64: the same as limbs of V 2^61 (fixed.h); else null
     const T *e;                   // [nr] off-diagonal -ce_i of the radial operator
     const T *piv;                 // [nm][nz][nr] inverse pivots of the Thomas factorisation
     const T *cpr;                 // [nm][nz][nr] upper multipliers of the Thomas factorisation
+    const T *f, *fq;              // [nm][nz][nr], [nm][nz][TRI_Q]: its factors as tri_rows (coarse.h) takes them
     // composite domain (nact > 0): dense solve over the nact active cells,
     // A_m = A_0 + lambda_m diag(mu) = M^(-1/2) Q (Lambda + lambda_m) Q^T M^(-1/2) with M = diag(mu)
     int nact;
@@ -241,6 +244,7 @@ struct Ctrl {
     int done_cycles[kMaxBatch];
     unsigned rbegin[kMaxBatch];   // residual-norm partials of problem p: [rbegin, rend)
     unsigned rend[kMaxBatch];
+    unsigned arrived;             // blocks that have come to a test of launch_deep_solve
 };
 
 // First stage of the residual-norm reduction: each block sums PSUM_CHUNK
@@ -337,6 +341,10 @@ cudaError_t launch_interp(const TabRef<T> &tab, unsigned grid, cudaStream_t st, 
 template <class T>
 cudaError_t launch_rhs_restrict(const TabRef<T> &tab, unsigned grid, cudaStream_t st, bool masked = false);
 
+// f and Q of a coarsest level from its factorisation.
+template <class T> cudaError_t launch_tri_factors(const CoarseDev<T> &D, cudaStream_t st);
+// V 2^61 of n entries in limbs (CoarseDev::Vl).
+cudaError_t launch_limbs_v(const double *V, int2 *Vl, int n, cudaStream_t st);
 // The limb tables of a level from its binary64 ones (ntab entries of [ncls][nr][nm]).
 cudaError_t launch_limbs(const LevelDev<double> &L, size_t ntab, cudaStream_t st);
 
@@ -422,6 +430,41 @@ constexpr size_t BOTTOM_MAX_SMEM = 200 * 1024;
 template <class T> size_t bottom_smem_bytes(int nr, int nz, int ncls, int ncr, int ncz);
 template <class T> cudaError_t launch_bottom(const BottomTab<T> *tab, unsigned grid, size_t smem, cudaStream_t st);
 
+// V-cycles of the lower levels in the shared memory of one cluster per mode
+// (deep.cu): levels l .. L-2 smoothed, level L-1 solved exactly.
+constexpr int DEEP_THREADS = 512;
+constexpr int DEEP_LEVELS = 8;
+constexpr size_t DEEP_MAX_SMEM = 225 * 1024;
+constexpr int DEEP_MAX_NZ = 64;          // rows of the coarsest level
+// Entries (cells x modes) of the first level up to which it takes that way: above,
+// the level kernels fill the chip and are as fast or faster.  Measured (us, with
+// launches / in shared memory): whole hierarchies 90 x 32 x 70 FP64 520 / 319,
+// 152 x 32 x 90 FP64 690 / 641, 128 x 64 x 96 mixed 656 / 470, 256 x 32 x 128 mixed
+// 981 / 875; below level 0, 139 k entries 981 / 916, 208 k 5,060 / 5,077, 832 k
+// 5,060 / 5,280 (FP64 9,600 / 10,470).
+constexpr size_t DEEP_MAX_WHOLE = 600000, DEEP_MAX_LOWER = 160000;
+template <class T> struct DeepLevel {
+    LevelDev<T> L;
+    int fz, fr, zmul;             // coarsening to the next level; rows per row of the coarsest level
+    unsigned u, bh, b, tab;       // shared-memory offsets
+};
+template <class T> struct DeepArg {
+    int nl = 0;                   // smoothed levels (0: not available)
+    int C = 1;                    // blocks per cluster; the coarsest level has at least as many rows
+    int pre = 0, post = 0, red_only = 0, black_only = 0;
+    int top_b = 0;                // the first level's b is held in shared memory too
+    int bottom = 0;               // a full-multigrid start solves the two coarsest levels together
+    unsigned bc = 0, fo = 0, ws = 0, V = 0, ps = 0, fs = 0, cs = 0, Q = 0, ecol = 0, smem = 0;
+    CoarseDev<T> D{};
+    DeepLevel<T> lv[DEEP_LEVELS]{};
+};
+template <class T> size_t deep_layout(DeepArg<T> &A, int C);   // sets C and the offsets, returns the bytes
+template <class T> int deep_resident(const DeepArg<T> &A);      // clusters of A that the device holds at a time
+template <class T> cudaError_t launch_deep(const DeepArg<T> &A, bool from_zero, int cycles, cudaStream_t st);
+// The whole solve in one cooperative launch; every cluster must be resident.
+// start: 0 from the level's iterate, 1 from zero, 2 a full-multigrid start; partials: two per block.
+cudaError_t launch_deep_solve(const DeepArg<double> &A, int start, Ctrl *ctrl, double *partials, cudaStream_t st);
+
 // Pieces of the separable coarsest-level solve shared by k_coarse (mg.cu) and
 // k_bottom (bottom.cu).
 //
@@ -438,36 +481,6 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 __device__ __forceinline__ void cp_async_group_close() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_group_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
-// The radial tridiagonal solves of the separable coarsest solve, one per
-// axial eigenvector j < nz, in place on the rows ws[j][0 .. nr) (row stride
-// lw): forward y_i = (w_i - e_(i-1) y_(i-1)) piv_i, back x_i = y_i - cpr_i x_(i+1),
-// with the factorisation piv, cpr ([nz][lw]) and e ([nr - 1]) staged in shared
-// memory, so that a step of the recurrence waits on shared memory rather than
-// on L2.  The nz recurrences are spread over the block's first four warps
-// (one per SM sub-partition; the block has at least 128 threads).
-template <class T>
-__device__ __forceinline__ void thomas_rows(T *ws, const T *ps, const T *cs, const T *es, int nz, int nr, int lw) {
-    const int w = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31), per = (nz + 3) >> 2;
-    if (w >= 4) return;
-    for (int l = lane; l < per; l += 32) {
-        const int j = w * per + l;
-        if (j >= nz) break;
-        const T *piv = ps + (size_t)j * lw, *cpr = cs + (size_t)j * lw;
-        T *row = ws + (size_t)j * lw;
-        T y = row[0] * piv[0];
-        row[0] = y;
-        for (int i = 1; i < nr; ++i) {
-            y = (row[i] - es[i - 1] * y) * piv[i];
-            row[i] = y;
-        }
-        T x = y;
-        for (int i = nr - 2; i >= 0; --i) {
-            x = row[i] - cpr[i] * x;
-            row[i] = x;
-        }
-    }
 }
 
 constexpr int FFT_TI = 32;        // radial columns per transform CTA

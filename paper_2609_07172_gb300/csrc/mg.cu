@@ -28,6 +28,7 @@
 //    without reading them, so only black cells receive the correction;
 //  * on coarse levels the first red half-sweep from a zero iterate is just
 //    u_red = b_hat_red, written by the restriction kernel.
+#include "coarse.h"
 #include "fixed.h"
 #include "internal.h"
 
@@ -459,6 +460,11 @@ k_residual_restrict(const __grid_constant__ LevelArg<T> arg, double *__restrict_
         const LaunchTab<T> *__restrict__ tab = arg.tab;
         const int p = find_problem(tab->start, tab->n, blockIdx.x);
         if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
+        if constexpr (sizeof(T) == sizeof(float)) {
+            const LevelDev<T> F = tab->f[p], C = tab->c[p];
+            restrict_body<T, RED_ONLY, MASK, false>(F, C, blockIdx.x - tab->start[p], red, partials);
+            return;
+        }
         __shared__ LevelDev<T> F, C;
         stage_view(&F, &tab->f[p]);
         stage_view(&C, &tab->c[p]);
@@ -741,7 +747,10 @@ __global__ void __launch_bounds__(MG_THREADS) k_update(const DefectTab *__restri
 // Q_k = b_k - b_(nz-1-k), (V^T b)_j sums V[k][j] P_k (even j) or V[k][j] Q_k
 // (odd j) over the first half only, and u_k, u_(nz-1-k) = E_k +- O_k with E, O
 // the sums over even and odd j -- half the FP64 multiply-adds of the plain
-// products.  Only rows k < ceil(nz/2) of V are read.
+// products.  Only rows k < ceil(nz/2) of V are read.  The transforms of a binary64
+// level are sums of integers and its recurrences run on eight lanes each
+// (coarse.h): 45 x 35 of 17 modes 34 -> 28 us a launch, now mostly the loads of
+// the factorisation.
 template <class T>
 __global__ void __launch_bounds__(MG_THREADS) k_coarse(const CoarseTab<T> *__restrict__ tab) {
     extern __shared__ unsigned char smraw[];
@@ -755,64 +764,38 @@ __global__ void __launch_bounds__(MG_THREADS) k_coarse(const CoarseTab<T> *__res
     const int lb = (int)(blockIdx.x - tab->start[p]);
     const int m = lb >> 1, comp = lb & 1;
     // (a composite domain or non-uniform axial mesh takes the dense solve of csrc/dense.cu)
-    const int h = nz >> 1, hz = nz - h;      // mirror pairs, rows with k <= nz-1-k
+    const int hz = nz - (nz >> 1);           // rows of V that are read
     T *bs = (T *)smraw;                      // [nz][nr]: b, then P (rows < hz) and Q (row nz-1-k)
-    const int lw = nr + 1;                   // padded rows: the Thomas threads walk rows
+    const int lw = nr + 1;                   // padded rows: the tridiagonal solves walk rows
     T *ws = bs + (size_t)nz * nr;            // [nz][lw]
     T *Vs = ws + (size_t)nz * lw;            // [hz][nz]
     T *ps = Vs + (size_t)hz * nz;            // [nz][lw] this mode's inverse pivots
     T *cs = ps + (size_t)nz * lw;            // [nz][lw] and upper multipliers
-    T *es = cs + (size_t)nz * lw;            // [nr] off-diagonal
+    T *fs = cs + (size_t)nz * lw;            // [nz][lw] its factors (tri_rows)
+    T *Qs = fs + (size_t)nz * lw;            // [nz][TRI_Q]
+    int *ecol = (int *)(Qs + (size_t)nz * TRI_Q);   // [nr] columns' exponents
     // every load of the block is in flight before the one wait (cp.async)
-    const T *bg = (const T *)L.b + comp;
+    const T *bg = (const T *)L.b + comp, *V = D.Vl ? (const T *)D.Vl : D.V;
     for (int f = threadIdx.x; f < nz * nr; f += blockDim.x) cp_async_elem(bs + f, bg + 2 * ((size_t)f * nm + m));
-    for (int f = threadIdx.x; f < hz * nz; f += blockDim.x) cp_async_elem(Vs + f, D.V + f);
+    for (int f = threadIdx.x; f < hz * nz; f += blockDim.x) cp_async_elem(Vs + f, V + f);
     {
-        const T *gp = D.piv + (size_t)m * nz * nr, *gc = D.cpr + (size_t)m * nz * nr;
+        const size_t base = (size_t)m * nz * nr;
         for (int f = threadIdx.x; f < nz * nr; f += blockDim.x) {
             const int j = f / nr, i = f - j * nr;
-            cp_async_elem(ps + j * lw + i, gp + f);
-            cp_async_elem(cs + j * lw + i, gc + f);
+            cp_async_elem(ps + j * lw + i, D.piv + base + f);
+            cp_async_elem(cs + j * lw + i, D.cpr + base + f);
+            cp_async_elem(fs + j * lw + i, D.f + base + f);
         }
-        for (int i = threadIdx.x; i + 1 < nr; i += blockDim.x) cp_async_elem(es + i, D.e + i);
+        if (nr > TRI_SERIAL)
+            for (int f = threadIdx.x; f < nz * TRI_Q; f += blockDim.x) cp_async_elem(Qs + f, D.fq + (size_t)m * nz * TRI_Q + f);
     }
     cp_async_wait_all();
     __syncthreads();
-    for (int f = threadIdx.x; f < h * nr; f += blockDim.x) {
-        const int k = f / nr, i = f - k * nr;
-        const T lo = bs[k * nr + i], hi = bs[(nz - 1 - k) * nr + i];
-        bs[k * nr + i] = lo + hi;
-        bs[(nz - 1 - k) * nr + i] = lo - hi;
-    }
+    coarse_forward(bs, ws, Vs, ecol, nr, nz, lw);   // w[j][i] = sum_k V[k][j] b[k][i]
+    tri_rows<T, 1>(ws, ps, fs, cs, Qs, nz, nr, lw);   // along r, one per axial eigenvector j
     __syncthreads();
-    // w[j][i] = sum_k V[k][j] b[k][i], folded
-    for (int f = threadIdx.x; f < nz * nr; f += blockDim.x) {
-        const int j = f / nr, i = f - j * nr;
-        T a = 0;
-        if ((j & 1) == 0) {
-            for (int k = 0; k < hz; ++k) a = fma(Vs[k * nz + j], bs[k * nr + i], a);
-        } else {
-            for (int k = 0; k < h; ++k) a = fma(Vs[k * nz + j], bs[(nz - 1 - k) * nr + i], a);
-        }
-        ws[j * lw + i] = a;
-    }
-    __syncthreads();
-    // tridiagonal solves along r, one per axial eigenvector j
-    thomas_rows(ws, ps, cs, es, nz, nr, lw);
-    __syncthreads();
-    // u[k][i] = sum_j V[k][j] w[j][i] = E +- O for the mirror pair (k, nz-1-k)
     T *ug = (T *)L.u + comp;
-    for (int f = threadIdx.x; f < hz * nr; f += blockDim.x) {
-        const int k = f / nr, i = f - k * nr;
-        T e = 0, o = 0;
-        for (int j = 0; j + 1 < nz; j += 2) {
-            e = fma(Vs[k * nz + j], ws[j * lw + i], e);
-            o = fma(Vs[k * nz + j + 1], ws[(j + 1) * lw + i], o);
-        }
-        if (nz & 1) e = fma(Vs[k * nz + nz - 1], ws[(nz - 1) * lw + i], e);
-        ug[2 * ((size_t)(k * nr + i) * nm + m)] = e + o;
-        if (nz - 1 - k != k) ug[2 * ((size_t)((nz - 1 - k) * nr + i) * nm + m)] = e - o;
-    }
+    coarse_back(ws, Vs, ecol, nr, nz, lw, [&](int k, int i, T v) { ug[2 * ((size_t)(k * nr + i) * nm + m)] = v; });
 }
 
 // 0 <= x <= 1 as a coefficient (fixed.h): limbs of m 2^61 and e, x = m 2^-e.
@@ -820,6 +803,16 @@ __device__ __forceinline__ int2 to_coef(double x) {
     const int e = 1022 - f64_exp(x), lim = min(max(e, 0), 127);   // (1 has m = 1, e = 0)
     const ufx m = f64_exp(x) ? (e < 0 ? 2 * (f64_mant(x) >> 2) : (f64_mant(x) >> 2) >> min(e - lim, 63)) : 0;
     return make_int2((int)(m >> 31), (int)((unsigned)m & 0x7fffff80u) | lim);
+}
+template <class T> __global__ void __launch_bounds__(64) k_tri_factors(const CoarseDev<T> D) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= D.nm * D.nz) return;
+    const size_t b = (size_t)t * D.nr;
+    tri_factors(D.e, D.piv + b, D.cpr + b, D.nr, const_cast<T *>(D.f) + b, const_cast<T *>(D.fq) + (size_t)t * TRI_Q);
+}
+__global__ void __launch_bounds__(256) k_limbs_v(const double *__restrict__ V, int2 *__restrict__ Vl, int n) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < n) Vl[t] = fx_split(f64_to_fx(V[t], max(1024 - f64_exp(V[t]), 1)));   // |V| <= 1
 }
 // x 2^q, exactly (x 0 or normal, as is the result).
 __device__ __forceinline__ double times_pow2(double x, int q) {
@@ -1114,6 +1107,18 @@ cudaError_t launch_update(const DefectTab *tab, unsigned grid, const Ctrl *ctrl,
 
 cudaError_t launch_limbs(const LevelDev<double> &L, size_t ntab, cudaStream_t st) {
     k_limbs<<<(unsigned)((ntab + 255) / 256), 256, 0, st>>>(L, ntab);
+    return cudaGetLastError();
+}
+
+template <class T> cudaError_t launch_tri_factors(const CoarseDev<T> &D, cudaStream_t st) {
+    k_tri_factors<T><<<(unsigned)((D.nm * D.nz + 63) / 64), 64, 0, st>>>(D);
+    return cudaGetLastError();
+}
+template cudaError_t launch_tri_factors<double>(const CoarseDev<double> &, cudaStream_t);
+template cudaError_t launch_tri_factors<float>(const CoarseDev<float> &, cudaStream_t);
+
+cudaError_t launch_limbs_v(const double *V, int2 *Vl, int n, cudaStream_t st) {
+    k_limbs_v<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(V, Vl, n);
     return cudaGetLastError();
 }
 

@@ -696,7 +696,8 @@ template <class T> void carve_coarse(const ProblemPlan &q, Carver &c, CoarseDev<
     cd.nact = q.nact;
     if (q.nact > 0) {   // composite domain: dense solve (coarse_factors' tables are not used)
         const size_t na = (size_t)q.nact;
-        cd.V = cd.e = cd.piv = cd.cpr = nullptr;
+        cd.V = cd.e = cd.piv = cd.cpr = cd.f = cd.fq = nullptr;
+        cd.Vl = nullptr;
         cd.aidx = c.take<int>(na);
         cd.amap = c.take<int>((size_t)h.nr * h.nz);
         cd.Q = c.take<float>(na * na);
@@ -714,8 +715,11 @@ template <class T> void carve_coarse(const ProblemPlan &q, Carver &c, CoarseDev<
     cd.Y = cd.Z = nullptr;
     cd.up = nullptr;
     cd.V = c.take<T>((size_t)h.nz * h.nz);
+    cd.Vl = std::is_same<T, double>::value ? c.take<int2>((size_t)h.nz * h.nz) : nullptr;
     cd.e = c.take<T>(h.nr);
     cd.piv = c.take<T>(nf);
+    cd.f = c.take<T>(nf);
+    cd.fq = c.take<T>((size_t)q.nm * h.nz * TRI_Q);
     cd.cpr = c.take<T>(nf);
 }
 
@@ -797,7 +801,7 @@ void carve(pic_poisson_plan_s &P, Carver &c) {
         const LevelHost &h0 = q.lv[0];
         const size_t n0 = (size_t)h0.nr * h0.nz * q.nm;
         g_fft += (size_t)h0.nz * ((h0.nr + FFT_TI - 1) / FFT_TI);
-        if (q.L > 1) g_restr0 += mg_blocks((size_t)q.lv[1].nr * q.lv[1].nz * q.nm);
+        if (q.L > 1) g_restr0 += std::max<size_t>(mg_blocks((size_t)q.lv[1].nr * q.lv[1].nz * q.nm), 16 * (size_t)q.nm);
         else g_single += mg_blocks(n0);
         g_defect += mg_blocks(n0);
         if (p == 0) g_api = mg_blocks(n0);
@@ -862,6 +866,74 @@ template <class T> void upload_level(const LevelHost &h, const LevelDev<T> &v, c
 }
 
 // Launch tables of one precision's hierarchy.  views(q) is problem q's level list.
+// V-cycles in shared memory (deep.cu): which levels, and how many blocks a mode gets.
+template <class T, class Views, class Coarse>
+void build_deep(const pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse) {
+    H.deep_from = -1;
+    H.deep_solve = false;
+    H.deep.clear();
+    const ProblemPlan &q = P.pr[0];
+    if (P.n != 1 || P.masked || P.shared.local_bottom != 0 || P.shared.omega != 1.0 || q.L < 2 || !q.lv[0].rcls.empty()) return;
+    if (q.lv[q.L - 1].nz > DEEP_MAX_NZ) return;
+    const std::vector<LevelDev<T>> &v = views(q);
+    const CoarseDev<T> &D = coarse(q);
+    int resident[9];   // clusters of C blocks, one block per SM
+    for (int C = 1; C <= 8; ++C) {
+        DeepArg<T> A;
+        A.D = D;
+        A.C = C;
+        A.smem = (unsigned)DEEP_MAX_SMEM;
+        resident[C] = deep_resident(A);
+        if (!resident[C]) return;
+    }
+    H.deep.resize(q.L - 1);
+    int zmul = 1;
+    for (int l = q.L - 2; l >= 0; --l) {
+        const LevelDev<T> &f = v[l], &c = v[l + 1];
+        const int fz = f.nz / c.nz, fr = f.nr / c.nr;
+        zmul *= fz;
+        if (f.nr % 2 || fz * c.nz != f.nz || fr * c.nr != f.nr || fz * fr > 4 || fz * fr < 2) break;
+        if constexpr (std::is_same<T, double>::value)
+            if (!f.hzw || !f.rzw) break;
+        if (q.L - 1 - l > DEEP_LEVELS) break;
+        if ((size_t)f.nr * f.nz * f.nm > (l == 0 ? DEEP_MAX_WHOLE : DEEP_MAX_LOWER)) break;
+        DeepArg<T> A;
+        A.nl = q.L - 1 - l;
+        A.pre = P.shared.pre_sweeps;
+        A.post = P.shared.post_sweeps;
+        A.red_only = A.pre > 0;
+        A.black_only = A.post > 0;
+        A.bottom = q.bottom;
+        A.D = D;
+        int zm = zmul;
+        for (int d = 0; d < A.nl; ++d) {
+            A.lv[d].L = v[l + d];
+            A.lv[d].fz = v[l + d].nz / v[l + d + 1].nz;
+            A.lv[d].fr = v[l + d].nr / v[l + d + 1].nr;
+            A.lv[d].zmul = zm;
+            zm /= A.lv[d].fz;
+        }
+        // the smallest cluster that holds the levels; a larger one while a half-sweep of the
+        // first level is more than a cell per thread and the modes stay resident
+        int C = 0;
+        for (int b = 1; b >= 0 && !C; --b)
+            for (int n = 1; n <= 8 && n <= D.nz && !C; ++n) {
+                A.top_b = b;
+                if (deep_layout(A, n) <= DEEP_MAX_SMEM) C = n;
+            }
+        if (!C) break;
+        const size_t cells = (size_t)f.nr / 2 * f.nz;
+        while (C < 8 && C < D.nz && f.nm <= resident[C + 1] && cells > (size_t)C * DEEP_THREADS) ++C;
+        if (std::is_same<T, double>::value && l == 0) {   // (the whole solve or nothing)
+            if (f.nm > resident[C]) break;
+            H.deep_solve = true;
+        }
+        deep_layout(A, C);
+        H.deep[l] = A;
+        H.deep_from = l;
+    }
+}
+
 template <class T, class Views, class Coarse>
 void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, cudaStream_t st, cudaError_t &err) {
     const int nl = std::max(P.Lmax - 1, 0);
@@ -1045,8 +1117,8 @@ void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, c
         tc.f[tc.n] = views(q)[q.L - 1];
         tc.c[tc.n] = cd;
         tc.start[tc.n + 1] = tc.start[tc.n] + 2u * (unsigned)q.nm;   // (mode, real / imaginary part)
-        const size_t sm = ((size_t)cd.nr * cd.nz + 3 * (size_t)(cd.nr + 1) * cd.nz +
-                           (size_t)(cd.nz - cd.nz / 2) * cd.nz + (size_t)cd.nr) * sizeof(T);
+        const size_t sm = ((size_t)cd.nr * cd.nz + 4 * (size_t)(cd.nr + 1) * cd.nz +
+                           (size_t)(cd.nz - cd.nz / 2) * cd.nz + (size_t)cd.nz * TRI_Q + (size_t)cd.nr) * sizeof(T);
         tc.smem = std::max(tc.smem, sm);
         ++tc.n;
     }
@@ -1059,6 +1131,7 @@ void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, c
     H.g_bottom = tb.start[tb.n];
     H.smem_bottom = smem_b;
     if (tb.n) blob_to_dev(tb, H.bottom, st, err);
+    build_deep(P, H, views, coarse);
 }
 
 int upload(pic_poisson_plan_s &P) {
@@ -1093,9 +1166,15 @@ int upload(pic_poisson_plan_s &P) {
                 to_dev(e, cd.e, st, err);
                 to_dev(piv, cd.piv, st, err);
                 to_dev(cpr, cd.cpr, st, err);
+                if (err == cudaSuccess) err = launch_tri_factors(cd, st);
             };
-            if (!mixed) put(q.cd);
-            else put(q.cf);
+            if (!mixed) {
+                put(q.cd);
+                if (err == cudaSuccess)
+                    err = launch_limbs_v(q.cd.V, const_cast<int2 *>(q.cd.Vl), q.cd.nz * q.cd.nz, st);
+            } else {
+                put(q.cf);
+            }
         }
         const int nt = q.d.ntheta, M = nt / 2;
         std::vector<int> tw(8 * (size_t)(M + 1), 0);   // e^{-2 pi i m / nt} in limbs

@@ -67,6 +67,9 @@ template <class T> struct Hier {
     BottomTab<T> *bottom = nullptr;           // problems with a mode-local bottom
     unsigned g_bottom = 0;
     size_t smem_bottom = 0;
+    int deep_from = -1;                       // first level whose V-cycles run in shared memory (-1: none)
+    bool deep_solve = false;                  // FP64: the whole solve is one launch
+    std::vector<DeepArg<T>> deep;             // V-cycles from level l (csrc/deep.cu), l >= deep_from
 };
 
 // Algorithmic traffic / arithmetic / launches recorded per kernel class.

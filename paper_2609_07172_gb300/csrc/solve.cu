@@ -222,6 +222,38 @@ int coarse_and_bottom(Runner &R, const Hier<T> &H) {
     return PIC_POISSON_OK;
 }
 
+// Complex entries of level l of a plan of one problem, and of its smoothed levels from l on.
+double deep_entries(const pic_poisson_plan_s &P, int l, double *below) {
+    const ProblemPlan &q = P.pr[0];
+    *below = 0;
+    for (int d = l; d + 1 < q.L; ++d) *below += (double)q.lv[d].nr * q.lv[d].nz * q.nm;
+    return (double)q.lv[l].nr * q.lv[l].nz * q.nm;
+}
+// V-cycles from level l down, in shared memory (H.deep): `from_zero` one whose
+// level l holds b and b_hat only, else from the level's iterate.
+template <class T>
+int deep_cycles(Runner &R, const Hier<T> &H, int l, bool from_zero, int cycles) {
+    const int ph = l == 0 ? PIC_POISSON_PHASE_SMOOTH : PIC_POISSON_PHASE_COARSE;
+    double below = 0;
+    const double n = deep_entries(R.P, l, &below);
+    RUN(R, ph, launch_deep(H.deep[l], from_zero, cycles, R.st));
+    R.account(ph, (from_zero ? 3.0 : 4.0) * n * sizeof(V2<T>),
+              cycles * below * (14.0 * (R.P.shared.pre_sweeps + R.P.shared.post_sweeps) + 18.0));
+    return PIC_POISSON_OK;
+}
+
+// A whole FP64 solve in one launch, the convergence loop included (booked as
+// one pass: the number of cycles is known on the device only).
+int deep_solve(Runner &R, int start) {
+    pic_poisson_plan_s &P = R.P;
+    double below = 0;
+    const double n = deep_entries(P, 0, &below);
+    RUN(R, PIC_POISSON_PHASE_SMOOTH, launch_deep_solve(P.h64.deep[0], start, P.ctrl, P.partials, R.st));
+    R.account(PIC_POISSON_PHASE_SMOOTH, (start ? 2.5 : 3.5) * n * sizeof(double2),
+              below * (14.0 * (P.shared.pre_sweeps + P.shared.post_sweeps) + 22.0));
+    return PIC_POISSON_OK;
+}
+
 // Coarse-grid correction below level lend: level lend + 1 holds the
 // restricted residual and its initialised iterate; returns with the
 // correction prolongated into level lend and post-smoothed there (lend = 0:
@@ -230,15 +262,17 @@ template <class T>
 int descend_ascend(Runner &R, const Hier<T> &H, int lend = 0) {
     pic_poisson_plan_s &P = R.P;
     const int nl = P.Lmax - 1, pre = P.shared.pre_sweeps, post = P.shared.post_sweeps;
-    for (int l = lend + 1; l < nl; ++l) {
+    // the levels from `deep` on, where they fit, in one launch
+    const int deep = H.deep_from >= 0 ? std::max(lend + 1, H.deep_from) : nl;
+    for (int l = lend + 1; l < std::min(deep, nl); ++l) {
         int rc = smooth_level(R, H, l, pre, pre > 0, false);
         if (rc) return rc;
         rc = restrict_level(R, H, l, nullptr);
         if (rc) return rc;
     }
-    int rc0 = coarse_and_bottom(R, H);
+    int rc0 = deep < nl ? deep_cycles(R, H, deep, true, 1) : coarse_and_bottom(R, H);
     if (rc0) return rc0;
-    for (int l = nl - 1; l >= lend; --l) {
+    for (int l = std::min(deep, nl) - 1; l >= lend; --l) {
         if (!H.prolong[l]) continue;
         // the red half-sweep that follows overwrites the red cells unread
         // (Gauss-Seidel only: an over-relaxed update reads the old value)
@@ -316,6 +350,11 @@ int fmg_start(Runner &R) {
         const double n = level_entries<double>(P, l), frac = H.interp_black ? 0.5 : 1.0;
         R.account(PIC_POISSON_PHASE_PROLONG, n * sizeof(double2) * (0.25 + frac), 16.0 * frac * n);
         if (l == 0) break;   // the main iteration takes over on level 0
+        if (H.deep_from >= 0 && l >= H.deep_from) {
+            rc = deep_cycles(R, H, l, false, 1);
+            if (rc) return rc;
+            continue;
+        }
         rc = smooth_level(R, H, l, pre, false, false);
         if (rc) return rc;
         rc = restrict_level(R, H, l, nullptr);
@@ -360,6 +399,11 @@ int fmg_correction(Runner &R) {
             launch_interp(H.interp[l], H.g_interp[l], R.st, R.P.masked, H.interp_black));
         const double n = level_entries<double>(P, l), frac = H.interp_black ? 0.5 : 1.0;
         R.account(PIC_POISSON_PHASE_PROLONG, n * sizeof(double2) * (0.25 + frac), 16.0 * frac * n);
+        if (H.deep_from >= 0 && l >= H.deep_from) {
+            rc = deep_cycles(R, H, l, false, 1);
+            if (rc) return rc;
+            continue;
+        }
         rc = smooth_level(R, H, l, pre, false, false);
         if (rc) return rc;
         rc = restrict_level(R, H, l, nullptr);
@@ -394,6 +438,7 @@ int enqueue_prologue(Runner &R, int guess) {
         RUN(R, PIC_POISSON_PHASE_FORWARD, launch_copy_guess(P.guess, P.g_fft, R.st));
         R.account(PIC_POISSON_PHASE_FORWARD, 2.0 * n0 * sizeof(double2), 0.0);
     }
+    if (guess == 0 && P.h64.deep_solve) return deep_solve(R, P.shared.fmg ? 2 : 1);
     if (guess != 0) {
         if (!mixed && P.shared.fmg && P.Lmax > 1) {
             int rc = fmg_correction(R);   // full-multigrid start on the given iterate's correction
@@ -409,6 +454,7 @@ int enqueue_prologue(Runner &R, int guess) {
         }
     }
     if (mixed) return mixed_defect_and_check(R, 0, guess == 0);
+    if (P.h64.deep_solve) return deep_solve(R, 0);
     if (P.Lmax > 1) {
         int rc = smooth_level(R, P.h64, 0, P.shared.pre_sweeps, false, false);
         if (rc) return rc;
@@ -434,7 +480,12 @@ int enqueue_body(Runner &R, bool first = false) {
         return fp64_residual_and_check(R, 1);
     }
     const int inner = first ? P.shared.inner_first : P.shared.inner_cycles;
-    for (int c = 0; c < inner; ++c) {
+    const bool deep = P.h32.deep_from == 0;
+    if (deep) {
+        int rc = deep_cycles(R, P.h32, 0, true, inner);
+        if (rc) return rc;
+    }
+    for (int c = 0; c < inner && !deep; ++c) {
         if (P.Lmax > 1) {
             int rc = smooth_level(R, P.h32, 0, pre, c == 0 && pre > 0, false);
             if (rc) return rc;
@@ -559,7 +610,7 @@ int capture_graph(pic_poisson_plan_s &P, int guess) {
     PP_CUDA(cudaStreamBeginCapture(P.cap0, mode));
     cudaStreamCaptureStatus status;
     if (cudaStreamGetCaptureInfo(P.cap0, &status, nullptr, &graph, nullptr, nullptr, nullptr) != cudaSuccess ||
-        cudaGraphConditionalHandleCreate(&P.handle, graph, 0, 0) != cudaSuccess) {
+        (!P.h64.deep_solve && cudaGraphConditionalHandleCreate(&P.handle, graph, 0, 0) != cudaSuccess)) {
         set_error("graph conditional handle creation failed");
         return fail(PIC_POISSON_ECUDA);
     }
@@ -611,6 +662,7 @@ int capture_graph(pic_poisson_plan_s &P, int guess) {
             return fail(PIC_POISSON_ECUDA);
         }
     }
+    if (!P.h64.deep_solve) {   // (a solve in one launch loops by itself)
     cudaGraphNodeParams cp{};
     cp.type = cudaGraphNodeTypeConditional;
     cp.conditional.handle = P.handle;
@@ -636,6 +688,7 @@ int capture_graph(pic_poisson_plan_s &P, int guess) {
     if (cudaStreamEndCapture(P.cap1, &body) != cudaSuccess) {
         set_error("capturing the loop body failed");
         return fail(PIC_POISSON_ECUDA);
+    }
     }
     Runner R2(P, P.cap0, false, false, P.seg[v][2]);
     rc = enqueue_epilogue(R2);
