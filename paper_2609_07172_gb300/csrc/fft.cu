@@ -33,6 +33,10 @@
 // the unpack (pack) of the real transform treats modes m and M - m together,
 // sharing one twiddle product.  A column that holds an infinity or a NaN comes
 // out as NaN.
+// The modes take the place of the transform's rows (X_M a row of its own), so
+// that 256 points need 68 KB of shared memory and not 133, three blocks per SM
+// instead of one: 128 x 256 x 96 forward 81 -> 52 us, and a batch's largest problem
+// no longer costs the others their room.
 // 512 x 128 x 400: forward 586 -> 312 us (with b_hat and the norm, in a solve,
 // 653 -> 330), inverse 496 -> 272 us; both now bound by integer instructions
 // and their latency (ALU pipe 44 to 48 %, three CTAs per SM).
@@ -205,14 +209,29 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
     return s;
 }
 
+// f(entry, mode, column) for this thread's entries of a block of n entries, mode fastest
+// (the division by nm is carried along).
+template <int nm, class F> __device__ __forceinline__ void entries(int n, F f) {
+    constexpr int dm = FFT_THREADS % nm, dc = FFT_THREADS / nm;
+    int m = (int)threadIdx.x % nm, c = (int)threadIdx.x / nm;
+    for (int e = threadIdx.x; e < n; e += FFT_THREADS) {
+        f(e, m, c);
+        m += dm;
+        c += dc;
+        if (m >= nm) {
+            m -= nm;
+            ++c;
+        }
+    }
+}
+
 // LG = log2 M: the loops' bounds and the shared-memory offsets are constants.
 template <int LG>
 __device__ __forceinline__ void forward_body(const FFTProb &P, int lb, double2 *sm, double *red, int *wmax, int *wsum,
                                              double *__restrict__ partials) {
     constexpr int M = 1 << LG, nt = 2 * M, nm = M + 1;
     const int nr = P.nr, nz = P.nz;
-    double2 *buf = sm;              // [M][LD]
-    double2 *outb = sm + M * LD;    // [TI][nm]
+    double2 *buf = sm;              // [M + 1][LD]
 
     const int tiles = (nr + TI - 1) / TI;
     const int k = lb / tiles;
@@ -256,7 +275,8 @@ __device__ __forceinline__ void forward_body(const FFTProb &P, int lb, double2 *
     //   X_m = hs (S - i T),  X_{M-m} = hs conj(S + i T);
     // X_0 = 2 hs (Re Z_0 + Im Z_0), X_M = 2 hs (Re Z_0 - Im Z_0), both exactly real.
     // |S - i T| = 2 |sum of the inputs times roots of unity| < 2^62; D is halved
-    // for the product.  hs multiplies as a 63-bit mantissa.
+    // for the product.  hs multiplies as a 63-bit mantissa.  In place: a pair's rows
+    // are read and written by one thread, X_M takes the row after the last.
     // s_i, or per cell in a composite domain (zero outside its patches)
     const size_t si = valid ? (P.s_rows ? (size_t)k * nr + i : (size_t)i) : 0;
     const double hs = (P.s ? P.s[si] : 1.0) * P.half_inv_n;
@@ -266,15 +286,15 @@ __device__ __forceinline__ void forward_body(const FFTProb &P, int lb, double2 *
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     auto out = [&](fx r, int e) { return bad ? nan : fx_to_f64(__mul64hi(r, hm), e); };
     double acc_in = 0.0, acc_edge = 0.0;   // Parseval weight 2 (0 < m < M) and 1 (m = 0, M)
-    double2 *ob = outb + lane * nm;
+    double2 *ob = buf + lane;
     for (int m = 1 + warp; 2 * m < M; m += NW) {
         const ci A = ld(buf + m * LD + lane), B = ld(buf + (M - m) * LD + lane);
         const ci S = {A.x + B.x, A.y - B.y};
         const ci T = tw_mul(twiddle<false>(P.tw, m), {(A.x - B.x) >> 1, (A.y + B.y) >> 1});   // W^m D / 2
         const double2 xm = make_double2(out(S.x + 2 * T.y, be), out(S.y - 2 * T.x, be));
         const double2 xp = make_double2(out(S.x - 2 * T.y, be), out(-S.y - 2 * T.x, be));
-        ob[m] = xm;
-        ob[M - m] = xp;
+        ob[m * LD] = xm;
+        ob[(M - m) * LD] = xp;
         acc_in = fma(xm.x, xm.x, fma(xm.y, xm.y, acc_in));
         acc_in = fma(xp.x, xp.x, fma(xp.y, xp.y, acc_in));
     }
@@ -285,28 +305,28 @@ __device__ __forceinline__ void forward_body(const FFTProb &P, int lb, double2 *
         if (P.bD && valid) x0 += P.bD[(size_t)k * nr + i];
         acc_edge = fma(x0, x0, fma(xM, xM, acc_edge));
         ob[0] = make_double2(x0, 0.0);
-        ob[M] = make_double2(xM, 0.0);
+        ob[M * LD] = make_double2(xM, 0.0);
     }
     if (M >= 2 && warp == NW - 1) {   // m = M/2 pairs with itself: X = 2 hs conj Z
         const ci z = ld(buf + (M >> 1) * LD + lane);
         const double2 x = make_double2(out(z.x, be + 1), out(-z.y, be + 1));
-        ob[M >> 1] = x;
+        ob[(M >> 1) * LD] = x;
         acc_in = fma(x.x, x.x, fma(x.y, x.y, acc_in));
     }
     __syncthreads();
     const int ncols = min(TI, nr - i0);
     double2 *dst = P.b + ((size_t)k * nr + i0) * nm;
-    for (int f = threadIdx.x; f < ncols * nm; f += FFT_THREADS) dst[f] = outb[f];
+    entries<nm>(ncols * nm, [&](int f, int m, int c) { dst[f] = buf[m * LD + c]; });
     if (P.bh && P.invd) {
         // b_hat = b / diag for the smoother (row class of plane k, cells i0.., all modes)
         const int cls = P.rcls ? P.rcls[k] : (k == 0 ? 0 : (k == nz - 1 ? P.ncls - 1 : 1));
         const double *inv = P.invd + ((size_t)cls * nr + i0) * nm;
         double2 *dh = P.bh + ((size_t)k * nr + i0) * nm;
-        for (int f = threadIdx.x; f < ncols * nm; f += FFT_THREADS) {
-            const double2 x = outb[f];
+        entries<nm>(ncols * nm, [&](int f, int m, int c) {
+            const double2 x = buf[m * LD + c];
             const double v = inv[f];
             dh[f] = make_double2(x.x * v, x.y * v);
-        }
+        });
     }
     if (partials) {
         const double tot = block_sum(valid ? fma(2.0, acc_in, acc_edge) : 0.0, red);
@@ -318,8 +338,8 @@ template <int LG>
 __device__ __forceinline__ void inverse_body(const FFTProb &P, int lb, double2 *sm, int *wmax, int *wsum) {
     constexpr int M = 1 << LG, nt = 2 * M, nm = M + 1;
     const int nr = P.nr;
-    double2 *buf = sm;              // [M][LD]
-    double2 *inb = sm + M * LD;     // [TI][nm]
+    double2 *buf = sm;              // [M + 1][LD]: X_m, then Z_m, in row(m)
+    auto row = [](int m) { return (m == M ? M : bitrev<LG>(m)) * LD; };
 
     const int tiles = (nr + TI - 1) / TI;
     const int k = lb / tiles;
@@ -330,21 +350,20 @@ __device__ __forceinline__ void inverse_body(const FFTProb &P, int lb, double2 *
     const int ncols = min(TI, nr - i0);
 
     const double2 *src = P.uhat + ((size_t)k * nr + i0) * nm;
-    for (int f = threadIdx.x; f < TI * nm; f += FFT_THREADS)
-        inb[f] = f < ncols * nm ? src[f] : make_double2(0.0, 0.0);
+    entries<nm>(TI * nm, [&](int f, int m, int c) { buf[row(m) + c] = f < ncols * nm ? src[f] : make_double2(0.0, 0.0); });
     __syncthreads();
 
     // The column's bounds; X_0 and X_M enter through their real parts only.
-    const double2 *ib = inb + lane * nm;
+    const double2 *ib = buf + lane;
     int em = 0;
     for (int m = warp; m <= M; m += NW) {
-        const double2 x = ib[m];
+        const double2 x = ib[row(m)];
         em = max(em, max(f64_exp(x.x), m == 0 || m == M ? 0 : f64_exp(x.y)));
     }
     em = column_max(em, wmax, lane, warp);
     unsigned mag = 0;
     for (int m = warp; m <= M; m += NW) {
-        const double2 x = ib[m];
+        const double2 x = ib[row(m)];
         mag += magnitude(x.x, em) + (m == 0 || m == M ? 0u : magnitude(x.y, em));
     }
     const int bl = column_bits<true>(mag, wsum, lane, warp);
@@ -359,20 +378,20 @@ __device__ __forceinline__ void inverse_body(const FFTProb &P, int lb, double2 *
     //   Z_m = S + i T,  Z_{M-m} = conj(S - i T);
     // Z_0 = (X_0 + X_M) + i (X_0 - X_M).
     for (int m = 1 + warp; 2 * m < M; m += NW) {
-        const double2 a = ib[m], b = ib[M - m];
+        const double2 a = ib[row(m)], b = ib[row(M - m)];
         const ci A = {in(a.x), in(a.y)}, B = {in(b.x), in(b.y)};
         const ci S = {A.x + B.x, A.y - B.y};
         const ci T = tw_mul(twiddle<true>(P.tw, m), {A.x - B.x, A.y + B.y});
-        st(buf + bitrev<LG>(m) * LD + lane, {S.x - T.y, S.y + T.x});
-        st(buf + bitrev<LG>(M - m) * LD + lane, {S.x + T.y, T.x - S.y});
+        st(buf + row(m) + lane, {S.x - T.y, S.y + T.x});
+        st(buf + row(M - m) + lane, {S.x + T.y, T.x - S.y});
     }
     if (warp == 0) {
-        const fx a = in(ib[0].x), b = in(ib[M].x);
+        const fx a = in(ib[0].x), b = in(ib[row(M)].x);
         st(buf + lane, {a + b, a - b});
     }
     if (M >= 2 && warp == NW - 1) {   // m = M/2 pairs with itself: Z = 2 conj X
-        const double2 x = ib[M >> 1];
-        st(buf + bitrev<LG>(M >> 1) * LD + lane, {2 * in(x.x), -2 * in(x.y)});
+        const double2 x = ib[row(M >> 1)];
+        st(buf + row(M >> 1) + lane, {2 * in(x.x), -2 * in(x.y)});
     }
     __syncthreads();
     fft_stages<true, LG>(buf, P.tw, lane, warp);
@@ -450,8 +469,7 @@ cudaError_t launch_copy_guess(const FFTTab *tab, unsigned grid, cudaStream_t st)
 }
 
 size_t fft_smem_bytes(int nt) {
-    const int M = nt / 2, nm = M + 1;
-    return (size_t)(M * LD + TI * nm) * sizeof(double2);
+    return (size_t)(nt / 2 + 1) * LD * sizeof(double2);
 }
 
 cudaError_t launch_forward(const FFTTab *tab, unsigned grid, size_t smem, double *partials, cudaStream_t st) {
