@@ -133,9 +133,17 @@ template <class T> struct LaunchTab {
     const int *done;
     int pid[kMaxBatch];           // problem index of each entry (entries list only the problems that take part)
     unsigned start[kMaxBatch + 1];
+    int chunk;                    // consecutive pieces of a block's size that each block works on
     LevelDev<T> f[kMaxBatch];
     LevelDev<T> c[kMaxBatch];
 };
+// A block of a batch looks its problem up and copies its level views, a chain of
+// some ten dependent loads, before it has work: it then works on `chunk` pieces,
+// as many as leave the launch four times the blocks that the chip holds.
+inline int batch_chunk(size_t blocks) {
+    const size_t c = blocks / (152 * 6 * 4);
+    return (int)(c < 1 ? 1 : c > 8 ? 8 : c);
+}
 
 // What a launch over a table gets: the table and, for a plan of one problem,
 // its entry by value.  The kernel then reads the level views from its own

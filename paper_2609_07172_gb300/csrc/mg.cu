@@ -366,14 +366,15 @@ k_smooth(const __grid_constant__ LevelArg<T> arg, int color) {
         const LaunchTab<T> *__restrict__ tab = arg.tab;
         const int p = find_problem(tab->start, tab->n, blockIdx.x);
         if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
+        const unsigned first = (blockIdx.x - tab->start[p]) * (unsigned)tab->chunk, last = first + (unsigned)tab->chunk;
         if constexpr (sizeof(T) == sizeof(double) && S == 0 && !SOR && !RW) {
             __shared__ LevelDev<T> L;
             stage_view(&L, &tab->f[p]);
             __syncthreads();
-            smooth_body<T, NT, S, SOR, RW, false>(L, blockIdx.x - tab->start[p], color);
+            for (unsigned c = first; c < last; ++c) smooth_body<T, NT, S, SOR, RW, false>(L, c, color);
         } else {
             const LevelDev<T> L = tab->f[p];
-            smooth_body<T, NT, S, SOR, RW, false>(L, blockIdx.x - tab->start[p], color);
+            for (unsigned c = first; c < last; ++c) smooth_body<T, NT, S, SOR, RW, false>(L, c, color);
         }
     }
 }
@@ -383,9 +384,9 @@ k_smooth(const __grid_constant__ LevelArg<T> arg, int color) {
 // with optional Parseval-weighted squared-norm partials.  RED_ONLY: only the
 // two red fine cells (after a black half-sweep the black residuals vanish).
 // F.init selects what else the coarse level receives (see internal.h).
+// Returns this thread's part of the norm.
 template <class T, bool RED_ONLY, bool MASK, bool EARLY>
-__device__ __forceinline__ void restrict_body(const LevelDev<T> &F, const LevelDev<T> &C, unsigned blk, double *red,
-                                              double *__restrict__ partials) {
+__device__ __forceinline__ double restrict_body(const LevelDev<T> &F, const LevelDev<T> &C, unsigned blk, bool partials) {
     const unsigned e = blk * MG_THREADS + threadIdx.x;
     if (EARLY) {
         pdl_wait();
@@ -444,32 +445,35 @@ __device__ __forceinline__ void restrict_body(const LevelDev<T> &F, const LevelD
         }
         if (partials) acc *= parseval_w(m, F.nt);
     }
-    if (partials) {
-        const double tot = block_sum(acc, red);
-        if (threadIdx.x == 0) partials[blockIdx.x] = tot;
-    }
+    return acc;
 }
 
 template <class T, bool RED_ONLY, bool MASK, bool ONE>
 __global__ void __launch_bounds__(MG_THREADS)
 k_residual_restrict(const __grid_constant__ LevelArg<T> arg, double *__restrict__ partials) {
     __shared__ double red[MG_THREADS];
+    double acc = 0.0;
     if constexpr (ONE) {
-        restrict_body<T, RED_ONLY, MASK, true>(arg.f, arg.c, blockIdx.x, red, partials);
+        acc = restrict_body<T, RED_ONLY, MASK, true>(arg.f, arg.c, blockIdx.x, partials != nullptr);
     } else {
         const LaunchTab<T> *__restrict__ tab = arg.tab;
         const int p = find_problem(tab->start, tab->n, blockIdx.x);
         if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
+        const unsigned first = (blockIdx.x - tab->start[p]) * (unsigned)tab->chunk, last = first + (unsigned)tab->chunk;
         if constexpr (sizeof(T) == sizeof(float)) {
             const LevelDev<T> F = tab->f[p], C = tab->c[p];
-            restrict_body<T, RED_ONLY, MASK, false>(F, C, blockIdx.x - tab->start[p], red, partials);
-            return;
+            for (unsigned c = first; c < last; ++c) acc += restrict_body<T, RED_ONLY, MASK, false>(F, C, c, partials != nullptr);
+        } else {
+            __shared__ LevelDev<T> F, C;
+            stage_view(&F, &tab->f[p]);
+            stage_view(&C, &tab->c[p]);
+            __syncthreads();
+            for (unsigned c = first; c < last; ++c) acc += restrict_body<T, RED_ONLY, MASK, false>(F, C, c, partials != nullptr);
         }
-        __shared__ LevelDev<T> F, C;
-        stage_view(&F, &tab->f[p]);
-        stage_view(&C, &tab->c[p]);
-        __syncthreads();
-        restrict_body<T, RED_ONLY, MASK, false>(F, C, blockIdx.x - tab->start[p], red, partials);
+    }
+    if (partials) {
+        const double tot = block_sum(acc, red);
+        if (threadIdx.x == 0) partials[blockIdx.x] = tot;
     }
 }
 
@@ -593,7 +597,8 @@ __global__ void __launch_bounds__(MG_THREADS) k_prolong(const __grid_constant__ 
         const int p = find_problem(tab->start, tab->n, blockIdx.x);
         if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
         const LevelDev<T> F = tab->f[p], C = tab->c[p];
-        prolong_body<T, BLACK_ONLY, ASSIGN, MASK, false>(F, C, blockIdx.x - tab->start[p]);
+        const unsigned first = (blockIdx.x - tab->start[p]) * (unsigned)tab->chunk, last = first + (unsigned)tab->chunk;
+        for (unsigned c = first; c < last; ++c) prolong_body<T, BLACK_ONLY, ASSIGN, MASK, false>(F, C, c);
     }
 }
 

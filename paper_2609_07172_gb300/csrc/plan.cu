@@ -939,10 +939,21 @@ void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, c
     const int nl = std::max(P.Lmax - 1, 0);
     const int pre = P.shared.pre_sweeps, post = P.shared.post_sweeps;
     auto put = [&](const LaunchTab<T> &t, TabRef<T> &r) {
-        blob_to_dev(t, r.tab, st, err);
+        blob_to_dev(t, r.tab, st, err);   // (t.chunk: 1 unless chunked() was called on it)
         r.one = P.n == 1;
         r.f = t.f[0];
         r.c = t.c[0];
+    };
+    // a batch's blocks take several pieces each (LaunchTab::chunk)
+    auto chunked = [&](LaunchTab<T> &t) {
+        t.chunk = P.n > 1 ? batch_chunk(t.start[t.n]) : 1;
+        unsigned at = 0, old = 0;
+        for (int p = 0; p < t.n; ++p) {
+            const unsigned end = t.start[p + 1];
+            at += (end - old + t.chunk - 1) / t.chunk;
+            old = end;
+            t.start[p + 1] = at;
+        }
     };
     H.g_smooth.assign(nl, 0);
     H.g_restr.assign(nl, 0);
@@ -1028,6 +1039,11 @@ void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, c
             ++tr.n;
             ++tp.n;
         }
+        ts.chunk = 1;
+        if (strip == 0) chunked(ts);
+        chunked(tr);
+        chunked(tp);
+        if (l == 0) H.restr0_start.assign(tr.start, tr.start + tr.n + 1);
         H.g_smooth[l] = ts.start[ts.n];
         H.g_restr[l] = tr.start[tr.n];
         H.g_prolong[l] = tp.start[tp.n];
@@ -1074,6 +1090,8 @@ void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, c
                     ++tin.n;
                 }
             }
+            trh.chunk = 1;
+            chunked(tin);
             H.g_rhs[l] = trh.start[trh.n];
             H.g_interp[l] = tin.start[tin.n];
             if (trh.n) put(trh, H.rhs[l]);
@@ -1421,8 +1439,7 @@ int upload(pic_poisson_plan_s &P) {
     C.inc_first = mixed ? P.shared.inner_first : 1;
     const unsigned g_restr0 = (!mixed && P.Lmax > 1) ? P.h64.g_restr[0] : 0;
     P.res_single_offset = g_restr0;
-    unsigned b0 = 0;
-    int is = 0;
+    int i0 = 0, is = 0;
     for (int p = 0; p < P.n; ++p) {
         const ProblemPlan &q = P.pr[p];
         C.count[p] = (double)q.lv[0].nr * q.lv[0].nz * q.d.ntheta;
@@ -1431,10 +1448,9 @@ int upload(pic_poisson_plan_s &P) {
             C.rend[p] = dt.start[p + 1];
         } else if (q.L > 1) {
             // the level-0 restriction table lists the multi-level problems in order
-            const unsigned nb = mg_blocks((size_t)q.lv[1].nr * q.lv[1].nz * q.nm);
-            C.rbegin[p] = b0;
-            C.rend[p] = b0 + nb;
-            b0 += nb;
+            C.rbegin[p] = P.h64.restr0_start[i0];
+            C.rend[p] = P.h64.restr0_start[i0 + 1];
+            ++i0;
         } else {
             C.rbegin[p] = g_restr0 + rs.start[is];
             C.rend[p] = g_restr0 + rs.start[is + 1];

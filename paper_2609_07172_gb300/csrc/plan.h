@@ -50,6 +50,7 @@ struct ProblemPlan {
 template <class T> struct Hier {
     std::vector<TabRef<T>> smooth, restr, prolong;        // tables (null when no problem takes part)
     std::vector<unsigned> g_smooth, g_restr, g_prolong;   // grids
+    std::vector<unsigned> restr0_start;                   // level 0's restriction: first block of each entry
     std::vector<int> strip;                               // smoother strip per level
     bool fused = false;                                   // FP32 fused smoother (pre: u -> u2, post: u2 -> u)
     std::vector<FusedTab *> fpre, fpost;
