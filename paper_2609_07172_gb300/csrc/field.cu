@@ -10,13 +10,19 @@
 // charge (discrete Gauss law): sum over faces of area E.n = rho V / eps0 for
 // the discrete solution.
 //
-// One thread per cell, r fastest (coalesced): each cell writes its lower r,
-// azimuthal (j + 1/2) and lower z face, and the cells next to the upper walls
-// also the wall face.  The differences are binary64 (one subtraction and one
-// multiplication by a precomputed inverse distance per face), so on this GPU
-// the kernel is bound by the FP64 pipe rather than by its 4 arrays of traffic.
+// Each cell writes its lower r, azimuthal (j + 1/2) and lower z face, and the cells
+// next to the upper walls also the wall face: one subtraction and one product by a
+// precomputed inverse distance per face.  With both in the FP64 unit the kernel
+// took 401 us at 512 x 128 x 400 (845 MB, 123 us at the copy rate); with the
+// products by integer multiplies, bit for bit those of binary64, and a walk along z
+// that keeps factors and the plane before in registers 193 us, bound by latency and
+// the subtractions (32 registers, eight blocks per SM and the next plane's load
+// ahead of its use: 237 us with 48 registers and no load ahead).
 // Non-uniform axial faces and composite domains take a variant with an axial
 // distance table and, for patches, exposed faces (k_face_field_gen).
+#include <algorithm>
+
+#include "fixed.h"
 #include "plan.h"
 
 namespace pp {
@@ -33,27 +39,63 @@ struct FieldArgs {
     double *er, *ea, *ez;                      // (nz, nt, nr + 1), (nz, nt, nr), (nz + 1, nt, nr)
 };
 
-__global__ void __launch_bounds__(256) k_face_field(const FieldArgs a) {
-    const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
-    const unsigned nr = (unsigned)a.nr, row_n = (unsigned)a.nz * (unsigned)a.nt;
-    if (e >= row_n * nr) return;
-    const unsigned row = e / nr;                     // k * nt + j
-    const int i = (int)(e - row * nr);
-    const int k = (int)(row / (unsigned)a.nt), j = (int)(row - (unsigned)k * a.nt);
-    const double p = a.phi[e];
-    // radial face i (between cells i - 1 and i; the inner wall for i = 0)
-    const size_t fr = (size_t)row * (nr + 1) + i;
-    const double pw = i > 0 ? a.phi[e - 1] : a.win[k];
-    a.er[fr] = (pw - p) * a.inv_rd[i];
-    if (i == a.nr - 1) a.er[fr + 1] = (p - a.wout[k]) * a.inv_rd[a.nr];
-    // azimuthal face j + 1/2, periodic
-    const int jn = j + 1 == a.nt ? 0 : j + 1;
-    a.ea[e] = (p - a.phi[((size_t)k * a.nt + jn) * nr + i]) * a.inv_rda[i];
-    // axial face k (between cells k - 1 and k; the wall z0 for k = 0)
-    const size_t plane = (size_t)a.nt * nr;
-    const double ps = k > 0 ? a.phi[e - plane] : a.phi_z0;
-    a.ez[e] = (ps - p) * (k > 0 ? a.inv_dz : a.inv_hdz);
-    if (k == a.nz - 1) a.ez[e + plane] = (p - a.phi_z1) * a.inv_hdz;
+// A positive binary64 constant to multiply by: its mantissa in 64 bits (top bit
+// set), exponent field and value.
+struct Factor {
+    ufx m;
+    int e;
+    double v;
+};
+__device__ __forceinline__ Factor factor(double c) { return {f64_mant(c) << 1, f64_exp(c), c}; }
+// d c, rounded to nearest: the upper half of the mantissas' product, by integer
+// multiplies.  What may be a tie (one product in a thousand), zeros, subnormals,
+// infinities, NaN and results outside the normal range go to the FP64 unit.
+// (Not inlined: predicated, that multiplication would hold the unit all the same.)
+__device__ __noinline__ double times_f64(double d, double c) { return d * c; }
+__device__ __forceinline__ double times(double d, const Factor &c) {
+    const int hi = __double2hiint(d), e = (hi >> 20) & 0x7ff;
+    const ufx p = __umul64hi(f64_mant(d), c.m);                // in [2^61, 2^63)
+    const unsigned big = (unsigned)(p >> 62);
+    const int E = e + c.e - 1023 + (int)big;                   // biased exponent, before a carry
+    const ufx q = p << (1 - big);
+    const ufx bits = ((q + (1ull << 9)) >> 10) + ((ufx)(unsigned)(E - 1) << 52);
+    double r = __longlong_as_double((fx)(bits | (ufx)((unsigned)hi & 0x80000000u) << 32));
+    if ((unsigned)(e - 1) >= 0x7feu || (unsigned)(E - 1) >= 0x7fdu || ((unsigned)q & 0x3ffu) == 0x200u) r = times_f64(d, c.v);
+    return r;
+}
+
+// One thread per (j, i), r fastest, over `chunk` planes: the plane before stays in a
+// register, the radial factors too.
+__global__ void __launch_bounds__(256, 8) k_face_field(const FieldArgs a, int chunk) {
+    const unsigned c = blockIdx.x * blockDim.x + threadIdx.x, nr = (unsigned)a.nr, plane = (unsigned)a.nt * nr;
+    if (c >= plane) return;
+    const unsigned j = c / nr, i = c - j * nr;
+    const int k0 = (int)blockIdx.y * chunk, k1 = min(k0 + chunk, a.nz);
+    const Factor fr = factor(a.inv_rd[i]), fa = factor(a.inv_rda[i]), fz = factor(a.inv_dz);
+    const double inv_out = i + 1 == nr ? a.inv_rd[nr] : 0.0;
+    const size_t e0 = (size_t)k0 * plane + c;
+    const double *phi = a.phi + e0;
+    // row j + 1 of the plane, periodic
+    const double *next = a.phi + (e0 - c) + (j + 1 == (unsigned)a.nt ? i : c + nr);
+    double *er = a.er + e0 + (size_t)k0 * a.nt + j, *ea = a.ea + e0, *ez = a.ez + e0;   // (er: rows of nr + 1)
+    double ps = k0 > 0 ? *(phi - plane) : a.phi_z0, p = 0.0, pn = *phi;
+#pragma unroll 1
+    for (int k = k0; k < k1; ++k) {
+        p = pn;
+        if (k + 1 < k1) pn = phi[plane];
+        const double pw = i > 0 ? *(phi - 1) : a.win[k];
+        *er = times(pw - p, fr);
+        if (i + 1 == nr) er[1] = (p - a.wout[k]) * inv_out;
+        *ea = times(p - *next, fa);
+        *ez = k > 0 ? times(ps - p, fz) : (ps - p) * a.inv_hdz;
+        ps = p;
+        phi += plane;
+        next += plane;
+        er += plane + a.nt;
+        ea += plane;
+        ez += plane;
+    }
+    if (k1 == a.nz) *ez = (p - a.phi_z1) * a.inv_hdz;
 }
 
 // The same on non-uniform axial faces and composite domains.  Axial
@@ -155,7 +197,10 @@ extern "C" int pic_poisson_face_field(pic_poisson_plan_t plan, const double *phi
     const size_t n = (size_t)a.nz * a.nt * a.nr;
     const unsigned grid = (unsigned)((n + 255) / 256);
     if (h.act.empty() && h.zf.empty()) {
-        k_face_field<<<grid, 256, 0, plan->stream>>>(a);
+        // planes per block: as many as leave the chip twice the blocks it holds
+        const unsigned cols = (unsigned)(((size_t)a.nt * a.nr + 255) / 256);
+        const int chunk = (int)std::min<size_t>(std::max<size_t>((size_t)cols * a.nz / (152 * 8 * 2), 1), 16);
+        k_face_field<<<dim3(cols, (unsigned)((a.nz + chunk - 1) / chunk)), 256, 0, plan->stream>>>(a, chunk);
     } else {   // non-uniform axial faces and / or a composite domain
         FieldGenArgs g{};
         g.a = a;
