@@ -18,10 +18,12 @@
 //                 complex layout.
 //
 // FP32 for both hierarchies: a coarse-grid correction needs no FP64
-// accuracy, and the FP32 pipe runs at 64 times the FP64 rate.  Each dot
-// product accumulates its n terms in index order with one fused multiply-add
-// per term, the order of the per-block loops it replaces, so the result is
-// bitwise the same.
+// accuracy, and the FP32 pipe runs at 64 times the FP64 rate.  A problem has a
+// few outputs per thread of the chip, so a product is bound by the latency of its
+// walk along the contraction: from DENSE_SPLIT cells four groups of a block take
+// every fourth chunk each, and their sums are added in group order (800 cells, 65
+// modes: 26 us less for the two products, a stretched 512 x 128 x 400 solve
+// 9,081 -> 8,770 us; with 150 cells, five chunks, 2 % more for the solve).
 #include "internal.h"
 
 namespace pp {
@@ -31,6 +33,7 @@ constexpr int TR = 32;   // output rows (cells or eigenvectors) per block
 constexpr int TC = 32;   // right-hand sides per block
 constexpr int TK = 32;   // contraction chunk staged in shared memory
 constexpr int DENSE_THREADS = 256;
+constexpr int DENSE_SPLIT = 384;
 
 __device__ __forceinline__ int find_problem(const unsigned *__restrict__ start, int n, unsigned blk) {
     int lo = 0, hi = n;
@@ -85,16 +88,17 @@ __global__ void __launch_bounds__(DENSE_THREADS) k_dense_prep(const DenseTab<T> 
         if (D.amap[f] < 0) ug[2 * ((size_t)f * nm + m)] = T(0);
 }
 
-// C[col][r] = sum_k A[r][k] B[col][k] for a TR x TC tile, k in order.
+// C[col][r] = sum_k A[r][k] B[col][k] for a TR x TC tile.
 // STAGE 1: A = Q^T (row j of Q^T is column j of Q), B = y; writes
 // z[col][j] = C / (lambda_j + lambda_m).  STAGE 2: A = Q, B = z; writes
 // u at cell aidx[a] of mode m, part comp: C M^(-1/2) times the scale.
-template <class T, int STAGE>
-__global__ void __launch_bounds__(DENSE_THREADS) k_dense_gemm(const DenseTab<T> *__restrict__ tab) {
+// KG: groups of the block, one chunk of the contraction each at a time.
+template <class T, int STAGE, int KG>
+__global__ void __launch_bounds__(KG * DENSE_THREADS) k_dense_gemm(const DenseTab<T> *__restrict__ tab) {
     // A row-major (a lane's row, conflict-free); B k-major so that a thread's
     // four adjacent columns are one 16-byte broadcast load per k
-    __shared__ float As[TR][TK + 1];
-    __shared__ __align__(16) float Bs[TK][TC + 4];
+    __shared__ float Asm[KG][TR][TK + 1];
+    __shared__ __align__(16) float Bsm[KG][TK][TC + 4];
     const int p = find_problem(tab->gstart, tab->n, blockIdx.x);
     const LevelDev<T> &L = tab->f[p];
     const CoarseDev<T> &D = tab->c[p];
@@ -104,7 +108,9 @@ __global__ void __launch_bounds__(DENSE_THREADS) k_dense_gemm(const DenseTab<T> 
     const int r0 = (lb % rtiles) * TR, c0 = (lb / rtiles) * TC;
     const float *A = STAGE == 1 ? D.QT : D.Q;
     const float *B = STAGE == 1 ? D.Y : D.Z;
-    const int t = threadIdx.x;
+    const int t = threadIdx.x % DENSE_THREADS, g = threadIdx.x / DENSE_THREADS;
+    float(*As)[TK + 1] = Asm[g];
+    float(*Bs)[TC + 4] = Bsm[g];
     const int tr = t % TR, tc = t / TR;   // row of the tile; columns 4 tc .. 4 tc + 3
     static_assert(TC == 4 * (DENSE_THREADS / TR), "four adjacent columns per thread");
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
@@ -125,8 +131,8 @@ __global__ void __launch_bounds__(DENSE_THREADS) k_dense_gemm(const DenseTab<T> 
     pdl_wait();
     pdl_go();
     if (tab->done && tab->done[tab->pid[p]]) return;
-    load(0);
-    for (int k0 = 0; k0 < n; k0 += TK) {
+    load(g * TK);
+    for (int k0 = g * TK; k0 < n + g * TK; k0 += KG * TK) {   // (the same count in every group; zeros beyond n)
 #pragma unroll
         for (int i = 0; i < PER; ++i) {
             const int e = t + i * DENSE_THREADS, x = e / TK, kk = e - x * TK;
@@ -134,10 +140,9 @@ __global__ void __launch_bounds__(DENSE_THREADS) k_dense_gemm(const DenseTab<T> 
             Bs[kk][x] = rb[i];
         }
         __syncthreads();
-        if (k0 + TK < n) load(k0 + TK);
-        const int kmax = min(TK, n - k0);   // padded terms are not accumulated: the order and count match
+        load(k0 + KG * TK);
 #pragma unroll 8
-        for (int kk = 0; kk < kmax; ++kk) {
+        for (int kk = 0; kk < TK; ++kk) {
             const float a = As[tr][kk];
             const float4 b = *reinterpret_cast<const float4 *>(&Bs[kk][4 * tc]);
             acc[0] = fmaf(a, b.x, acc[0]);
@@ -146,6 +151,18 @@ __global__ void __launch_bounds__(DENSE_THREADS) k_dense_gemm(const DenseTab<T> 
             acc[3] = fmaf(a, b.w, acc[3]);
         }
         __syncthreads();
+    }
+    float4 *sums = reinterpret_cast<float4 *>(&Bsm[0][0][0]);   // [KG][DENSE_THREADS]
+    static_assert(KG * DENSE_THREADS * sizeof(float4) <= sizeof(Bsm), "the groups' sums take the tiles' place");
+    sums[g * DENSE_THREADS + t] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    __syncthreads();
+    if (g > 0) return;
+    for (int q = 1; q < KG; ++q) {
+        const float4 x = sums[q * DENSE_THREADS + t];
+        acc[0] += x.x;
+        acc[1] += x.y;
+        acc[2] += x.z;
+        acc[3] += x.w;
     }
     const int r = r0 + tr;
     if (r >= n) return;
@@ -170,15 +187,15 @@ unsigned dense_gemm_blocks(int nact, int nm) {
 }
 
 template <class T>
-cudaError_t launch_dense(const DenseTab<T> *tab, int stage, unsigned g_prep, unsigned g_gemm, cudaStream_t st) {
-    switch (stage) {
-    case 0: return launch_pdl(k_dense_prep<T>, g_prep, DENSE_THREADS, 0, st, tab);
-    case 1: return launch_pdl(k_dense_gemm<T, 1>, g_gemm, DENSE_THREADS, 0, st, tab);
-    default: return launch_pdl(k_dense_gemm<T, 2>, g_gemm, DENSE_THREADS, 0, st, tab);
-    }
+cudaError_t launch_dense(const DenseTab<T> *tab, int stage, unsigned g_prep, unsigned g_gemm, int nmax, cudaStream_t st) {
+    const bool split = nmax >= DENSE_SPLIT;
+    const int threads = (split ? 4 : 1) * DENSE_THREADS;
+    if (stage == 0) return launch_pdl(k_dense_prep<T>, g_prep, DENSE_THREADS, 0, st, tab);
+    if (stage == 1) return launch_pdl(split ? k_dense_gemm<T, 1, 4> : k_dense_gemm<T, 1, 1>, g_gemm, threads, 0, st, tab);
+    return launch_pdl(split ? k_dense_gemm<T, 2, 4> : k_dense_gemm<T, 2, 1>, g_gemm, threads, 0, st, tab);
 }
 
-template cudaError_t launch_dense<double>(const DenseTab<double> *, int, unsigned, unsigned, cudaStream_t);
-template cudaError_t launch_dense<float>(const DenseTab<float> *, int, unsigned, unsigned, cudaStream_t);
+template cudaError_t launch_dense<double>(const DenseTab<double> *, int, unsigned, unsigned, int, cudaStream_t);
+template cudaError_t launch_dense<float>(const DenseTab<float> *, int, unsigned, unsigned, int, cudaStream_t);
 
 }  // namespace pp

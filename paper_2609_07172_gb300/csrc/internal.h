@@ -336,9 +336,10 @@ cudaError_t launch_prolong(const TabRef<T> &tab, unsigned grid, bool black_only,
                            bool masked = false);
 template <class T>
 cudaError_t launch_coarse(const CoarseTab<T> *tab, unsigned grid, size_t smem, cudaStream_t st);
-// Dense coarsest solves, in stage order: 0 preparation (g_prep blocks), 1 and 2 the two GEMMs (g_gemm blocks).
+// Dense coarsest solves, in stage order: 0 preparation (g_prep blocks), 1 and 2 the two GEMMs (g_gemm blocks);
+// nmax: active cells of the largest.
 template <class T>
-cudaError_t launch_dense(const DenseTab<T> *tab, int stage, unsigned g_prep, unsigned g_gemm, cudaStream_t st);
+cudaError_t launch_dense(const DenseTab<T> *tab, int stage, unsigned g_prep, unsigned g_gemm, int nmax, cudaStream_t st);
 unsigned dense_gemm_blocks(int nact, int nm);   // GEMM blocks of one problem
 // Full-multigrid start: u_f = P u_c on every fine cell (black_only: on the
 // black ones, for a red Gauss-Seidel half-sweep to follow); coarse b =

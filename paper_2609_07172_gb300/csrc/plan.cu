@@ -1124,6 +1124,7 @@ void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, c
         }
         if (cd.nact > 0) {   // dense coarsest solve: two GEMMs over all modes
             td.pid[td.n] = p;
+            H.dense_max = std::max(H.dense_max, cd.nact);
             td.f[td.n] = views(q)[q.L - 1];
             td.c[td.n] = cd;
             td.start[td.n + 1] = td.start[td.n] + 2u * (unsigned)q.nm;

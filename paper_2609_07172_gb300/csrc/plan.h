@@ -59,6 +59,7 @@ template <class T> struct Hier {
     CoarseTab<T> *coarse = nullptr;           // problems solved by k_coarse (separable coarsest level)
     DenseTab<T> *dense = nullptr;             // problems with a dense coarsest solve (csrc/dense.cu)
     unsigned g_dense_prep = 0, g_dense_gemm = 0;
+    int dense_max = 0;                        // active cells of the largest
     unsigned g_coarse = 0;
     size_t smem_coarse = 0;
     std::vector<TabRef<T>> rhs, interp;       // full-multigrid start: b restricted to l + 1, u_l = P u_(l+1)

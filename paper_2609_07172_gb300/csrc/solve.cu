@@ -198,10 +198,10 @@ int coarse_and_bottom(Runner &R, const Hier<T> &H) {
         double qb = 0, df = 0;
         const double dn = dense_work(P, &qb, &df);
         // y: b in, y out; each GEMM: Q, one FP32 column block in, one out
-        RUN(R, PIC_POISSON_PHASE_COARSE, launch_dense(H.dense, 0, H.g_dense_prep, H.g_dense_gemm, R.st));
+        RUN(R, PIC_POISSON_PHASE_COARSE, launch_dense(H.dense, 0, H.g_dense_prep, H.g_dense_gemm, H.dense_max, R.st));
         R.account(PIC_POISSON_PHASE_COARSE, dn * (sizeof(V2<T>) + sizeof(float2)), 0.0);
         for (int stage = 1; stage <= 2; ++stage) {
-            RUN(R, PIC_POISSON_PHASE_COARSE, launch_dense(H.dense, stage, H.g_dense_prep, H.g_dense_gemm, R.st));
+            RUN(R, PIC_POISSON_PHASE_COARSE, launch_dense(H.dense, stage, H.g_dense_prep, H.g_dense_gemm, H.dense_max, R.st));
             R.account(PIC_POISSON_PHASE_COARSE, 0.5 * qb + dn * (stage == 1 ? 2 * sizeof(float2) : sizeof(float2) + sizeof(V2<T>)),
                       0.5 * df);
         }
