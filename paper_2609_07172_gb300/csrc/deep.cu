@@ -163,7 +163,7 @@ template <class T> __device__ __forceinline__ V2<T> update(const Cell<T> &c, con
     const V2<T> us = *(r - nr), un = r[nr], uw = c.w ? *(x - 1) : zero, ue = c.e ? *x : zero;
     V2<T> v;
     v.x = fma(c.he, ue.x, fma(c.hw, uw.x, fma(c.hz, us.x + un.x, c.b.x)));
-    if constexpr (sizeof(T) == 8) v.y = fx_update(c.b.y, us.y, un.y, uw.y, ue.y, c.zw, c.ev);
+    if constexpr (sizeof(T) == 8) v.y = fx_update<true>(c.b.y, us.y, un.y, uw.y, ue.y, c.zw, c.ev);
     else v.y = fma(c.he, ue.y, fma(c.hw, uw.y, fma(c.hz, us.y + un.y, c.b.y)));
     return v;
 }
@@ -217,7 +217,7 @@ __device__ __forceinline__ V2<T> residual(const Lv &v, const Tab<T> &t, const V2
     q.x = fma(-d, uc.x, fma(ce, ue.x, fma(cw, uw.x, fma(cz, us.x + un.x, bv.x))));
     if constexpr (sizeof(T) == 8) {
         const int4 zw = t.rzw[e];
-        q.y = fx_residual(bv.y, us.y, un.y, uw.y, ue.y, uc.y, make_int2(zw.x, zw.y), make_int2(zw.z, zw.w), t.rev[e],
+        q.y = fx_residual<true>(bv.y, us.y, un.y, uw.y, ue.y, uc.y, make_int2(zw.x, zw.y), make_int2(zw.z, zw.w), t.rev[e],
                           t.rdg[tb], v.rq);
     } else {
         q.y = fma(-d, uc.y, fma(ce, ue.y, fma(cw, uw.y, fma(cz, us.y + un.y, bv.y))));

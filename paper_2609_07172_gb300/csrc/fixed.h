@@ -113,11 +113,25 @@ __device__ __forceinline__ double fx_to_f64_normal(fx r, int be) {
     const double d = __ll2double_rn(r);
     return r ? __hiloint2double(__double2hiint(d) + ((be - 1086) << 20), __double2loint(d)) : 0.0;
 }
+// The same by integer instructions, ties to even: bit for bit the conversion's.
+__device__ __forceinline__ double fx_to_f64_int(fx r, int be) {
+    const ufx a = r < 0 ? 0ull - (ufx)r : (ufx)r;
+    const int lz = __clzll((fx)a);
+    const ufx m = a << (lz & 63);
+    const ufx q = m + 0x3ffu + ((unsigned)(m >> 11) & 1u);         // (below 2^64: m < 2^64 - 2^10 for |r| < 2^63)
+    const ufx bits = (q >> 11) + ((ufx)(unsigned)(be - lz - 1) << 52);
+    const double d = __longlong_as_double((fx)(bits | (ufx)((unsigned)((ufx)r >> 32) & 0x80000000u) << 32));
+    return r ? d : 0.0;
+}
 __device__ __forceinline__ int coef_exp(int2 c) { return (c.y & 127) << 20; }
 __device__ __forceinline__ Limbs coef_limbs(int2 c) { return {c.x, c.y & ~127}; }
 
 // b + hz (s + n) + hw w + he e (a Gauss-Seidel update).  All terms below 2^60.
-__device__ __forceinline__ double fx_update(double b, double s, double n, double w, double e, int2 hz, int2 hw,
+// INT: the conversion by integer instructions -- where few warps are in flight, or
+// the FP64 unit has more to do besides than the integer pipes (a half-sweep of many
+// waves: 74 us with the unit, 79 without; a restriction 65 and 61; 48 x 16 x 20 in
+// shared memory 282 and 270).
+template <bool INT = false> __device__ __forceinline__ double fx_update(double b, double s, double n, double w, double e, int2 hz, int2 hw,
                                             int2 he) {
     const int ez = coef_exp(hz), eb = exp_bits(b), es = exp_bits(s) - ez, en = exp_bits(n) - ez;
     const int ew = exp_bits(w) - coef_exp(hw), ee = exp_bits(e) - coef_exp(he);
@@ -136,13 +150,14 @@ __device__ __forceinline__ double fx_update(double b, double s, double n, double
     m2 += (fx)zl * f.h;
     hi += (fx)zh * f.h;
     const fx r = 2 * hi + (m1 >> 30) + (m2 >> 30) + fx_align<3>(b, eb, em);
-    return fx_ends(fx_to_f64_normal(r, (em >> 20) + 4), em);
+    return fx_ends(INT ? fx_to_f64_int(r, (em >> 20) + 4) : fx_to_f64_normal(r, (em >> 20) + 4), em);
 }
+template <bool INT = false>
 __device__ __forceinline__ double fx_update(double b, double s, double n, double w, double e, int4 zw, int2 ev) {
-    return fx_update(b, s, n, w, e, make_int2(zw.x, zw.y), make_int2(zw.z, zw.w), ev);
+    return fx_update<INT>(b, s, n, w, e, make_int2(zw.x, zw.y), make_int2(zw.z, zw.w), ev);
 }
 // b + cz (s + n) + cw w + ce e - d u, the coefficients given times 2^q (|q| < 60).
-__device__ __forceinline__ double fx_residual(double b, double s, double n, double w, double e, double u, int2 cz,
+template <bool INT = false> __device__ __forceinline__ double fx_residual(double b, double s, double n, double w, double e, double u, int2 cz,
                                               int2 cw, int2 ce, int2 cd, int q) {
     const int ez = coef_exp(cz), es = exp_bits(s) - ez, en = exp_bits(n) - ez, eb = exp_bits(b) + q * (1 << 20);
     const int ew = exp_bits(w) - coef_exp(cw), ee = exp_bits(e) - coef_exp(ce), eu = exp_bits(u) - coef_exp(cd);
@@ -166,7 +181,8 @@ __device__ __forceinline__ double fx_residual(double b, double s, double n, doub
     hi -= (fx)vh * g.h;
     const fx r = 2 * hi + (m1 >> 30) + (m2 >> 30) + fx_align<3>(b, eb, em);
     const int emq = em - q * (1 << 20);
-    return fx_ends(fx_to_f64_normal(r, (emq >> 20) + 4), min(em, emq), max(em, emq));
+    const int be = (emq >> 20) + 4;
+    return fx_ends(INT ? fx_to_f64_int(r, be) : fx_to_f64_normal(r, be), min(em, emq), max(em, emq));
 }
 // u + (9 c0 + 3 (+-c1) + 3 (+-c2) +- c3) / 16: bilinear interpolation, s1 s2 set for a minus.
 __device__ __forceinline__ double fx_bilinear(double u, double c0, double c1, double c2, double c3, bool s1, bool s2) {

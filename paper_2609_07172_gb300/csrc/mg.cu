@@ -99,7 +99,7 @@ template <class T> __device__ __forceinline__ void stage_view(LevelDev<T> *dst, 
 }
 
 // b - A_m u at entry (k, i, m), Eq. matrix_free_mode_operator.
-template <class T, bool MASK>
+template <class T, bool MASK, bool INT = false>
 __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i, int m, size_t idx) {
     const size_t rowstride = (size_t)L.nr * L.nm;
     if (MASK && L.rcls) {
@@ -128,7 +128,7 @@ __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i,
             const int4 zw = L.rzw[i];
             const int2 ev = L.rev[i], dg = L.rdg[tb];
             return mk<T>(fma(-L.diag[tb], uc.x, fma(L.ce[i], ue.x, fma(L.cw[i], uw.x, fma(L.cz[i], us.x + un.x, b.x)))),
-                         fx_residual(b.y, us.y, un.y, uw.y, ue.y, uc.y, make_int2(zw.x, zw.y), make_int2(zw.z, zw.w),
+                         fx_residual<INT>(b.y, us.y, un.y, uw.y, ue.y, uc.y, make_int2(zw.x, zw.y), make_int2(zw.z, zw.w),
                                      ev, dg, L.rq));
         }
     }
@@ -418,11 +418,11 @@ __device__ __forceinline__ double restrict_body(const LevelDev<T> &F, const Leve
         };
         int k, i;
         cell(0, k, i);
-        V2<T> sum = residual_at<T, MASK>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
+        V2<T> sum = residual_at<T, MASK, true>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
         if (partials) acc = fma((double)sum.y, (double)sum.y, (double)sum.x * (double)sum.x);
         auto more = [&](int c) {
             cell(c, k, i);
-            const V2<T> r = residual_at<T, MASK>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
+            const V2<T> r = residual_at<T, MASK, true>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
             sum = mk<T>(sum.x + r.x, sum.y + r.y);
             if (partials) acc = fma((double)r.y, (double)r.y, fma((double)r.x, (double)r.x, acc));
         };
