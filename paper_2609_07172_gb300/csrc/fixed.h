@@ -184,6 +184,53 @@ template <bool INT = false> __device__ __forceinline__ double fx_residual(double
     const int be = (emq >> 20) + 4;
     return fx_ends(INT ? fx_to_f64_int(r, be) : fx_to_f64_normal(r, be), min(em, emq), max(em, emq));
 }
+// The same with four couplings of their own (per-row tables): b + hs s + hw w + he e + hn n.
+struct FxCell {                  // sums of products of aligned operands with coefficients
+    fx hi = 0, m1 = 0, m2 = 0;
+    __device__ __forceinline__ void add(fx x, int2 c) {
+        const Limbs l = coef_limbs(c);
+        const int xh = (int)(x >> 31), xl = (int)((unsigned)x & 0x7fffffffu);
+        hi += (fx)xh * l.h;
+        m1 += (fx)xh * l.l;
+        m2 += (fx)xl * l.h;
+    }
+    __device__ __forceinline__ void sub(fx x, int2 c) {
+        const Limbs l = coef_limbs(c);
+        const int xh = (int)(x >> 31), xl = (int)((unsigned)x & 0x7fffffffu);
+        hi -= (fx)xh * l.h;
+        m1 -= (fx)xh * l.l;
+        m2 -= (fx)xl * l.h;
+    }
+    __device__ __forceinline__ fx total() const { return 2 * hi + (m1 >> 30) + (m2 >> 30); }
+};
+__device__ __forceinline__ double fx_update(double b, double s, double w, double e, double n, int4 sw, int4 en) {
+    const int2 hs = make_int2(sw.x, sw.y), hw = make_int2(sw.z, sw.w), he = make_int2(en.x, en.y), hn = make_int2(en.z, en.w);
+    const int eb = exp_bits(b), es = exp_bits(s) - coef_exp(hs), ew = exp_bits(w) - coef_exp(hw);
+    const int ee = exp_bits(e) - coef_exp(he), et = exp_bits(n) - coef_exp(hn);
+    const int em = max(max(max(es, et), max(ew, ee)), eb);
+    FxCell t;
+    t.add(fx_align<3>(s, es, em), hs);
+    t.add(fx_align<3>(w, ew, em), hw);
+    t.add(fx_align<3>(e, ee, em), he);
+    t.add(fx_align<3>(n, et, em), hn);
+    return fx_ends(fx_to_f64_normal(t.total() + fx_align<3>(b, eb, em), (em >> 20) + 4), em);
+}
+// b + cs s + cw w + ce e + cn n - d u, the coefficients given times 2^q.
+__device__ __forceinline__ double fx_residual(double b, double s, double w, double e, double n, double u, int4 sw, int4 en,
+                                              int2 d, int q) {
+    const int2 cs = make_int2(sw.x, sw.y), cw = make_int2(sw.z, sw.w), ce = make_int2(en.x, en.y), cn = make_int2(en.z, en.w);
+    const int eb = exp_bits(b) + q * (1 << 20), es = exp_bits(s) - coef_exp(cs), ew = exp_bits(w) - coef_exp(cw);
+    const int ee = exp_bits(e) - coef_exp(ce), et = exp_bits(n) - coef_exp(cn), eu = exp_bits(u) - coef_exp(d);
+    const int em = max(max(max(es, et), max(ew, ee)), max(eb, eu));
+    FxCell t;
+    t.add(fx_align<3>(s, es, em), cs);
+    t.add(fx_align<3>(w, ew, em), cw);
+    t.add(fx_align<3>(e, ee, em), ce);
+    t.add(fx_align<3>(n, et, em), cn);
+    t.sub(fx_align<3>(u, eu, em), d);
+    const int emq = em - q * (1 << 20);
+    return fx_ends(fx_to_f64_int(t.total() + fx_align<3>(b, eb, em), (emq >> 20) + 4), min(em, emq), max(em, emq));
+}
 // u + (9 c0 + 3 (+-c1) + 3 (+-c2) +- c3) / 16: bilinear interpolation, s1 s2 set for a minus.
 __device__ __forceinline__ double fx_bilinear(double u, double c0, double c1, double c2, double c3, bool s1, bool s2) {
     const int em = max(max(max(exp_bits(u), exp_bits(c0)), max(exp_bits(c1), exp_bits(c2))), exp_bits(c3));

@@ -85,6 +85,8 @@ template <class T> struct LevelDev {
     const int4 *rzw;              // FP64 levels without per-row tables: cz, cw [nr], ce [nr] and
     const int2 *rev, *rdg;        // diag [ncls][nr][nm] times 2^rq in limbs; else null
     int rq;
+    const int4 *hen, *ren;        // FP64 levels with per-row tables of few classes: (he, hn) in limbs beside hzw, which
+                                  // then holds (hz, hw), and (cce, ccn) beside rzw, (ccs, ccw), [ncls][nr]; else null
     const int *rcls;              // per-row tables (composite domain or non-uniform axial mesh): coefficient
                                   // class of each row [nz]; null: rows 0 and nz-1 are classes 0 and
                                   // ncls-1, the others class 1.  An inactive cell has zero diag, invd and

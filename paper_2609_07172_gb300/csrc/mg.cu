@@ -111,6 +111,17 @@ __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i,
         // a cell outside a composite domain's patches (zero diagonal) has no
         // residual: nothing else is loaded for it
         if (d == T(0)) return mk<T>(0, 0);
+        if constexpr (sizeof(T) == sizeof(double)) {
+            if (L.ren) {   // real part on the FP64 unit, imaginary part in fixed point
+                const V2<T> zero = mk<T>(0, 0), *u = L.u + idx;
+                const V2<T> us = k > 0 ? *(u - rowstride) : zero, un = k < L.nz - 1 ? u[rowstride] : zero;
+                const V2<T> uw = i > 0 ? *(u - L.nm) : zero, ue = i < L.nr - 1 ? u[L.nm] : zero, uc = *u, b = L.b[idx];
+                T x = fma(L.ccn[ci], un.x, fma(L.ccs[ci], us.x, b.x));
+                x = fma(L.cce[ci], ue.x, fma(L.ccw[ci], uw.x, x));
+                return mk<T>(fma(-d, uc.x, x), fx_residual(b.y, us.y, uw.y, ue.y, un.y, uc.y, L.rzw[ci], L.ren[ci],
+                                                           L.rdg[ci * L.nm + m], L.rq));
+            }
+        }
         V2<T> acc = L.b[idx];
         if (k > 0) acc = fma2<T>(L.ccs[ci], L.u[idx - rowstride], acc);
         if (k < L.nz - 1) acc = fma2<T>(L.ccn[ci], L.u[idx + rowstride], acc);
@@ -211,6 +222,17 @@ __device__ __forceinline__ void smooth_body(const LevelDev<T> &L, unsigned blk, 
         }
         V2<T> acc;
         if (RW && L.holes && L.invd[tb] == T(0)) return;   // outside a composite domain: u stays 0
+        if constexpr (RW && !SOR && sizeof(T) == sizeof(double)) {
+            if (L.hen) {   // real part on the FP64 unit, imaginary part in fixed point
+                const V2<T> zero = mk<T>(0, 0), *u = L.u + idx;
+                const V2<T> us = k > 0 ? *(u - rowstride) : zero, un = k < L.nz - 1 ? u[rowstride] : zero;
+                const V2<T> uw = i > 0 ? *(u - nm) : zero, ue = i < L.nr - 1 ? u[nm] : zero, b = L.bh[idx];
+                const T x = fma(L.hn[tb], un.x, fma(L.hz[tb], us.x, b.x));
+                L.u[idx] = mk<T>(fma(L.he[tb], ue.x, fma(L.hw[tb], uw.x, x)),
+                                 fx_update(b.y, us.y, uw.y, ue.y, un.y, L.hzw[tb], L.hen[tb]));
+                return;
+            }
+        }
         if (RW && L.rcls && sizeof(T) == sizeof(double)) {   // per-row tables, FP64: south (hz) and
                                                              // north (hn) couplings apart
             acc = L.bh[idx];
@@ -319,6 +341,17 @@ __device__ __forceinline__ void smooth_body(const LevelDev<T> &L, unsigned blk, 
                 south = vn[t];
                 continue;
             }
+            if constexpr (RW && !SOR && sizeof(T) == sizeof(double)) {
+                if (L.hen) {   // imaginary part in fixed point, as above
+                    const size_t tb = (size_t)L.rcls[k] * rs + tcol;
+                    const T x = fma(L.hn[tb], vn[t].x, fma(L.hz[tb], south.x, vb[t].x));
+                    L.u[idx0 + (size_t)(2 * t) * rs] =
+                        mk<T>(fma(L.he[tb], ve[t].x, fma(L.hw[tb], vw[t].x, x)),
+                              fx_update(vb[t].y, south.y, vw[t].y, ve[t].y, vn[t].y, L.hzw[tb], L.hen[tb]));
+                    south = vn[t];
+                    continue;
+                }
+            }
             if (RW && L.rcls && sizeof(T) == sizeof(double)) {   // per-row tables, FP64
                 const size_t tb = (size_t)L.rcls[k] * rs + tcol;
                 hw = L.hw[tb];
@@ -358,7 +391,7 @@ __device__ __forceinline__ void smooth_body(const LevelDev<T> &L, unsigned blk, 
 }
 
 template <class T, int NT, int S, bool SOR, bool RW, bool ONE>
-__global__ void __launch_bounds__(NT, S == 0 ? (sizeof(T) == 8 && !RW && !SOR ? 1536 : 2048) / NT : 1)
+__global__ void __launch_bounds__(NT, S == 0 ? (sizeof(T) == 8 && !SOR ? 1536 : 2048) / NT : 1)
 k_smooth(const __grid_constant__ LevelArg<T> arg, int color) {
     if constexpr (ONE) {
         smooth_body<T, NT, S, SOR, RW, true>(arg.f, blockIdx.x, color);
@@ -367,7 +400,10 @@ k_smooth(const __grid_constant__ LevelArg<T> arg, int color) {
         const int p = find_problem(tab->start, tab->n, blockIdx.x);
         if (tab->done && tab->done[tab->pid[p]]) return;   // stopped problem of a batch
         const unsigned first = (blockIdx.x - tab->start[p]) * (unsigned)tab->chunk, last = first + (unsigned)tab->chunk;
-        if constexpr (sizeof(T) == sizeof(double) && S == 0 && !SOR && !RW) {
+        if constexpr (RW && sizeof(T) == sizeof(float)) {   // (no room for a loop in 32 registers: chunk is 1)
+            const LevelDev<T> L = tab->f[p];
+            smooth_body<T, NT, S, SOR, RW, false>(L, first, color);
+        } else if constexpr (S == 0 && (RW || (sizeof(T) == sizeof(double) && !SOR))) {
             __shared__ LevelDev<T> L;
             stage_view(&L, &tab->f[p]);
             __syncthreads();
@@ -828,9 +864,22 @@ __global__ void __launch_bounds__(256) k_limbs(const LevelDev<double> L, size_t 
     if (t >= ntab) return;
     const int2 z = to_coef(L.hz[t]), w = to_coef(L.hw[t]);
     const_cast<int4 *>(L.hzw)[t] = make_int4(z.x, z.y, w.x, w.y);
-    const_cast<int2 *>(L.hev)[t] = to_coef(L.he[t]);
+    if (L.hen) {
+        const int2 e = to_coef(L.he[t]), n = to_coef(L.hn[t]);
+        const_cast<int4 *>(L.hen)[t] = make_int4(e.x, e.y, n.x, n.y);
+    } else {
+        const_cast<int2 *>(L.hev)[t] = to_coef(L.he[t]);
+    }
     if (!L.rzw) return;
     const_cast<int2 *>(L.rdg)[t] = to_coef(times_pow2(L.diag[t], L.rq));
+    if (L.ren) {
+        if (t >= (size_t)L.ncls * L.nr) return;
+        const int2 s = to_coef(times_pow2(L.ccs[t], L.rq)), a = to_coef(times_pow2(L.ccw[t], L.rq));
+        const int2 e = to_coef(times_pow2(L.cce[t], L.rq)), n = to_coef(times_pow2(L.ccn[t], L.rq));
+        const_cast<int4 *>(L.rzw)[t] = make_int4(s.x, s.y, a.x, a.y);
+        const_cast<int4 *>(L.ren)[t] = make_int4(e.x, e.y, n.x, n.y);
+        return;
+    }
     if (t < (size_t)L.nr) {
         const int2 a = to_coef(times_pow2(L.cz[t], L.rq)), b = to_coef(times_pow2(L.cw[t], L.rq));
         const_cast<int4 *>(L.rzw)[t] = make_int4(a.x, a.y, b.x, b.y);
@@ -926,23 +975,30 @@ __global__ void __launch_bounds__(1024) k_check(Ctrl *__restrict__ ctrl, const d
     __shared__ double wsum[32];
     __shared__ double sums[kMaxBatch];
     __shared__ int s_any;
+    // What the tests before and the norm of b left is read before the wait (the
+    // kernel before this one writes partials only, and started after theirs ended).
+    const int n = ctrl->n, max_cycles = ctrl->max_cycles, scaled = ctrl->scaled;
+    const int cycles = ctrl->cycles + (counting == 2 ? ctrl->inc_first : counting ? ctrl->inc : 0);
+    const double tol = ctrl->tol;
+    const bool mine = (int)threadIdx.x < n;
+    const int done = mine ? ctrl->done[threadIdx.x] : 1;
+    const double bb = mine ? ctrl->bnorm2[threadIdx.x] : 0.0, best = mine ? ctrl->best[threadIdx.x] : 0.0;
+    const double su = mine ? ctrl->sigma_next[threadIdx.x] : 1.0, count = mine ? ctrl->count[threadIdx.x] : 1.0;
+    static_assert(kMaxBatch <= 1024, "a thread per problem");
+    if (threadIdx.x == 0) s_any = 0;
     pdl_wait();
     pdl_go();
-    const int cycles = ctrl->cycles + (counting == 2 ? ctrl->inc_first : counting ? ctrl->inc : 0);
-    if (threadIdx.x == 0) s_any = 0;
-    range_sums(partials, ctrl->rbegin, ctrl->rend, ctrl->n, sums, wsum);
-    const double tol = ctrl->tol;
-    for (int p = threadIdx.x; p < ctrl->n; p += blockDim.x) {
-        if (ctrl->done[p]) continue;   // stopped: its kernels no longer run, rel stays the reported one
+    range_sums(partials, ctrl->rbegin, ctrl->rend, n, sums, wsum);
+    if (mine && !done) {   // (stopped: its kernels no longer run, rel stays the reported one)
+        const int p = (int)threadIdx.x;
         double rr2 = sums[p];
-        if (ctrl->scaled) {
-            const double su = ctrl->sigma_next[p];
+        if (scaled) {   // sigma is a power of two: its inverse and these products are exact
+            const double inv = __hiloint2double((2046 << 20) - __double2hiint(su), 0);
             ctrl->sigma_used[p] = su;
-            ctrl->inv_sigma_used[p] = 1.0 / su;
-            rr2 = rr2 / (su * su);
-            ctrl->sigma_next[p] = pow2_scale(rr2, ctrl->count[p]);
+            ctrl->inv_sigma_used[p] = inv;
+            rr2 = (rr2 * inv) * inv;
+            ctrl->sigma_next[p] = pow2_scale(rr2, count);
         }
-        const double bb = ctrl->bnorm2[p];
         const double rel = bb > 0.0 ? sqrt(rr2 / bb) : sqrt(rr2);
         ctrl->rel[p] = rel;
         if (!counting) ctrl->rel_first[p] = rel;
@@ -953,13 +1009,13 @@ __global__ void __launch_bounds__(1024) k_check(Ctrl *__restrict__ ctrl, const d
                 status = PIC_POISSON_ENONFINITE;
             } else if (tol > 0.0) {
                 stop = rel <= tol;
-            } else if (rel < 0.5 * ctrl->best[p]) {   // halved since the last reference point
+            } else if (rel < 0.5 * best) {   // halved since the last reference point
                 ctrl->best[p] = rel;
                 ctrl->stall[p] = 0;
             } else {   // rounding floor: no halving within kFloorWindow tests in a row
                 stop = ++ctrl->stall[p] >= kFloorWindow;
             }
-            if (!stop && cycles >= ctrl->max_cycles) {
+            if (!stop && cycles >= max_cycles) {
                 stop = 1;
                 status = PIC_POISSON_ENOTCONVERGED;
             }

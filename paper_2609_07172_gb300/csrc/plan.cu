@@ -655,11 +655,16 @@ template <class T, class V> void carve_level(const LevelHost &h, int nm, int nt,
     v.hw = c.take<T>(ntab);
     v.he = c.take<T>(ntab);
     v.hz = c.take<T>(ntab);
-    const bool fxt = std::is_same<T, double>::value && h.rcls.empty();
+    // per-row tables: only where the classes are few (a composite domain) -- on a
+    // stretched axial mesh every row has its own and the tables are as large as u
+    const bool rows = !h.rcls.empty();
+    const bool fxt = std::is_same<T, double>::value && (!rows || 2 * h.ncls <= h.nz);
     v.hzw = fxt ? c.take<int4>(ntab) : nullptr;
-    v.hev = fxt ? c.take<int2>(ntab) : nullptr;
-    v.rzw = fxt ? c.take<int4>(h.nr) : nullptr;
-    v.rev = fxt ? c.take<int2>(h.nr) : nullptr;
+    v.hev = fxt && !rows ? c.take<int2>(ntab) : nullptr;
+    v.hen = fxt && rows ? c.take<int4>(ntab) : nullptr;
+    v.rzw = fxt ? c.take<int4>(rows ? (size_t)h.ncls * h.nr : h.nr) : nullptr;
+    v.rev = fxt && !rows ? c.take<int2>(h.nr) : nullptr;
+    v.ren = fxt && rows ? c.take<int4>((size_t)h.ncls * h.nr) : nullptr;
     v.rdg = fxt ? c.take<int2>(ntab) : nullptr;
     int rq = 0;   // the largest diagonal times 2^rq in [1/2, 1)
     if (fxt) {
@@ -669,7 +674,7 @@ template <class T, class V> void carve_level(const LevelHost &h, int nm, int nt,
         if (dmax > 0.0 && std::abs(rq) < 60) {
             v.rq = -rq;
         } else {   // (coefficients out of that range: the FP64 unit computes both parts)
-            v.rzw = nullptr;
+            v.rzw = v.ren = nullptr;
             v.rev = v.rdg = nullptr;
             v.rq = 0;
         }
@@ -1040,7 +1045,7 @@ void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, c
             ++tp.n;
         }
         ts.chunk = 1;
-        if (strip == 0) chunked(ts);
+        if (strip == 0 && !(std::is_same<T, float>::value && P.masked)) chunked(ts);
         chunked(tr);
         chunked(tp);
         if (l == 0) H.restr0_start.assign(tr.start, tr.start + tr.n + 1);
