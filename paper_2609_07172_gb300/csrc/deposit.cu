@@ -363,22 +363,13 @@ FixAxis fix_axis(double lo, double hi, int n) {
     while ((n >> (b + 1)) != 0) ++b;
     a.F = 61 - b;                                          // n 2^F in [2^61, 2^62)
     const u64 num = (u64)n << a.F, den = a.span << a.sh;   // K = floor(num 2^64 / den), num < den
-    u64 rem = num, K = 0;
-    for (int k = 0; k < 64; ++k) {
-        rem <<= 1;
-        K <<= 1;
-        if (rem >= den) {
-            rem -= den;
-            K |= 1;
-        }
-    }
-    a.K = K;
+    a.K = den ? (u64)(((unsigned __int128)num << 64) / den) : 0;
     if (a.span == 0 || num >= den) a.span = 0;             // degenerate: every particle takes the binary64 arithmetic
     return a;
 }
 
 struct ProjectArgs {
-    int nr, nt, nz, accumulate;
+    int nr, nt, nz, accumulate, walk;   // walk: axial cells per warp
     double charge;
     const double *flo, *fhi;   // [nr] radial shares of a cell's lower / upper corner nodes
     const double *nodes;
@@ -392,17 +383,18 @@ struct ProjectArgs {
 // and gets the next radius' sum from the next lane -- 2 additions and 2
 // multiply-adds per cell where one thread per cell took 7 and 4 FP64
 // instructions, which bound the kernel (26.2 M cells: 545 us, now 264, the FP64 unit 72 % busy).
+// Fewer cells per walk where that leaves too few warps (320 x 8 x 21: 7.1 -> 3.4 us).
 constexpr int PROJ_K = 8, PROJ_WARPS = 8;
 
 template <bool MASK>
 __global__ void __launch_bounds__(PROJ_WARPS * 32) k_project(const ProjectArgs a) {
     const int lane = threadIdx.x & 31;
     const unsigned item = blockIdx.x * PROJ_WARPS + (threadIdx.x >> 5);   // (k block, j, radial block), radial fastest
-    const unsigned rb = (unsigned)(a.nr + 30) / 31u, kb = (unsigned)(a.nz + PROJ_K - 1) / PROJ_K;
+    const unsigned rb = (unsigned)(a.nr + 30) / 31u, kb = (unsigned)(a.nz + a.walk - 1) / a.walk;
     if (item >= rb * (unsigned)a.nt * kb) return;
     const unsigned row = item / rb;
     const int i = (int)(item - row * rb) * 31 + lane;
-    const int k0 = (int)(row / (unsigned)a.nt) * PROJ_K, j = (int)(row % (unsigned)a.nt);
+    const int k0 = (int)(row / (unsigned)a.nt) * a.walk, j = (int)(row % (unsigned)a.nt);
     const int jn = j + 1 == a.nt ? 0 : j + 1;
     const size_t rs = (size_t)a.nr + 1, ps = (size_t)a.nt * rs;
     const int in = min(i, a.nr);                                           // (lanes beyond the last node radius)
@@ -411,7 +403,7 @@ __global__ void __launch_bounds__(PROJ_WARPS * 32) k_project(const ProjectArgs a
     const double flo = cell ? s * a.flo[i] : 0.0, fhi = cell ? s * a.fhi[i] : 0.0;
     const double *n0 = a.nodes + (size_t)k0 * ps + (size_t)j * rs + in, *n1 = a.nodes + (size_t)k0 * ps + (size_t)jn * rs + in;
     double lower = *n0 + *n1;
-    const int k1 = min(a.nz, k0 + PROJ_K);
+    const int k1 = min(a.nz, k0 + a.walk);
     for (int k = k0; k < k1; ++k) {
         n0 += ps;
         n1 += ps;
@@ -530,7 +522,9 @@ extern "C" int pic_poisson_project(pic_poisson_plan_t plan, const double *nodes_
     a.nodes = nodes_dev;
     a.rho = rho_dev;
     a.act = q.act0;
-    const size_t items = (size_t)((a.nr + 30) / 31) * a.nt * ((a.nz + PROJ_K - 1) / PROJ_K);
+    const size_t rows = (size_t)((a.nr + 30) / 31) * a.nt;   // of warps
+    a.walk = (int)std::min<size_t>(std::max<size_t>(rows * a.nz / (152 * 64 * 2), 1), PROJ_K);
+    const size_t items = rows * ((a.nz + a.walk - 1) / a.walk);
     const unsigned grid = (unsigned)((items + PROJ_WARPS - 1) / PROJ_WARPS);
     if (q.act0) k_project<true><<<grid, PROJ_WARPS * 32, 0, plan->stream>>>(a);
     else k_project<false><<<grid, PROJ_WARPS * 32, 0, plan->stream>>>(a);
