@@ -356,8 +356,14 @@ cudaError_t launch_rhs_restrict(const TabRef<T> &tab, unsigned grid, cudaStream_
 template <class T> cudaError_t launch_tri_factors(const CoarseDev<T> &D, cudaStream_t st);
 // V 2^61 of n entries in limbs (CoarseDev::Vl).
 cudaError_t launch_limbs_v(const double *V, int2 *Vl, int n, cudaStream_t st);
-// The limb tables of a level from its binary64 ones (ntab entries of [ncls][nr][nm]).
-cudaError_t launch_limbs(const LevelDev<double> &L, size_t ntab, cudaStream_t st);
+// The limb tables of levels from their binary64 ones (ntab entries of [ncls][nr][nm] each).
+struct LimbSet {
+    static constexpr int MAX = 12;
+    int n = 0;
+    size_t ntab[MAX];
+    LevelDev<double> L[MAX];
+};
+cudaError_t launch_limbs(const LimbSet &set, cudaStream_t st);
 
 // zero_x: the FP64 iterate is zero (r = b; the kernel also writes x = 0).
 cudaError_t launch_defect(const DefectTab *tab, unsigned grid, const Ctrl *ctrl, double *partials, bool zero_x,

@@ -28,6 +28,8 @@
 //    without reading them, so only black cells receive the correction;
 //  * on coarse levels the first red half-sweep from a zero iterate is just
 //    u_red = b_hat_red, written by the restriction kernel.
+#include <algorithm>
+
 #include "coarse.h"
 #include "fixed.h"
 #include "internal.h"
@@ -859,9 +861,10 @@ __global__ void __launch_bounds__(256) k_limbs_v(const double *__restrict__ V, i
 __device__ __forceinline__ double times_pow2(double x, int q) {
     return f64_exp(x) ? __hiloint2double(__double2hiint(x) + q * (1 << 20), __double2loint(x)) : 0.0;
 }
-__global__ void __launch_bounds__(256) k_limbs(const LevelDev<double> L, size_t ntab) {
+__global__ void __launch_bounds__(256) k_limbs(const __grid_constant__ LimbSet set) {
+    const LevelDev<double> &L = set.L[blockIdx.y];
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= ntab) return;
+    if (t >= set.ntab[blockIdx.y]) return;
     const int2 z = to_coef(L.hz[t]), w = to_coef(L.hw[t]);
     const_cast<int4 *>(L.hzw)[t] = make_int4(z.x, z.y, w.x, w.y);
     if (L.hen) {
@@ -1166,8 +1169,10 @@ cudaError_t launch_update(const DefectTab *tab, unsigned grid, const Ctrl *ctrl,
     return launch_pdl(k_update, grid, MG_THREADS, 0, st, tab, ctrl);
 }
 
-cudaError_t launch_limbs(const LevelDev<double> &L, size_t ntab, cudaStream_t st) {
-    k_limbs<<<(unsigned)((ntab + 255) / 256), 256, 0, st>>>(L, ntab);
+cudaError_t launch_limbs(const LimbSet &set, cudaStream_t st) {
+    size_t most = 0;
+    for (int l = 0; l < set.n; ++l) most = std::max(most, set.ntab[l]);
+    if (most) k_limbs<<<dim3((unsigned)((most + 255) / 256), (unsigned)set.n), 256, 0, st>>>(set);
     return cudaGetLastError();
 }
 

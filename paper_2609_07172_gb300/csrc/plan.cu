@@ -865,9 +865,6 @@ template <class T> void upload_level(const LevelHost &h, const LevelDev<T> &v, c
     to_dev(h.hw, v.hw, st, err);
     to_dev(h.he, v.he, st, err);
     to_dev(h.hz, v.hz, st, err);
-    if constexpr (std::is_same<T, double>::value) {   // the same coefficients in limbs
-        if (v.hzw && err == cudaSuccess) err = launch_limbs(v, h.hz.size(), st);
-    }
 }
 
 // Launch tables of one precision's hierarchy.  views(q) is problem q's level list.
@@ -882,15 +879,17 @@ void build_deep(const pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coa
     if (q.lv[q.L - 1].nz > DEEP_MAX_NZ) return;
     const std::vector<LevelDev<T>> &v = views(q);
     const CoarseDev<T> &D = coarse(q);
-    int resident[9];   // clusters of C blocks, one block per SM
-    for (int C = 1; C <= 8; ++C) {
-        DeepArg<T> A;
-        A.D = D;
-        A.C = C;
-        A.smem = (unsigned)DEEP_MAX_SMEM;
-        resident[C] = deep_resident(A);
-        if (!resident[C]) return;
-    }
+    int known[9] = {0};
+    auto resident = [&](int C) {   // clusters of C blocks, one block per SM, that the device holds
+        if (!known[C]) {
+            DeepArg<T> A;
+            A.D = D;
+            A.C = C;
+            A.smem = (unsigned)DEEP_MAX_SMEM;
+            known[C] = std::max(deep_resident(A), 0) + 1;
+        }
+        return known[C] - 1;
+    };
     H.deep.resize(q.L - 1);
     int zmul = 1;
     for (int l = q.L - 2; l >= 0; --l) {
@@ -928,9 +927,9 @@ void build_deep(const pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coa
             }
         if (!C) break;
         const size_t cells = (size_t)f.nr / 2 * f.nz;
-        while (C < 8 && C < D.nz && f.nm <= resident[C + 1] && cells > (size_t)C * DEEP_THREADS) ++C;
+        while (C < 8 && C < D.nz && cells > (size_t)C * DEEP_THREADS && f.nm <= resident(C + 1)) ++C;
         if (std::is_same<T, double>::value && l == 0) {   // (the whole solve or nothing)
-            if (f.nm > resident[C]) break;
+            if (f.nm > resident(C)) break;
             H.deep_solve = true;
         }
         deep_layout(A, C);
@@ -1164,7 +1163,19 @@ int upload(pic_poisson_plan_s &P) {
     const bool mixed = P.shared.precision == PIC_POISSON_MIXED;
     for (int p = 0; p < P.n; ++p) {
         ProblemPlan &q = P.pr[p];
-        for (size_t l = 0; l < q.dl.size(); ++l) upload_level(q.lv[l], q.dl[l], st, err);
+        LimbSet limbs;   // the FP64 levels' coefficients once more, as limbs (one launch)
+        auto flush = [&] {
+            if (limbs.n && err == cudaSuccess) err = launch_limbs(limbs, st);
+            limbs.n = 0;
+        };
+        for (size_t l = 0; l < q.dl.size(); ++l) {
+            upload_level(q.lv[l], q.dl[l], st, err);
+            if (!q.dl[l].hzw) continue;
+            limbs.L[limbs.n] = q.dl[l];
+            limbs.ntab[limbs.n++] = q.lv[l].hz.size();
+            if (limbs.n == LimbSet::MAX) flush();
+        }
+        flush();
         for (size_t l = 0; l < q.fl.size(); ++l) upload_level(q.lv[l], q.fl[l], st, err);
         std::vector<double> V, e, piv, cpr;
         if (q.nact > 0) {   // composite domain: dense coarsest solve

@@ -1,4 +1,6 @@
 """V-cycles in shared memory (one cluster per mode) against the level kernels: bitwise equal."""
+import threading
+
 import pytest
 import torch
 
@@ -52,3 +54,28 @@ def test_from_a_given_iterate(dims, fmg):
     a, ca = _level_kernels(p, rho, g, fmg=fmg, initial_guess=True)
     b, cb = _solve(p, rho, g, fmg=fmg, initial_guess=True)
     assert ca == cb and torch.equal(a, b)
+
+
+def test_two_threads_on_their_own_streams():
+    """Two solves of one launch each that fill most of the chip, at the same time: neither waits on the other's blocks."""
+    p = W.annulus(64, 64, 64)
+    rho = torch.from_numpy(W.rho_plasma(p, 9)).cuda()
+    want, _ = _solve(p, rho)
+    torch.cuda.synchronize()
+    errors = []
+
+    def work():
+        try:
+            st = torch.cuda.Stream()
+            with torch.cuda.stream(st), Plan(p, graph=True) as plan:
+                for _ in range(40):
+                    phi, info = plan.solve(rho, tol=1e-10)
+                    assert info["status"] == 0 and torch.equal(phi, want)
+        except BaseException as e:      # noqa: B036 (reported by the test's thread)
+            errors.append(e)
+    threads = [threading.Thread(target=work) for _ in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
