@@ -49,7 +49,7 @@ extern "C" {
 #define PIC_POISSON_OK 0
 #define PIC_POISSON_EINVAL 1          /* bad descriptor, size or argument */
 #define PIC_POISSON_ENOMEM 2          /* device or host allocation failed */
-#define PIC_POISSON_ECUDA 3           /* a CUDA call failed (see last_error) */
+#define PIC_POISSON_ECUDA 3           /* a CUDA call failed or a kernel's bounded wait ran out (see last_error) */
 #define PIC_POISSON_ENOTCONVERGED 4   /* tolerance not met in max_cycles; phi holds the last iterate */
 #define PIC_POISSON_ENONFINITE 5      /* non-finite right-hand side or residual */
 
@@ -236,6 +236,16 @@ int pic_poisson_plan_batch(const pic_poisson_desc *descs, int n, void *stream, p
 
 /* Replace the plan's stream (later calls enqueue there). */
 int pic_poisson_set_stream(pic_poisson_plan_t plan, void *stream);
+
+/*
+ * How many times a block of a small FP64 solve that runs as one launch
+ * (local_bottom = 0) looks for the other blocks' norms in a convergence test
+ * before it gives up (default 2^22, seconds; a test waits for microseconds).
+ * A solve that gives up returns PIC_POISSON_ECUDA with a NaN residual; phi is
+ * then an unconverged iterate, and the plan can be used again.  Applies to the
+ * solves that follow.
+ */
+int pic_poisson_set_poll_limit(pic_poisson_plan_t plan, int polls);
 
 /*
  * Full solve: rho_dev (nz, ntheta, nr) FP64 charge density -> phi_dev (same

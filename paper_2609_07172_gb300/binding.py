@@ -22,7 +22,7 @@ NPHASE = len(PHASES)
 
 EXPORTS = (
     "pic_poisson_query", "pic_poisson_cell_coeffs", "pic_poisson_plan", "pic_poisson_plan_batch",
-    "pic_poisson_set_stream", "pic_poisson_solve_batch",
+    "pic_poisson_set_stream", "pic_poisson_set_poll_limit", "pic_poisson_solve_batch",
     "pic_poisson_solve", "pic_poisson_solve_host", "pic_poisson_forward", "pic_poisson_inverse",
     "pic_poisson_face_field", "pic_poisson_deposit", "pic_poisson_project",
     "pic_poisson_mode_residual", "pic_poisson_destroy", "pic_poisson_last_error",
@@ -131,6 +131,7 @@ def load(build_if_missing: bool = True):
         "pic_poisson_plan_batch": ([vp, ip, vp, vp], ip),
         "pic_poisson_solve_batch": ([vp, vp, vp, dp, vp], ip),
         "pic_poisson_set_stream": ([vp, vp], ip),
+        "pic_poisson_set_poll_limit": ([vp, ip], ip),
         "pic_poisson_solve": ([vp, vp, vp, dp, vp], ip),
         "pic_poisson_solve_host": ([vp, vp, vp, dp, vp], ip),
         "pic_poisson_forward": ([vp, vp, vp], ip),
@@ -283,6 +284,10 @@ class Plan:
     def set_stream(self, stream):
         self.stream = stream
         _check(load().pic_poisson_set_stream(self._plan, ctypes.c_void_p(stream.cuda_stream)))
+
+    def set_poll_limit(self, polls):
+        """Polls after which a block of a one-launch solve gives up waiting (default 2^22)."""
+        _check(load().pic_poisson_set_poll_limit(self._plan, int(polls)))
 
     def solve(self, rho, phi=None, tol=1e-10):
         """Solve into phi (allocated if None); returns (phi, info dict).

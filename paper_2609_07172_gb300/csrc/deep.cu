@@ -563,14 +563,14 @@ template <class T> __device__ __forceinline__ void fmg(const Ctx<T> &X) {
 // FP64 problem).  Every block adds its part; the first block of each cluster
 // waits for all of them, adds them in the same order and tells its cluster.  The
 // grid is resident as a whole (a cooperative launch); a wait that runs out all
-// the same ends the solve with an error status.
+// the same (Ctrl::polls) ends the solve with the status ECUDA and a NaN residual.
+// Clusters whose own wait was met go on to the next test and give up there.
 struct Test {
     double best, rr_first, rr;
     int stall, cycles, epoch, status;
 };
 __device__ __forceinline__ int converged(Ctrl *ctrl, Test &t) {
     const double tol = ctrl->tol, bb = ctrl->bnorm2[0];
-    if (t.epoch == 1) t.rr_first = t.rr;
     // far from the tolerance: no division, no square root
     if (tol > 0.0 && t.cycles < ctrl->max_cycles && bb > 0.0 && t.rr < 1e300 && t.rr > 1.001 * tol * tol * bb) return 0;
     const double rel = bb > 0.0 ? sqrt(t.rr / bb) : sqrt(t.rr);
@@ -614,7 +614,7 @@ __device__ __forceinline__ bool test(const Ctx<T> &X, Ctrl *ctrl, double *partia
             if (threadIdx.x == 0) {
                 const unsigned want = (unsigned)t.epoch * gridDim.x;
                 ok = 0;
-                for (int n = 0; n < (1 << 22) && !ok; ++n) {
+                for (int n = 0, polls = ctrl->polls; n < polls && !ok; ++n) {
                     unsigned got;
                     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(&ctrl->arrived) : "memory");
                     ok = got >= want;
@@ -626,7 +626,8 @@ __device__ __forceinline__ bool test(const Ctx<T> &X, Ctrl *ctrl, double *partia
                 for (unsigned b = threadIdx.x; b < gridDim.x; b += 32) s += __ldcg(part + b);
             for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if (threadIdx.x == 0) {
-                t.rr = s;
+                t.rr = ok ? s : __longlong_as_double(0x7ff8000000000000ll);
+                if (t.epoch == 1) t.rr_first = t.rr;
                 int stop = 1;
                 if (ok) stop = converged(ctrl, t);
                 else t.status = PIC_POISSON_ECUDA;

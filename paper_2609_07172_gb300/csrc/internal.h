@@ -255,6 +255,7 @@ struct Ctrl {
     unsigned rbegin[kMaxBatch];   // residual-norm partials of problem p: [rbegin, rend)
     unsigned rend[kMaxBatch];
     unsigned arrived;             // blocks that have come to a test of launch_deep_solve
+    int polls;                    // per solve: reads of `arrived` after which a test's wait gives up
 };
 
 // First stage of the residual-norm reduction: each block sums PSUM_CHUNK
@@ -453,6 +454,7 @@ constexpr int DEEP_THREADS = 512;
 constexpr int DEEP_LEVELS = 8;
 constexpr size_t DEEP_MAX_SMEM = 225 * 1024;
 constexpr int DEEP_MAX_NZ = 64;          // rows of the coarsest level
+constexpr int DEEP_POLLS = 1 << 22;      // default of Ctrl::polls: seconds, where a test's wait takes microseconds
 // Entries (cells x modes) of the first level up to which it takes that way: above,
 // the level kernels fill the chip and are as fast or faster.  Measured (us, with
 // launches / in shared memory): whole hierarchies 90 x 32 x 70 FP64 520 / 319,

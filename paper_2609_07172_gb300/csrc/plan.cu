@@ -1728,6 +1728,17 @@ int pic_poisson_set_stream(pic_poisson_plan_t plan, void *stream) {
     return PIC_POISSON_OK;
 }
 
+int pic_poisson_set_poll_limit(pic_poisson_plan_t plan, int polls) {
+    int rc = plan_enter(plan);
+    if (rc) return rc;
+    if (polls < 0) {
+        set_error("the poll limit is negative (%d)", polls);
+        return PIC_POISSON_EINVAL;
+    }
+    plan->polls = polls;
+    return PIC_POISSON_OK;
+}
+
 int pic_poisson_destroy(pic_poisson_plan_t plan) {
     if (!plan) return PIC_POISSON_OK;
     cudaSetDevice(plan->device);

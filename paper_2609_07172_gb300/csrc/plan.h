@@ -111,6 +111,7 @@ struct pic_poisson_plan_s {
 
     pp::Ctrl *ctrl = nullptr;                   // device
     pp::Ctrl hctrl{};                           // per-solve initial state
+    int polls = pp::DEEP_POLLS;                 // pic_poisson_set_poll_limit
     pp::Ctrl *hctrl_out = nullptr;              // pinned, results
     double *partials = nullptr, *partials_fwd = nullptr;
     size_t npartials = 0, npartials_fwd = 0;

@@ -539,6 +539,7 @@ int set_io(pic_poisson_plan_s &P, const double *const *rho, double *const *phi, 
     C.max_cycles = P.shared.max_cycles;
     C.cycles = 0;
     C.cont = 1;
+    C.polls = P.polls;
     for (int p = 0; p < P.n; ++p) {
         C.rel[p] = 1.0;
         C.rel_first[p] = 1.0;
@@ -752,7 +753,9 @@ int solve_batch(pic_poisson_plan_s &P, const double *const *rho, double *const *
     int worst = PIC_POISSON_OK;
     for (int p = 0; p < P.n; ++p) {
         const int s = C.status[p];
-        if (s == PIC_POISSON_ENONFINITE || (s == PIC_POISSON_ENOTCONVERGED && worst == PIC_POISSON_OK)) worst = s;
+        // a solve that gave up outranks values that are not finite, these a tolerance not reached
+        auto rank = [](int v) { return v == PIC_POISSON_OK ? 0 : v == PIC_POISSON_ENOTCONVERGED ? 1 : v == PIC_POISSON_ENONFINITE ? 2 : 3; };
+        if (rank(s) > rank(worst)) worst = s;
         if (!infos) continue;
         pic_poisson_info &I = infos[p];
         memset(&I, 0, sizeof I);
@@ -772,7 +775,8 @@ int solve_batch(pic_poisson_plan_s &P, const double *const *rho, double *const *
         }
     }
     if (worst == PIC_POISSON_ENONFINITE) set_error("non-finite right-hand side or residual");
-    if (worst == PIC_POISSON_ENOTCONVERGED) set_error("tolerance not reached in max_cycles");
+    else if (worst == PIC_POISSON_ENOTCONVERGED) set_error("tolerance not reached in max_cycles");
+    else if (worst != PIC_POISSON_OK) set_error("a wait between the blocks of the solve ran out (poll limit %d)", P.polls);
     return worst;
 }
 
