@@ -305,7 +305,7 @@ template <class T> size_t bottom_smem_bytes(int nr, int nz, int ncls, int ncr, i
 }
 
 template <class T> cudaError_t launch_bottom(const BottomTab<T> *tab, unsigned grid, size_t smem, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(k_bottom<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_bottom<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BOTTOM_MAX_SMEM);
     if (e != cudaSuccess) return e;
     return launch_pdl(k_bottom<T>, grid, BOTTOM_THREADS, smem, st, tab);
 }

@@ -746,8 +746,15 @@ int conv_tc_occupancy(int which, int threads, size_t smem, unsigned tmem_cols_pe
     return PIC_POISSON_OK;
 }
 
+// (the kernels' ceiling, not this launch's size: other layers set it too, on other
+// threads.  The most that a layer takes is 149 KB: 32 mixed channels to 80.)
+constexpr size_t CONV_MAX_SMEM = 200 * 1024;
 int set_smem(const void *kernel, size_t smem) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem > CONV_MAX_SMEM) {
+        set_error("conv3x3 (tcgen05): %zu bytes of shared memory, at most %zu", smem, CONV_MAX_SMEM);
+        return PIC_POISSON_EINVAL;
+    }
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CONV_MAX_SMEM);
     if (e == cudaSuccess)   // all of the SM's unified memory as shared memory, so several CTAs fit
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  (int)cudaSharedmemCarveoutMaxShared);

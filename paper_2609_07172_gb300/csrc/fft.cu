@@ -473,14 +473,14 @@ size_t fft_smem_bytes(int nt) {
 }
 
 cudaError_t launch_forward(const FFTTab *tab, unsigned grid, size_t smem, double *partials, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(k_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_smem_bytes(kMaxNtheta));
     if (e != cudaSuccess) return e;
     k_forward<<<grid, FFT_THREADS, smem, st>>>(tab, partials);
     return cudaGetLastError();
 }
 
 cudaError_t launch_inverse(const FFTTab *tab, unsigned grid, size_t smem, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(k_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_smem_bytes(kMaxNtheta));
     if (e != cudaSuccess) return e;
     k_inverse<<<grid, FFT_THREADS, smem, st>>>(tab);
     return cudaGetLastError();

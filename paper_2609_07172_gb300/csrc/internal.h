@@ -100,7 +100,6 @@ template <class T> struct LevelDev {
 };
 
 // Coarsest level: separable direct solve (z eigenbasis, tridiagonal in r).
-constexpr int TRI_Q = 48;         // products of factors per row of the tridiagonal solves (coarse.h)
 template <class T> struct CoarseDev {
     int nr, nz, nm;
     const T *V;                   // [nz][nz] orthonormal eigenvectors of the axial operator, V[k*nz+j]
@@ -303,6 +302,27 @@ cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size
     c.numAttrs = overlap ? 1 : 0;
     return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
+
+// ------------------------------------------------------------------ dynamic shared memory
+// A kernel's limit of dynamic shared memory belongs to the process, not to a
+// launch: the launchers set it to the kernel's ceiling below, never to the size
+// of their own launch, which a plan with smaller arrays on another thread would
+// lower between the call and the launch ("too many resources requested").
+constexpr int kMaxNtheta = 256;           // azimuthal cells
+constexpr int kMaxCoarseCells = 4096;     // cells and rows of an exactly solved coarsest level
+constexpr int kMaxCoarseNz = 64;
+constexpr int TRI_Q = 48;         // products of factors per row of the tridiagonal solves (coarse.h)
+// Elements that k_coarse holds of an nr x nz level: b, then four padded arrays, the
+// rows of V that it reads, the products of the factors, the columns' exponents.
+constexpr size_t coarse_smem_elems(int nr, int nz) {
+    return (size_t)nr * nz + 4 * (size_t)(nr + 1) * nz + (size_t)(nz - nz / 2) * nz + (size_t)nz * TRI_Q + (size_t)nr;
+}
+// (5 nr nz + nr + 52 nz + nz ceil(nz / 2): with nr nz given it is largest at one end of the range of nz)
+constexpr size_t COARSE_MAX_ELEMS =
+    coarse_smem_elems(kMaxCoarseCells / kMaxCoarseNz, kMaxCoarseNz) > coarse_smem_elems(kMaxCoarseCells, 1)
+        ? coarse_smem_elems(kMaxCoarseCells / kMaxCoarseNz, kMaxCoarseNz)
+        : coarse_smem_elems(kMaxCoarseCells, 1);
+static_assert(COARSE_MAX_ELEMS * sizeof(double) <= 227 * 1024, "the largest exact solve fits one block");
 
 // ------------------------------------------------------------------ launchers
 // All launchers enqueue on `st` and return cudaGetLastError().  `grid` is the

@@ -1149,7 +1149,7 @@ cudaError_t launch_rhs_restrict(const TabRef<T> &tab, unsigned grid, cudaStream_
 
 template <class T>
 cudaError_t launch_coarse(const CoarseTab<T> *tab, unsigned grid, size_t smem, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(k_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(COARSE_MAX_ELEMS * sizeof(T)));
     if (e != cudaSuccess) return e;
     return launch_pdl(k_coarse<T>, grid, MG_THREADS, smem, st, tab);
 }

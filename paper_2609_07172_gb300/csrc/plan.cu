@@ -32,9 +32,6 @@ namespace {
 
 constexpr double kPi = 3.14159265358979323846;
 constexpr double kEps0 = 8.8541878128e-12;   // F/m, CODATA 2018
-constexpr int kMaxNtheta = 256;
-constexpr int kMaxCoarseCells = 4096;
-constexpr int kMaxCoarseNz = 64;
 constexpr unsigned kKnownFlags =
     PIC_POISSON_USE_INITIAL_GUESS | PIC_POISSON_PROFILE | PIC_POISSON_GRAPH | PIC_POISSON_HOST_STAGED;
 
@@ -1140,9 +1137,7 @@ void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, c
         tc.f[tc.n] = views(q)[q.L - 1];
         tc.c[tc.n] = cd;
         tc.start[tc.n + 1] = tc.start[tc.n] + 2u * (unsigned)q.nm;   // (mode, real / imaginary part)
-        const size_t sm = ((size_t)cd.nr * cd.nz + 4 * (size_t)(cd.nr + 1) * cd.nz +
-                           (size_t)(cd.nz - cd.nz / 2) * cd.nz + (size_t)cd.nz * TRI_Q + (size_t)cd.nr) * sizeof(T);
-        tc.smem = std::max(tc.smem, sm);
+        tc.smem = std::max(tc.smem, coarse_smem_elems(cd.nr, cd.nz) * sizeof(T));
         ++tc.n;
     }
     H.g_coarse = tc.start[tc.n];
