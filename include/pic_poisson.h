@@ -360,7 +360,9 @@ int pic_poisson_solve_host(pic_poisson_plan_t plan, const double *rho_host, doub
  * run of equal cells issues the FP64 atomics, so cell-sorted particles are
  * cheapest; any order is correct (the order of the atomics, hence rounding,
  * varies from run to run).  Offsets, weights' products and those sums are
- * 64-bit fixed point (2^-54 of a particle); the atomics are binary64.
+ * 64-bit fixed point where that holds a weight to 2^-45 of itself, else
+ * binary64 (a particle so close to a cell's corner that a weight is below
+ * about 2^-14); the atomics are binary64.
  * Particles outside the domain deposit nothing.  On non-uniform faces
  * (r_faces, z_faces) the cell is the one the face arrays define (max{a :
  * face[a] <= x}, found by a lookup guess and exact binary64 comparisons) and

@@ -20,18 +20,24 @@
 //
 // Fixed point.  The FP64 unit (1/64 of the FP32 rate) bound this kernel: about
 // 23 of its instructions per particle for the position and 16 per cell for the
-// corners, 5.8 of the 5.8 ms per 105 M particles.  Offsets in the cell, their
-// products and every sum are 64-bit integers instead (scale 2^-54): a cell's
-// particles are summed as the eight moments 1, x, y, z, xy, xz, yz, xyz -- sums
-// that round nothing -- and the corner weights follow from them by exact
-// subtractions.  A particle's products are within 2^-54 of exact, where the
-// double-float products before were within 2^-48 relative.  The position goes
-// to a cell and an offset by one 64-bit multiplication; a particle near a cell
-// boundary (2^-24 of a cell) or outside takes the binary64 arithmetic, which
-// alone decides those cases.  210 M cell-sorted particles of two species, 4 per
-// cell and species, at 512 x 128 x 400: 11.6 ms, now 2.25 (integer instructions and
-// their issue, both two thirds busy; against a quadruple-precision deposit the nodes
-// are within 5.6e-14 as before, the largest error 2.0e-13 instead of 4.8e-13).
+// corners, 5.8 of the 5.8 ms per 105 M particles.  Offsets in the cell (64 fraction
+// bits), their products and every sum are 64-bit integers instead (units of 2^-61): a
+// cell's particles are summed as the eight moments 1, x, y, z, xy, xz, yz, xyz --
+// sums that round nothing -- and the corner weights follow from them by exact
+// subtractions.  Their error is absolute, three units per particle; a run with a
+// corner sum below 2^47 units per particle (2^-14 of one; 2 to 3 % of single particles
+// of a uniform density, one in 10^8 of four) goes to the nodes particle by particle
+// in binary64, so that every weight holds 2^-45 of itself as double-float
+// products did.  The position goes to a cell and an offset by one 64-bit
+// multiplication; a particle near a cell boundary (2^-24 of a cell) or outside takes
+// the binary64 arithmetic, which alone decides those cases, and one whose
+// coordinate has bits below the fixed point's, close to the lower wall, takes that too.
+// 210 M cell-sorted particles of two species, 4 per cell and species, at
+// 512 x 128 x 400: 11.6 ms with double-float, now 2.55 (integer instructions and their
+// issue, both two thirds busy).  In units of 2^-54 without the second way it was 2.3, but
+// a weight of 1e-12 kept four digits; 96-bit products hold every weight without it and
+// took 3.1.  Against a quadruple-precision deposit of 1.6 M particles the nodes are
+// within 5.6e-14 (L2), all forms alike: the rounding of the node volumes.
 //
 // Non-uniform faces and composite domains (FACES): the cell comes
 // from the face arrays (a bin lookup guesses, binary64 comparisons decide),
@@ -61,11 +67,14 @@ typedef unsigned long long u64;
 
 // One uniform axis in fixed point: x -> X = x 2^(62 - E) (|x| < 2^E over the
 // domain), D = X - base in [0, span), and D 2^sh K / 2^64 = the position in
-// cells with F fraction bits.
+// cells with F fraction bits, the product's low word giving the bits below.
+// K is cut by less than 2^-62 of it, and so is the position.  X is exact for
+// |x| >= 2^(E - 10); below, or where the wall is cut, D is off by up to two units.
 struct FixAxis {
     long long base;
     u64 span, K;
     int e1;                 // E + 1023
+    int smax;               // shift up to which X is exact (0: the wall is cut)
     int sh, F;
 };
 
@@ -74,7 +83,7 @@ struct DepositArgs {
     long long np;
     double r_in, z0, inv_dr, inv_da, inv_dz;
     FixAxis fr, fa, fz;
-    double wscale;          // the weight times 2^-54
+    double weight;
     int vec;                // the arrays allow 16-byte loads
     const double *r, *al, *z;
     const double *inv_vr;   // [nr + 1] 1 / (radial integral of r dr of node a's interval)
@@ -112,11 +121,17 @@ __device__ __forceinline__ int find_cell(double x, const double *f, int n, const
 
 constexpr int DEP_PPT = 4;   // consecutive particles per thread
 constexpr int DEP_THREADS = 256;
+constexpr u64 DEP_NEAR = 1ull << 48;   // least D of a coordinate or wall that is cut
 
 // A particle in its cell: indices and offsets, 64 fraction bits.
 struct Place {
     int ir, ia, iz;
     u64 x, y, z;
+};
+// The same with binary64 offsets.
+struct Spot {
+    int ir, ia, iz;
+    double x, y, z;
 };
 
 // A binary64 offset in [0, 1] as a 64-bit fraction (cut; 1 becomes 1 - 2^-64).
@@ -129,49 +144,36 @@ __device__ __forceinline__ u64 frac64(double f) {
 }
 
 // Cell and offset of x on a uniform axis; false where the binary64 arithmetic
-// has to decide: outside, not finite, or within 2^-24 of a cell boundary.
+// has to decide (outside, not finite, within 2^-24 of a cell boundary) or keeps
+// more of the offset (`near` above: close to the lower wall).
 __device__ __forceinline__ bool fix_place(const FixAxis &a, double x, int &cell, u64 &f) {
     const int hi = __double2hiint(x);
     const unsigned lo = (unsigned)__double2loint(x);
     const int s = a.e1 - ((hi >> 20) & 0x7ff);
     u64 X = ((((u64)((hi & 0xfffff) | 0x100000)) << 32 | lo) << 10) >> min(max(s, 0), 63);
     if (hi < 0) X = 0ull - X;
-    const u64 D = X - (u64)a.base;
-    const u64 t = __umul64hi(D << a.sh, a.K);
+    const u64 D = X - (u64)a.base, d = D << a.sh;
+    const u64 t = __umul64hi(d, a.K);
     cell = (int)(t >> a.F);
-    f = t << (64 - a.F);
-    return s >= 1 && D < a.span && (unsigned)(f >> 32) + 0x100u >= 0x200u;
+    f = t << (64 - a.F) | (d * a.K) >> a.F;
+    return s >= 1 && D < a.span && (s <= a.smax || D >= DEP_NEAR) && (unsigned)(f >> 32) + 0x100u >= 0x200u;
 }
 
 // Cell and offsets of particle (r, al, z) by binary64 arithmetic; false when
 // it is outside.
-__device__ __noinline__ bool place_exact(const DepositArgs &a, double r, double al, double z, Place &q) {
+__device__ __forceinline__ bool locate(const DepositArgs &a, double r, double al, double z, Spot &q) {
     const double tr = (r - a.r_in) * a.inv_dr, ta = al * a.inv_da, tz = (z - a.z0) * a.inv_dz;
     const double fr = floor(tr), fa = floor(ta), fz = floor(tz);
     // in range before any conversion (NaN compares false)
     if (!(fr >= 0.0 && fr < (double)a.nr && fa >= 0.0 && fa < (double)a.nt && fz >= 0.0 && fz < (double)a.nz))
         return false;
-    q.ir = (int)fr;
-    q.ia = (int)fa;
-    q.iz = (int)fz;
-    q.x = frac64(tr - fr);   // exact differences, in [0, 1)
-    q.y = frac64(ta - fa);
-    q.z = frac64(tz - fz);
-    return true;
-}
-
-__device__ __forceinline__ bool place(const DepositArgs &a, double r, double al, double z, Place &q) {
-    const bool ok = fix_place(a.fr, r, q.ir, q.x) & fix_place(a.fa, al, q.ia, q.y) & fix_place(a.fz, z, q.iz, q.z);
-    if (ok) return true;
-    Place e;   // (q stays in registers)
-    if (!place_exact(a, r, al, z, e)) return false;
-    q = e;
+    q = {(int)fr, (int)fa, (int)fz, tr - fr, ta - fa, tz - fz};   // exact differences, in [0, 1)
     return true;
 }
 
 // The same on face arrays; false also for a particle in an inactive cell.
-__device__ __forceinline__ bool place_faces(const DepositArgs &a, const DepositGeo &g, double r, double al, double z,
-                                            Place &q) {
+__device__ __forceinline__ bool locate_faces(const DepositArgs &a, const DepositGeo &g, double r, double al, double z,
+                                             Spot &q) {
     const double ta = al * a.inv_da, fa = floor(ta);
     if (!(fa >= 0.0 && fa < (double)a.nt)) return false;
     q.ir = find_cell(r, g.rf, a.nr, g.rbin, g.nrbin, g.r0f, g.inv_rbw);
@@ -180,14 +182,34 @@ __device__ __forceinline__ bool place_faces(const DepositArgs &a, const DepositG
     if (g.act && !g.act[(size_t)q.iz * a.nr + q.ir]) return false;   // inactive cell: nothing deposited
     q.ia = (int)fa;
     // the products may round to 1 at the upper face; the weights stay in [0, 1]
-    q.x = frac64(fmin((r - g.rf[q.ir]) * g.inv_wr[q.ir], 1.0));
-    q.y = frac64(ta - fa);
-    q.z = frac64(fmin((z - g.zf[q.iz]) * g.inv_wz[q.iz], 1.0));
+    q.x = fmin((r - g.rf[q.ir]) * g.inv_wr[q.ir], 1.0);
+    q.y = ta - fa;
+    q.z = fmin((z - g.zf[q.iz]) * g.inv_wz[q.iz], 1.0);
     return true;
 }
 
-// Moments of a cell's particles in units of 2^-54 (the count apart); at most
-// the 128 particles of a warp, so every sum stays below 2^61.
+// One particle's eight weights in binary64 straight to the nodes.
+template <bool V2D> __device__ __forceinline__ void spread(const DepositArgs &a, const double *inv_v2, const Spot &q) {
+    const int ja = q.ia + 1 == a.nt ? 0 : q.ia + 1;
+    const size_t rs = (size_t)a.nr + 1, ps = (size_t)a.nt * rs;
+#pragma unroll 1
+    for (int c = 0; c < 8; ++c) {
+        const int nzi = q.iz + (c >> 2), nai = (c & 2) ? ja : q.ia, nri = q.ir + (c & 1);
+        const double w = ((c & 4) ? q.z : 1.0 - q.z) * ((c & 2) ? q.y : 1.0 - q.y) * ((c & 1) ? q.x : 1.0 - q.x);
+        const double f = V2D ? a.weight * inv_v2[(size_t)nzi * rs + nri] : a.weight * a.inv_vr[nri] * a.inv_vz[nzi];
+        atomicAdd(a.nodes + (size_t)nzi * ps + (size_t)nai * rs + nri, w * f);
+    }
+}
+// Particle p by itself.
+template <bool FACES, bool V2D> __device__ __noinline__ void stray(const DepositArgs &a, const DepositGeo &g, long long p) {
+    Spot q;
+    if (FACES ? locate_faces(a, g, a.r[p], a.al[p], a.z[p], q) : locate(a, a.r[p], a.al[p], a.z[p], q)) spread<V2D>(a, g.inv_v2, q);
+}
+
+// Moments of a cell's particles, the count apart.  A thread's (at most four) are in
+// units of 2^-61; where runs cross lanes a warp's (at most 128) are cut to 2^-56.
+// Every sum stays below 2^63, two runs' below 2^64.
+constexpr int DEP_UNIT = 61, DEP_WIDE = 56;
 struct Moments {
     unsigned n;
     u64 m[7];   // x, y, z, xy, xz, yz, xyz
@@ -197,9 +219,10 @@ struct Moments {
         for (int e = 0; e < 7; ++e) m[e] = 0;
     }
     __device__ __forceinline__ void add(const Place &q) {
-        const u64 y = q.y >> 10, z = q.z >> 10, yz = __umul64hi(q.y, z);
+        constexpr int S = 64 - DEP_UNIT;
+        const u64 y = q.y >> S, z = q.z >> S, yz = __umul64hi(q.y, z);
         ++n;
-        m[0] += q.x >> 10;
+        m[0] += q.x >> S;
         m[1] += y;
         m[2] += z;
         m[3] += __umul64hi(q.x, y);
@@ -207,9 +230,11 @@ struct Moments {
         m[5] += yz;
         m[6] += __umul64hi(q.x, yz);
     }
-    // Corner sums (corner 4 dz + 2 dalpha + dr).  The cut of the products can
-    // bring a sum that is 0 a few units below it.
-    __device__ __forceinline__ void corners(u64 c[8]) const {
+    // Corner sums (corner 4 dz + 2 dalpha + dr), each off by less than three units per
+    // particle (four per lane where the moments are cut).  Returns whether every sum is
+    // 2^47 units per particle or more, which makes that 2^-45 of it, the accuracy of
+    // double-float products.
+    __device__ __forceinline__ bool corners(u64 c[8], int unit) const {
         c[7] = m[6];
         c[3] = m[3] - m[6];
         c[5] = m[4] - m[6];
@@ -217,54 +242,72 @@ struct Moments {
         c[1] = m[0] - m[3] - c[5];
         c[2] = m[1] - m[3] - c[6];
         c[4] = m[2] - m[4] - c[6];
-        c[0] = ((u64)n << 54) - m[0] - c[2] - c[4] - c[6];
+        c[0] = ((u64)n << unit) - m[0] - c[2] - c[4] - c[6];
+        int least = (int)(c[0] >> 32);
 #pragma unroll
-        for (int e = 0; e < 7; ++e)
-            if ((long long)c[e] < 0) c[e] = 0;
+        for (int e = 1; e < 8; ++e) least = min(least, (int)(c[e] >> 32));
+        return least >= (int)(n << 15);
     }
 };
 
-// The nearest binary64 value of an integer below 2^63 (integer instructions;
-// the FP64 unit's conversion takes several of its slots).
-__device__ __forceinline__ double to_f64(u64 c) {
+// The nearest binary64 value of c 2^-unit (integer instructions; the FP64 unit's
+// conversion takes several of its slots).
+__device__ __forceinline__ double to_f64(u64 c, int unit) {
     const int lz = __clzll((long long)c);
     const u64 m = c << (lz & 63);
-    const u64 bits = ((u64)(1085 - lz) << 52) + (m >> 11) + ((m >> 10) & 1u);
+    const u64 bits = ((u64)(unsigned)(1085 - unit - lz) << 52) + (m >> 11) + ((m >> 10) & 1u);
     return c ? __longlong_as_double((long long)bits) : 0.0;
 }
 
 // Add four corner sums to the nodes at radius index nri around cell (ia, iz):
 // (alpha, z) = (0, 0), (1, 0), (0, 1), (1, 1).
 template <bool V2D>
-__device__ __forceinline__ void add4(const DepositArgs &a, const double *inv_v2, int nri, int ia, int iz, u64 c00,
+__device__ __forceinline__ void add4(const DepositArgs &a, const double *inv_v2, int unit, int nri, int ia, int iz, u64 c00,
                                      u64 c10, u64 c01, u64 c11) {
     const int ja = ia + 1 == a.nt ? 0 : ia + 1;
     const size_t rs = (size_t)a.nr + 1, ps = (size_t)a.nt * rs;
     double f0, f1;
     if (V2D) {   // composite domain: node volumes of active octants
-        f0 = a.wscale * inv_v2[(size_t)iz * rs + nri];
-        f1 = a.wscale * inv_v2[(size_t)(iz + 1) * rs + nri];
+        f0 = a.weight * inv_v2[(size_t)iz * rs + nri];
+        f1 = a.weight * inv_v2[(size_t)(iz + 1) * rs + nri];
     } else {
-        const double fr = a.wscale * a.inv_vr[nri];
+        const double fr = a.weight * a.inv_vr[nri];
         f0 = fr * a.inv_vz[iz];
         f1 = fr * a.inv_vz[iz + 1];
     }
     double *p = a.nodes + (size_t)iz * ps + nri;
-    atomicAdd(p + (size_t)ia * rs, to_f64(c00) * f0);
-    atomicAdd(p + (size_t)ja * rs, to_f64(c10) * f0);
-    atomicAdd(p + ps + (size_t)ia * rs, to_f64(c01) * f1);
-    atomicAdd(p + ps + (size_t)ja * rs, to_f64(c11) * f1);
+    atomicAdd(p + (size_t)ia * rs, to_f64(c00, unit) * f0);
+    atomicAdd(p + (size_t)ja * rs, to_f64(c10, unit) * f0);
+    atomicAdd(p + ps + (size_t)ia * rs, to_f64(c01, unit) * f1);
+    atomicAdd(p + ps + (size_t)ja * rs, to_f64(c11, unit) * f1);
 }
 
 // FACES: face arrays or a composite domain; V2D: a composite domain.
+//
+// What a run's sums would not hold to 2^-45 goes to the nodes particle by particle
+// in binary64: a run with a corner sum too small for its units, a particle that
+// fix_place leaves to that arithmetic.  The block queues these and works on them
+// together at its end -- an FP64 instruction of a warp holds the unit for 16
+// cycles whether one lane needs it or all.
 template <bool FACES, bool V2D>
-__global__ void __launch_bounds__(DEP_THREADS) k_deposit(const DepositArgs a, const DepositGeo g) {
+__global__ void __launch_bounds__(DEP_THREADS) k_deposit(const __grid_constant__ DepositArgs a, const __grid_constant__ DepositGeo g) {
     constexpr int W = DEP_THREADS / 32;
     __shared__ long long s_first[W], s_last[W];   // labels of each warp's first and last lane
     __shared__ u64 s_hi[W][4];                    // outer corners of its last run
-    const long long t0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * DEP_PPT;
+    __shared__ unsigned short s_queue[DEP_THREADS * DEP_PPT];
+    __shared__ int s_queued;
+    const long long b0 = (long long)blockIdx.x * (DEP_THREADS * DEP_PPT), t0 = b0 + (int)threadIdx.x * DEP_PPT;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned full = 0xffffffffu;
+    if (threadIdx.x == 0) s_queued = 0;
+    __syncthreads();
+    auto queue = [&](unsigned mask) {             // of the thread's particles; a particle once
+        while (mask) {
+            const int t = __ffs((int)mask) - 1;
+            mask &= mask - 1;
+            s_queue[atomicAdd(&s_queued, 1)] = (unsigned short)(threadIdx.x * DEP_PPT + t);
+        }
+    };
     double pr[DEP_PPT], pa[DEP_PPT], pz[DEP_PPT];
     const int have_p = (int)min((long long)DEP_PPT, max(0ll, a.np - t0));
     if (a.vec && have_p == DEP_PPT) {
@@ -283,44 +326,71 @@ __global__ void __launch_bounds__(DEP_THREADS) k_deposit(const DepositArgs a, co
     Moments M;
     M.clear();
     int cr = 0, ca = 0, cz = 0;
-    bool have = false;
+    unsigned mine = 0, lone = 0;                  // particles of the current run, of the queue
     u64 c[8];
 #pragma unroll
     for (int t = 0; t < DEP_PPT; ++t) {
         Place q;
         if (t >= have_p) continue;
-        if (!(FACES ? place_faces(a, g, pr[t], pa[t], pz[t], q) : place(a, pr[t], pa[t], pz[t], q))) continue;
-        if (have && (q.ir != cr || q.ia != ca || q.iz != cz)) {   // the finished run straight to the nodes
-            M.corners(c);
-            add4<V2D>(a, g.inv_v2, cr, ca, cz, c[0], c[2], c[4], c[6]);
-            add4<V2D>(a, g.inv_v2, cr + 1, ca, cz, c[1], c[3], c[5], c[7]);
+        if constexpr (FACES) {
+            Spot s;
+            if (!locate_faces(a, g, pr[t], pa[t], pz[t], s)) continue;
+            q = {s.ir, s.ia, s.iz, frac64(s.x), frac64(s.y), frac64(s.z)};
+        } else if (!(fix_place(a.fr, pr[t], q.ir, q.x) & fix_place(a.fa, pa[t], q.ia, q.y) &
+                     fix_place(a.fz, pz[t], q.iz, q.z))) {
+            lone |= 1u << t;
+            continue;
+        }
+        if (mine && (q.ir != cr || q.ia != ca || q.iz != cz)) {   // the finished run straight to the nodes
+            if (M.corners(c, DEP_UNIT)) {
+                add4<V2D>(a, g.inv_v2, DEP_UNIT, cr, ca, cz, c[0], c[2], c[4], c[6]);
+                add4<V2D>(a, g.inv_v2, DEP_UNIT, cr + 1, ca, cz, c[1], c[3], c[5], c[7]);
+            } else {
+                lone |= mine;
+            }
             M.clear();
+            mine = 0;
         }
         cr = q.ir;
         ca = q.ia;
         cz = q.iz;
-        have = true;
+        mine |= 1u << t;
         M.add(q);
     }
     // runs of lanes with the same last cell (lanes with nothing left: a run each)
-    const long long label = have ? ((long long)cz * a.nt + ca) * a.nr + cr : -1 - lane;
-    const long long prev = __shfl_up_sync(full, label, 1), next = __shfl_down_sync(full, label, 1);
-    const unsigned heads = __ballot_sync(full, lane == 0 || prev != label);
+    const long long cell = mine ? ((long long)cz * a.nt + ca) * a.nr + cr : -1 - lane;
+    const long long prev = __shfl_up_sync(full, cell, 1);
+    const unsigned heads = __ballot_sync(full, lane == 0 || prev != cell);
     const unsigned upto = lane == 31 ? full : ((2u << lane) - 1u);
-    const int start = 31 - __clz(heads & upto);   // first lane of this lane's run
-    for (int off = 1; __any_sync(full, lane - off >= start); off <<= 1) {
-        const bool in = lane - off >= start;
-        const unsigned yn = __shfl_up_sync(full, M.n, off);
-        if (in) M.n += yn;
+    const int start = 31 - __clz(heads & upto);   // first and last lane of this lane's run
+    const int end = (heads & ~upto) ? __ffs((int)(heads & ~upto)) - 2 : 31;
+    const bool wide = heads != full;              // (the same for the whole warp)
+    const int unit = wide ? DEP_WIDE : DEP_UNIT;
+    if (wide) {
 #pragma unroll
-        for (int e = 0; e < 7; ++e) {
-            const u64 y = __shfl_up_sync(full, M.m[e], off);
-            if (in) M.m[e] += y;
+        for (int e = 0; e < 7; ++e) M.m[e] >>= DEP_UNIT - DEP_WIDE;
+        for (int off = 1; __any_sync(full, lane - off >= start); off <<= 1) {
+            const bool in = lane - off >= start;
+            const unsigned yn = __shfl_up_sync(full, M.n, off);
+            if (in) M.n += yn;
+#pragma unroll
+            for (int e = 0; e < 7; ++e) {
+                const u64 y = __shfl_up_sync(full, M.m[e], off);
+                if (in) M.m[e] += y;
+            }
         }
     }
-    M.corners(c);
+    const bool small = !M.corners(c, unit);
+    if (__shfl_sync(full, small, end)) {          // (the run's sums are those of its last lane)
+        lone |= mine;
+        mine = 0;
+    }
+    if (lone) queue(lone);
     // the outer corners of the run before go to this run when its cell is the
-    // radial neighbour; the warps' ends meet through shared memory
+    // radial neighbour (and its units are the same); the warps' ends meet through
+    // shared memory
+    const long long label = mine ? 2 * cell + (wide ? 1 : 0) : -2 - lane;
+    const long long next = __shfl_down_sync(full, label, 1);
     if (lane == 0) s_first[warp] = label;
     if (lane == 31) {
         s_last[warp] = label;
@@ -338,15 +408,16 @@ __global__ void __launch_bounds__(DEP_THREADS) k_deposit(const DepositArgs a, co
 #pragma unroll
         for (int e = 0; e < 4; ++e) hi[e] = s_hi[warp > 0 ? warp - 1 : 0][e];
     }
-    const bool last = lane == 31 || ((heads >> (lane + 1)) & 1u);
-    if (!(have && last)) return;
-    if (pl >= 0 && pl + 1 == label && cr > 0) {
+    if (mine && lane == end) {
+        if (pl >= 0 && pl + 2 == label && cr > 0) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) c[2 * e] += hi[e];
+            for (int e = 0; e < 4; ++e) c[2 * e] += hi[e];
+        }
+        add4<V2D>(a, g.inv_v2, unit, cr, ca, cz, c[0], c[2], c[4], c[6]);
+        const long long nl = lane < 31 ? next : (warp + 1 < W ? s_first[warp + 1] : -1);
+        if (!(nl == label + 2 && cr + 1 < a.nr)) add4<V2D>(a, g.inv_v2, unit, cr + 1, ca, cz, c[1], c[3], c[5], c[7]);
     }
-    add4<V2D>(a, g.inv_v2, cr, ca, cz, c[0], c[2], c[4], c[6]);
-    const long long nl = lane < 31 ? next : (warp + 1 < W ? s_first[warp + 1] : -1);
-    if (!(nl == label + 1 && cr + 1 < a.nr)) add4<V2D>(a, g.inv_v2, cr + 1, ca, cz, c[1], c[3], c[5], c[7]);
+    for (int e = threadIdx.x; e < s_queued; e += DEP_THREADS) stray<FACES, V2D>(a, g, b0 + s_queue[e]);
 }
 
 // The fixed-point form of a uniform axis of n cells over [lo, hi).
@@ -356,6 +427,7 @@ FixAxis fix_axis(double lo, double hi, int n) {
     std::frexp(std::max(std::fabs(lo), std::fabs(hi)), &E);
     a.e1 = E + 1023;
     a.base = (long long)std::ldexp(lo, 62 - E);   // (cut where lo has bits below 2^(E - 62))
+    a.smax = std::ldexp((double)a.base, E - 62) == lo ? 10 : 0;
     a.span = (u64)((long long)std::ldexp(hi, 62 - E) - a.base);
     a.sh = 0;
     while (a.span && !((a.span << a.sh) >> 62)) ++a.sh;    // span 2^sh in [2^62, 2^63)
@@ -456,7 +528,7 @@ extern "C" int pic_poisson_deposit(pic_poisson_plan_t plan, const double *r_dev,
     a.inv_dr = 1.0 / h.dr;
     a.inv_da = q.d.ntheta / q.d.theta_span;
     a.inv_dz = 1.0 / h.dz;
-    a.wscale = std::ldexp(weight, -54);
+    a.weight = weight;
     a.vec = ((reinterpret_cast<uintptr_t>(r_dev) | reinterpret_cast<uintptr_t>(alpha_dev) |
               reinterpret_cast<uintptr_t>(z_dev)) & 15) == 0;
     a.r = r_dev;
