@@ -100,8 +100,10 @@ template <class T> __device__ __forceinline__ void stage_view(LevelDev<T> *dst, 
         reinterpret_cast<unsigned long long *>(dst)[w] = reinterpret_cast<const unsigned long long *>(src)[w];
 }
 
-// b - A_m u at entry (k, i, m), Eq. matrix_free_mode_operator.
-template <class T, bool MASK, bool INT = false>
+// b - A_m u at entry (k, i, m), Eq. matrix_free_mode_operator.  FX: binary64
+// levels with limb tables compute the imaginary part in fixed point, which takes
+// values of 2^-863 to 2^977 (the norms of a solve hold less); else both parts in T.
+template <class T, bool MASK, bool FX, bool INT = false>
 __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i, int m, size_t idx) {
     const size_t rowstride = (size_t)L.nr * L.nm;
     if (MASK && L.rcls) {
@@ -113,7 +115,7 @@ __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i,
         // a cell outside a composite domain's patches (zero diagonal) has no
         // residual: nothing else is loaded for it
         if (d == T(0)) return mk<T>(0, 0);
-        if constexpr (sizeof(T) == sizeof(double)) {
+        if constexpr (FX && sizeof(T) == sizeof(double)) {
             if (L.ren) {   // real part on the FP64 unit, imaginary part in fixed point
                 const V2<T> zero = mk<T>(0, 0), *u = L.u + idx;
                 const V2<T> us = k > 0 ? *(u - rowstride) : zero, un = k < L.nz - 1 ? u[rowstride] : zero;
@@ -131,7 +133,7 @@ __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i,
         if (i < L.nr - 1) acc = fma2<T>(L.cce[ci], L.u[idx + L.nm], acc);
         return fma2<T>(-d, L.u[idx], acc);
     }
-    if constexpr (sizeof(T) == sizeof(double)) {
+    if constexpr (FX && sizeof(T) == sizeof(double)) {
         if (L.rzw) {   // real part on the FP64 unit, imaginary part in fixed point (fixed.h)
             const unsigned rs = (unsigned)L.nr * (unsigned)L.nm;
             const V2<T> zero = mk<T>(0, 0), *u = L.u + idx;
@@ -456,11 +458,11 @@ __device__ __forceinline__ double restrict_body(const LevelDev<T> &F, const Leve
         };
         int k, i;
         cell(0, k, i);
-        V2<T> sum = residual_at<T, MASK, true>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
+        V2<T> sum = residual_at<T, MASK, true, true>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
         if (partials) acc = fma((double)sum.y, (double)sum.y, (double)sum.x * (double)sum.x);
         auto more = [&](int c) {
             cell(c, k, i);
-            const V2<T> r = residual_at<T, MASK, true>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
+            const V2<T> r = residual_at<T, MASK, true, true>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
             sum = mk<T>(sum.x + r.x, sum.y + r.y);
             if (partials) acc = fma((double)r.y, (double)r.y, fma((double)r.x, (double)r.x, acc));
         };
@@ -517,7 +519,7 @@ k_residual_restrict(const __grid_constant__ LevelArg<T> arg, double *__restrict_
 
 // r = b - A_m u on level f (r written to c.u when write_r), Parseval-weighted
 // squared norms of r into partials[block] and, when stride > 0, of b into
-// partials[stride + block].
+// partials[stride + block].  The stage call's kernel: both parts in T, over its whole range.
 template <class T, bool MASK>
 __global__ void __launch_bounds__(MG_THREADS)
 k_residual(const LaunchTab<T> *__restrict__ tab, int write_r, double *__restrict__ partials, unsigned stride) {
@@ -533,7 +535,7 @@ k_residual(const LaunchTab<T> *__restrict__ tab, int write_r, double *__restrict
         const int m = (int)(e - c * nm);
         const int k = (int)fdiv(c, (unsigned)L.nr, L.rnr);
         const int i = (int)(c - (unsigned)k * L.nr);
-        const V2<T> r = residual_at<T, MASK>(L, k, i, m, e);
+        const V2<T> r = residual_at<T, MASK, false>(L, k, i, m, e);
         if (write_r) tab->c[p].u[e] = r;
         const V2<T> b = L.b[e];
         const double w = parseval_w(m, L.nt);
@@ -743,7 +745,7 @@ k_defect(const DefectTab *__restrict__ tab, const Ctrl *__restrict__ ctrl, doubl
             r = D.b[e];
             D.u[e] = make_double2(0.0, 0.0);
         } else {
-            r = residual_at<double, MASK>(D, k, i, m, e);
+            r = residual_at<double, MASK, true>(D, k, i, m, e);
         }
         const float2 b32 = make_float2(f64_to_f32_pow2(r.x, ls), f64_to_f32_pow2(r.y, ls));
         const float w = (m == 0 || 2 * m == D.nt) ? 1.f : 2.f;
