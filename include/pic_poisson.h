@@ -417,7 +417,8 @@ int pic_poisson_face_field(pic_poisson_plan_t plan, const double *phi_dev, doubl
  * Step a-1 alone: bhat_dev (mode layout) = s * rho_hat + b^D delta_m0 where
  * rho_hat is the forward DFT of rho_dev along theta with scale 1/N_theta
  * (Eqs. azimuthal_dft, mode_rhs).  Imaginary parts of m = 0 and m = N/2 are
- * written as exactly 0.
+ * written as exactly 0.  An infinity or a NaN in rho makes every mode of its
+ * (r, z) cell NaN (likewise pic_poisson_analyze and, for phi, pic_poisson_inverse).
  */
 int pic_poisson_forward(pic_poisson_plan_t plan, const double *rho_dev, double *bhat_dev);
 

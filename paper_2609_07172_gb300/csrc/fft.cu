@@ -32,7 +32,8 @@
 // values held in registers, halving the shared-memory round trips and barriers;
 // the unpack (pack) of the real transform treats modes m and M - m together,
 // sharing one twiddle product.  A column that holds an infinity or a NaN comes
-// out as NaN.
+// out as NaN; one of values near or below the normal range is scaled up first, and
+// results below it are rounded to subnormals.
 // The modes take the place of the transform's rows (X_M a row of its own), so
 // that 256 points need 68 KB of shared memory and not 133, three blocks per SM
 // instead of one: 128 x 256 x 96 forward 81 -> 52 us, and a batch's largest problem
@@ -49,6 +50,26 @@ namespace {
 constexpr int TI = FFT_TI;
 constexpr int LD = TI + 1;   // padded row of the transform buffer (conflict-free 16-byte lanes)
 constexpr int NW = FFT_THREADS / 32;
+// A column whose largest exponent field is below SMALL is scaled by 2^UP first (by
+// integers: a column of zeros comes here too): beside larger values a subnormal is
+// less than a unit of the column, so that the conversions take it for 0.
+constexpr int SMALL = 64, UP = 128;
+__device__ __noinline__ double2 scaled_up(double2 v) {
+    double *x = &v.x;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const ufx b = (ufx)__double_as_longlong(x[i]), m = b & ~(1ull << 63);
+        if (m == 0) continue;
+        const int lz = __clzll((fx)m) - 11;      // of a subnormal: to bit 52
+        const ufx r = m >> 52 ? b + ((ufx)UP << 52) : ((m << (lz & 63)) & ~(1ull << 52)) + ((ufx)(UP + 1 - lz) << 52) + (b & (1ull << 63));
+        x[i] = __longlong_as_double((fx)r);
+    }
+    return v;
+}
+__device__ __forceinline__ void scale_up(double2 *e) {
+    const double2 v = *e;
+    if (((ufx)__double_as_longlong(v.x) | (ufx)__double_as_longlong(v.y)) << 1) *e = scaled_up(v);
+}
 
 template <int LG> __device__ __forceinline__ int bitrev(int n) {
     return LG == 0 ? 0 : (int)(__brev((unsigned)n) >> (32 - LG));
@@ -253,6 +274,15 @@ __device__ __forceinline__ void forward_body(const FFTProb &P, int lb, double2 *
         buf[bitrev<LG>(n) * LD + lane] = make_double2(a, b);
     }
     em = column_max(em, wmax, lane, warp);
+    int down = 0;
+    if (em < SMALL && valid) {   // (values that may be subnormal: brought into the normal range)
+        for (int n = warp; n < M; n += NW) {
+            double2 *e = buf + bitrev<LG>(n) * LD + lane;
+            scale_up(e);
+        }
+        down = UP;
+        em = max(em, 1) + UP;
+    }
     unsigned mag = 0;
 #pragma unroll 4
     for (int n = warp; n < M; n += NW) {   // (a thread's own entries: no barrier between these passes)
@@ -281,10 +311,9 @@ __device__ __forceinline__ void forward_body(const FFTProb &P, int lb, double2 *
     const size_t si = valid ? (P.s_rows ? (size_t)k * nr + i : (size_t)i) : 0;
     const double hs = (P.s ? P.s[si] : 1.0) * P.half_inv_n;
     const fx hm = f64_exp(hs) ? (hs < 0.0 ? -(fx)f64_mant(hs) : (fx)f64_mant(hs)) : 0;
-    const int be = em + bl - 18 + f64_exp(hs) - 1021;     // biased exponent of r hm = 2^63 2^64
-    const bool bad = em == 0x7ff;
-    const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    auto out = [&](fx r, int e) { return bad ? nan : fx_to_f64(__mul64hi(r, hm), e); };
+    const int be = em == 0x7ff ? FX_NAN : em - down + bl - 18 + f64_exp(hs) - 1021;   // biased exponent of r hm = 2^63 2^64
+    const bool rare = fx_rare(be);
+    auto out = [&](fx r, int e) { return fx_to_f64(__mul64hi(r, hm), e, rare); };
     double acc_in = 0.0, acc_edge = 0.0;   // Parseval weight 2 (0 < m < M) and 1 (m = 0, M)
     double2 *ob = buf + lane;
     for (int m = 1 + warp; 2 * m < M; m += NW) {
@@ -361,6 +390,15 @@ __device__ __forceinline__ void inverse_body(const FFTProb &P, int lb, double2 *
         em = max(em, max(f64_exp(x.x), m == 0 || m == M ? 0 : f64_exp(x.y)));
     }
     em = column_max(em, wmax, lane, warp);
+    int down = 0;
+    if (em < SMALL && valid) {   // (as in the forward transform; column_bits has a barrier)
+        for (int m = warp; m <= M; m += NW) {
+            double2 *e = buf + row(m) + lane;
+            scale_up(e);
+        }
+        down = UP;
+        em = max(em, 1) + UP;
+    }
     unsigned mag = 0;
     for (int m = warp; m <= M; m += NW) {
         const double2 x = ib[row(m)];
@@ -397,15 +435,14 @@ __device__ __forceinline__ void inverse_body(const FFTProb &P, int lb, double2 *
     fft_stages<true, LG>(buf, P.tw, lane, warp);
 
     if (valid) {
-        const int be = em + bl - 16;
-        const bool bad = em == 0x7ff;
-        const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        const int be = em == 0x7ff ? FX_NAN : em - down + bl - 16;
+        const bool rare = fx_rare(be);
         double *dst = P.phi + (size_t)k * nt * nr + i;
-    #pragma unroll 4
-    for (int n = warp; n < M; n += NW) {
+#pragma unroll 4
+        for (int n = warp; n < M; n += NW) {
             const ci z = ld(buf + n * LD + lane);
-            dst[(size_t)(2 * n) * nr] = bad ? nan : fx_to_f64(z.x, be);
-            dst[(size_t)(2 * n + 1) * nr] = bad ? nan : fx_to_f64(z.y, be);
+            dst[(size_t)(2 * n) * nr] = fx_to_f64(z.x, be, rare);
+            dst[(size_t)(2 * n + 1) * nr] = fx_to_f64(z.y, be, rare);
         }
     }
 }

@@ -33,18 +33,31 @@ __device__ __forceinline__ fx f64_to_fx(double x, int s) {
 }
 
 // The nearest binary64 value of r 2^(be - 1086) (be: the biased exponent that
-// |r| = 2^63 would get); |r| <= 2^63.  Results below the normal range become
-// signed zero, above it infinite.
-__device__ __forceinline__ double fx_to_f64(fx r, int be) {
+// |r| = 2^63 would get); |r| <= 2^63.  `rare` (fx_rare of be, the same for a whole
+// column): the result may lie outside the normal range, or be is FX_NAN or more, NaN.
+constexpr int FX_NAN = 1 << 20;
+static __device__ __noinline__ double fx_to_f64_rare(fx r, int be) {
+    const ufx a = r < 0 ? 0ull - (ufx)r : (ufx)r;
+    const int lz = __clzll((fx)a), e = be - lz;
+    const ufx m = a << (lz & 63);
+    ufx bits = ((ufx)(unsigned)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1u);
+    if (e <= 0) bits = e < -52 ? 0 : ((m >> (11 - e)) + 1) >> 1;   // units of 2^-1074
+    if (e >= 0x7ff) bits = 0x7ffull << 52;
+    if (a == 0) bits = 0;
+    if (be >= FX_NAN) bits = 0x7ff8ull << 48;
+    return __longlong_as_double((fx)(bits | (ufx)((unsigned)((ufx)r >> 32) & 0x80000000u) << 32));
+}
+__device__ __forceinline__ bool fx_rare(int be) { return (unsigned)(be - 64) >= 0x7ffu - 65u; }   // be + 1 too
+__device__ __forceinline__ double fx_to_f64(fx r, int be, bool rare) {
     const ufx a = r < 0 ? 0ull - (ufx)r : (ufx)r;
     const int lz = __clzll((fx)a);
     const ufx m = a << (lz & 63);
-    const int e = be - lz;
     const unsigned sign = (unsigned)((ufx)r >> 32) & 0x80000000u;
-    ufx bits = ((ufx)(unsigned)(e - 1) << 52) + (m >> 11) + ((m >> 10) & 1u);
-    if (e >= 0x7ff) bits = 0x7ffull << 52;
-    if (a == 0 || e <= 0) bits = 0;
-    return __longlong_as_double((fx)(bits | (ufx)sign << 32));
+    ufx bits = ((ufx)(unsigned)(be - lz - 1) << 52) + (m >> 11) + ((m >> 10) & 1u);
+    if (a == 0) bits = 0;
+    double v = __longlong_as_double((fx)(bits | (ufx)sign << 32));
+    if (rare && (a != 0 || be >= FX_NAN)) v = fx_to_f64_rare(r, be);
+    return v;
 }
 
 // A constant |c| <= 1 as two 31-bit limbs: c 2^61 = h 2^31 + l, 0 <= l < 2^31.
