@@ -188,16 +188,24 @@ __device__ __forceinline__ bool locate_faces(const DepositArgs &a, const Deposit
     return true;
 }
 
-// One particle's eight weights in binary64 straight to the nodes.
+// One particle's eight weights in binary64 straight to the nodes (21 FP64
+// instructions beside the atomics).
 template <bool V2D> __device__ __forceinline__ void spread(const DepositArgs &a, const double *inv_v2, const Spot &q) {
     const int ja = q.ia + 1 == a.nt ? 0 : q.ia + 1;
     const size_t rs = (size_t)a.nr + 1, ps = (size_t)a.nt * rs;
-#pragma unroll 1
-    for (int c = 0; c < 8; ++c) {
-        const int nzi = q.iz + (c >> 2), nai = (c & 2) ? ja : q.ia, nri = q.ir + (c & 1);
-        const double w = ((c & 4) ? q.z : 1.0 - q.z) * ((c & 2) ? q.y : 1.0 - q.y) * ((c & 1) ? q.x : 1.0 - q.x);
-        const double f = V2D ? a.weight * inv_v2[(size_t)nzi * rs + nri] : a.weight * a.inv_vr[nri] * a.inv_vz[nzi];
-        atomicAdd(a.nodes + (size_t)nzi * ps + (size_t)nai * rs + nri, w * f);
+    const double w0 = 1.0 - q.y, wr[2] = {1.0 - q.x, q.x}, wz[2] = {1.0 - q.z, q.z};
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+        const int nri = q.ir + d;
+        const double f = V2D ? a.weight * wr[d] : a.weight * a.inv_vr[nri] * wr[d];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int nzi = q.iz + e;
+            const double g = f * (V2D ? inv_v2[(size_t)nzi * rs + nri] * wz[e] : a.inv_vz[nzi] * wz[e]);
+            double *p = a.nodes + (size_t)nzi * ps + nri;
+            atomicAdd(p + (size_t)q.ia * rs, g * w0);
+            atomicAdd(p + (size_t)ja * rs, g * q.y);
+        }
     }
 }
 // Particle p by itself.
@@ -207,9 +215,10 @@ template <bool FACES, bool V2D> __device__ __noinline__ void stray(const Deposit
 }
 
 // Moments of a cell's particles, the count apart.  A thread's (at most four) are in
-// units of 2^-61; where runs cross lanes a warp's (at most 128) are cut to 2^-56.
-// Every sum stays below 2^63, two runs' below 2^64.
-constexpr int DEP_UNIT = 61, DEP_WIDE = 56;
+// units of 2^-61; in a warp with a run over more than one lane all are cut to as many
+// bits fewer as the longest run's sum needs.  Every sum stays below 2^63, two runs'
+// below 2^64.
+constexpr int DEP_UNIT = 61;
 struct Moments {
     unsigned n;
     u64 m[7];   // x, y, z, xy, xz, yz, xyz
@@ -364,12 +373,13 @@ __global__ void __launch_bounds__(DEP_THREADS) k_deposit(const __grid_constant__
     const unsigned upto = lane == 31 ? full : ((2u << lane) - 1u);
     const int start = 31 - __clz(heads & upto);   // first and last lane of this lane's run
     const int end = (heads & ~upto) ? __ffs((int)(heads & ~upto)) - 2 : 31;
-    const bool wide = heads != full;              // (the same for the whole warp)
-    const int unit = wide ? DEP_WIDE : DEP_UNIT;
-    if (wide) {
+    int unit = DEP_UNIT;                          // (the same for the whole warp)
+    if (heads != full) {
+        const int longest = (int)__reduce_max_sync(full, (unsigned)(lane - start)), cut = 32 - __clz(longest);
+        unit -= cut;
 #pragma unroll
-        for (int e = 0; e < 7; ++e) M.m[e] >>= DEP_UNIT - DEP_WIDE;
-        for (int off = 1; __any_sync(full, lane - off >= start); off <<= 1) {
+        for (int e = 0; e < 7; ++e) M.m[e] >>= cut;
+        for (int off = 1; off <= longest; off <<= 1) {
             const bool in = lane - off >= start;
             const unsigned yn = __shfl_up_sync(full, M.n, off);
             if (in) M.n += yn;
@@ -389,7 +399,7 @@ __global__ void __launch_bounds__(DEP_THREADS) k_deposit(const __grid_constant__
     // the outer corners of the run before go to this run when its cell is the
     // radial neighbour (and its units are the same); the warps' ends meet through
     // shared memory
-    const long long label = mine ? 2 * cell + (wide ? 1 : 0) : -2 - lane;
+    const long long label = mine ? 64 * cell + unit : -2 - lane;
     const long long next = __shfl_down_sync(full, label, 1);
     if (lane == 0) s_first[warp] = label;
     if (lane == 31) {
@@ -409,13 +419,13 @@ __global__ void __launch_bounds__(DEP_THREADS) k_deposit(const __grid_constant__
         for (int e = 0; e < 4; ++e) hi[e] = s_hi[warp > 0 ? warp - 1 : 0][e];
     }
     if (mine && lane == end) {
-        if (pl >= 0 && pl + 2 == label && cr > 0) {
+        if (pl >= 0 && pl + 64 == label && cr > 0) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) c[2 * e] += hi[e];
         }
         add4<V2D>(a, g.inv_v2, unit, cr, ca, cz, c[0], c[2], c[4], c[6]);
         const long long nl = lane < 31 ? next : (warp + 1 < W ? s_first[warp + 1] : -1);
-        if (!(nl == label + 2 && cr + 1 < a.nr)) add4<V2D>(a, g.inv_v2, unit, cr + 1, ca, cz, c[1], c[3], c[5], c[7]);
+        if (!(nl == label + 64 && cr + 1 < a.nr)) add4<V2D>(a, g.inv_v2, unit, cr + 1, ca, cz, c[1], c[3], c[5], c[7]);
     }
     for (int e = threadIdx.x; e < s_queued; e += DEP_THREADS) stray<FACES, V2D>(a, g, b0 + s_queue[e]);
 }
