@@ -191,12 +191,37 @@ __global__ void __launch_bounds__(WG_WARPS * 32, 2) k_wgrad_mma(const WgradArgs 
         a.partb[(size_t)blockIdx.x * a.cout + co0 + threadIdx.x] = red[9 * 256 + threadIdx.x];
 }
 
+// Weight e's sum over the pixels of rows [row0, row1) of all images, by scalar FMAs:
+// only products of pixels inside the image and gradients that are not zero.
+__device__ __noinline__ float wgrad_scalar(const WgradArgs &a, int e, long row0, long row1) {
+    const int ci = e % a.cin, co = e / a.cin % a.cout, tap = e / a.cin / a.cout;
+    float s = 0.f;
+    for (long r = row0; r < row1; ++r) {
+        const long img = r / a.h * a.h;
+        const int y = (int)(r - img) + tap / 3 - 1;
+        if ((unsigned)y >= (unsigned)a.h) continue;
+        for (int x0 = 0; x0 < a.wd; ++x0) {
+            const float g = __bfloat162float(a.dout[(r * a.wd + x0) * a.cout + co]);
+            const int x = x0 + tap % 3 - 1;
+            if (g == 0.f || (unsigned)x >= (unsigned)a.wd) continue;
+            const bf16 *v = ci < a.cu ? a.up + (((img >> 1) + (y >> 1)) * (a.wd >> 1) + (x >> 1)) * a.cu + ci
+                                      : a.in + ((img + y) * a.wd + x) * (a.cin - a.cu) + (ci - a.cu);
+            s = fmaf(g, __bfloat162float(*v), s);
+        }
+    }
+    return s;
+}
+
 // Sum of the CTAs' partials: 32 outputs per block, each summed by eight
-// threads over eighths of the partials, then those eight in order.
-__global__ void __launch_bounds__(256) k_wgrad_reduce_split(const float *__restrict__ part, const float *__restrict__ partb,
-                                                            int parts, int nw, int cout, float *__restrict__ dw,
+// threads over eighths of the partials, then those eight in order.  The MMAs also
+// multiply the zeros around the images and gradients that are zero; where the other
+// factor is infinite or NaN that gives NaN, so a weight whose sum is not finite is
+// summed again without them (a diverged step: every weight takes the scalar loop).
+__global__ void __launch_bounds__(256) k_wgrad_reduce_split(const __grid_constant__ WgradArgs a, int parts, float *__restrict__ dw,
                                                             float *__restrict__ db) {
     __shared__ float red[8][32];
+    const float *__restrict__ part = a.part, *__restrict__ partb = a.partb;
+    const int nw = 9 * a.cout * a.cin, cout = a.cout;
     const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
     const int e = (int)blockIdx.x * 32 + lane;   // weights, then biases
     const int eighth = (parts + 7) / 8, c0 = seg * eighth, c1 = min(parts, c0 + eighth);
@@ -208,8 +233,18 @@ __global__ void __launch_bounds__(256) k_wgrad_reduce_split(const float *__restr
     }
     red[seg][lane] = s;
     __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s = k ? s + red[k][lane] : red[0][lane];   // (every segment the same sum)
+    const bool again = e < nw && !isfinite(s);
+    if (__any_sync(0xffffffffu, again)) {   // (the same in the block's eight warps)
+        __syncthreads();
+        const long rows = (long)a.n * a.h, eighth_r = (rows + 7) / 8;
+        if (again) red[seg][lane] = wgrad_scalar(a, e, min(rows, seg * eighth_r), min(rows, (seg + 1) * eighth_r));
+        __syncthreads();
+        if (again)
+            for (int k = 0; k < 8; ++k) s = k ? s + red[k][lane] : red[0][lane];
+    }
     if (seg == 0) {
-        for (int k = 1; k < 8; ++k) s += red[k][lane];
         if (e < nw) dw[e] = s;
         else if (db && e - nw < cout) db[e - nw] = s;
     }
@@ -258,7 +293,7 @@ cudaError_t launch_wgrad_mma(const void *up, int cu, const void *in, int cin, co
     cudaError_t e = cudaFuncSetAttribute(k_wgrad_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     k_wgrad_mma<<<dim3((unsigned)used, (unsigned)blocks), WG_WARPS * 32, smem, st>>>(a);
-    k_wgrad_reduce_split<<<(unsigned)((nw + cout + 31) / 32), 256, 0, st>>>(a.part, a.partb, used, nw, cout, dw, dbias);
+    k_wgrad_reduce_split<<<(unsigned)((nw + cout + 31) / 32), 256, 0, st>>>(a, used, dw, dbias);
     return cudaGetLastError();
 }
 
