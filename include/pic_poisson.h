@@ -163,6 +163,9 @@ typedef struct {
     int launches_phase[PIC_POISSON_NPHASE];/* launches per kernel class */
     double bytes_phase[PIC_POISSON_NPHASE];/* algorithmic (compulsory) DRAM bytes per kernel class */
     double flops_phase[PIC_POISSON_NPHASE];/* algorithmic floating-point operations per kernel class */
+    /* V-cycles that run inside one launch (local_bottom = 0) are booked with it, all four of the above:
+       a small problem's as SMOOTH, another's lower levels as COARSE.  Their bytes are those of the
+       first level; the levels stay on the chip. */
 } pic_poisson_info;
 
 #define PIC_POISSON_MAX_TUNE 96

@@ -77,6 +77,7 @@ template <class T> struct Hier {
 // Algorithmic traffic / arithmetic / launches recorded per kernel class.
 struct Tally {
     double bytes[PIC_POISSON_NPHASE] = {0}, flops[PIC_POISSON_NPHASE] = {0};
+    double flops_cycle[PIC_POISSON_NPHASE] = {0};   // per cycle of a solve whose loop is inside a launch
     int launches[PIC_POISSON_NPHASE] = {0};
 };
 

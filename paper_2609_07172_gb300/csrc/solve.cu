@@ -222,35 +222,54 @@ int coarse_and_bottom(Runner &R, const Hier<T> &H) {
     return PIC_POISSON_OK;
 }
 
-// Complex entries of level l of a plan of one problem, and of its smoothed levels from l on.
-double deep_entries(const pic_poisson_plan_s &P, int l, double *below) {
+// Arithmetic of the V-cycles in shared memory (deep.cu) by the models above, of a
+// plan of one problem.  half: half-sweeps on level l.
+struct DeepWork {
+    const pic_poisson_plan_s &P;
     const ProblemPlan &q = P.pr[0];
-    *below = 0;
-    for (int d = l; d + 1 < q.L; ++d) *below += (double)q.lv[d].nr * q.lv[d].nz * q.nm;
-    return (double)q.lv[l].nr * q.lv[l].nz * q.nm;
-}
+    const int nl = q.L - 1, pre = P.shared.pre_sweeps, post = P.shared.post_sweeps;
+    double n(int l) const { return (double)q.lv[l].nr * q.lv[l].nz * q.nm; }
+    double halves(int l, int half) const { return 7.0 * half * n(l); }
+    double restriction(int l, bool norm) const { return n(l) * ((pre > 0 ? 0.5 : 1.0) * (norm ? 22.0 : 18.0) + 1.0); }
+    double prolongation(int l, bool black) const { return n(l) * (black ? 8.0 : 16.0); }
+    double coarse() const { return n(nl) * (4.0 * q.lv[nl].nz + 12.0); }
+    // from level l down and back up; skip: its first red half-sweep was done
+    double cycle(int l, bool skip) const {
+        double f = coarse();
+        for (int d = l; d < nl; ++d)
+            f += halves(d, 2 * (pre + post) - ((d > l || skip) && pre > 0 ? 1 : 0)) + restriction(d, false) + prolongation(d, post > 0);
+        return f;
+    }
+    double fmg(bool bottom) const {
+        double f = bottom ? cycle(nl - 1, true) : coarse();
+        for (int l = 0; l < nl; ++l) f += 0.5 * n(l);
+        for (int l = bottom ? nl - 2 : nl - 1; l >= 0; --l) f += prolongation(l, pre > 0) + (l > 0 ? cycle(l, false) : 0.0);
+        return f;
+    }
+};
 // V-cycles from level l down, in shared memory (H.deep): `from_zero` one whose
 // level l holds b and b_hat only, else from the level's iterate.
 template <class T>
 int deep_cycles(Runner &R, const Hier<T> &H, int l, bool from_zero, int cycles) {
     const int ph = l == 0 ? PIC_POISSON_PHASE_SMOOTH : PIC_POISSON_PHASE_COARSE;
-    double below = 0;
-    const double n = deep_entries(R.P, l, &below);
+    const DeepWork W{R.P};
     RUN(R, ph, launch_deep(H.deep[l], from_zero, cycles, R.st));
-    R.account(ph, (from_zero ? 3.0 : 4.0) * n * sizeof(V2<T>),
-              cycles * below * (14.0 * (R.P.shared.pre_sweeps + R.P.shared.post_sweeps) + 18.0));
+    R.account(ph, (from_zero ? 3.0 : 4.0) * W.n(l) * sizeof(V2<T>), W.cycle(l, from_zero) + (cycles - 1) * W.cycle(l, false));
     return PIC_POISSON_OK;
 }
 
-// A whole FP64 solve in one launch, the convergence loop included (booked as
-// one pass: the number of cycles is known on the device only).
+// A whole FP64 solve in one launch, the convergence loop included: the levels are
+// read and the iterate written once; a cycle's arithmetic is booked once and counted
+// when the number of cycles is back.
 int deep_solve(Runner &R, int start) {
     pic_poisson_plan_s &P = R.P;
-    double below = 0;
-    const double n = deep_entries(P, 0, &below);
+    const DeepWork W{P};
     RUN(R, PIC_POISSON_PHASE_SMOOTH, launch_deep_solve(P.h64.deep[0], start, P.ctrl, P.partials, R.st));
-    R.account(PIC_POISSON_PHASE_SMOOTH, (start ? 2.5 : 3.5) * n * sizeof(double2),
-              below * (14.0 * (P.shared.pre_sweeps + P.shared.post_sweeps) + 22.0));
+    const double top = W.halves(0, 2 * W.pre) + W.restriction(0, true);   // pre-smoothing, residual and its norm
+    R.account(PIC_POISSON_PHASE_SMOOTH, (start ? 2.5 : 3.5) * W.n(0) * sizeof(double2),
+              top + (start == 2 ? W.fmg(P.h64.deep[0].bottom != 0) : 0.0));
+    R.tally.flops_cycle[PIC_POISSON_PHASE_SMOOTH] +=
+        (W.nl > 1 ? W.cycle(1, true) : W.coarse()) + W.prolongation(0, W.post > 0) + W.halves(0, 2 * W.post) + top;
     return PIC_POISSON_OK;
 }
 
@@ -748,8 +767,10 @@ int solve_batch(pic_poisson_plan_s &P, const double *const *rho, double *const *
             tally.flops[ph] = sg[0].flops[ph] + passes * sg[1].flops[ph] + sg[2].flops[ph] + fp * sg[3].flops[ph];
             tally.launches[ph] =
                 sg[0].launches[ph] + passes * sg[1].launches[ph] + sg[2].launches[ph] + fp * sg[3].launches[ph];
+            tally.flops_cycle[ph] = sg[0].flops_cycle[ph];
         }
     }
+    for (int ph = 0; ph < PIC_POISSON_NPHASE; ++ph) tally.flops[ph] += C.cycles * tally.flops_cycle[ph];
     int worst = PIC_POISSON_OK;
     for (int p = 0; p < P.n; ++p) {
         const int s = C.status[p];
