@@ -102,9 +102,11 @@ template <class T> __device__ void tri_factors(const T *e, const T *piv, const T
         }
 }
 
-// One real part's transforms by a whole block (nr x nz, nz <= 64), mirror-folded.
+// One real part's transforms by a whole block (nr x nz), mirror-folded.
 // Binary64 in fixed point, V then as limbs (CoarseDev::Vl), each column aligned
-// to its largest value: one warp per column, exponents in ecol [nr].
+// to its largest value: one warp per column, exponents in ecol [nr].  A lane takes one
+// mirror pair and two rows, and a sum of 64 products fits FxSum:
+static_assert(kMaxCoarseNz <= 64, "the planner's limit is the transforms'");
 
 // bs [nz][nr] -> ws [nz][lw] = V^T b; bs is overwritten.
 template <class T>

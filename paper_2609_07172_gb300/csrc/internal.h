@@ -473,7 +473,7 @@ template <class T> cudaError_t launch_bottom(const BottomTab<T> *tab, unsigned g
 constexpr int DEEP_THREADS = 512;
 constexpr int DEEP_LEVELS = 8;
 constexpr size_t DEEP_MAX_SMEM = 225 * 1024;
-constexpr int DEEP_MAX_NZ = 64;          // rows of the coarsest level
+constexpr int DEEP_MAX_NZ = kMaxCoarseNz;   // rows of the coarsest level
 constexpr int DEEP_POLLS = 1 << 22;      // default of Ctrl::polls: seconds, where a test's wait takes microseconds
 // Entries (cells x modes) of the first level up to which it takes that way: above,
 // the level kernels fill the chip and are as fast or faster.  Measured (us, with
