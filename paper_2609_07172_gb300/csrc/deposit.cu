@@ -605,7 +605,7 @@ extern "C" int pic_poisson_project(pic_poisson_plan_t plan, const double *nodes_
     a.rho = rho_dev;
     a.act = q.act0;
     const size_t rows = (size_t)((a.nr + 30) / 31) * a.nt;   // of warps
-    a.walk = (int)std::min<size_t>(std::max<size_t>(rows * a.nz / (152 * 64 * 2), 1), PROJ_K);
+    a.walk = (int)std::min<size_t>(std::max<size_t>(rows * a.nz / (kSMs * 64 * 2), 1), PROJ_K);
     const size_t items = rows * ((a.nz + a.walk - 1) / a.walk);
     const unsigned grid = (unsigned)((items + PROJ_WARPS - 1) / PROJ_WARPS);
     if (q.act0) k_project<true><<<grid, PROJ_WARPS * 32, 0, plan->stream>>>(a);

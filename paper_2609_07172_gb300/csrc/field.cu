@@ -200,7 +200,7 @@ extern "C" int pic_poisson_face_field(pic_poisson_plan_t plan, const double *phi
         // planes per block: as many as leave the chip twice the blocks it holds
         const unsigned cols = (unsigned)(((size_t)a.nt * a.nr + 255) / 256);
         // (and no more pieces than the grid's second dimension holds)
-        const int fill = (int)std::min<size_t>(std::max<size_t>((size_t)cols * a.nz / (152 * 8 * 2), 1), 16);
+        const int fill = (int)std::min<size_t>(std::max<size_t>((size_t)cols * a.nz / (kSMs * 8 * 2), 1), 16);
         const int chunk = std::max(fill, (a.nz + 65534) / 65535);
         k_face_field<<<dim3(cols, (unsigned)((a.nz + chunk - 1) / chunk)), 256, 0, plan->stream>>>(a, chunk);
     } else {   // non-uniform axial faces and / or a composite domain

@@ -34,6 +34,7 @@ template <> struct V2t<float> { using type = float2; };
 template <class T> using V2 = typename V2t<T>::type;
 
 constexpr int kMaxBatch = PIC_POISSON_MAX_BATCH;
+constexpr int kSMs = 152;                 // of this GPU: what launches are sized for (any number runs them)
 
 // ------------------------------------------------------------------ one multigrid level
 // Coefficients of A_m on a uniform level (appendix Eqs. interior_face_conductances,
@@ -142,7 +143,7 @@ template <class T> struct LaunchTab {
 // some ten dependent loads, before it has work: it then works on `chunk` pieces,
 // as many as leave the launch four times the blocks that the chip holds.
 inline int batch_chunk(size_t blocks) {
-    const size_t c = blocks / (152 * 6 * 4);
+    const size_t c = blocks / (kSMs * 6 * 4);
     return (int)(c < 1 ? 1 : c > 8 ? 8 : c);
 }
 
@@ -284,7 +285,7 @@ struct PsumTab {
 // of these the views alone give 592, 1,308 and 2,812 us.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-constexpr size_t PDL_MAX_THREADS = size_t(152) * 2048;
+constexpr size_t PDL_MAX_THREADS = size_t(kSMs) * 2048;
 template <class... P, class... A>
 cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchConfig_t c{};

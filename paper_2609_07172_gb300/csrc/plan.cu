@@ -977,7 +977,7 @@ void build_hier(pic_poisson_plan_s &P, Hier<T> &H, Views views, Coarse coarse, c
             }
         H.fres[l] = res;
         // fused smoother blocks per problem: one wave of two blocks per SM
-        const int target = std::max(1, 2 * 152 / std::max(nprob, 1));
+        const int target = std::max(1, 2 * kSMs / std::max(nprob, 1));
         // smoother strip (0: one entry per thread); a strip longer than the
         // level's rows of one parity is cut to the next power of two that fits
         int strip = P.shared.smooth_strip;

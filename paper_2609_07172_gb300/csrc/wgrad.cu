@@ -281,7 +281,7 @@ cudaError_t launch_wgrad_mma(const void *up, int cu, const void *in, int cin, co
     const int blocks = a.tci * ((cout + 15) / 16);
     // two CTAs per SM over all channel blocks, as many times as keep a CTA to WG_CHAIN
     // tiles; no more partials than the scratch holds (one per 2048 pixels)
-    const int fill = (2 * 152 + blocks - 1) / blocks;
+    const int fill = (2 * kSMs + blocks - 1) / blocks;
     const long waves = std::max(1l, ((long)a.tiles + (long)fill * WG_CHAIN - 1) / ((long)fill * WG_CHAIN));
     const int parts = (int)std::max(1l, std::min({(long)max_parts, (long)a.tiles, fill * waves}));
     a.per = (a.tiles + parts - 1) / parts;
