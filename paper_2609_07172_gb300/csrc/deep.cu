@@ -21,9 +21,11 @@
 // Bound by the latency of dependent steps (a half-sweep some 850 cycles in FP64,
 // 290 in FP32, plus the barrier): levels of one cell per thread keep their
 // coefficients in registers, and the level's description is read from shared
-// memory.  Measured with launches / here: 32 x 16 x 32 FP64 496 / 296 us,
-// 90 x 32 x 70 FP64 520 / 320, 152 x 32 x 90 FP64 690 / 640, 64 x 64 x 64 mixed
-// 718 / 348, 128 x 64 x 96 mixed 778 / 470 us.
+// memory.  Solves in one graph, us, by launches only (local_bottom = -1) / with the
+// lower levels here (DEEP_MAX_WHOLE = 0) / as chosen: FP64 32 x 16 x 32 556 / 472 /
+// 302, 90 x 32 x 70 528 / 530 / 342, 128 x 64 x 64 1,011 / 888 / 625, 152 x 32 x 90 (only
+// the lower levels fit) 677 / 628; mixed 64 x 64 x 64 814 / 455 / 346, 128 x 64 x 96 876 /
+// 578 / 467, 96 x 128 x 96 973 / 681 / 517, 192 x 32 x 192 1,182 / 788 / 631 us.
 #include <algorithm>
 
 #include "coarse.h"

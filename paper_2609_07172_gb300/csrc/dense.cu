@@ -23,7 +23,11 @@
 // walk along the contraction: from DENSE_SPLIT cells four groups of a block take
 // every fourth chunk each, and their sums are added in group order (800 cells, 65
 // modes: 26 us less for the two products, a stretched 512 x 128 x 400 solve
-// 9,081 -> 8,770 us; with 150 cells, five chunks, 2 % more for the solve).
+// 9,081 -> 8,770 us).  Whole mixed solves of stretched meshes with 17 and 65 modes,
+// by cells of the coarsest level, time with the split over time without: 165 1.013 and
+// 1.009, 208 0.993 and 0.993, 240 0.979 and 0.979, 323 0.976 and 0.987, 408 0.997 and
+// 0.989, 644 0.971 and 0.918, 800 0.959 and 0.881; FP64 composite domains of 10 to 30
+// active cells 1.011 to 1.028, 120 0.992, 150 1.021, 350 0.991.
 #include "internal.h"
 
 namespace pp {
@@ -33,7 +37,7 @@ constexpr int TR = 32;   // output rows (cells or eigenvectors) per block
 constexpr int TC = 32;   // right-hand sides per block
 constexpr int TK = 32;   // contraction chunk staged in shared memory
 constexpr int DENSE_THREADS = 256;
-constexpr int DENSE_SPLIT = 384;
+constexpr int DENSE_SPLIT = 200;
 
 __device__ __forceinline__ int find_problem(const unsigned *__restrict__ start, int n, unsigned blk) {
     int lo = 0, hi = n;

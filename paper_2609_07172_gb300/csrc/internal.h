@@ -263,7 +263,11 @@ struct Ctrl {
 // block) adds a few dozen numbers instead of tens of thousands -- on one SM
 // the FP64 additions alone took longer than the rest of the test.
 constexpr int PSUM_CHUNK = 2048;
-constexpr unsigned PSUM_MIN = 4096;   // partials below which the test adds them itself
+// Up to PSUM_MIN partials the test adds them itself, which saves the launch of k_psum.  Solves
+// without that launch over solves with it, by partials: FP64 1,000 0.984, 2,100 0.988, 4,200
+// 0.993, 6,200 0.999, 8,300 1.000; mixed 1,600 0.965, 4,200 0.991, 8,300 0.990, 10,400 0.995,
+// 12,500 1.000, 16,600 1.003, 25,000 1.009.
+constexpr unsigned PSUM_MIN = 10000;
 struct PsumTab {
     int n;
     unsigned start[kMaxBatch + 1];    // blocks (chunks) of problem p: [start[p], start[p+1])
@@ -476,13 +480,13 @@ constexpr int DEEP_LEVELS = 8;
 constexpr size_t DEEP_MAX_SMEM = 225 * 1024;
 constexpr int DEEP_MAX_NZ = kMaxCoarseNz;   // rows of the coarsest level
 constexpr int DEEP_POLLS = 1 << 22;      // default of Ctrl::polls: seconds, where a test's wait takes microseconds
-// Entries (cells x modes) of the first level up to which it takes that way: above,
-// the level kernels fill the chip and are as fast or faster.  Measured (us, with
-// launches / in shared memory): whole hierarchies 90 x 32 x 70 FP64 520 / 319,
-// 152 x 32 x 90 FP64 690 / 641, 128 x 64 x 96 mixed 656 / 470, 256 x 32 x 128 mixed
-// 981 / 875; below level 0, 139 k entries 981 / 916, 208 k 5,060 / 5,077, 832 k
-// 5,060 / 5,280 (FP64 9,600 / 10,470).
-constexpr size_t DEEP_MAX_WHOLE = 600000, DEEP_MAX_LOWER = 160000;
+// Entries (cells x modes) of the first level up to which it takes that way.  Whole
+// hierarchies: whatever the shared memory of 8 blocks per mode holds is faster (deep.cu;
+// of 40 sizes of 230 thousand to 2.4 million entries none above 626 thousand fits).
+// Lower levels: above, the level kernels fill the chip and are as fast or faster --
+// solves with launches / in shared memory from a level of 139 k entries 981 / 916 us,
+// 208 k 5,060 / 5,077, 832 k 5,060 / 5,280 (FP64 9,600 / 10,470).
+constexpr size_t DEEP_MAX_WHOLE = 640000, DEEP_MAX_LOWER = 160000;
 template <class T> struct DeepLevel {
     LevelDev<T> L;
     int fz, fr, zmul;             // coarsening to the next level; rows per row of the coarsest level

@@ -1471,8 +1471,7 @@ int upload(pic_poisson_plan_s &P) {
     }
     // two-stage norm reduction: k_psum sums chunks of each problem's partials,
     // the convergence test reads the chunk sums -- or, when there are few, the
-    // partials themselves: a launch costs about 3 us, 4096 additions by one block
-    // about 1 us
+    // partials themselves
     PsumTab ps{};
     ps.n = P.n;
     unsigned total = 0;
