@@ -144,8 +144,8 @@ __device__ __forceinline__ Limbs coef_limbs(int2 c) { return {c.x, c.y & ~127}; 
 // the FP64 unit has more to do besides than the integer pipes (a half-sweep of many
 // waves: 74 us with the unit, 79 without; a restriction 65 and 61; 48 x 16 x 20 in
 // shared memory 282 and 270).
-template <bool INT = false> __device__ __forceinline__ double fx_update(double b, double s, double n, double w, double e, int2 hz, int2 hw,
-                                            int2 he) {
+template <bool INT = false>
+__device__ __forceinline__ double fx_update(double b, double s, double n, double w, double e, int2 hz, int2 hw, int2 he) {
     const int ez = coef_exp(hz), eb = exp_bits(b), es = exp_bits(s) - ez, en = exp_bits(n) - ez;
     const int ew = exp_bits(w) - coef_exp(hw), ee = exp_bits(e) - coef_exp(he);
     const int em = max(max(max(eb, es), max(en, ew)), ee);
@@ -170,8 +170,9 @@ __device__ __forceinline__ double fx_update(double b, double s, double n, double
     return fx_update<INT>(b, s, n, w, e, make_int2(zw.x, zw.y), make_int2(zw.z, zw.w), ev);
 }
 // b + cz (s + n) + cw w + ce e - d u, the coefficients given times 2^q (|q| < 60).
-template <bool INT = false> __device__ __forceinline__ double fx_residual(double b, double s, double n, double w, double e, double u, int2 cz,
-                                              int2 cw, int2 ce, int2 cd, int q) {
+template <bool INT = false>
+__device__ __forceinline__ double fx_residual(double b, double s, double n, double w, double e, double u, int2 cz, int2 cw,
+                                              int2 ce, int2 cd, int q) {
     const int ez = coef_exp(cz), es = exp_bits(s) - ez, en = exp_bits(n) - ez, eb = exp_bits(b) + q * (1 << 20);
     const int ew = exp_bits(w) - coef_exp(cw), ee = exp_bits(e) - coef_exp(ce), eu = exp_bits(u) - coef_exp(cd);
     const int em = max(max(max(es, en), max(ew, ee)), max(eu, eb));

@@ -81,10 +81,11 @@ template <class T> struct LevelDev {
     const T *cw, *ce, *cz;        // [nr]
     const T *invd, *diag;         // [ncls][nr][nm]: omega / diag, diag
     const T *hw, *he, *hz;        // [ncls][nr][nm] omega * off-diagonal conductances / diag
-    const int4 *hzw;              // FP64 levels without per-row tables, omega = 1: the h tables in limbs
-    const int2 *hev;              // (fixed.h), (hz, hw) and he, [ncls][nr][nm]; else null
+    const int4 *hzw;              // FP64 levels: the h tables in limbs (fixed.h), (hz, hw), [ncls][nr][nm]; null with
+    const int2 *hev;              // per-row tables of many classes.  he beside it without per-row tables; else null.
+                                  // (Made for any omega; the over-relaxed smoother does not read them)
     const int4 *rzw;              // FP64 levels without per-row tables: cz, cw [nr], ce [nr] and
-    const int2 *rev, *rdg;        // diag [ncls][nr][nm] times 2^rq in limbs; else null
+    const int2 *rev, *rdg;        // diag [ncls][nr][nm] times 2^rq in limbs; with per-row tables: hen, ren below
     int rq;
     const int4 *hen, *ren;        // FP64 levels with per-row tables of few classes: (he, hn) in limbs beside hzw, which
                                   // then holds (hz, hw), and (cce, ccn) beside rzw, (ccs, ccw), [ncls][nr]; else null
@@ -279,7 +280,7 @@ struct PsumTab {
 // The solve's kernels are launched so that a kernel's blocks may start while
 // the one before still runs (programmatic dependent launch): they read their
 // launch table and level view -- written at plan time -- and work out their
-// indices, then pdl_wait() blocks until the kernel before has completed and
+// indices; pdl_wait() then blocks until the kernel before has completed and
 // its writes are visible.  Nothing a kernel of the solve writes is read before
 // that.  pdl_go(), after the wait, lets the next kernel start likewise.  Most
 // kernels below level 0 run for 2 to 4 us, of which launch, table reads and

@@ -20,8 +20,9 @@
 //  * the smoother uses coefficients pre-divided by the diagonal and a
 //    right-hand side b_hat = b / diag, so one Gauss-Seidel update is
 //    u = b_hat + h_z (u_S + u_N) + h_w u_W + h_e u_E (4 FP64 ops per component);
-//  * on levels without per-row tables the imaginary part is computed in 64-bit
-//    fixed point by the integer pipes while the FP64 unit does the real part;
+//  * FP64 levels compute the imaginary part in 64-bit fixed point by the integer
+//    pipes while the FP64 unit does the real part (with per-row tables where their
+//    classes are few: composite domains, not stretched meshes);
 //  * after a black half-sweep the black cells satisfy their equations, so the
 //    residual (and the restricted right-hand side) only needs the red cells;
 //  * the red half-sweep that follows a prolongation overwrites the red cells

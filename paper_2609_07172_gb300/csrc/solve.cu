@@ -524,8 +524,8 @@ int enqueue_epilogue(Runner &R) {
     pic_poisson_plan_s &P = R.P;
     double x3 = 0;
     const double ff = fft_flops_all(P, &x3), n0 = level0_entries(P, 0);
-    // binary64 in both forms: an error in phi reaches the residual amplified by
-    // the operator (up to ~N^2 for its high frequencies), an error in b does not
+    // (the 64-bit transform in both forms: an error in phi reaches the residual amplified
+    // by the operator, up to ~N^2 for its high frequencies, an error in b does not)
     RUN(R, PIC_POISSON_PHASE_INVERSE, launch_inverse(P.inv, P.g_fft, P.smem_fft, R.st));
     R.account(PIC_POISSON_PHASE_INVERSE, x3 + n0 * sizeof(double2), ff);
     return PIC_POISSON_OK;
@@ -683,32 +683,32 @@ int capture_graph(pic_poisson_plan_s &P, int guess) {
         }
     }
     if (!P.h64.deep_solve) {   // (a solve in one launch loops by itself)
-    cudaGraphNodeParams cp{};
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = P.handle;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    cudaGraphNode_t cnode;
-    if (cudaGraphAddNode(&cnode, graph, deps, nullptr, ndeps, &cp) != cudaSuccess ||
-        cudaStreamUpdateCaptureDependencies(P.cap0, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies) !=
-            cudaSuccess) {
-        set_error("adding the while node failed");
-        return fail(PIC_POISSON_ECUDA);
-    }
-    cudaGraph_t body = cp.conditional.phGraph_out[0];
-    if (cudaStreamBeginCaptureToGraph(P.cap1, body, nullptr, nullptr, 0, mode) != cudaSuccess) {
-        set_error("capturing the loop body failed to start");
-        return fail(PIC_POISSON_ECUDA);
-    }
-    body_open = true;
-    Runner R1(P, P.cap1, false, true, P.seg[v][1]);
-    rc = enqueue_body(R1);
-    if (rc) return fail(rc);
-    body_open = false;
-    if (cudaStreamEndCapture(P.cap1, &body) != cudaSuccess) {
-        set_error("capturing the loop body failed");
-        return fail(PIC_POISSON_ECUDA);
-    }
+        cudaGraphNodeParams cp{};
+        cp.type = cudaGraphNodeTypeConditional;
+        cp.conditional.handle = P.handle;
+        cp.conditional.type = cudaGraphCondTypeWhile;
+        cp.conditional.size = 1;
+        cudaGraphNode_t cnode;
+        if (cudaGraphAddNode(&cnode, graph, deps, nullptr, ndeps, &cp) != cudaSuccess ||
+            cudaStreamUpdateCaptureDependencies(P.cap0, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies) !=
+                cudaSuccess) {
+            set_error("adding the while node failed");
+            return fail(PIC_POISSON_ECUDA);
+        }
+        cudaGraph_t body = cp.conditional.phGraph_out[0];
+        if (cudaStreamBeginCaptureToGraph(P.cap1, body, nullptr, nullptr, 0, mode) != cudaSuccess) {
+            set_error("capturing the loop body failed to start");
+            return fail(PIC_POISSON_ECUDA);
+        }
+        body_open = true;
+        Runner R1(P, P.cap1, false, true, P.seg[v][1]);
+        rc = enqueue_body(R1);
+        if (rc) return fail(rc);
+        body_open = false;
+        if (cudaStreamEndCapture(P.cap1, &body) != cudaSuccess) {
+            set_error("capturing the loop body failed");
+            return fail(PIC_POISSON_ECUDA);
+        }
     }
     Runner R2(P, P.cap0, false, false, P.seg[v][2]);
     rc = enqueue_epilogue(R2);
