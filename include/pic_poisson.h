@@ -121,7 +121,12 @@ typedef struct {
                                   half-sweeps */
     int local_bottom;          /* 0: the lower levels -- at least the level above the coarsest and the
                                   coarsest solve, of small problems all of them -- run per mode in shared
-                                  memory where they fit (omega = 1); -1: never (separate launches) */
+                                  memory where they fit (omega = 1); -1: never (separate launches).  A
+                                  small FP64 problem (up to some 500 thousand cells x modes) is then
+                                  solved by one cooperative launch of up to a block per SM with up to
+                                  225 KB of shared memory each, which starts when all of these SMs are
+                                  free: beside a kernel that keeps SMs until this solve has ended (one
+                                  that waits for it on another stream) use -1 */
     int fmg;                   /* FP64: 1 starts a solve with a full-multigrid pass: from a zero iterate,
                                   the right-hand side restricted to every level, coarsest solve, then
                                   prolongation and one V-cycle per level up to the finest; from a given
