@@ -264,7 +264,7 @@ struct Ctrl {
 // block) adds a few dozen numbers instead of tens of thousands -- on one SM
 // the FP64 additions alone took longer than the rest of the test.
 constexpr int PSUM_CHUNK = 2048;
-// Up to PSUM_MIN partials the test adds them itself, which saves the launch of k_psum.  Solves
+// Up to PSUM_MIN partials the test adds them itself, which saves the launch of k_psum (a batch: plan.cu).  Solves
 // without that launch over solves with it, by partials: FP64 1,000 0.984, 2,100 0.988, 4,200
 // 0.993, 6,200 0.999, 8,300 1.000; mixed 1,600 0.965, 4,200 0.991, 8,300 0.990, 10,400 0.995,
 // 12,500 1.000, 16,600 1.003, 25,000 1.009.

@@ -1474,10 +1474,13 @@ int upload(pic_poisson_plan_s &P) {
     // partials themselves
     PsumTab ps{};
     ps.n = P.n;
-    unsigned total = 0;
-    for (int p = 0; p < P.n; ++p) total += C.rend[p] - C.rbegin[p];
+    // (the test gives each problem of a batch its share of 32 warps, one at least, and
+    // takes 32 problems at a time: what counts is the longest sum by that share)
+    size_t longest = 0;
+    for (int p = 0; p < P.n; ++p) longest = std::max<size_t>(longest, C.rend[p] - C.rbegin[p]);
+    const int share = std::max(32 / P.n, 1), rounds = (P.n + 31) / 32;
     P.g_psum = 0;
-    if (total > PSUM_MIN) {
+    if (longest * (32 / share) * rounds > PSUM_MIN) {
         for (int p = 0; p < P.n; ++p) {
             const unsigned len = C.rend[p] - C.rbegin[p];
             const unsigned chunks = std::max(1u, (len + PSUM_CHUNK - 1) / PSUM_CHUNK);
