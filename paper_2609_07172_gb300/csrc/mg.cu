@@ -101,10 +101,31 @@ template <class T> __device__ __forceinline__ void stage_view(LevelDev<T> *dst, 
         reinterpret_cast<unsigned long long *>(dst)[w] = reinterpret_cast<const unsigned long long *>(src)[w];
 }
 
-// b - A_m u at entry (k, i, m), Eq. matrix_free_mode_operator.  FX: binary64
-// levels with limb tables compute the imaginary part in fixed point, which takes
-// values of 2^-863 to 2^977 (the norms of a solve hold less); else both parts in T.
-template <class T, bool MASK, bool FX, bool INT = false>
+// f(b, s, n, w, e, u), a fixed-point sum of products, over the whole range of binary64
+// (fx_ends cuts it to 2^-863 .. 2^977): operands beyond 2^877 or all below 2^-623 are
+// scaled by a power of two first -- the same bits --, and one that is not finite gives
+// NaN whatever its coefficient.
+template <class F>
+__device__ __forceinline__ double fx_whole_range(F f, double b, double s, double n, double w, double e, double u) {
+    const int r = max(max(max(exp_bits(b), exp_bits(s)), max(exp_bits(n), exp_bits(w))), max(exp_bits(e), exp_bits(u)));
+    double y = f(b, s, n, w, e, u);
+    if (r >= (1900 << 20) || r < (400 << 20)) {
+        const auto bits = [](double x) { return (ufx)__double_as_longlong(x); };
+        if (r == (2047 << 20)) {
+            y = __longlong_as_double(0x7ff8000000000000ll);
+        } else if ((bits(b) | bits(s) | bits(n) | bits(w) | bits(e) | bits(u)) << 1) {
+            const bool big = r >= (1900 << 20);
+            const double up = big ? 0x1p-300 : 0x1p400, down = big ? 0x1p300 : 0x1p-400;
+            y = f(b * up, s * up, n * up, w * up, e * up, u * up) * down;
+        }
+    }
+    return y;
+}
+
+// b - A_m u at entry (k, i, m), Eq. matrix_free_mode_operator.  Binary64 levels with
+// limb tables compute the imaginary part in fixed point, which takes values of 2^-863
+// to 2^977 (the norms of a solve hold less); WHOLE: of binary64's whole range.
+template <class T, bool MASK, bool WHOLE, bool INT = false>
 __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i, int m, size_t idx) {
     const size_t rowstride = (size_t)L.nr * L.nm;
     if (MASK && L.rcls) {
@@ -116,15 +137,20 @@ __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i,
         // a cell outside a composite domain's patches (zero diagonal) has no
         // residual: nothing else is loaded for it
         if (d == T(0)) return mk<T>(0, 0);
-        if constexpr (FX && sizeof(T) == sizeof(double)) {
+        if constexpr (sizeof(T) == sizeof(double)) {
             if (L.ren) {   // real part on the FP64 unit, imaginary part in fixed point
                 const V2<T> zero = mk<T>(0, 0), *u = L.u + idx;
                 const V2<T> us = k > 0 ? *(u - rowstride) : zero, un = k < L.nz - 1 ? u[rowstride] : zero;
                 const V2<T> uw = i > 0 ? *(u - L.nm) : zero, ue = i < L.nr - 1 ? u[L.nm] : zero, uc = *u, b = L.b[idx];
                 T x = fma(L.ccn[ci], un.x, fma(L.ccs[ci], us.x, b.x));
                 x = fma(L.cce[ci], ue.x, fma(L.ccw[ci], uw.x, x));
-                return mk<T>(fma(-d, uc.x, x), fx_residual(b.y, us.y, uw.y, ue.y, un.y, uc.y, L.rzw[ci], L.ren[ci],
-                                                           L.rdg[ci * L.nm + m], L.rq));
+                const int4 sw = L.rzw[ci], en = L.ren[ci];
+                const int2 dg = L.rdg[ci * L.nm + m];
+                const auto f = [&](double b, double s, double n, double w, double e, double u) {
+                    return fx_residual(b, s, w, e, n, u, sw, en, dg, L.rq);
+                };
+                return mk<T>(fma(-d, uc.x, x), WHOLE ? fx_whole_range(f, b.y, us.y, un.y, uw.y, ue.y, uc.y)
+                                                     : f(b.y, us.y, un.y, uw.y, ue.y, uc.y));
             }
         }
         V2<T> acc = L.b[idx];
@@ -134,7 +160,7 @@ __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i,
         if (i < L.nr - 1) acc = fma2<T>(L.cce[ci], L.u[idx + L.nm], acc);
         return fma2<T>(-d, L.u[idx], acc);
     }
-    if constexpr (FX && sizeof(T) == sizeof(double)) {
+    if constexpr (sizeof(T) == sizeof(double)) {
         if (L.rzw) {   // real part on the FP64 unit, imaginary part in fixed point (fixed.h)
             const unsigned rs = (unsigned)L.nr * (unsigned)L.nm;
             const V2<T> zero = mk<T>(0, 0), *u = L.u + idx;
@@ -143,9 +169,12 @@ __device__ __forceinline__ V2<T> residual_at(const LevelDev<T> &L, int k, int i,
             const unsigned tb = (unsigned)row_class(k, L.nz, L.ncls) * rs + (unsigned)i * (unsigned)L.nm + (unsigned)m;
             const int4 zw = L.rzw[i];
             const int2 ev = L.rev[i], dg = L.rdg[tb];
+            const auto f = [&](double b, double s, double n, double w, double e, double u) {
+                return fx_residual<INT>(b, s, n, w, e, u, make_int2(zw.x, zw.y), make_int2(zw.z, zw.w), ev, dg, L.rq);
+            };
             return mk<T>(fma(-L.diag[tb], uc.x, fma(L.ce[i], ue.x, fma(L.cw[i], uw.x, fma(L.cz[i], us.x + un.x, b.x)))),
-                         fx_residual<INT>(b.y, us.y, un.y, uw.y, ue.y, uc.y, make_int2(zw.x, zw.y), make_int2(zw.z, zw.w),
-                                     ev, dg, L.rq));
+                         WHOLE ? fx_whole_range(f, b.y, us.y, un.y, uw.y, ue.y, uc.y)
+                               : f(b.y, us.y, un.y, uw.y, ue.y, uc.y));
         }
     }
     V2<T> s = mk<T>(0, 0);
@@ -459,11 +488,11 @@ __device__ __forceinline__ double restrict_body(const LevelDev<T> &F, const Leve
         };
         int k, i;
         cell(0, k, i);
-        V2<T> sum = residual_at<T, MASK, true, true>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
+        V2<T> sum = residual_at<T, MASK, false, true>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
         if (partials) acc = fma((double)sum.y, (double)sum.y, (double)sum.x * (double)sum.x);
         auto more = [&](int c) {
             cell(c, k, i);
-            const V2<T> r = residual_at<T, MASK, true, true>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
+            const V2<T> r = residual_at<T, MASK, false, true>(F, k, i, m, ((size_t)k * F.nr + i) * nm + m);
             sum = mk<T>(sum.x + r.x, sum.y + r.y);
             if (partials) acc = fma((double)r.y, (double)r.y, fma((double)r.x, (double)r.x, acc));
         };
@@ -520,7 +549,7 @@ k_residual_restrict(const __grid_constant__ LevelArg<T> arg, double *__restrict_
 
 // r = b - A_m u on level f (r written to c.u when write_r), Parseval-weighted
 // squared norms of r into partials[block] and, when stride > 0, of b into
-// partials[stride + block].  The stage call's kernel: both parts in T, over its whole range.
+// partials[stride + block].  The stage call's kernel: over binary64's whole range.
 template <class T, bool MASK>
 __global__ void __launch_bounds__(MG_THREADS)
 k_residual(const LaunchTab<T> *__restrict__ tab, int write_r, double *__restrict__ partials, unsigned stride) {
@@ -536,7 +565,7 @@ k_residual(const LaunchTab<T> *__restrict__ tab, int write_r, double *__restrict
         const int m = (int)(e - c * nm);
         const int k = (int)fdiv(c, (unsigned)L.nr, L.rnr);
         const int i = (int)(c - (unsigned)k * L.nr);
-        const V2<T> r = residual_at<T, MASK, false>(L, k, i, m, e);
+        const V2<T> r = residual_at<T, MASK, true>(L, k, i, m, e);
         if (write_r) tab->c[p].u[e] = r;
         const V2<T> b = L.b[e];
         const double w = parseval_w(m, L.nt);
@@ -746,7 +775,7 @@ k_defect(const DefectTab *__restrict__ tab, const Ctrl *__restrict__ ctrl, doubl
             r = D.b[e];
             D.u[e] = make_double2(0.0, 0.0);
         } else {
-            r = residual_at<double, MASK, true>(D, k, i, m, e);
+            r = residual_at<double, MASK, false>(D, k, i, m, e);
         }
         const float2 b32 = make_float2(f64_to_f32_pow2(r.x, ls), f64_to_f32_pow2(r.y, ls));
         const float w = (m == 0 || 2 * m == D.nt) ? 1.f : 2.f;
