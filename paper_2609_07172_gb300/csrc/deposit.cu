@@ -33,7 +33,7 @@
 // the binary64 arithmetic, which alone decides those cases, and one whose
 // coordinate has bits below the fixed point's, close to the lower wall, takes that too.
 // 210 M cell-sorted particles of two species, 4 per cell and species, at
-// 512 x 128 x 400: 11.6 ms with double-float, now 2.55 (integer instructions and their
+// 512 x 128 x 400: 11.6 ms with double-float, now 2.5 (integer instructions and their
 // issue, both two thirds busy).  In units of 2^-54 without the second way it was 2.3, but
 // a weight of 1e-12 kept four digits; 96-bit products hold every weight without it and
 // took 3.1.  Against a quadruple-precision deposit of 1.6 M particles the nodes are
@@ -155,7 +155,7 @@ __device__ __forceinline__ bool fix_place(const FixAxis &a, double x, int &cell,
     const u64 D = X - (u64)a.base, d = D << a.sh;
     const u64 t = __umul64hi(d, a.K);
     cell = (int)(t >> a.F);
-    f = t << (64 - a.F) | (d * a.K) >> a.F;
+    f = t << (64 - a.F) | (unsigned)((d * a.K) >> 32) >> (a.F - 32);   // (the low word's upper half: F >= 32, n < 2^30)
     return s >= 1 && D < a.span && (s <= a.smax || D >= DEP_NEAR) && (unsigned)(f >> 32) + 0x100u >= 0x200u;
 }
 
@@ -446,7 +446,7 @@ FixAxis fix_axis(double lo, double hi, int n) {
     a.F = 61 - b;                                          // n 2^F in [2^61, 2^62)
     const u64 num = (u64)n << a.F, den = a.span << a.sh;   // K = floor(num 2^64 / den), num < den
     a.K = den ? (u64)(((unsigned __int128)num << 64) / den) : 0;
-    if (a.span == 0 || num >= den) a.span = 0;             // degenerate: every particle takes the binary64 arithmetic
+    if (num >= den || a.F < 32) a.span = 0;                // degenerate: every particle takes the binary64 arithmetic
     return a;
 }
 
