@@ -38,9 +38,9 @@
 // that 256 points need 68 KB of shared memory and not 133, three blocks per SM
 // instead of one: 128 x 256 x 96 forward 81 -> 52 us, and a batch's largest problem
 // no longer costs the others their room.
-// 512 x 128 x 400: forward 586 -> 312 us (with b_hat and the norm, in a solve,
-// 653 -> 330), inverse 496 -> 272 us; both now bound by integer instructions
-// and their latency (ALU pipe 44 to 48 %, three CTAs per SM).
+// 512 x 128 x 400: forward 586 -> 306 us (with b_hat and the norm, in a solve,
+// 653 -> 346), inverse 496 -> 274 us; both now bound by integer instructions
+// and their latency (ALU pipe 47 to 52 %, three CTAs per SM).
 #include "fixed.h"
 #include "internal.h"
 
